@@ -192,7 +192,7 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         ea.uni_scale = h->uni_scale;
         ea.species_slot = h->d_species + d.T; ea.n_present = (int)h->present.size();
         ea.frames = nb.batch ? nb.frames : nullptr; ea.frame_of = nb.frame_of;
-        ea.row_ptr = nb.row_ptr; ea.src = nb.src; ea.shift = nb.shift;
+        ea.row_ptr = nb.row_ptr; ea.nbr = nb.nbr;
         ea.Lx = nb.L[0]; ea.Ly = nb.L[1]; ea.Lz = nb.L[2];
         for (int k = 0; k < 9; ++k) ea.H[k] = nb.H[k];
         ea.tri = nb.tri;
@@ -360,10 +360,10 @@ int ensure_device_model(umlmd_t* h) {
 }
 
 int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type, const double cell[9],
-               const int pbc[3], double skin) {
+               const int pbc[3], double skin, const BuildFetch* fetch) {
     int rc = ensure_device_model(h);
     if (rc != UMLMD_OK) return rc;
-    { Scope sc(h, kNeighbor, 7); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, h->st, &h->err); }
+    { Scope sc(h, kNeighbor, 5 + (fetch && N > 0)); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, fetch, h->st, &h->err); }
     if (rc != UMLMD_OK) { h->have_list = false; return rc; }
     h->have_list = true;
     h->have_edge_grad = false;       // edges were renumbered
@@ -378,6 +378,17 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
         if (h->nb.E > h->nb.E_owned)
             API_CUDA(h, cudaMemsetAsync(h->g + 3 * (size_t)h->nb.E_owned, 0, sizeof(float) * 3 * (size_t)(h->nb.E - h->nb.E_owned), h->st));
     }
+    return UMLMD_OK;
+}
+
+int ensure_species_buffers(umlmd_t* h) {
+    int rc = ensure_device_model(h);
+    if (rc != UMLMD_OK || h->d_species) return rc;
+    const size_t T = (size_t)h->d.T;
+    void* p = nullptr;
+    API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * T));
+    h->d_species = (int*)p;
+    API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * T));
     return UMLMD_OK;
 }
 
@@ -501,26 +512,18 @@ int umlmd_build_neighbors(umlmd_t* h, int64_t N, const double* d_pos, const int3
         for (int i = 0; i < 3; ++i)
             if (!(cell[4 * i] > 0.0)) return fail(h, UMLMD_E_UNSUPPORTED_CELL, "cell edges must be positive");
     h->have_md = false;
-    int rc = build_list(h, N, d_pos, d_type, cell, pbc, skin);
+    // which species occur: few enough of them get per-pair amplitude tables (see below); comes back with
+    // the edge count, and with what the device found wrong (non-finite positions, image range, species)
+    int rc = ensure_species_buffers(h);
     if (rc != UMLMD_OK) return rc;
-    if (N > 0) API_CUDA(h, cudaMemcpyAsync(h->type_o, d_type, sizeof(int) * N, cudaMemcpyDeviceToDevice, h->st));
-    // which species occur: few enough of them get per-pair amplitude tables (see below)
-    const int T = h->d.T;
-    if (!h->d_species) {
-        void* p = nullptr;
-        API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * (size_t)T));
-        h->d_species = (int*)p;
-        API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * (size_t)T));
-    }
-    API_CUDA(h, launch_species_present(N, d_type, T, h->d_species, h->d_err, h->st));
-    h->launches_total += N > 0;
-    API_CUDA(h, cudaMemcpyAsync(h->h_species, h->d_species, sizeof(int) * (size_t)T, cudaMemcpyDeviceToHost, h->st));
-    // surface device-side findings of the build (non-finite positions, image range)
-    API_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-    API_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
-    API_CUDA(h, cudaStreamSynchronize(h->st));
+    *h->h_err = 0;
+    for (int t = 0; t < h->d.T; ++t) h->h_species[t] = 0;
+    const BuildFetch fetch = {h->d.T, h->d_species, h->h_species, h->h_err};
+    rc = build_list(h, N, d_pos, d_type, cell, pbc, skin, &fetch);
+    if (rc != UMLMD_OK) return rc;
     rc = decode_device_errors(h, *h->h_err);
     if (rc != UMLMD_OK) { h->have_list = false; return rc; }
+    if (N > 0) API_CUDA(h, cudaMemcpyAsync(h->type_o, d_type, sizeof(int) * N, cudaMemcpyDeviceToDevice, h->st));
     return setup_pair_tables(h);
 }
 
@@ -579,7 +582,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t A = N + 1;
     t += buf(3 * A, 8) * 3 + buf(6 * A, 4) + buf(A, 4) * 2 + buf(A + 1, 8) + buf(A, 4) * 4 + buf(A + 1, 4);
     t += buf(8 * N + 64 + 2, 4);
-    t += grown(n_edges, 4) * 2 + grown(n_edges, 8);
+    t += grown(n_edges, 8) * 2;
     t += 16 * A + (2 << 20);
     // evaluation workspace of one node tile, per-edge gradients, per-atom results, MD forces
     const int64_t Bt = N < h->node_tile ? N : h->node_tile;
@@ -659,29 +662,17 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
     const int64_t N = frame_offsets[n_frames];
     if (N > 0x7fff0000LL) return fail(h, UMLMD_E_INVALID_ARG, "too many atoms for 32-bit indices");
     if (N > 0 && (!d_pos || !d_type)) return fail(h, UMLMD_E_INVALID_ARG, "null positions or species");
-    int rc = ensure_device_model(h);
+    int rc = ensure_species_buffers(h);
     if (rc != UMLMD_OK) return rc;
     h->have_list = false; h->have_md = false; h->have_edge_grad = false;     // the handle's list is replaced
     ++h->list_serial;
-    { Scope sc(h, kNeighbor, 5); rc = neighbor_build_batch(&h->nb, n_frames, frame_offsets, cells, pbc, d_pos, d_type, h->d.T, h->hm.rc, h->d_err, h->st, &h->err); }
+    const BuildFetch fetch = {h->d.T, h->d_species, h->h_species, h->h_err};
+    { Scope sc(h, kNeighbor, 5); rc = neighbor_build_batch(&h->nb, n_frames, frame_offsets, cells, pbc, d_pos, d_type, h->d.T, h->hm.rc, h->d_err, &fetch, h->st, &h->err); }
     if (rc != UMLMD_OK) return rc;
     const bool want_grad = d_force != nullptr || virials != nullptr;
     if (N > 0) {
-        if ((rc = ensure_workspace(h)) != UMLMD_OK) return rc;
-        const int T = h->d.T;
-        if (!h->d_species) {
-            void* p = nullptr;
-            API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * (size_t)T));
-            h->d_species = (int*)p;
-            API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * (size_t)T));
-        }
-        API_CUDA(h, launch_species_present(N, h->nb.type_s, T, h->d_species, h->d_err, h->st));
-        h->launches_total += 1;
-        API_CUDA(h, cudaMemcpyAsync(h->h_species, h->d_species, sizeof(int) * (size_t)T, cudaMemcpyDeviceToHost, h->st));
-        API_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-        API_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
-        API_CUDA(h, cudaStreamSynchronize(h->st));
         if ((rc = decode_device_errors(h, *h->h_err)) != UMLMD_OK) return rc;
+        if ((rc = ensure_workspace(h)) != UMLMD_OK) return rc;
         if ((rc = setup_pair_tables(h)) != UMLMD_OK) return rc;
         if ((rc = enqueue_compute(h, d_pos, want_grad, d_force, d_atom_energy)) != UMLMD_OK) return rc;
     }
@@ -755,7 +746,7 @@ static int maybe_rebuild(umlmd_t* h, int rebuild_every) {
         // to look at what the steps since the previous build reported: a list that went stale, or a
         // non-finite value, ends the run here instead of after the last step.
         API_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-        int rc = build_list(h, N, h->md_pos, h->type_o, cell, pbc, skin);
+        int rc = build_list(h, N, h->md_pos, h->type_o, cell, pbc, skin, nullptr);
         if (rc != UMLMD_OK) return rc;
         const int word = *h->h_err;                  // the build has synchronised the stream since the copy
         if (word) {

@@ -54,8 +54,8 @@ __global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const ei
 // -1/2 sum_{e in row(i)} (g_e - g_rev(e)) (x) r_e (the reverse edge has the opposite vector).
 // Edge vectors are recomputed in double from the positions of the last evaluation.
 struct CellRowsA { double h[9]; };
-__global__ void k_atom_virial(int N, const eidx_t* __restrict__ row_ptr, const int* __restrict__ src,
-                              const int* __restrict__ shift, const eidx_t* __restrict__ rev,
+__global__ void k_atom_virial(int N, const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
+                              const eidx_t* __restrict__ rev,
                               const float* __restrict__ g, const double* __restrict__ xs, CellRowsA H,
                               const int* __restrict__ perm, double* __restrict__ out) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -72,7 +72,7 @@ __global__ void k_atom_virial(int N, const eidx_t* __restrict__ row_ptr, const i
         double d[3] = {(double)a[0], (double)a[1], (double)a[2]};
         const eidx_t r = rev[e];
         if (r >= 0) { const float* b = g + 3 * (size_t)r; d[0] -= (double)b[0]; d[1] -= (double)b[1]; d[2] -= (double)b[2]; }
-        const int j = src[e], s = shift[e];
+        const int j = nbr[e].x, s = nbr[e].y;
         const double nx = (double)(signed char)(s & 0xff), ny = (double)(signed char)((s >> 8) & 0xff),
                      nz = (double)(signed char)((s >> 16) & 0xff);
         const double* xj = xs + 3 * (size_t)j;
@@ -151,8 +151,8 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // when asked, -g (x) r over the edges of the frame's rows (edge vectors recomputed from the
 // positions and the frame's cell); thread-strided partial sums, then one fixed-order block sum.
 __global__ void __launch_bounds__(kRedBlock) k_frame_reduce(const FrameCell* __restrict__ frames, const double* __restrict__ e_atom,
-                                                            const eidx_t* __restrict__ row_ptr, const int* __restrict__ src,
-                                                            const int* __restrict__ shift, const float* __restrict__ g,
+                                                            const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
+                                                            const float* __restrict__ g,
                                                             const double* __restrict__ xs, bool want_virial,
                                                             double* __restrict__ out) {
     __shared__ double sh[kRedBlock / 32];
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kRedBlock) k_frame_reduce(const FrameCell* __r
         if (!want_virial) continue;
         const double xi = xs[3 * (size_t)i], yi = xs[3 * (size_t)i + 1], zi = xs[3 * (size_t)i + 2];
         for (eidx_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-            const int j = src[k], s = shift[k];
+            const int j = nbr[k].x, s = nbr[k].y;
             const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff), nz = (int)(signed char)((s >> 16) & 0xff);
             const double r[3] = {(xs[3 * (size_t)j] + ((nx * fc.H[0] + ny * fc.H[3]) + nz * fc.H[6])) - xi,
                                  (xs[3 * (size_t)j + 1] + ((nx * fc.H[1] + ny * fc.H[4]) + nz * fc.H[7])) - yi,
@@ -321,7 +321,7 @@ cudaError_t launch_atom_virial(const NeighborDev& nb, const float* g, double* d_
     if (N == 0) return cudaSuccess;
     CellRowsA H;
     for (int k = 0; k < 9; ++k) H.h[k] = nb.H[k];
-    k_atom_virial<<<(N + 7) / 8, 256, 0, st>>>(N, nb.row_ptr, nb.src, nb.shift, nb.rev, g, nb.xs, H, nb.perm, d_out);
+    k_atom_virial<<<(N + 7) / 8, 256, 0, st>>>(N, nb.row_ptr, nb.nbr, nb.rev, g, nb.xs, H, nb.perm, d_out);
     return cudaGetLastError();
 }
 
@@ -343,7 +343,7 @@ cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_so
 cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
                                 double* d_out, cudaStream_t st) {
     if (nb.n_frames <= 0) return cudaSuccess;
-    k_frame_reduce<<<nb.n_frames, kRedBlock, 0, st>>>(nb.frames, e_atom, nb.row_ptr, nb.src, nb.shift, g, nb.xs, want_virial, d_out);
+    k_frame_reduce<<<nb.n_frames, kRedBlock, 0, st>>>(nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial, d_out);
     return cudaGetLastError();
 }
 

@@ -118,6 +118,8 @@ __host__ __device__ inline void tab_unpack(unsigned w, float k2, float k3, float
 struct FrameCell {
     double H[9];      // cell vectors as rows
     double Hinv[9];   // inverse (fractional coordinates f = r Hinv)
+    double reach[3];  // cutoff in fractional coordinates along each cell vector, rounded up
+    float near_tol;   // band around the squared cutoff inside which the scan decides in double precision
     int m[3];         // periodic images to visit along each cell vector (0 for an open direction)
     int pbc[3];
     int a0, a1;       // atoms [a0, a1) of the concatenated arrays
@@ -143,8 +145,7 @@ struct NeighborDev {
     // (x_hi, y_hi, z_hi, species bits), (x_lo, y_lo, z_lo, 0) with x = (double)x_hi + (double)x_lo
     float4* rec = nullptr;
     eidx_t* row_ptr = nullptr;   // [N+1]
-    int* src = nullptr;          // [E] sorted index of the neighbour
-    int* shift = nullptr;        // [E] packed int8 x3 image n
+    int2* nbr = nullptr;         // [E] x: sorted index of the neighbour, y: its image n, packed int8 x3
     eidx_t* rev = nullptr;       // [E] index of the reverse edge, -1 if absent
     // batched evaluation: per-frame cells and the frame of every atom (null for a single system)
     FrameCell* frames = nullptr; int64_t frames_cap = 0; int n_frames = 0;
@@ -154,6 +155,7 @@ struct NeighborDev {
     int* key = nullptr; int* key2 = nullptr; int* idx = nullptr; int* idx2 = nullptr;
     int* cell_start = nullptr; int64_t ncell_cap = 0;
     int* deg = nullptr;
+    eidx_t* h_totals = nullptr;  // pinned [2]: edges in all, edges of owned atoms
     void* cub_tmp = nullptr; size_t cub_bytes = 0;
 };
 

@@ -46,8 +46,8 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     g.dx = g.dy = g.dz = 0.f; g.rho = 1.f; g.inv_rho = 1.f; g.ux = g.uy = g.uz = 0.f;
     g.chi = 0.f; g.dchi = 0.f; g.t = 0.f; g.row = 0; g.pair = 0;
     if (!in_range) return g;
-    const int j = a.src[e];
-    const int s = a.shift[e];
+    const int2 js = __ldg(a.nbr + e);
+    const int j = js.x, s = js.y;
     const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff),
               nz = (int)(signed char)((s >> 16) & 0xff);
     // the neighbour's record: position as float pairs (exact to 2^-48 of the coordinate) and species

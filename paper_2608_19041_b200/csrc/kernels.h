@@ -8,6 +8,10 @@
 namespace umd {
 
 // ---- neighbor.cu ---------------------------------------------------------------------
+// What a build brings back to the host with the edge count, in its one synchronisation: which of the
+// T species occur, and the device error word, which is cleared (an image index out of range, a
+// non-finite position or a bad species are all found before that point).
+struct BuildFetch { int T; int* d_flags; int* h_flags; int* h_err; };
 // Full build: fold + bin + sort + count + scan + fill + reverse map.  Synchronises once
 // (to learn the edge count and grow the edge arrays).  Returns a UMLMD_* code.
 // n_owned < N: the atoms with caller index >= n_owned are ghosts; they come after all owned atoms
@@ -15,7 +19,7 @@ namespace umd {
 // [0, n_owned) are the owned atoms' and nb->E_owned edges belong to them.
 int neighbor_build(NeighborDev* nb, int64_t N, int64_t n_owned, const double* d_pos, const int32_t* d_type,
                    const double cell[9], const int pbc[3], double skin, double rc, int* d_err,
-                   cudaStream_t st, std::string* err);   // cell: the three cell vectors as rows
+                   const BuildFetch* fetch, cudaStream_t st, std::string* err);   // cell: the three cell vectors as rows
 void neighbor_free(NeighborDev* nb);
 // Export the list in caller numbering (device buffers of the caller).
 int neighbor_export(NeighborDev* nb, int32_t* d_row_ptr, int32_t* d_src, int8_t* d_shift,
@@ -24,8 +28,8 @@ int neighbor_export(NeighborDev* nb, int32_t* d_row_ptr, int32_t* d_src, int8_t*
 // offsets[f] .. offsets[f+1]-1 with cell cells[9 f ..]), list radius rc, by exhaustive search inside
 // each frame (meant for many small frames); atoms keep the caller's order.  Returns a UMLMD_* code.
 int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, const double* cells, const int pbc[3],
-                         const double* d_pos, const int32_t* d_type, int T, double rc, int* d_err, cudaStream_t st,
-                         std::string* err);
+                         const double* d_pos, const int32_t* d_type, int T, double rc, int* d_err, const BuildFetch* fetch,
+                         cudaStream_t st, std::string* err);
 // per-frame energy and virial: out[10 f] = sum of e_atom over the frame, out[10 f + 1 ..] = -sum over
 // the frame's edges of g (x) r, each by one block in a fixed order
 cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
@@ -47,8 +51,7 @@ struct EdgeArgs {
     const float4* rec;      // [N][2] positions (as float pairs) and species, one record per atom
     const int* type_s;
     const eidx_t* row_ptr;
-    const int* src;
-    const int* shift;
+    const int2* nbr;        // [E] neighbour (sorted index) and its image
     double Lx, Ly, Lz;
     double H[9];            // cell vectors as rows, used instead of Lx, Ly, Lz when tri
     int tri;

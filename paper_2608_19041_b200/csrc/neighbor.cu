@@ -2,14 +2,17 @@
 //
 // Atoms are folded into the cell, binned into cells at least r_list wide, sorted by cell
 // (stable radix sort, so the internal numbering is deterministic) and renumbered in that
-// order.  One warp per centre then walks the surrounding cells twice -- a count pass and a
-// fill pass with an in-warp prefix count that keeps candidates in traversal order -- so the
-// edge list comes out grouped by destination with no atomics and a reproducible order.
-// A last pass finds, for every edge (i <- j, n), the slot of its reverse (j <- i, -n).
+// order.  A warp takes a few centres of one cell and walks the surrounding cells twice -- a
+// count pass and a fill pass with an in-warp prefix count that keeps candidates in traversal
+// order -- so the edge list comes out grouped by destination with no atomics and a
+// reproducible order.  A last pass finds, for every edge (i <- j, n), the slot of its reverse
+// (j <- i, -n).
 //
 // The distance predicate is the paper's neighbor-set definition evaluated in double
 // precision with explicit round-to-nearest adds and multiplies (no contraction into fused
-// multiply-adds), which makes the edge set reproducible bit for bit.
+// multiply-adds), which makes the edge set reproducible bit for bit.  The scans decide in
+// single precision every candidate whose distance is further from the list radius than single
+// precision can be wrong (Near), and evaluate that predicate for the others.
 #include <cub/cub.cuh>
 #include <thrust/iterator/transform_iterator.h>
 
@@ -159,130 +162,271 @@ __global__ void k_fold_bin(int N, const double* __restrict__ pos, Grid g, double
     idx[i] = i;
 }
 
-__global__ void k_cell_start(int ncell, int N, const int* __restrict__ skey, int* __restrict__ cell_start) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c > ncell) return;
-    int lo = 0, hi = N;
-    while (lo < hi) {
-        const int mid = lo + ((hi - lo) >> 1);     // lo + hi would pass 2^31 in a long list
-        if (skey[mid] < c) lo = mid + 1; else hi = mid;
-    }
-    cell_start[c] = lo;
-}
-
-__global__ void k_gather_sorted(int N, const int* __restrict__ sidx, const double* __restrict__ wpos,
-                                const int* __restrict__ img_o, const int* __restrict__ type,
+// gather the per-atom arrays into sorted order; where the sorted key rises from one atom to the next,
+// the cells in between start at the latter (a gap of more than four cells is filled by the whole warp)
+__global__ void k_gather_sorted(int N, int nkeys, const int* __restrict__ skey, const int* __restrict__ sidx,
+                                const double* __restrict__ wpos, const int* __restrict__ img_o, const int* __restrict__ type,
                                 int* __restrict__ perm, double* __restrict__ xs0, double* __restrict__ xs,
-                                int* __restrict__ img, int* __restrict__ type_s) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+                                float4* __restrict__ rec, int* __restrict__ img, int* __restrict__ type_s,
+                                int* __restrict__ cell_start) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    int lo = 0, n = 0;                           // this atom's gap: cells lo .. lo + n - 1 start at atom i
+    if (i <= N) {
+        lo = i > 0 ? skey[i - 1] + 1 : 0;
+        n = (i < N ? skey[i] : nkeys) - lo + 1;
+    }
+    if (n <= 4) for (int c = 0; c < n; ++c) cell_start[lo + c] = i;
+    unsigned wide = __ballot_sync(0xffffffffu, n > 4);
+    while (wide) {
+        const int l = __ffs(wide) - 1;
+        wide &= wide - 1;
+        const int lo_l = __shfl_sync(0xffffffffu, lo, l), n_l = __shfl_sync(0xffffffffu, n, l), i_l = i - lane + l;
+        for (int c = lane; c < n_l; c += 32) cell_start[lo_l + c] = i_l;
+    }
     if (i >= N) return;
     const int o = sidx[i];
     perm[i] = o;
     type_s[i] = type[o];
+    float hi[3];
     for (int k = 0; k < 3; ++k) {
         const double w = wpos[3 * (size_t)o + k];
         xs0[3 * (size_t)i + k] = w;
         xs[3 * (size_t)i + k] = w;
         img[3 * (size_t)i + k] = img_o[3 * (size_t)o + k];
+        hi[k] = (float)w;
     }
+    rec[2 * (size_t)i] = make_float4(hi[0], hi[1], hi[2], 0.f);   // what the scans read; the evaluation rewrites the records
 }
 
-// One warp per centre.  FILL = false: count accepted candidates.  FILL = true: write them.
-template <bool FILL>
-__global__ void k_scan_cells(int N, Grid g, double rl2, const int* __restrict__ skey,
-                             const int* __restrict__ cell_start, const double* __restrict__ xs0,
-                             int* __restrict__ deg, const eidx_t* __restrict__ row_ptr,
-                             int* __restrict__ src, int* __restrict__ shift, int* __restrict__ err) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= N) return;
-    const int i = warp;
-    int key = skey[i];
-    if (key >= g.ncell) key -= g.ncell;         // a ghost's own bin
-    const int cx = key % g.nc[0], cy = (key / g.nc[0]) % g.nc[1], cz = key / (g.nc[0] * g.nc[1]);
-    const double xi = xs0[3 * (size_t)i], yi = xs0[3 * (size_t)i + 1], zi = xs0[3 * (size_t)i + 2];
-    int count = 0;
-    const eidx_t base_out = FILL ? row_ptr[i] : 0;
+// Squared list radius, its single-precision value, and a band around that outside of which a squared
+// distance computed in single precision from rounded coordinates falls on the right side of it.
+struct Near { double rl2; float mid, tol; };
+
+// X bounds the magnitude of the coordinates.  With u = 2^-24 a rounded candidate is off by u X, its
+// rounded image shift by u (2 X + r), their sum by u (X + r), the rounded centre by u X and the
+// difference, near the list radius r, by u r: err = u (5 X + 3 r) in all.  The square sum is then off
+// by 2 sqrt(3) r err + 3 err^2 and the rounding of products and sums, 8 u r^2; the band is twice that.
+inline Near near_band(double r, double X) {
+    const double u = 5.9604644775390625e-8, err = u * (5.0 * X + 3.0 * r);
+    Near nr;
+    nr.rl2 = r * r;
+    nr.mid = (float)nr.rl2;
+    const double tol = 2.0 * (3.4641016151377546 * r * err + 3.0 * err * err + 8.0 * u * r * r);
+    nr.tol = tol < 1.0e30 ? (float)tol : 1.0e30f;
+    return nr;
+}
+
+__device__ __forceinline__ bool exact_inside(const double* __restrict__ xj, double sx, double sy, double sz, double xi, double yi,
+                                             double zi, double rl2) {
+    const double ddx = __dsub_rn(__dadd_rn(xj[0], sx), xi), ddy = __dsub_rn(__dadd_rn(xj[1], sy), yi),
+                 ddz = __dsub_rn(__dadd_rn(xj[2], sz), zi);
+    return __dadd_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)), __dmul_rn(ddz, ddz)) < rl2;
+}
+// component c of the shift vector n . H, built up one cell vector after another without fused
+// multiply-add; for an orthorhombic cell all but one term of each component are exact zeros
+__device__ __forceinline__ double image_shift(const Grid& g, int nx, int ny, int nz, int c) {
+    return __dadd_rn(__dadd_rn(__dmul_rn((double)nz, g.H[6 + c]), __dmul_rn((double)ny, g.H[3 + c])), __dmul_rn((double)nx, g.H[c]));
+}
+
+// A warp takes G centres of one cell; its lanes are 32 candidates at a time, tested against all G
+// centres (held in registers of every lane), so that the walk over the cells, the candidate loads
+// and the loop around them are paid once per G centres.  The walk is cut into runs: bins that follow
+// one another along x under the same image hold consecutive atoms.  The warp lays out 32 runs at a
+// time, a lane each, and then goes through their candidates end to end, so that short runs leave no
+// lane idle.  FILL = false: count the neighbours.  FILL = true: write them, in the order of the walk.
+// Bound by instruction issue: nine instructions per centre and 32 candidates in the count pass,
+// about twenty in the fill pass.
+template <bool FILL, int G>
+__global__ void __launch_bounds__(128) k_scan_cells(Grid g, Near nr, const int* __restrict__ cell_start, const float4* __restrict__ rec,
+                                                    const double* __restrict__ xs0, int* __restrict__ deg,
+                                                    const eidx_t* __restrict__ row_ptr, int2* __restrict__ nbr, int* __restrict__ err) {
+    struct Run { int end, first, code; float sx, sy, sz; };   // candidates before its end; atom of candidate 0; image
+    __shared__ Run runs_s[4][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    Run* const runs = runs_s[warp];
     const unsigned lt_mask = (1u << lane) - 1u;
     const int wz = 2 * g.m[2] + 1, wy = 2 * g.m[1] + 1, wx = 2 * g.m[0] + 1;
+    const int n_keys = g.halves * g.ncell;
+    for (int key0 = blockIdx.x; key0 < n_keys; key0 += gridDim.x) {
+    const int c_end = cell_start[key0 + 1], first_i = cell_start[key0] + G * (warp + n_warps * blockIdx.y);
+    if (first_i >= c_end) continue;
+    const int key = key0 < g.ncell ? key0 : key0 - g.ncell;         // a ghost's own bin
+    const int cx = key % g.nc[0], cy = (key / g.nc[0]) % g.nc[1], cz = key / (g.nc[0] * g.nc[1]);
     const int sz0 = walk_start(cz, g.m[2], g.nc[2], g.pbc[2], g.sorted);
     const int sy0 = walk_start(cy, g.m[1], g.nc[1], g.pbc[1], g.sorted);
     const int sx0 = walk_start(cx, g.m[0], g.nc[0], g.pbc[0], g.sorted);
+    // the walk along x, the same on every line of bins: the run at offset tx of the walk, and how far
+    // it goes (a run that is off the grid of an open direction is empty)
+    auto x_run = [&](int tx, int* xc, int* nx) {
+        int dx = sx0 + tx;
+        if (dx > g.m[0]) dx -= wx;
+        *xc = cx + dx; *nx = 0;
+        if (g.pbc[0]) {
+            *nx = floor_div(*xc, g.nc[0]);
+            *xc -= *nx * g.nc[0];
+            return min(min(g.nc[0] - *xc, g.m[0] - dx + 1), wx - tx);
+        }
+        return *xc < 0 ? -*xc : min(max(g.nc[0] - *xc, 1), wx - tx);
+    };
+    int per_line = 0;
+    for (int tx = 0, xc, nx; tx < wx; ++per_line) tx += x_run(tx, &xc, &nx);
+    const int n_runs = wz * wy * per_line;
+    for (int i0 = first_i; i0 < c_end; i0 += G * n_warps * gridDim.y) {
+    const int gn = min(G, c_end - i0);
+    // lane k < G keeps centre k in double precision; every lane has all of them in single precision
+    double xi = 0, yi = 0, zi = 0;
+    if (lane < gn) { const double* x = xs0 + 3 * (size_t)(i0 + lane); xi = x[0]; yi = x[1]; zi = x[2]; }
+    float fx[G], fy[G], fz[G];
+    int cnt[G];                                  // FILL: next slot, counted from the first centre's row
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+        fx[k] = __shfl_sync(0xffffffffu, lane < gn ? (float)xi : -3.0e18f, k);
+        fy[k] = __shfl_sync(0xffffffffu, (float)yi, k); fz[k] = __shfl_sync(0xffffffffu, (float)zi, k);
+        cnt[k] = FILL && k < gn ? (int)(row_ptr[i0 + k] - row_ptr[i0]) : 0;
+    }
+    int2* const out = FILL ? nbr + row_ptr[i0] : nullptr;
     // with ghosts the bins are walked twice, owned atoms first: ghosts follow every owned atom in
     // the internal order, so the row still ascends in the neighbour index
     for (int half = 0; half < g.halves; ++half)
-    for (int tz = 0; tz < wz; ++tz) {
-        int dz = sz0 + tz;
-        if (dz > g.m[2]) dz -= wz;
-        int zc = cz + dz, nz = 0;
-        if (g.pbc[2]) { nz = floor_div(zc, g.nc[2]); zc -= nz * g.nc[2]; }
-        else if (zc < 0 || zc >= g.nc[2]) continue;
-        // shift vector n . H, built up one cell vector per loop level without fused multiply-add;
-        // for an orthorhombic cell all but one term of each component are exact zeros
-        const double szx = __dmul_rn((double)nz, g.H[6]), szy = __dmul_rn((double)nz, g.H[7]),
-                     szz = __dmul_rn((double)nz, g.H[8]);
-        for (int ty = 0; ty < wy; ++ty) {
-            int dy = sy0 + ty;
+    for (int r0 = 0; r0 < n_runs; r0 += 32) {
+        int n = 0;
+        Run my = {0, 0, 0, 0.f, 0.f, 0.f};
+        if (r0 + lane < n_runs) {
+            const int line = (r0 + lane) / per_line, seg = (r0 + lane) - line * per_line;
+            int dz = sz0 + line / wy, dy = sy0 + line % wy;
+            if (dz > g.m[2]) dz -= wz;
             if (dy > g.m[1]) dy -= wy;
-            int yc = cy + dy, ny = 0;
+            int zc = cz + dz, yc = cy + dy, xc = 0, nx = 0, ny = 0, nz = 0, run = 0;
+            bool in = true;
+            if (g.pbc[2]) { nz = floor_div(zc, g.nc[2]); zc -= nz * g.nc[2]; }
+            else if (zc < 0 || zc >= g.nc[2]) in = false;
             if (g.pbc[1]) { ny = floor_div(yc, g.nc[1]); yc -= ny * g.nc[1]; }
-            else if (yc < 0 || yc >= g.nc[1]) continue;
-            const double syx = __dadd_rn(szx, __dmul_rn((double)ny, g.H[3])), syy = __dadd_rn(szy, __dmul_rn((double)ny, g.H[4])),
-                         syz = __dadd_rn(szz, __dmul_rn((double)ny, g.H[5]));
-            for (int tx = 0, run = 1; tx < wx; tx += run) {
-                int dx = sx0 + tx;
-                if (dx > g.m[0]) dx -= wx;
-                int xc = cx + dx, nx = 0;
-                run = 1;
-                if (g.pbc[0]) { nx = floor_div(xc, g.nc[0]); xc -= nx * g.nc[0]; }
-                else if (xc < 0 || xc >= g.nc[0]) continue;
-                // bins that follow one another along x with the same image hold consecutive atoms:
-                // they are scanned as one range (same candidates in the same order, fuller warps)
-                while (g.sorted && tx + run < wx) {
-                    int dx2 = sx0 + tx + run;
-                    if (dx2 > g.m[0]) dx2 -= wx;
-                    int xc2 = cx + dx2, nx2 = 0;
-                    if (g.pbc[0]) { nx2 = floor_div(xc2, g.nc[0]); xc2 -= nx2 * g.nc[0]; }
-                    else if (xc2 < 0 || xc2 >= g.nc[0]) break;
-                    if (nx2 != nx || xc2 != xc + run) break;
-                    ++run;
-                }
-                const double sx = __dadd_rn(syx, __dmul_rn((double)nx, g.H[0])), sy = __dadd_rn(syy, __dmul_rn((double)nx, g.H[1])),
-                             sz = __dadd_rn(syz, __dmul_rn((double)nx, g.H[2]));
+            else if (yc < 0 || yc >= g.nc[1]) in = false;
+            for (int q = 0, tx = 0; q <= seg; ++q) { tx += run; run = x_run(tx, &xc, &nx); }
+            if (xc < 0 || xc >= g.nc[0]) in = false;
+            if (in) {
                 const int cell = (zc * g.nc[1] + yc) * g.nc[0] + xc + half * g.ncell;
-                const int beg = cell_start[cell], end = cell_start[cell + run];
-                const bool self_img = (nx == 0 && ny == 0 && nz == 0);
-                for (int b = beg; b < end; b += 32) {
-                    const int j = b + lane;
-                    bool ok = false;
-                    if (j < end) {
-                        const double ddx = __dsub_rn(__dadd_rn(xs0[3 * (size_t)j], sx), xi);
-                        const double ddy = __dsub_rn(__dadd_rn(xs0[3 * (size_t)j + 1], sy), yi);
-                        const double ddz = __dsub_rn(__dadd_rn(xs0[3 * (size_t)j + 2], sz), zi);
-                        const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)),
-                                                    __dmul_rn(ddz, ddz));
-                        ok = (d2 < rl2) && !(self_img && j == i);
-                    }
-                    const unsigned mask = __ballot_sync(0xffffffffu, ok);
-                    if (FILL && ok) {
-                        const eidx_t p = base_out + count + __popc(mask & lt_mask);
-                        src[p] = j;
-                        shift[p] = pack_shift(nx, ny, nz);
-                    }
-                    count += __popc(mask);
+                my.first = cell_start[cell];
+                n = cell_start[cell + run] - my.first;
+                my.code = pack_shift(nx, ny, nz);
+                my.sx = (float)image_shift(g, nx, ny, nz, 0); my.sy = (float)image_shift(g, nx, ny, nz, 1);
+                my.sz = (float)image_shift(g, nx, ny, nz, 2);
+                if (nx < -127 || nx > 127 || ny < -127 || ny > 127 || nz < -127 || nz > 127) atomicOr(err, kErrShiftRange);
+            }
+        }
+        my.end = n;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, my.end, off);
+            if (lane >= off) my.end += v;
+        }
+        my.first -= my.end - n;
+        const int total = __shfl_sync(0xffffffffu, my.end, 31);
+        __syncwarp();
+        runs[lane] = my;
+        __syncwarp();
+        int r = 0, j_next = 0, code_next = 0;
+        float4 p_next = make_float4(3.0e18f, 0.f, 0.f, 0.f);
+        auto fetch = [&](int f) {                // candidate f of these runs, its image applied
+            p_next = make_float4(3.0e18f, 0.f, 0.f, 0.f);
+            j_next = -1; code_next = 0;
+            if (f < total) {
+                while (f >= runs[r].end) ++r;
+                j_next = runs[r].first + f;
+                code_next = runs[r].code;
+                p_next = __ldg(rec + 2 * (size_t)j_next);
+            }
+        };
+        fetch(lane);
+        for (int f0 = 0; f0 < total; f0 += 32) {
+            float4 p = p_next;
+            const int j = j_next, code = code_next;
+            if (code != 0) { p.x += runs[r].sx; p.y += runs[r].sy; p.z += runs[r].sz; }
+            fetch(f0 + 32 + lane);
+            auto distance = [&](int k) {         // squared, minus the squared list radius
+                const float ddx = p.x - fx[k], ddy = p.y - fy[k], ddz = p.z - fz[k];
+                return fmaf(ddx, ddx, fmaf(ddy, ddy, fmaf(ddz, ddz, -nr.mid)));
+            };
+            float closest = 1.0e30f;
+            unsigned hit[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const float off = distance(k);
+                closest = fminf(closest, fabsf(off));
+                if (FILL) hit[k] = __ballot_sync(0xffffffffu, off < 0.f);
+                else cnt[k] += off < 0.f;
+            }
+            if (__any_sync(0xffffffffu, closest <= nr.tol)) {
+                const int nx = (int)(signed char)(code & 0xff), ny = (int)(signed char)((code >> 8) & 0xff), nz = (int)(signed char)((code >> 16) & 0xff);
+                const double sx = image_shift(g, nx, ny, nz, 0), sy = image_shift(g, nx, ny, nz, 1), sz = image_shift(g, nx, ny, nz, 2);
+#pragma unroll
+                for (int k = 0; k < G; ++k) {
+                    const double xk = __shfl_sync(0xffffffffu, xi, k), yk = __shfl_sync(0xffffffffu, yi, k), zk = __shfl_sync(0xffffffffu, zi, k);
+                    const bool in = j >= 0 && k < gn && exact_inside(xs0 + 3 * (size_t)j, sx, sy, sz, xk, yk, zk, nr.rl2);
+                    if (FILL) hit[k] = __ballot_sync(0xffffffffu, in);
+                    else cnt[k] += (int)in - (int)(distance(k) < 0.f);
                 }
-                if (nx < -127 || nx > 127 || ny < -127 || ny > 127 || nz < -127 || nz > 127)
-                    if (lane == 0) atomicOr(err, kErrShiftRange);
+            }
+            if (FILL) {
+                const bool self = code == 0 && (unsigned)(j - i0) < (unsigned)G;    // no atom is its own neighbour
+                if (__any_sync(0xffffffffu, self)) {
+#pragma unroll
+                    for (int k = 0; k < G; ++k) hit[k] &= ~__ballot_sync(0xffffffffu, self && j - i0 == k);
+                }
+#pragma unroll
+                for (int k = 0; k < G; ++k) {
+                    if (!hit[k]) continue;
+                    if ((hit[k] >> lane) & 1u) out[cnt[k] + __popc(hit[k] & lt_mask)] = make_int2(j, code);
+                    cnt[k] += __popc(hit[k]);
+                }
             }
         }
     }
-    if (!FILL && lane == 0) deg[i] = count;
+    if (!FILL) {
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const int v = __reduce_add_sync(0xffffffffu, cnt[k]);
+            if (k < gn && lane == k) deg[i0 + k] = max(v - 1, 0);    // the walk meets the centre itself once (unless it is not a number)
+        }
+    }
+    }
+    }
 }
 
-// rev[e] = slot of (j <- i, -n) for e = (i <- j, n); -1 when absent (can only happen for
-// pairs whose two orientations round to opposite sides of the list radius).
-__global__ void k_reverse_map(int N, int sorted, const eidx_t* __restrict__ row_ptr, const int* __restrict__ src,
-                              const int* __restrict__ shift, eidx_t* __restrict__ rev) {
+// How the rows of a list are ordered, i.e. how the reverse of an edge is searched for.
+//   kByIndex   ascending in the neighbour index, each neighbour at most once
+//   kByBin     by the neighbour's bin counted across images (z, then y, then x), then by index:
+//              boxes so small that a walk visits a bin under several images
+//   kByImage   by image (z, then y, then x), then by index: batched frames
+enum RowOrder { kByIndex = 0, kByBin = 1, kByImage = 2 };
+
+// position of neighbour (s, n) in the order of a row
+template <int ORDER>
+__device__ __forceinline__ unsigned long long order_key(const Grid& g, const int* __restrict__ skey, int s, int n) {
+    const int nx = (int)(signed char)(n & 0xff), ny = (int)(signed char)((n >> 8) & 0xff), nz = (int)(signed char)((n >> 16) & 0xff);
+    unsigned long long k = 0;
+    if (ORDER == kByBin) {
+        int c = skey[s], half = 0;
+        if (c >= g.ncell) { c -= g.ncell; half = 1; }
+        // bins are counted from -m, fewer than 2^18 of them (127 images of at most 1024 bins)
+        const int uz = c / (g.nc[0] * g.nc[1]) + nz * g.nc[2] + (1 << 17), uy = (c / g.nc[0]) % g.nc[1] + ny * g.nc[1] + (1 << 17),
+                  ux = c % g.nc[0] + nx * g.nc[0] + (1 << 17);
+        k = ((((unsigned long long)half << 18 | (unsigned)uz) << 18 | (unsigned)uy) << 18) | (unsigned)ux;
+    } else {
+        k = (((unsigned)(nz + 128) << 8 | (unsigned)(ny + 128)) << 8) | (unsigned)(nx + 128);
+    }
+    return k;
+}
+
+// rev[e] = slot of (j <- i, -n) for e = (i <- j, n); stays at the -1 it comes with when absent (can only
+// happen for pairs whose two orientations round to opposite sides of the list radius).  Rows that
+// ascend in the neighbour index are searched for the neighbours above the row's own index only: an
+// edge and its reverse are each other's reverse, so one search fills both slots.
+// Bound by the tag lookups of its uncoalesced probes (eight per search, one lane each): 1.11 ms when every
+// edge was searched for, 0.65 now (59 M edges, rows of 273).
+template <int ORDER>
+__global__ void k_reverse_map(int N, Grid g, const int* __restrict__ skey, const eidx_t* __restrict__ row_ptr,
+                              const int2* __restrict__ nbr, eidx_t* __restrict__ rev) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= N) return;
@@ -291,29 +435,30 @@ __global__ void k_reverse_map(int N, int sorted, const eidx_t* __restrict__ row_
     const int len = (int)(row_ptr[i + 1] - e0);
     for (int k = lane; k < len; k += 32) {
         const eidx_t e = e0 + k;
-        const int j = src[e];
-        const int s = shift[e];
-        const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff),
-                  nz = (int)(signed char)((s >> 16) & 0xff);
-        const int want = pack_shift(-nx, -ny, -nz);
-        eidx_t found = -1;
+        const int2 js = nbr[e];
+        const int j = js.x, s = js.y;
+        if (ORDER == kByIndex && j <= i) continue;
+        const int want = pack_shift(-(int)(signed char)(s & 0xff), -(int)(signed char)((s >> 8) & 0xff), -(int)(signed char)((s >> 16) & 0xff));
         const eidx_t f0 = row_ptr[j];
         const int flen = (int)(row_ptr[j + 1] - f0);
-        const int* srow = src + f0;
-        const int* hrow = shift + f0;
-        if (sorted) {          // rows ascend in the neighbour index, each neighbour at most once
-            int lo = 0, hi = flen;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;            // offsets inside one row: no overflow
-                if (srow[mid] < i) lo = mid + 1; else hi = mid;
+        const int2* row = nbr + f0;
+        int lo = 0, hi = flen;                                 // offsets inside one row: no overflow
+        unsigned long long target = 0;
+        if constexpr (ORDER != kByIndex) target = order_key<ORDER>(g, skey, i, want);
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const int2 at = row[mid];
+            bool below = at.x < i;
+            if constexpr (ORDER != kByIndex) {
+                const unsigned long long km = order_key<ORDER>(g, skey, at.x, at.y);
+                below = km < target || (km == target && below);
             }
-            if (lo < flen && srow[lo] == i && hrow[lo] == want) found = f0 + lo;
-        } else {
-            for (int f = 0; f < flen; ++f) {
-                if (srow[f] == i && hrow[f] == want) { found = f0 + f; break; }
-            }
+            if (below) lo = mid + 1; else hi = mid;
         }
-        rev[e] = found;
+        if (lo < flen && row[lo].x == i && row[lo].y == want) {
+            rev[e] = f0 + lo;
+            if (ORDER == kByIndex) rev[f0 + lo] = e;
+        }
     }
 }
 
@@ -353,45 +498,58 @@ __global__ void k_batch_fold(const FrameCell* __restrict__ frames, const double*
 }
 
 // One warp per centre: every atom of the centre's frame under every image within reach, in the
-// order image (z slowest), then atom; the same double-precision predicate as the cell-list scan.
+// order image (z slowest), then atom; the same predicate as the cell-list scan.  An image is left out
+// when the planes that bound it along some cell vector are further than the cutoff from the centre.
 template <bool FILL>
-__global__ void k_batch_scan(int N, const FrameCell* __restrict__ frames, const int* __restrict__ frame_of, double rl2,
-                             const double* __restrict__ xs, int* __restrict__ deg, const eidx_t* __restrict__ row_ptr,
-                             int* __restrict__ src, int* __restrict__ shift) {
+__global__ void k_batch_scan(int N, const FrameCell* __restrict__ frames, const int* __restrict__ frame_of, double rc,
+                             const double* __restrict__ xs, const float4* __restrict__ rec, int* __restrict__ deg,
+                             const eidx_t* __restrict__ row_ptr, int2* __restrict__ nbr) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= N) return;
     const int i = warp;
     const FrameCell& fc = frames[frame_of[i]];
     const double xi = xs[3 * (size_t)i], yi = xs[3 * (size_t)i + 1], zi = xs[3 * (size_t)i + 2];
+    const double rl2 = rc * rc;
+    const float mid = (float)rl2, tol = fc.near_tol;
     const unsigned lt_mask = (1u << lane) - 1u;
     const eidx_t base_out = FILL ? row_ptr[i] : 0;
     int count = 0;
-    for (int nz = -fc.m[2]; nz <= fc.m[2]; ++nz) {
+    // image n along cell vector k can reach the centre for n in [lo, hi]: its atoms lie at fractional
+    // coordinates [n, n + 1) (within rounding), the cutoff spans `reach` of them
+    int lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) {
+        const double f = xi * fc.Hinv[k] + yi * fc.Hinv[3 + k] + zi * fc.Hinv[6 + k];
+        lo[k] = hi[k] = 0;
+        if (fc.pbc[k]) {
+            lo[k] = max(-fc.m[k], (int)floor(f - fc.reach[k]));
+            hi[k] = min(fc.m[k], (int)floor(f + fc.reach[k]));
+        }
+    }
+    for (int nz = lo[2]; nz <= hi[2]; ++nz) {
         const double szx = __dmul_rn((double)nz, fc.H[6]), szy = __dmul_rn((double)nz, fc.H[7]), szz = __dmul_rn((double)nz, fc.H[8]);
-        for (int ny = -fc.m[1]; ny <= fc.m[1]; ++ny) {
+        for (int ny = lo[1]; ny <= hi[1]; ++ny) {
             const double syx = __dadd_rn(szx, __dmul_rn((double)ny, fc.H[3])), syy = __dadd_rn(szy, __dmul_rn((double)ny, fc.H[4])),
                          syz = __dadd_rn(szz, __dmul_rn((double)ny, fc.H[5]));
-            for (int nx = -fc.m[0]; nx <= fc.m[0]; ++nx) {
+            for (int nx = lo[0]; nx <= hi[0]; ++nx) {
                 const double sx = __dadd_rn(syx, __dmul_rn((double)nx, fc.H[0])), sy = __dadd_rn(syy, __dmul_rn((double)nx, fc.H[1])),
                              sz = __dadd_rn(syz, __dmul_rn((double)nx, fc.H[2]));
                 const bool self_img = nx == 0 && ny == 0 && nz == 0;
+                const float fx = (float)(xi - sx), fy = (float)(yi - sy), fz = (float)(zi - sz);
                 for (int b = fc.a0; b < fc.a1; b += 32) {
                     const int j = b + lane;
-                    bool ok = false;
+                    bool ok = false, unsure = false;
                     if (j < fc.a1) {
-                        const double ddx = __dsub_rn(__dadd_rn(xs[3 * (size_t)j], sx), xi);
-                        const double ddy = __dsub_rn(__dadd_rn(xs[3 * (size_t)j + 1], sy), yi);
-                        const double ddz = __dsub_rn(__dadd_rn(xs[3 * (size_t)j + 2], sz), zi);
-                        const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)), __dmul_rn(ddz, ddz));
-                        ok = (d2 < rl2) && !(self_img && j == i);
+                        const float4 p = __ldg(rec + 2 * (size_t)j);
+                        const float ddx = p.x - fx, ddy = p.y - fy, ddz = p.z - fz;
+                        const float off = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz)) - mid;
+                        ok = off < 0.f;
+                        unsure = fabsf(off) <= tol;
                     }
-                    const unsigned mask = __ballot_sync(0xffffffffu, ok);
-                    if (FILL && ok) {
-                        const eidx_t p = base_out + count + __popc(mask & lt_mask);
-                        src[p] = j;
-                        shift[p] = pack_shift(nx, ny, nz);
-                    }
+                    if (__any_sync(0xffffffffu, unsure) && unsure) ok = exact_inside(xs + 3 * (size_t)j, sx, sy, sz, xi, yi, zi, rl2);
+                    const unsigned mask = __ballot_sync(0xffffffffu, ok && !(self_img && j == i));
+                    if (FILL && ((mask >> lane) & 1u))
+                        nbr[base_out + count + __popc(mask & lt_mask)] = make_int2(j, pack_shift(nx, ny, nz));
                     count += __popc(mask);
                 }
             }
@@ -437,8 +595,7 @@ __global__ void k_export_deg(int N, const int* __restrict__ perm, const eidx_t* 
 }
 
 __global__ void k_export_rows(int N, const int* __restrict__ perm, const eidx_t* __restrict__ row_ptr,
-                              const int* __restrict__ src, const int* __restrict__ shift,
-                              const int* __restrict__ row_ptr_o, int* __restrict__ src_o,
+                              const int2* __restrict__ nbr, const int* __restrict__ row_ptr_o, int* __restrict__ src_o,
                               signed char* __restrict__ shift_o) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -447,8 +604,8 @@ __global__ void k_export_rows(int N, const int* __restrict__ perm, const eidx_t*
     const eidx_t e0 = row_ptr[i];
     const int n = (int)(row_ptr[i + 1] - e0), q0 = row_ptr_o[o];
     for (int k = lane; k < n; k += 32) {
-        const int s = shift[e0 + k];
-        src_o[q0 + k] = perm[src[e0 + k]];
+        const int s = nbr[e0 + k].y;
+        src_o[q0 + k] = perm[nbr[e0 + k].x];
         shift_o[3 * (size_t)(q0 + k)] = (signed char)(s & 0xff);
         shift_o[3 * (size_t)(q0 + k) + 1] = (signed char)((s >> 8) & 0xff);
         shift_o[3 * (size_t)(q0 + k) + 2] = (signed char)((s >> 16) & 0xff);
@@ -467,8 +624,8 @@ __global__ void k_export_deg_range(int N, int first, int n, const int* __restric
 }
 
 __global__ void k_export_rows_range(int N, int first, int n, const int* __restrict__ perm,
-                                    const eidx_t* __restrict__ row_ptr, const int* __restrict__ src,
-                                    const int* __restrict__ shift, const long long* __restrict__ row_ptr_o,
+                                    const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
+                                    const long long* __restrict__ row_ptr_o,
                                     long long cap, int* __restrict__ src_o, signed char* __restrict__ shift_o) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -480,8 +637,8 @@ __global__ void k_export_rows_range(int N, int first, int n, const int* __restri
     const long long q0 = row_ptr_o[o];
     for (int k = lane; k < len; k += 32) {
         if (q0 + k >= cap) break;
-        const int s = shift[e0 + k];
-        src_o[q0 + k] = perm[src[e0 + k]];
+        const int s = nbr[e0 + k].y;
+        src_o[q0 + k] = perm[nbr[e0 + k].x];
         shift_o[3 * (size_t)(q0 + k)] = (signed char)(s & 0xff);
         shift_o[3 * (size_t)(q0 + k) + 1] = (signed char)((s >> 8) & 0xff);
         shift_o[3 * (size_t)(q0 + k) + 2] = (signed char)((s >> 16) & 0xff);
@@ -504,17 +661,43 @@ struct WidenDeg {
 }  // namespace
 
 void neighbor_free(NeighborDev* nb) {
-    void* ptrs[] = {nb->frames, nb->rec, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->src,
-                    nb->shift, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
+    void* ptrs[] = {nb->frames, nb->rec, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->nbr, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
                     nb->cub_tmp, nb->bounds};
     for (void* p : ptrs)
         dev_free(p);
+    if (nb->h_totals) cudaFreeHost(nb->h_totals);
     *nb = NeighborDev();
+}
+
+// The one synchronisation of a build: the edge counts come back, with whatever else the caller wants to
+// know by then, and the edge arrays grow to hold the list.
+static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, int* d_err, const BuildFetch* fetch, cudaStream_t st,
+                       std::string* err) {
+    if (!nb->h_totals) NB_CHECK(cudaMallocHost((void**)&nb->h_totals, 2 * sizeof(eidx_t)));
+    NB_CHECK(cudaMemcpyAsync(nb->h_totals, nb->row_ptr + N, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
+    if (n_owned < N) NB_CHECK(cudaMemcpyAsync(nb->h_totals + 1, nb->row_ptr + n_owned, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
+    if (fetch) {
+        NB_CHECK(launch_species_present(N, d_type, fetch->T, fetch->d_flags, d_err, st));
+        NB_CHECK(cudaMemcpyAsync(fetch->h_flags, fetch->d_flags, sizeof(int) * (size_t)fetch->T, cudaMemcpyDeviceToHost, st));
+        NB_CHECK(cudaMemcpyAsync(fetch->h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        NB_CHECK(cudaMemsetAsync(d_err, 0, sizeof(int), st));
+    }
+    NB_CHECK(cudaStreamSynchronize(st));
+    const int64_t total = nb->h_totals[0];
+    nb->E = total;
+    nb->E_owned = n_owned < N ? nb->h_totals[1] : total;
+    if (total > nb->E_cap) {
+        int64_t c;
+        c = 0; NB_CHECK(dev_ensure(&nb->nbr, &c, total, 1.1));
+        c = 0; NB_CHECK(dev_ensure(&nb->rev, &c, total, 1.1));
+        nb->E_cap = c;
+    }
+    return UMLMD_OK;
 }
 
 int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double* d_pos, const int32_t* d_type,
                    const double cell[9], const int pbc[3], double skin, double rc, int* d_err,
-                   cudaStream_t st, std::string* err) {
+                   const BuildFetch* fetch, cudaStream_t st, std::string* err) {
     if (N64 > 0x7fff0000LL) { *err = "too many atoms for 32-bit indices"; return UMLMD_E_INVALID_ARG; }
     const int N = (int)N64;
     const int n_owned = n_owned64 < 0 || n_owned64 > N64 ? N : (int)n_owned64;
@@ -569,6 +752,14 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     for (int k = 0; k < 3; ++k) {
         g.L[k] = L[k]; g.lo[k] = lo[k]; g.pbc[k] = pbc[k] ? 1 : 0;
         int nc = (int)std::floor(ext[k] * unit[k] / rl_pad);
+        // a periodic box of less than three list radii: bins of a half, third or quarter of the list
+        // radius still give 2 m + 1 distinct bins (from 2.5, 2.33 and 2.25 list radii on), and with them
+        // rows sorted by neighbour index
+        if (pbc[k] && nc == 2)
+            for (int q = 2; q <= 4; ++q) {
+                const int fine = (int)std::floor(q * ext[k] * unit[k] / rl_pad);
+                if (fine >= 2 * q + 1) { nc = fine; break; }
+            }
         if (nc < 1) nc = 1;
         if (nc > 1024) nc = 1024;
         g.nc[k] = nc;
@@ -591,6 +782,14 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     g.sorted = 1;
     for (int k = 0; k < 3; ++k)
         if (g.pbc[k] && g.nc[k] < 2 * g.m[k] + 1) g.sorted = 0;
+    double X = 0;                               // bound of the coordinates' magnitude
+    for (int c = 0; c < 3; ++c) {
+        double v = 0;
+        if (g.tri) for (int k = 0; k < 3; ++k) v += std::fmax(std::fabs(lo[k]), std::fabs(lo[k] + ext[k])) * std::fabs(cell[3 * k + c]);
+        else v = std::fmax(std::fabs(lo[c]), std::fabs(lo[c] + ext[c]));
+        X = std::fmax(X, v);
+    }
+    const Near nr = near_band(r_list, X);
     g.ncell = (int)ncell; g.n_owned = n_owned; g.halves = n_owned < N ? 2 : 1;
     const int64_t nkeys = (int64_t)g.halves * ncell;
 
@@ -644,34 +843,29 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     size_t tmp_bytes = nb->cub_bytes;
     NB_CHECK(cub::DeviceRadixSort::SortPairs(nb->cub_tmp, tmp_bytes, nb->key, nb->key2, nb->idx, nb->idx2, N,
                                              0, end_bit, st));
-    k_cell_start<<<(int)((nkeys + 1 + TB - 1) / TB), TB, 0, st>>>((int)nkeys, N, nb->key2, nb->cell_start);
-    k_gather_sorted<<<(N + TB - 1) / TB, TB, 0, st>>>(N, nb->idx2, nb->wpos, img_o, d_type, nb->perm, nb->xs0,
-                                                      nb->xs, nb->img, nb->type_s);
-    const double rl2 = r_list * r_list;
-    const int warps_per_block = TB / 32;
-    const int wb = (N + warps_per_block - 1) / warps_per_block;
-    k_scan_cells<false><<<wb, TB, 0, st>>>(N, g, rl2, nb->key2, nb->cell_start, nb->xs0, nb->deg, nullptr,
-                                           nullptr, nullptr, d_err);
+    k_gather_sorted<<<N / TB + 1, TB, 0, st>>>(N, (int)nkeys, nb->key2, nb->idx2, nb->wpos, img_o, d_type, nb->perm, nb->xs0,
+                                              nb->xs, nb->rec, nb->img, nb->type_s, nb->cell_start);
+    // Eight centres per warp and a block of four warps per cell; below 16384 atoms, where the cells are
+    // too few to fill the machine that way, two centres per warp and four blocks per cell (4000 atoms,
+    // 125 cells: count and fill 19 + 24 us; with one block per cell they took 34 + 45).
+    // Both are bound by instruction issue.  With one warp per centre and every test in double precision
+    // 216,000 atoms with 273 neighbours took 1.21 + 1.49 ms, so 0.32 + 0.52.
+    const bool few = N < 16384;
+    const dim3 scan_blocks((unsigned)(nkeys < 148 * 64 ? nkeys : 148 * 64), few ? 4 : 1);
+    const int scan_threads = 128;
+    auto scan = few ? k_scan_cells<false, 2> : k_scan_cells<false, 8>;
+    scan<<<scan_blocks, scan_threads, 0, st>>>(g, nr, nb->cell_start, nb->rec, nb->xs0, nb->deg, nullptr, nullptr, d_err);
     NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
     tmp_bytes = nb->cub_bytes;
     NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, N + 1, st));
-    eidx_t total = 0, total_owned = 0;
-    NB_CHECK(cudaMemcpyAsync(&total, nb->row_ptr + N, sizeof(total), cudaMemcpyDeviceToHost, st));
-    if (n_owned < N) NB_CHECK(cudaMemcpyAsync(&total_owned, nb->row_ptr + n_owned, sizeof(total_owned), cudaMemcpyDeviceToHost, st));
-    NB_CHECK(cudaStreamSynchronize(st));
-    nb->E = total;
-    nb->E_owned = n_owned < N ? total_owned : total;
-    if (total > nb->E_cap) {
-        int64_t c;
-        c = 0; NB_CHECK(dev_ensure(&nb->src, &c, total, 1.1));
-        c = 0; NB_CHECK(dev_ensure(&nb->shift, &c, total, 1.1));
-        c = 0; NB_CHECK(dev_ensure(&nb->rev, &c, total, 1.1));
-        nb->E_cap = c;
-    }
-    if (total > 0) {
-        k_scan_cells<true><<<wb, TB, 0, st>>>(N, g, rl2, nb->key2, nb->cell_start, nb->xs0, nullptr,
-                                              nb->row_ptr, nb->src, nb->shift, d_err);
-        k_reverse_map<<<wb, TB, 0, st>>>(N, g.sorted, nb->row_ptr, nb->src, nb->shift, nb->rev);
+    int code = read_totals(nb, N, n_owned, d_type, d_err, fetch, st, err);
+    if (code != UMLMD_OK) return code;
+    if (nb->E > 0) {
+        auto fill = few ? k_scan_cells<true, 2> : k_scan_cells<true, 8>;
+        fill<<<scan_blocks, scan_threads, 0, st>>>(g, nr, nb->cell_start, nb->rec, nb->xs0, nullptr, nb->row_ptr, nb->nbr, d_err);
+        NB_CHECK(cudaMemsetAsync(nb->rev, 0xff, sizeof(eidx_t) * (size_t)nb->E, st));
+        auto reverse = g.sorted ? k_reverse_map<kByIndex> : k_reverse_map<kByBin>;
+        reverse<<<(N + TB / 32 - 1) / (TB / 32), TB, 0, st>>>(N, g, nb->key2, nb->row_ptr, nb->nbr, nb->rev);
     }
     NB_CHECK(cudaGetLastError());
     return UMLMD_OK;
@@ -690,15 +884,15 @@ int neighbor_export(NeighborDev* nb, int32_t* d_row_ptr, int32_t* d_src, int8_t*
     NB_CHECK(cub::DeviceScan::ExclusiveSum(nb->cub_tmp, tmp_bytes, nb->deg, d_row_ptr, N + 1, st));
     const int wb = (N + TB / 32 - 1) / (TB / 32);
     if (nb->E > 0)
-        k_export_rows<<<wb, TB, 0, st>>>(N, nb->perm, nb->row_ptr, nb->src, nb->shift, d_row_ptr, d_src,
+        k_export_rows<<<wb, TB, 0, st>>>(N, nb->perm, nb->row_ptr, nb->nbr, d_row_ptr, d_src,
                                          (signed char*)d_shift);
     NB_CHECK(cudaGetLastError());
     return UMLMD_OK;
 }
 
 int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, const double* cells, const int pbc[3],
-                         const double* d_pos, const int32_t* d_type, int T, double rc, int* d_err, cudaStream_t st,
-                         std::string* err) {
+                         const double* d_pos, const int32_t* d_type, int T, double rc, int* d_err, const BuildFetch* fetch,
+                         cudaStream_t st, std::string* err) {
     const int64_t N = offsets[n_frames];
     std::vector<FrameCell> fr((size_t)n_frames);
     for (int f = 0; f < n_frames; ++f) {
@@ -721,9 +915,14 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
             const double nrm = std::sqrt(cr[k][0] * cr[k][0] + cr[k][1] * cr[k][1] + cr[k][2] * cr[k][2]);
             const double height = std::fabs(det) / nrm;
             c.pbc[k] = pbc[k] ? 1 : 0;
+            c.reach[k] = rc / height + 1e-6;
             c.m[k] = pbc[k] ? (int)std::ceil(rc / height) : 0;
             if (c.m[k] > 127) { *err = "frame cell much smaller than the cutoff (more than 127 images)"; return UMLMD_E_UNSUPPORTED_CELL; }
         }
+        // coordinates of a folded atom are bounded by the cell along periodic directions only
+        double X = 0;
+        for (int k = 0; k < 9; ++k) X = std::fmax(X, std::fabs(H[k]));
+        c.near_tol = pbc[0] && pbc[1] && pbc[2] ? near_band(rc, 3.0 * X).tol : 1.0e30f;
         c.a0 = (int)offsets[f]; c.a1 = (int)offsets[f + 1];
     }
     nb->N = N; nb->skin = 0; nb->r_list = rc; nb->tri = 1; nb->batch = true; nb->n_frames = n_frames;
@@ -752,8 +951,8 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
     }
     nb->frame_of = nb->key;                    // scratch of the cell-list build, free here
     NB_CHECK(dev_ensure(&nb->frames, &nb->frames_cap, (int64_t)n_frames));
+    // (pageable memory: the call returns once the frames have been staged)
     NB_CHECK(cudaMemcpyAsync(nb->frames, fr.data(), sizeof(FrameCell) * (size_t)n_frames, cudaMemcpyHostToDevice, st));
-    NB_CHECK(cudaStreamSynchronize(st));       // `fr` is pageable host memory
     auto deg_wide = thrust::make_transform_iterator(static_cast<const int*>(nb->deg), WidenDeg());
     size_t need_scan = 0;
     cub::DeviceScan::ExclusiveScan(nullptr, need_scan, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, (int)N + 1, st);
@@ -765,27 +964,18 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
     }
     const int TB = 256;
     k_batch_fold<<<n_frames, TB, 0, st>>>(nb->frames, d_pos, d_type, T, nb->xs, nb->rec, nb->type_s, nb->frame_of, nb->perm, d_err);
-    const double rl2 = rc * rc;
     const int wb = (int)((N + TB / 32 - 1) / (TB / 32));
-    k_batch_scan<false><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rl2, nb->xs, nb->deg, nullptr, nullptr, nullptr);
+    k_batch_scan<false><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rc, nb->xs, nb->rec, nb->deg, nullptr, nullptr);
     NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
     size_t tmp_bytes = nb->cub_bytes;
     NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, (int)N + 1, st));
-    eidx_t total = 0;
-    NB_CHECK(cudaMemcpyAsync(&total, nb->row_ptr + N, sizeof(total), cudaMemcpyDeviceToHost, st));
-    NB_CHECK(cudaStreamSynchronize(st));
-    nb->E = total;
-    nb->n_owned = N; nb->E_owned = total;
-    if (total > nb->E_cap) {
-        int64_t c;
-        c = 0; NB_CHECK(dev_ensure(&nb->src, &c, total, 1.1));
-        c = 0; NB_CHECK(dev_ensure(&nb->shift, &c, total, 1.1));
-        c = 0; NB_CHECK(dev_ensure(&nb->rev, &c, total, 1.1));
-        nb->E_cap = c;
-    }
-    if (total > 0) {
-        k_batch_scan<true><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rl2, nb->xs, nullptr, nb->row_ptr, nb->src, nb->shift);
-        k_reverse_map<<<wb, TB, 0, st>>>((int)N, 0, nb->row_ptr, nb->src, nb->shift, nb->rev);
+    nb->n_owned = N;
+    int code = read_totals(nb, (int)N, (int)N, nb->type_s, d_err, fetch, st, err);
+    if (code != UMLMD_OK) return code;
+    if (nb->E > 0) {
+        k_batch_scan<true><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rc, nb->xs, nb->rec, nullptr, nb->row_ptr, nb->nbr);
+        NB_CHECK(cudaMemsetAsync(nb->rev, 0xff, sizeof(eidx_t) * (size_t)nb->E, st));
+        k_reverse_map<kByImage><<<wb, TB, 0, st>>>((int)N, Grid(), nullptr, nb->row_ptr, nb->nbr, nb->rev);
     }
     NB_CHECK(cudaGetLastError());
     return UMLMD_OK;
@@ -806,7 +996,7 @@ int neighbor_export_rows(NeighborDev* nb, int64_t first, int64_t n, int64_t* d_r
                                             (eidx_t)0, (int)n + 1, st));
     if (cap > 0 && d_src && d_shift) {
         const int wb = (N + TB / 32 - 1) / (TB / 32);
-        k_export_rows_range<<<wb, TB, 0, st>>>(N, (int)first, (int)n, nb->perm, nb->row_ptr, nb->src, nb->shift,
+        k_export_rows_range<<<wb, TB, 0, st>>>(N, (int)first, (int)n, nb->perm, nb->row_ptr, nb->nbr,
                                                reinterpret_cast<const long long*>(d_row_ptr), (long long)cap, d_src,
                                                (signed char*)d_shift);
     }

@@ -1,0 +1,69 @@
+"""Neighbor scans at the sizes where their layout changes: boxes around two to three list radii (bins of
+a fraction of the list radius, rows ordered by bin), the atom count at which the work per warp changes,
+pairs whose distance rounds to either side of the list radius in single precision."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import dpa4c as orc
+from workloads import SMALL_PROFILES, make_blob
+
+pytestmark = pytest.mark.gpu
+RC = 6.0
+
+
+def _check_rows(m, pos, cell, pbc, r_list, centers):
+    row_ptr, src, shift = (t.cpu().numpy().astype(np.int64) for t in m.get_neighbors())
+    ref = orc.neighbor_rows(orc.wrap_positions(pos, cell, pbc), cell, pbc, r_list, centers=centers)
+    for c, want in zip(centers, ref):
+        a, b = row_ptr[c], row_ptr[c + 1]
+        got = np.concatenate([src[a:b, None], shift[a:b]], axis=1)
+        got = got[np.lexsort((got[:, 3], got[:, 2], got[:, 1], got[:, 0]))]
+        assert np.array_equal(got, want), c
+
+
+def _run(pos, cell, pbc, skin, centers):
+    from paper_2608_19041_b200 import binding
+    m = binding.Model(make_blob(SMALL_PROFILES["p8_2_0"], 3))
+    types = torch.as_tensor(np.arange(len(pos)) % 2, dtype=torch.int32).cuda()
+    p = torch.as_tensor(pos, dtype=torch.float64).cuda().contiguous()
+    m.build_neighbors(p, types, cell, pbc, skin)
+    _check_rows(m, pos, cell, pbc, RC + skin, centers)
+    # a wrong reverse slot breaks Newton's third law: the sum of 3 N forces is single-precision noise
+    F = m.compute(p)["forces"].cpu().numpy()
+    assert np.abs(F.sum(axis=0)).max() <= 2e-6 * max(np.abs(F).max(), 1e-6) * np.sqrt(len(pos)) * 10
+    m.close()
+
+
+# edge of the box in list radii: under several images of a bin (1.6, 2.2), quarter, third and half bins
+# (2.28, 2.4, 2.6), whole ones (3.1); the other edges differ
+@pytest.mark.parametrize("pbc", [(1, 1, 1), (1, 0, 1)])
+@pytest.mark.parametrize("edge", [1.6, 2.2, 2.28, 2.4, 2.6, 3.1])
+def test_rows_in_small_boxes(edge, pbc):
+    skin = 0.5
+    cell = np.diag(np.array([edge, edge + 0.15, edge + 0.35]) * (RC + skin))
+    n = int(np.prod(np.diag(cell)) * 0.04)
+    rng = np.random.Generator(np.random.PCG64(int(100 * edge)))
+    _run(rng.random((n, 3)) @ cell, cell, pbc, skin, np.arange(n))
+
+
+@pytest.mark.parametrize("n", [16383, 16384])
+def test_rows_at_the_switch_of_the_work_split(n):
+    rng = np.random.Generator(np.random.PCG64(n))
+    cell = np.diag([70.0, 66.0, 59.0])
+    _run(rng.random((n, 3)) @ cell, cell, (1, 1, 1), 1.0, np.sort(rng.choice(n, 64, replace=False)))
+
+
+@pytest.mark.parametrize("origin", [0.0, 9.0e3])
+def test_pairs_at_the_list_radius(origin):
+    """Dimers of length r (1 +- d), d down to 1e-13, far apart from one another: the exact predicate decides."""
+    rng = np.random.Generator(np.random.PCG64(5))
+    pos = []
+    for k in range(64):
+        u = rng.standard_normal(3)
+        u /= np.linalg.norm(u)
+        a = origin + np.array([40.0 * (k % 4), 40.0 * (k // 4 % 4), 40.0 * (k // 16)])
+        pos += [a, a + RC * (1.0 + (-1.0) ** k * 10.0 ** -rng.integers(3, 14)) * u]
+    pos = np.array(pos)
+    _run(pos, np.eye(3) * 400.0, (0, 0, 0), 0.0, np.arange(len(pos)))
