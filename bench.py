@@ -343,12 +343,15 @@ class Workload:
         prof = m.get_profile()
         m.set_profiling(False)
         work = work_model(self.p, self.N, self.e_rc, self.e_list, one_species=len(np.unique(self.s["types"])) == 1)
+        if not prof["mlp_backward"][1]:        # one kernel for both passes, under the forward pass's name
+            work["mlp_forward"] = dict(work["mlp_forward"], flops=work["mlp_forward"]["flops"] + work["mlp_backward"]["flops"],
+                                       bytes=work["mlp_forward"]["bytes"] + work["mlp_backward"]["bytes"])
         total_ms = sum(v[0] for v in prof.values()) or 1.0
         kernels = []
         for cname, (kms, kl) in prof.items():
             if kl == 0 or cname not in work:
                 continue
-            evals = steps if cname != "neighbor_build" else max(1, kl // 7)
+            evals = steps if cname != "neighbor_build" else max(1, kl // 5)
             ent = roofline_entry(cname, kms, kl, evals, work, peaks)
             if ent:
                 ent["share"] = round(kms / total_ms, 4)

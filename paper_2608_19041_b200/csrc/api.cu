@@ -27,6 +27,7 @@ struct umlmd {
     // workspace
     float* state = nullptr; float* desc = nullptr; float* pre = nullptr; float* hbuf = nullptr;
     __half* tc_hi = nullptr; __half* tc_lo = nullptr;   // half-precision split of the current GEMM's activations
+    float* fused_scratch = nullptr;      // per-CTA areas of the one-kernel MLP
     int64_t tile_cap = 0;
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
@@ -135,6 +136,11 @@ void fill_info(const Dims& d, umlmd_info* o) {
 constexpr int64_t kIntermediatesMaxAtoms = 65536;
 bool keeps_intermediates(const umlmd_t* h) { return h->nb.N < kIntermediatesMaxAtoms && h->nb.N <= h->node_tile; }
 
+// whether some evaluation of up to B rows runs its MLP as a chain of GEMMs
+bool mlp_needs_chain(const umlmd_t* h, int64_t B) {
+    return !(mlp_fused_pick(h->d, h->mlp_path, B, true) && mlp_fused_pick(h->d, h->mlp_path, B, false));
+}
+
 int ensure_workspace(umlmd_t* h) {
     const Dims& d = h->d;
     const int64_t N = h->nb.N, E = h->nb.E;
@@ -143,11 +149,16 @@ int ensure_workspace(umlmd_t* h) {
         int64_t c;
         c = 0; API_CUDA(h, dev_ensure(&h->state, &c, B * d.SP));
         c = 0; API_CUDA(h, dev_ensure(&h->desc, &c, B * d.DP));
-        c = 0; API_CUDA(h, dev_ensure(&h->pre, &c, B * d.F * d.n_hidden));
-        c = 0; API_CUDA(h, dev_ensure(&h->hbuf, &c, B * d.F * 2));
         const int64_t wmax = d.DP > d.F ? d.DP : d.F;
-        c = 0; API_CUDA(h, dev_ensure(&h->tc_hi, &c, 2 * B * wmax));
-        c = 0; API_CUDA(h, dev_ensure(&h->tc_lo, &c, 2 * B * wmax));
+        const bool chain = mlp_needs_chain(h, B);
+        if (chain) {
+            c = 0; API_CUDA(h, dev_ensure(&h->pre, &c, B * d.F * d.n_hidden));
+            c = 0; API_CUDA(h, dev_ensure(&h->hbuf, &c, B * d.F * 2));
+        }
+        const int64_t split = chain ? 2 * B * wmax : B * d.DP;      // the one-kernel MLP only reads the feature split
+        c = 0; API_CUDA(h, dev_ensure(&h->tc_hi, &c, split));
+        c = 0; API_CUDA(h, dev_ensure(&h->tc_lo, &c, split));
+        if (mlp_fused_pick(d, h->mlp_path, 1, true)) { c = 0; API_CUDA(h, dev_ensure(&h->fused_scratch, &c, mlp_fused_scratch_floats(d, B))); }
         h->tile_cap = B;
     }
     if (E > h->g_cap || !h->g) { API_CUDA(h, dev_ensure(&h->g, &h->g_cap, E * 3, 1.1)); h->g_cap /= 3; }
@@ -218,9 +229,10 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         ma.tc_slot = (size_t)h->tile_cap * (size_t)(d.DP > d.F ? d.DP : d.F);
         ma.spin_limit = h->gemm_spin_limit; ma.test_skip_kblock = h->fault_skip_stage;
         h->fault_skip_stage = 0;                      // one shot
-        { Scope sc(h, kMlpFwd, d.n_hidden + 1); API_CUDA(h, launch_mlp_forward(ma, h->st)); }
+        ma.fused_scratch = mlp_fused_pick(d, h->mlp_path, n, want_grad) ? h->fused_scratch : nullptr;
+        { Scope sc(h, kMlpFwd, ma.fused_scratch ? 1 : d.n_hidden + 1); API_CUDA(h, launch_mlp_forward(ma, h->st)); }
         if (want_grad) {
-            { Scope sc(h, kMlpBwd, d.n_hidden); API_CUDA(h, launch_mlp_backward(ma, h->st)); }
+            if (!ma.fused_scratch) { Scope sc(h, kMlpBwd, d.n_hidden); API_CUDA(h, launch_mlp_backward(ma, h->st)); }
             { Scope sc(h, kInvBwd, 1); API_CUDA(h, launch_invariants_backward(ia, h->st)); }
             int blocks = 0;
             { Scope sc(h, kEdgeBwd, 1); API_CUDA(h, launch_edge_backward(ea, &blocks, h->st)); }
@@ -465,7 +477,7 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->on_device) cudaStreamSynchronize(h->st);
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
-    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
+    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
                     h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->table_uni, h->d_species, h->uni_scale};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
@@ -587,7 +599,10 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     // evaluation workspace of one node tile, per-edge gradients, per-atom results, MD forces
     const int64_t Bt = N < h->node_tile ? N : h->node_tile;
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
-    t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4) + buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
+    t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
+    if (mlp_fused_pick(d, h->mlp_path, 1, true)) t += buf(mlp_fused_scratch_floats(d, Bt), 4);
+    if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
+    else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
     t += grown(3 * n_edges, 4);
     t += buf(N, 8) + buf(3 * N, 8) + buf(N, 4);
     const int64_t tiles = Bt > 0 ? (N + Bt - 1) / Bt : 0;

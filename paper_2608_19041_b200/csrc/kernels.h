@@ -116,7 +116,14 @@ struct MlpArgs {
     int* err;               // device error word
     int spin_limit;         // tensor-core path: polls before a pipeline wait gives up (0 = default)
     int test_skip_kblock;   // diagnostic, first layer of the forward pass only: see GemmArgs
+    float* fused_scratch;   // mlp_fused_scratch_floats(); null: one GEMM per layer
 };
+// mlp_fused.cu: forward layers, head and (grad) input gradient in one kernel.  Path 2, when the first layer has
+// no identity residual, a block's activations fit in shared memory (F <= 384) and n atoms are few enough for it
+// to be the faster way (true for n implies true for fewer).
+bool mlp_fused_pick(const Dims& d, int path, int64_t n, bool grad);
+int64_t mlp_fused_scratch_floats(const Dims& d, int64_t n_max);
+cudaError_t launch_mlp_fused(const MlpArgs& a, cudaStream_t st);
 cudaError_t launch_mlp_forward(const MlpArgs& a, cudaStream_t st);   // layers + head (+ backward seed)
 cudaError_t launch_mlp_backward(const MlpArgs& a, cudaStream_t st);  // needs a forward with want_grad
 

@@ -114,6 +114,7 @@ cudaError_t launch_mlp_forward(const MlpArgs& a, cudaStream_t st) {
     const Dims& d = a.d;
     const int n = a.n, F = d.F, NH = d.n_hidden;
     if (n <= 0) return cudaSuccess;
+    if (a.fused_scratch) return launch_mlp_fused(a, st);         // the backward pass is part of it
     const size_t layer = (size_t)n * F;
     float* hb[2] = {a.hbuf, a.hbuf + layer};
     const bool res0 = (d.D_out == F);
@@ -189,7 +190,7 @@ cudaError_t launch_mlp_forward(const MlpArgs& a, cudaStream_t st) {
 cudaError_t launch_mlp_backward(const MlpArgs& a, cudaStream_t st) {
     const Dims& d = a.d;
     const int n = a.n, F = d.F, NH = d.n_hidden;
-    if (n <= 0) return cudaSuccess;
+    if (n <= 0 || a.fused_scratch) return cudaSuccess;
     const size_t layer = (size_t)n * F;
     float* hb[2] = {a.hbuf, a.hbuf + layer};
     const bool res0 = (d.D_out == F);

@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "mlp_gemm.h"
+#include "tcgen05.cuh"
 
 namespace umd {
 
@@ -48,69 +49,6 @@ constexpr uint32_t BAR_BYTES = 128;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + BAR_BYTES;
 constexpr uint32_t TMEM_COLS = 256;                   // two accumulators: hi*hi, and the two cross terms
 constexpr int EPITCH = BN + 4;                        // epilogue staging pitch: 16-byte rows, odd in 16-byte units
-constexpr int kSpinLimit = 4000000;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Bounded wait.  After `limit` polls it gives up: the CTA's abort flag is raised, the error word
-// gets kErrPipelineTimeout, and from then on every wait of the CTA returns at once, the producer
-// stops issuing copies and the MMA warp stops issuing instructions, so that a wedged pipeline
-// ends with a wrong result and an error code instead of a hang.  Returns false on that path.
-__device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, int* err, volatile int* abort_flag, int limit) {
-    if (*abort_flag) return false;
-    for (int i = 0; i < limit; ++i) {
-        if (mbar_try(bar, parity)) return true;
-        if (i > 64) __nanosleep(32);
-    }
-    *abort_flag = 1;
-    if (err) atomicOr(err, kErrPipelineTimeout);
-    return false;
-}
-// plain bounded wait of the shutdown path (no flag, no error: the caller is already giving up)
-__device__ __forceinline__ void mbar_wait_quiet(uint32_t bar, uint32_t parity, int limit) {
-    for (int i = 0; i < limit; ++i) {
-        if (mbar_try(bar, parity)) return;
-        if (i > 64) __nanosleep(32);
-    }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
-}
-// shared-memory matrix descriptor: K-major tile, 64-byte swizzle, rows 64 B apart, 8-row
-// groups 512 B apart
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
-}
-__device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
     uint32_t r[32];
@@ -821,38 +759,6 @@ __global__ void k_split_f16(const float* __restrict__ A, int lda, int M, int K, 
         const float4 x = *reinterpret_cast<const float4*>(A + (size_t)m * lda + k);
         store_split4(hi, lo, (size_t)m * K + k, x);
     }
-}
-
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-    static EncodeFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeFn>(p);
-    }
-    return fn;
-}
-
-// 2-D map over a row-major [rows][cols] half-precision matrix with row pitch ld (elements); box =
-// 32 cols x 128 rows
-bool make_map(CUtensorMap* map, const __half* ptr, int rows, int cols, int ld, int box_rows = BM) {
-    EncodeFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {BK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
