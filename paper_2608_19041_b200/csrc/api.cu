@@ -33,6 +33,7 @@ struct umlmd {
     double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
     double* virial_part = nullptr; int64_t vpart_cap = 0;
     double* frame_out = nullptr; int64_t frame_out_cap = 0;     // batched evaluation: [n_frames][10] energy, virial
+    double* h_frame = nullptr; int64_t h_frame_cap = 0;         // pinned copy of it
     double* scratch = nullptr; double* d_out = nullptr; int* d_err = nullptr;
     double* h_out = nullptr; int* h_err = nullptr;      // pinned
     // per-pair amplitude tables of the species present (set up by umlmd_build_neighbors)
@@ -186,7 +187,8 @@ int decode_device_errors(umlmd_t* h, int word) {
 }
 
 // enqueue one full evaluation; results stay on the device (d_out[0] energy, d_out[1..9] virial)
-int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_force, double* d_atom_energy) {
+// (to_host: results and error word also go to h_out and h_err, and the word is cleared)
+int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_force, double* d_atom_energy, bool to_host = false) {
     const Dims& d = h->d;
     NeighborDev& nb = h->nb;
     const int N = (int)nb.N;
@@ -244,17 +246,20 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         Scope sc(h, kForce, 1);
         API_CUDA(h, launch_force_assembly(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, h->d_err, h->st));
     }
-    Scope sc(h, kReduce, (N <= 4096 ? 1 : 2) + (d_atom_energy ? 1 : 0));      // one reduction launch for a single slice of energies
-    API_CUDA(h, launch_reduce_energy_virial(h->e_atom, N, h->virial_part, vpart_used, h->scratch, h->d_out,
-                                            h->d_err, h->st));
-    if (d_atom_energy) API_CUDA(h, launch_scatter_atom_energy(nb, h->e_atom, d_atom_energy, h->st));
+    if (nb.batch) {                   // frames are reduced one by one
+        if (d_atom_energy) { Scope sc(h, kReduce, 1); API_CUDA(h, launch_scatter_atom_energy(nb, h->e_atom, d_atom_energy, h->st)); }
+        return UMLMD_OK;
+    }
+    Scope sc(h, kReduce, 1);
+    API_CUDA(h, launch_reduce_energy_virial(nb, h->e_atom, d_atom_energy, h->virial_part, vpart_used, h->scratch, (unsigned*)h->d_err + 1,
+                                            h->d_out, h->d_err, to_host ? h->h_out : nullptr, to_host ? h->h_err : nullptr, h->st));
     return UMLMD_OK;
 }
 
 // copy results and the error word to the host and clear the error word (enqueue_fetch), then
 // synchronise and decode (finish_fetch)
 int enqueue_fetch(umlmd_t* h, int n_out) {
-    API_CUDA(h, cudaMemcpyAsync(h->h_out, h->d_out, sizeof(double) * n_out, cudaMemcpyDeviceToHost, h->st));
+    if (n_out > 0) API_CUDA(h, cudaMemcpyAsync(h->h_out, h->d_out, sizeof(double) * n_out, cudaMemcpyDeviceToHost, h->st));
     API_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
     API_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
     return UMLMD_OK;
@@ -489,6 +494,7 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->h_out) cudaFreeHost(h->h_out);
     if (h->h_err) cudaFreeHost(h->h_err);
     if (h->h_species) cudaFreeHost(h->h_species);
+    if (h->h_frame) cudaFreeHost(h->h_frame);
     delete h;
     return UMLMD_OK;
 }
@@ -649,8 +655,7 @@ int umlmd_compute(umlmd_t* h, const double* d_pos, double* energy, double* d_for
         return UMLMD_OK;
     }
     int rc = run_replayed(h, h->rp_compute, d_pos, d_force, d_atom_energy, nullptr, 0.0, want_grad ? 1 : 0, [&]() {
-        int r = enqueue_compute(h, d_pos, want_grad, d_force, d_atom_energy);
-        return r != UMLMD_OK ? r : enqueue_fetch(h, 10);
+        return enqueue_compute(h, d_pos, want_grad, d_force, d_atom_energy, true);
     });
     if (rc != UMLMD_OK) return rc;
     rc = finish_fetch(h);
@@ -691,20 +696,26 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
         if ((rc = setup_pair_tables(h)) != UMLMD_OK) return rc;
         if ((rc = enqueue_compute(h, d_pos, want_grad, d_force, d_atom_energy)) != UMLMD_OK) return rc;
     }
-    API_CUDA(h, dev_ensure(&h->frame_out, &h->frame_out_cap, (int64_t)n_frames * 10));
+    const int64_t n_out = (int64_t)n_frames * 10;
+    API_CUDA(h, dev_ensure(&h->frame_out, &h->frame_out_cap, n_out));
+    if (n_out > h->h_frame_cap) {
+        if (h->h_frame) cudaFreeHost(h->h_frame);
+        h->h_frame = nullptr; h->h_frame_cap = 0;
+        API_CUDA(h, cudaMallocHost((void**)&h->h_frame, sizeof(double) * (size_t)n_out));
+        h->h_frame_cap = n_out;
+    }
     if (N > 0) {
         Scope sc(h, kReduce, 1);
-        API_CUDA(h, launch_frame_reduce(h->nb, h->e_atom, h->g, virials != nullptr, h->frame_out, h->st));
+        API_CUDA(h, launch_frame_reduce(h->nb, h->e_atom, h->g, virials != nullptr, h->frame_out, h->d_err, h->st));
     } else {
-        API_CUDA(h, cudaMemsetAsync(h->frame_out, 0, sizeof(double) * 10 * (size_t)n_frames, h->st));
+        API_CUDA(h, cudaMemsetAsync(h->frame_out, 0, sizeof(double) * (size_t)n_out, h->st));
     }
-    std::vector<double> host((size_t)n_frames * 10);
-    API_CUDA(h, cudaMemcpyAsync(host.data(), h->frame_out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->st));
-    if (N > 0) { if ((rc = fetch_results(h, 10)) != UMLMD_OK) return rc; }
+    API_CUDA(h, cudaMemcpyAsync(h->h_frame, h->frame_out, sizeof(double) * (size_t)n_out, cudaMemcpyDeviceToHost, h->st));
+    if (N > 0) { if ((rc = fetch_results(h, 0)) != UMLMD_OK) return rc; }
     else API_CUDA(h, cudaStreamSynchronize(h->st));
     for (int f = 0; f < n_frames; ++f) {
-        if (energies) energies[f] = host[10 * (size_t)f];
-        if (virials) for (int k = 0; k < 9; ++k) virials[9 * (size_t)f + k] = host[10 * (size_t)f + 1 + k];
+        if (energies) energies[f] = h->h_frame[10 * (size_t)f];
+        if (virials) for (int k = 0; k < 9; ++k) virials[9 * (size_t)f + k] = h->h_frame[10 * (size_t)f + 1 + k];
     }
     return UMLMD_OK;
 }
@@ -845,12 +856,12 @@ int umlmd_step_nvt(umlmd_t* h, int nsteps, double dt_ps, int rebuild_every, doub
         if ((rc = enqueue_compute(h, h->md_pos, true, h->md_force, nullptr)) != UMLMD_OK) return rc;
         h->have_force = true;
     }
-    double* d_ke = h->d_out + 10;
+    double* d_ke = h->d_out + 10;      // (only of a call without steps)
     double* d_scale = h->d_nhc + 2 * M;
     if (nsteps > 0) {      // opening half step of the chain for the first step
-        Scope sc(h, kIntegrate, 3);
-        API_CUDA(h, launch_kinetic_energy(N, h->md_vel, h->type_o, h->d_mass, h->scratch, d_ke, h->st));
-        API_CUDA(h, launch_nhc(h->d_nhc, d_ke, 1, p, h->st));
+        Scope sc(h, kIntegrate, 1);
+        API_CUDA(h, launch_kick_thermostat(N, h->md_vel, h->md_force, h->type_o, h->d_mass, h->d_inv_mass, dt_ps, false, h->scratch,
+                                           (unsigned*)h->d_err + 2, h->d_nhc, 1, p, h->st));
     }
     for (int s = 0; s < nsteps; ++s) {
         { Scope sc(h, kIntegrate, 1); API_CUDA(h, launch_vv_kick_drift(N, h->md_pos, h->md_vel, h->md_force, h->type_o, h->d_inv_mass, dt_ps, 1, true, d_scale, h->st)); }
@@ -860,11 +871,10 @@ int umlmd_step_nvt(umlmd_t* h, int nsteps, double dt_ps, int rebuild_every, doub
         auto body = [&]() {
             int r = enqueue_compute(h, h->md_pos, true, h->md_force, nullptr);
             if (r != UMLMD_OK) return r;
-            Scope sc(h, kIntegrate, 4);
-            API_CUDA(h, launch_vv_kick_drift(N, h->md_pos, h->md_vel, h->md_force, h->type_o, h->d_inv_mass, dt_ps, 1, false, nullptr, h->st));
-            API_CUDA(h, launch_kinetic_energy(N, h->md_vel, h->type_o, h->d_mass, h->scratch, d_ke, h->st));
-            // closing half step of the chain, and the next step's opening one in the same launch
-            API_CUDA(h, launch_nhc(h->d_nhc, d_ke, last ? 1 : 2, p, h->st));
+            Scope sc(h, kIntegrate, 1);
+            // closing half kick and half step of the chain, and the next step's opening one in the same launch
+            API_CUDA(h, launch_kick_thermostat(N, h->md_vel, h->md_force, h->type_o, h->d_mass, h->d_inv_mass, dt_ps, true, h->scratch,
+                                               (unsigned*)h->d_err + 2, h->d_nhc, last ? 1 : 2, p, h->st));
             return (int)UMLMD_OK;
         };
         // a middle step between two list builds launches the same sequence as the one before it (the

@@ -13,6 +13,8 @@ namespace {
 
 constexpr int kRedBlock = 256;
 constexpr int kRedMaxBlocks = 1024;
+constexpr int kReduceBlocks = 296;        // two per SM
+static_assert(kReduceBlocks * 10 >= kRedMaxBlocks, "one scratch area serves both kinds of reduction");
 
 // out (caller numbering, through perm) and / or f (sorted numbering) may be null
 __global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
@@ -147,71 +149,111 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return s;   // valid in thread 0
 }
 
+// Sums of K values over the threads of a block, in thread 0 .. K - 1's return value (sum of value
+// threadIdx.x); sh holds K doubles per warp.  Lanes by butterfly, then warps in order.
+template <int K>
+__device__ __forceinline__ double block_sums(double* v, double* sh) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+        if (lane == 0) sh[wid * K + k] = v[k];
+    }
+    __syncthreads();
+    double s = 0;
+    if (threadIdx.x < K) for (int w = 0; w < nw; ++w) s += sh[w * K + threadIdx.x];
+    return s;
+}
+
 // Segmented reduction of a batched evaluation: block f sums the atomic energies of frame f and,
 // when asked, -g (x) r over the edges of the frame's rows (edge vectors recomputed from the
-// positions and the frame's cell); thread-strided partial sums, then one fixed-order block sum.
-__global__ void __launch_bounds__(kRedBlock) k_frame_reduce(const FrameCell* __restrict__ frames, const double* __restrict__ e_atom,
-                                                            const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
-                                                            const float* __restrict__ g,
-                                                            const double* __restrict__ xs, bool want_virial,
-                                                            double* __restrict__ out) {
-    __shared__ double sh[kRedBlock / 32];
+// positions and the frame's cell): a warp per row, lanes over its edges, then one fixed-order block
+// sum.  Latency-bound: a frame is one block (64 frames of 54 to 108 atoms: 15 us; with a thread per row,
+// whose edges followed one another, 74 us).
+constexpr int kFrameBlock = 1024;
+__global__ void __launch_bounds__(kFrameBlock) k_frame_reduce(const FrameCell* __restrict__ frames, const double* __restrict__ e_atom,
+                                                              const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
+                                                              const float* __restrict__ g, const double* __restrict__ xs, bool want_virial,
+                                                              double* __restrict__ out, int* __restrict__ err) {
+    __shared__ double sh[kFrameBlock / 32 * 10];
     const FrameCell& fc = frames[blockIdx.x];
-    double e = 0, v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i = fc.a0 + threadIdx.x; i < fc.a1; i += kRedBlock) {
-        e += e_atom[i];
-        if (!want_virial) continue;
+    const int lane = threadIdx.x & 31;
+    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int i = fc.a0 + threadIdx.x; i < fc.a1; i += kFrameBlock) v[0] += e_atom[i];
+    for (int i = fc.a0 + (threadIdx.x >> 5); want_virial && i < fc.a1; i += kFrameBlock / 32) {
         const double xi = xs[3 * (size_t)i], yi = xs[3 * (size_t)i + 1], zi = xs[3 * (size_t)i + 2];
-        for (eidx_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-            const int j = nbr[k].x, s = nbr[k].y;
+        const eidx_t e1 = row_ptr[i + 1];
+        for (eidx_t k = row_ptr[i] + lane; k < e1; k += 32) {
+            const int2 js = nbr[k];
+            const int j = js.x, s = js.y;
             const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff), nz = (int)(signed char)((s >> 16) & 0xff);
             const double r[3] = {(xs[3 * (size_t)j] + ((nx * fc.H[0] + ny * fc.H[3]) + nz * fc.H[6])) - xi,
                                  (xs[3 * (size_t)j + 1] + ((nx * fc.H[1] + ny * fc.H[4]) + nz * fc.H[7])) - yi,
                                  (xs[3 * (size_t)j + 2] + ((nx * fc.H[2] + ny * fc.H[5]) + nz * fc.H[8])) - zi};
             const double gg[3] = {(double)g[3 * (size_t)k], (double)g[3 * (size_t)k + 1], (double)g[3 * (size_t)k + 2]};
+#pragma unroll
             for (int a = 0; a < 3; ++a)
-                for (int b = 0; b < 3; ++b) v[3 * a + b] += gg[a] * r[b];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) v[1 + 3 * a + b] += gg[a] * r[b];
         }
     }
-    const double es = block_sum(e, sh);
-    if (threadIdx.x == 0) out[10 * (size_t)blockIdx.x] = es;
-    for (int k = 0; k < 9; ++k) {
-        const double s = want_virial ? block_sum(v[k], sh) : 0.0;
-        if (threadIdx.x == 0) out[10 * (size_t)blockIdx.x + 1 + k] = -s;
+    const double s = block_sums<10>(v, sh);
+    if (threadIdx.x < 10) {
+        if (!isfinite(s)) atomicOr(err, kErrNonFinite);
+        out[10 * (size_t)blockIdx.x + threadIdx.x] = threadIdx.x ? -s : s;
     }
 }
 
-// pass 1: block b sums the contiguous slice [b*chunk, (b+1)*chunk) of x
-__global__ void __launch_bounds__(kRedBlock) k_sum_slices(const double* __restrict__ x, int64_t N, int64_t chunk,
-                                                          double* __restrict__ part) {
-    __shared__ double sh[kRedBlock / 32];
-    const int64_t lo = (int64_t)blockIdx.x * chunk;
-    const int64_t hi = lo + chunk < N ? lo + chunk : N;
-    double v = 0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += kRedBlock) v += x[i];
-    const double s = block_sum(v, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// pass 2 (ten blocks): block 0: out[0] = sum of slice partials; block 1 + k: out[1 + k] = -sum of
-// the k-th component of the virial partials
-__global__ void __launch_bounds__(kRedBlock) k_final_reduce(const double* __restrict__ part, int n_part,
-                                                            const double* __restrict__ vpart, int n_vpart,
-                                                            double* __restrict__ out, int* __restrict__ err) {
-    __shared__ double sh[kRedBlock / 32];
-    double v = 0;
-    if (blockIdx.x == 0) {
-        for (int i = threadIdx.x; i < n_part; i += kRedBlock) v += part[i];
-        const double s = block_sum(v, sh);
-        if (threadIdx.x == 0) {
-            out[0] = s;
-            if (!isfinite(s)) atomicOr(err, kErrNonFinite);
-        }
-    } else {
-        const int k = blockIdx.x - 1;
-        for (int i = threadIdx.x; i < n_vpart; i += kRedBlock) v += vpart[(size_t)i * 9 + k];
-        const double s = block_sum(v, sh);
-        if (threadIdx.x == 0) out[1 + k] = -s;
+// Energy and virial of an evaluation: out[0] = sum of the atomic energies, out[1 + k] = -sum of the k-th
+// component of the virial partials; e_out (may be null) receives the atomic energies in the caller's
+// numbering on the way.  Each block sums a strided share of both arrays; the last block to finish adds up
+// the blocks' sums in their order, so the result does not depend on which one it is.  h_out / h_err
+// (pinned host memory, may be null) get the results and the error word, which is then cleared: a caller
+// that waits for this call needs no copies.
+// Bound by latency (128,000 atoms, 32,000 partials of 72 bytes: 9.6 us; 108 atoms: 8.3 us.  One block per
+// component behind a pass over the energies took 28 and 11 us, and a copy of the energies 2.5 more).
+__global__ void __launch_bounds__(kRedBlock) k_reduce(const double* __restrict__ e_atom, int N, const int* __restrict__ perm,
+                                                      double* __restrict__ e_out, const double* __restrict__ vpart, int n_vpart,
+                                                      double* __restrict__ part, unsigned* __restrict__ done, double* __restrict__ out,
+                                                      int* __restrict__ err, double* __restrict__ h_out, int* __restrict__ h_err) {
+    __shared__ double sh[kRedBlock / 32 * 10];
+    __shared__ bool last;
+    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    const int first = blockIdx.x * kRedBlock + threadIdx.x, step = gridDim.x * kRedBlock;
+    for (int i = first; i < N; i += step) {
+        const double e = e_atom[i];
+        v[0] += e;
+        if (e_out) e_out[perm[i]] = e;
+    }
+    for (int i = first; i < n_vpart; i += step) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) v[1 + k] += vpart[(size_t)i * 9 + k];
+    }
+    const double s = block_sums<10>(v, sh);
+    if (threadIdx.x < 10) part[(size_t)blockIdx.x * 10 + threadIdx.x] = s;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < 10; ++k) v[k] = 0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedBlock) {
+#pragma unroll
+        for (int k = 0; k < 10; ++k) v[k] += __ldcg(part + (size_t)i * 10 + k);
+    }
+    const double t = block_sums<10>(v, sh);
+    if (threadIdx.x == 0 && !isfinite(t)) atomicOr(err, kErrNonFinite);
+    if (threadIdx.x < 10) {
+        const double r = threadIdx.x ? -t : t;
+        out[threadIdx.x] = r;
+        if (h_out) h_out[threadIdx.x] = r;
+    }
+    if (threadIdx.x == 0) {
+        *done = 0;
+        if (h_err) *h_err = atomicExch(err, 0);
     }
 }
 
@@ -237,15 +279,14 @@ __global__ void k_vv(int64_t N, double* __restrict__ pos, double* __restrict__ v
 }
 
 // Nose-Hoover chain of kNhcChain thermostats (Martyna-Tuckerman-Klein form): `halves` successive
-// half-step propagations of the chain given the current kinetic energy; returns the product of the
+// half-step propagations of the chain given the current kinetic energy; leaves the product of the
 // velocity scale factors and the kinetic energy after scaling.  One thread: the chain is a handful
 // of scalars.  st = [eta[M], v_eta[M], scale, kinetic energy]
-__global__ void k_nhc(double* __restrict__ st, const double* __restrict__ ke_in, int halves, NhcParams p) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__device__ void propagate_chain(double* __restrict__ st, double ke, int halves, const NhcParams& p) {
     constexpr int M = kNhcChain;
     double* eta = st;
     double* v = st + M;
-    double ke2 = 2.0 * (ke_in ? *ke_in : st[2 * M + 1]);
+    double ke2 = 2.0 * ke;
     double scale = 1.0;
     const double d2 = p.dt_half, d4 = 0.5 * d2, d8 = 0.25 * d2;
     for (int h = 0; h < halves; ++h) {
@@ -272,6 +313,46 @@ __global__ void k_nhc(double* __restrict__ st, const double* __restrict__ ke_in,
     st[2 * M + 1] = 0.5 * ke2;
 }
 
+// The closing half kick of a thermostatted step (kick), the kinetic energy after it and the chain's
+// propagation, in one launch: blocks sum a strided share, the last one to finish adds up the blocks'
+// sums in their order and propagates the chain.  Latency-bound: 9.0 us at 128,000 atoms (kick, sum in two
+// passes and chain as four launches took 6.8 + 14.3 + 2.6 + 3.6 us at 216,000).
+__global__ void __launch_bounds__(kRedBlock) k_kick_thermostat(int64_t N, double* __restrict__ vel, const double* __restrict__ force,
+                                                               const int* __restrict__ type, const double* __restrict__ mass,
+                                                               const double* __restrict__ inv_mass, double dt, bool kick,
+                                                               double* __restrict__ part, unsigned* __restrict__ done,
+                                                               double* __restrict__ st, int halves, NhcParams p) {
+    __shared__ double sh[kRedBlock / 32];
+    __shared__ bool last;
+    double v[1] = {0};
+    for (int64_t i = (int64_t)blockIdx.x * kRedBlock + threadIdx.x; i < N; i += (int64_t)gridDim.x * kRedBlock) {
+        const int t = type[i];
+        double u[3];
+        const double c = 0.5 * dt * kAccelUnit * inv_mass[t];
+        for (int k = 0; k < 3; ++k) {
+            u[k] = vel[3 * i + k];
+            if (kick) { u[k] = u[k] + c * force[3 * i + k]; vel[3 * i + k] = u[k]; }
+        }
+        v[0] += 0.5 * mass[t] * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) / kAccelUnit;
+    }
+    const double s = block_sums<1>(v, sh);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    v[0] = 0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedBlock) v[0] += __ldcg(part + i);
+    const double ke = block_sums<1>(v, sh);
+    if (threadIdx.x == 0) {
+        *done = 0;
+        propagate_chain(st, ke, halves, p);
+    }
+}
+
 __global__ void __launch_bounds__(kRedBlock) k_ke_slices(const double* __restrict__ vel, const int* __restrict__ type,
                                                          const double* __restrict__ mass, int64_t N, int64_t chunk,
                                                          double* __restrict__ part) {
@@ -296,7 +377,7 @@ __global__ void __launch_bounds__(kRedBlock) k_sum_small(const double* __restric
 }
 
 inline void slices(int64_t N, int* blocks, int64_t* chunk) {
-    int64_t b = (N + 4095) / 4096;
+    int64_t b = (N + 1023) / 1024;       // four atoms per thread, up to the 1024 partials there is room for
     if (b < 1) b = 1;
     if (b > kRedMaxBlocks) b = kRedMaxBlocks;
     *blocks = (int)b;
@@ -305,7 +386,7 @@ inline void slices(int64_t N, int* blocks, int64_t* chunk) {
 
 }  // namespace
 
-int reduce_scratch_doubles(int64_t) { return kRedMaxBlocks; }
+int reduce_scratch_doubles(int64_t) { return kReduceBlocks * 10; }      // (more than kRedMaxBlocks)
 
 // forces in sorted numbering (f_sorted) and / or scattered to the caller's numbering (d_force)
 cudaError_t launch_force_assembly(const NeighborDev& nb, const float* g, double* f_sorted, double* d_force,
@@ -333,32 +414,26 @@ cudaError_t launch_scatter_forces(const NeighborDev& nb, const double* f_sorted,
     return cudaGetLastError();
 }
 
+cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
+                                double* d_out, int* d_err, cudaStream_t st) {
+    if (nb.n_frames <= 0) return cudaSuccess;
+    k_frame_reduce<<<nb.n_frames, kFrameBlock, 0, st>>>(nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial, d_out, d_err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part,
+                                        int n_part, double* scratch, unsigned* counter, double* out, int* d_err, double* h_out,
+                                        int* h_err, cudaStream_t st) {
+    const int N = (int)nb.N, blocks = (N + 4 * kRedBlock - 1) / (4 * kRedBlock);
+    k_reduce<<<blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks), kRedBlock, 0, st>>>(
+        e_atom, N, nb.perm, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out, cudaStream_t st) {
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
     k_scatter1<<<(N + 255) / 256, 256, 0, st>>>(N, nb.perm, e_sorted, d_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
-                                double* d_out, cudaStream_t st) {
-    if (nb.n_frames <= 0) return cudaSuccess;
-    k_frame_reduce<<<nb.n_frames, kRedBlock, 0, st>>>(nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial, d_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_energy_virial(const double* e_atom, int64_t N, const double* virial_part, int n_part,
-                                        double* scratch, double* out, int* d_err, cudaStream_t st) {
-    int blocks; int64_t chunk;
-    slices(N, &blocks, &chunk);
-    if (blocks == 1) {
-        // a single slice: the second pass sums the atomic energies itself, in the order the first
-        // pass would have used (its own sum over one partial only adds zeros), and one launch less
-        k_final_reduce<<<10, kRedBlock, 0, st>>>(e_atom, (int)N, virial_part, n_part, out, d_err);
-        return cudaGetLastError();
-    }
-    k_sum_slices<<<blocks, kRedBlock, 0, st>>>(e_atom, N, chunk, scratch);
-    k_final_reduce<<<10, kRedBlock, 0, st>>>(scratch, blocks, virial_part, n_part, out, d_err);
     return cudaGetLastError();
 }
 
@@ -385,8 +460,12 @@ cudaError_t launch_vv_kick_drift(int64_t N, double* pos, double* vel, const doub
     return cudaGetLastError();
 }
 
-cudaError_t launch_nhc(double* d_state, const double* d_ke, int halves, const NhcParams& p, cudaStream_t st) {
-    k_nhc<<<1, 32, 0, st>>>(d_state, d_ke, halves, p);
+cudaError_t launch_kick_thermostat(int64_t N, double* vel, const double* force, const int* type, const double* mass,
+                                   const double* inv_mass, double dt, bool kick, double* scratch, unsigned* counter, double* d_state,
+                                   int halves, const NhcParams& p, cudaStream_t st) {
+    const int64_t blocks = (N + 2 * kRedBlock - 1) / (2 * kRedBlock);
+    k_kick_thermostat<<<(unsigned)(blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks)), kRedBlock, 0, st>>>(
+        N, vel, force, type, mass, inv_mass, dt, kick, scratch, counter, d_state, halves, p);
     return cudaGetLastError();
 }
 

@@ -33,7 +33,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
 // per-frame energy and virial: out[10 f] = sum of e_atom over the frame, out[10 f + 1 ..] = -sum over
 // the frame's edges of g (x) r, each by one block in a fixed order
 cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
-                                double* d_out, cudaStream_t st);
+                                double* d_out, int* d_err, cudaStream_t st);
 // Rows first .. first + n - 1 of the caller's numbering with 64-bit offsets: d_row_ptr [n + 1] is
 // always filled; edges are copied while they fit `cap` (cap = 0 or null buffers: offsets only).
 int neighbor_export_rows(NeighborDev* nb, int64_t first, int64_t n, int64_t* d_row_ptr, int32_t* d_src,
@@ -140,10 +140,12 @@ cudaError_t launch_scatter_forces(const NeighborDev& nb, const double* f_sorted,
                                   int* d_err, cudaStream_t st);
 cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out,
                                        cudaStream_t st);
-// out[0] = sum e_atom, out[1..9] = -sum virial partials (fixed order, double)
-cudaError_t launch_reduce_energy_virial(const double* e_atom, int64_t N, const double* virial_part,
-                                        int n_part, double* scratch, double* out, int* d_err,
-                                        cudaStream_t st);
+// out[0] = sum e_atom, out[1..9] = -sum virial partials (fixed order, double), in one launch; the atomic
+// energies go to d_atom_energy (caller's numbering, may be null) on the way.  counter: a zero that comes
+// back as zero.  h_out, h_err (pinned, may be null): results and error word for the host; clears the word.
+cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part,
+                                        int n_part, double* scratch, unsigned* counter, double* out, int* d_err, double* h_out,
+                                        int* h_err, cudaStream_t st);
 int reduce_scratch_doubles(int64_t N);
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width,
                                 float* out, cudaStream_t st);
@@ -155,7 +157,10 @@ cudaError_t launch_vv_kick_drift(int64_t N, double* pos, double* vel, const doub
 // propagation of `halves` half steps on the device; d_state = [eta[M], v_eta[M], scale, kinetic energy]
 constexpr int kNhcChain = 3;
 struct NhcParams { double dof, kT, Q[kNhcChain], dt_half; };
-cudaError_t launch_nhc(double* d_state, const double* d_ke, int halves, const NhcParams& p, cudaStream_t st);
+// closing half kick (if kick), kinetic energy and `halves` half-step propagations of the chain, one launch
+cudaError_t launch_kick_thermostat(int64_t N, double* vel, const double* force, const int* type, const double* mass,
+                                   const double* inv_mass, double dt, bool kick, double* scratch, unsigned* counter, double* d_state,
+                                   int halves, const NhcParams& p, cudaStream_t st);
 cudaError_t launch_kinetic_energy(int64_t N, const double* vel, const int* type, const double* mass,
                                   double* scratch, double* out, cudaStream_t st);
 
