@@ -46,7 +46,7 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     g.dx = g.dy = g.dz = 0.f; g.rho = 1.f; g.inv_rho = 1.f; g.ux = g.uy = g.uz = 0.f;
     g.chi = 0.f; g.dchi = 0.f; g.t = 0.f; g.row = 0; g.pair = 0;
     if (!in_range) return g;
-    const int2 js = __ldg(a.nbr + e);
+    const int2 js = a.nbr[e];      // (through the read-only path the forward kernel's loads were scheduled 6 % slower at C0 = 128)
     const int j = js.x, s = js.y;
     const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff),
               nz = (int)(signed char)((s >> 16) & 0xff);
@@ -196,9 +196,9 @@ __device__ __forceinline__ void table_eval1(const float* __restrict__ table, int
 }
 
 // Shared radial modes q_mu(rho) (and derivatives) of the first nb queued edges, one (edge, mode)
-// pair per lane, parked as qm[edge * kMaxR + mu]: evaluated once per edge here instead of once
+// pair per lane, parked as qm[edge * PQ + mu]: evaluated once per edge here instead of once
 // per lane in the channel-parallel phase.
-template <bool DERIV>
+template <bool DERIV, int PQ>
 __device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, int nb, int lane, float* qm, float* dqm) {
     const int R = a.d.R;
     for (int idx = lane; idx < nb * R; idx += 32) {
@@ -206,8 +206,8 @@ __device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, i
         const int4 es = qes[b];
         float qv, dqv = 0.f;
         table_eval1<DERIV>(a.table, a.d.CP, es.x, a.d.C0 + q, __int_as_float(es.z), a.d.tab_k2, a.d.tab_k3, &qv, &dqv);
-        qm[b * kMaxR + q] = qv;
-        if (DERIV) dqm[b * kMaxR + q] = dqv;
+        qm[b * PQ + q] = qv;
+        if (DERIV) dqm[b * PQ + q] = dqv;
     }
 }
 
@@ -265,22 +265,29 @@ template <int C0, int L, int G = 1> struct Widths {
     static constexpr int EPI = 32 / LPE;        // edges per replay step
     static constexpr int NL1 = C1 / 4;          // lanes of a group that hold degree-1 channels
     static constexpr int NHI = 3 * C1 + 5 * C2 + (L >= 3 ? 7 : 0) + (L >= 4 ? 9 : 0);   // sums of degree >= 1
-    static constexpr int NCH = (NHI + 31) / 32;
-    // row pitch (floats) of the per-edge amplitude staging; pitch/4 odd keeps 16-byte
-    // accesses of 8 consecutive lanes on distinct bank groups
-    // (forward, C0 = 128: a whole warp works on one edge, rows are written one or two at a time and
-    // read one at a time, so no padding is needed, and with degree 4 none fits in 48 KB)
-    static constexpr int PF = C0 / (4 * G) == 32 ? C1 : (((C1 / 4 + 1) & 1) ? C1 + 4 : C1 + 8);   // forward: psi
     static constexpr int PB = ((2 * C1 / 4 + 1) & 1) ? 2 * C1 + 4 : 2 * C1 + 8;   // backward: psi, dpsi
-    // forward, sums of degree >= 1: a job is four consecutive channels of one harmonic component
-    // (degrees 1 and 2) or one component of a one-channel degree (3, 4); a lane owns up to SLOTS jobs
-    static constexpr int J1 = 3 * (C1 / 4), J2 = 5 * (C2 / 4), J3 = L >= 3 ? 7 : 0, J4 = L >= 4 ? 9 : 0;
+    // Forward, sums of degree >= 1: a job is four multiply-adds per edge, a vector times a scalar.  Degrees 1
+    // and 2: four consecutive channels (vector) of one harmonic component (scalar).  Degrees 3 and 4 have
+    // one channel: where VECW, four components (vector) of it, else one component.  Below C0 = 128 the jobs
+    // are at most sixteen, so that EG groups of JW lanes take every EG-th edge each (with one group, 8 to 18
+    // lanes of 32 worked, over all edges: the forward kernel of 216,000 atoms with 158 neighbours at C0 = 8
+    // took 1.109 ms, so 0.867; C0 = 64: 4000 atoms 31.4 -> 29.1 us, 32,400 atoms with degree three 201 -> 198).
+    static constexpr bool VECW = C0 <= 64;
+    static constexpr int J1 = 3 * (C1 / 4), J2 = 5 * (C2 / 4), J3 = L >= 3 ? (VECW ? 2 : 7) : 0, J4 = L >= 4 ? (VECW ? 3 : 9) : 0;
     static constexpr int NJ = J1 + J2 + J3 + J4;
-    static constexpr int SLOTS = (NJ + 31) / 32;
-    static constexpr int NM = 3 + 5 + J3 + J4;  // harmonic components of all degrees >= 1
-    static constexpr int PW = NM | 1;           // odd row pitch of the parked weights
-    static constexpr int WOFF = 32 * PF;        // they sit behind the parked amplitudes (where the radial modes were)
-    static constexpr int SCRATCH = 32 * PF + (32 * PW > 32 * kMaxR ? 32 * PW : 32 * kMaxR);
+    static constexpr int JW = NJ <= 8 ? 8 : (NJ <= 16 ? 16 : 32), EG = 32 / JW;
+    static constexpr int SLOTS = (NJ + JW - 1) / JW;
+    // the parked row of an edge: leading C1 amplitudes, harmonic weights (degree 3 from 8 on, degree 4 from
+    // 15, or 16 where VECW).  VECW: one row, pitch / 4 odd, so that 16-byte accesses of eight consecutive
+    // lanes fall on distinct banks.  C0 = 128: a whole warp works on one edge, amplitude rows need no padding,
+    // and the weights sit behind them with an odd pitch, which takes less room (L1 is what is left over).
+    static constexpr int O4 = VECW ? 16 : 15;
+    static constexpr int NM = L >= 4 ? O4 + (VECW ? 12 : 9) : (L >= 3 ? (VECW ? 16 : 15) : 8);
+    static constexpr int PP = VECW ? (((C1 + NM) / 4) & 1 ? C1 + NM : C1 + NM + 4) : C1;      // pitch of the amplitudes
+    static constexpr int PW = VECW ? PP : (NM | 1);                                           // pitch of the weights
+    static constexpr int OW = VECW ? C1 : 32 * C1;                                            // offset of the weights
+    static constexpr int PQ = VECW ? PP : kMaxR;     // the radial modes sit where the weights come later
+    static constexpr int SCRATCH = VECW ? 32 * PP : 32 * C1 + (32 * PW > 32 * kMaxR ? 32 * PW : 32 * kMaxR);
 };
 
 // The channel-parallel phase of the backward pass waits on load latency, and what hides it best
@@ -309,10 +316,10 @@ template <int C0, int L, bool HASR> struct BwdSmem {          // dynamic shared 
 //      degree-0 sums accumulated in registers; the leading C1 amplitudes of each edge are
 //      parked in shared memory.
 //   3. lane = edge again: harmonics of the lane's own edge, parked as weights chi^2 B_lm; then
-//      lane = job: a lane owns four consecutive channels of one harmonic component (or one
-//      component of a one-channel degree) for the whole row, and for every edge of the batch adds
-//      weight x amplitudes from the two parked rows: two shared-memory reads per edge and warp,
-//      where summing per-edge products by transposition took six.
+//      lane = job: a lane owns four consecutive channels of one harmonic component (or up to four
+//      components of a one-channel degree) for the whole row, and for every edge of its group of
+//      edges adds vector x scalar from the parked row: two shared-memory reads per edge and group of
+//      lanes, where summing per-edge products by transposition took six.
 // Up to C0 = 64 a fourth group of eight resident warps per SM (64 registers, a few spilled words) is worth more
 // than the registers: the channel-parallel phase waits on load latency (measured: 6-10 % on the
 // forward kernel at C0 = 8 .. 64, 2 % the other way at C0 = 128, which stays at 24 warps).
@@ -320,8 +327,8 @@ template <int C0, int L, bool HASR, bool UNI>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 ? 4 : 3) * 8 / kWarpsPerBlock)
 k_edge_forward(const EdgeArgs a) {
     using W = Widths<C0, L>;
-    // scratch per warp: the parked amplitudes of the batch (row pitch PF), and behind them first the
-    // radial modes, then (once the amplitudes are done) the harmonic weights chi^2 B_lm (row pitch PW)
+    // scratch per warp: the parked amplitudes of the batch, first the radial modes and then (once the
+    // amplitudes are done) the harmonic weights chi^2 B_lm
     __shared__ __align__(16) float scratch[kWarpsPerBlock][W::SCRATCH];
     // queue of edges inside the cutoff: row, pair, t, chi (fetched with one 16-byte broadcast
     // load in the channel-parallel phase; shuffles would go through the same L1 data pipe as
@@ -331,9 +338,9 @@ k_edge_forward(const EdgeArgs a) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = a.a0 + blockIdx.x * kWarpsPerBlock + wid;
     if (i >= a.a1) return;
-    float* const psi_s = scratch[wid];      // [32][PF]
-    float* const qm = scratch[wid] + W::WOFF;      // [32][kMaxR] radial modes, behind the parked amplitudes
-    float* const wbs = scratch[wid] + W::WOFF;     // [32][PW] harmonic weights, in the same place later
+    float* const psi_s = scratch[wid];             // [32][PP]
+    float* const qm = scratch[wid] + W::OW;        // [32][PQ] radial modes
+    float* const wbs = scratch[wid] + W::OW;       // [32][PW] harmonic weights, in the same place later
     int4* const qes = q_es[wid];
     float* const qd = q_d[wid];
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
@@ -345,32 +352,40 @@ k_edge_forward(const EdgeArgs a) {
     const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
     const unsigned lt_mask = (1u << lane) - 1u;
     float acc0[4] = {0.f, 0.f, 0.f, 0.f};
-    // this lane's jobs of the degree >= 1 sums: offset of the four channels in an amplitude row,
-    // of the component in a weight row, of the result in the output block (negative: no job)
+    // this lane's jobs of the degree >= 1 sums: where its vector and its scalar are in the rows of edge 0, offset
+    // of the result in the output block, number of results (0: no job)
     float accJ[W::SLOTS][4];
-    int j_psi[W::SLOTS], j_w[W::SLOTS], j_out[W::SLOTS];
+    int j_v[W::SLOTS], j_s[W::SLOTS], j_out[W::SLOTS], j_n[W::SLOTS];
+    const int eg = lane / W::JW;
 #pragma unroll
     for (int sl = 0; sl < W::SLOTS; ++sl) {
         accJ[sl][0] = accJ[sl][1] = accJ[sl][2] = accJ[sl][3] = 0.f;
-        const int j = lane + 32 * sl;
+        const int j = lane % W::JW + W::JW * sl;
+        j_v[sl] = 0; j_s[sl] = W::OW; j_out[sl] = 0; j_n[sl] = 0;
         if (j < W::J1) {
             const int m = j / (W::C1 / 4), cb = j % (W::C1 / 4);
-            j_psi[sl] = 4 * cb; j_w[sl] = m; j_out[sl] = m * W::C1 + 4 * cb;
+            j_v[sl] = 4 * cb; j_s[sl] += m; j_out[sl] = m * W::C1 + 4 * cb; j_n[sl] = 4;
         } else if (j < W::J1 + W::J2) {
             const int jj = j - W::J1, m = jj / (W::C2 / 4), cb = jj % (W::C2 / 4);
-            j_psi[sl] = 4 * cb; j_w[sl] = 3 + m; j_out[sl] = 3 * W::C1 + m * W::C2 + 4 * cb;
+            j_v[sl] = 4 * cb; j_s[sl] += 3 + m; j_out[sl] = 3 * W::C1 + m * W::C2 + 4 * cb; j_n[sl] = 4;
         } else if (j < W::NJ) {
-            const int m = j - W::J1 - W::J2;             // degrees 3 and 4 follow each other in both layouts
-            j_psi[sl] = 0; j_w[sl] = 8 + m; j_out[sl] = 3 * W::C1 + 5 * W::C2 + m;
-        } else {
-            j_psi[sl] = 0; j_w[sl] = 0; j_out[sl] = -1;
+            const int jj = j - W::J1 - W::J2;
+            const bool deg3 = jj < W::J3;
+            const int first = W::VECW ? (deg3 ? 4 * jj : 4 * (jj - W::J3)) : (deg3 ? jj : jj - W::J3);   // component
+            j_out[sl] = 3 * W::C1 + 5 * W::C2 + (deg3 ? 0 : 7) + first;
+            if (W::VECW) {                  // vector: the weights, scalar: the channel's amplitude
+                j_v[sl] = W::OW + (deg3 ? 8 : W::O4) + first; j_s[sl] = 0;      // (one pitch for both)
+                j_n[sl] = min(4, (deg3 ? 7 : 9) - first);
+            } else {
+                j_s[sl] += (deg3 ? 8 : W::O4) + first; j_n[sl] = 1;
+            }
         }
     }
     double s0 = 0.0, s1 = 0.0;   // normaliser sums in double: the calibration subtracts their mean
 
     auto run_batch = [&](const int nb) {     // the first nb queue slots
         if (HASR) {
-            eval_modes<false>(a, qes, nb, lane, qm, nullptr);
+            eval_modes<false, W::PQ>(a, qes, nb, lane, qm, nullptr);
             __syncwarp();
         }
         int it = 0;
@@ -388,8 +403,8 @@ k_edge_forward(const EdgeArgs a) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc0[k] += cb * pb[k];
                 if (cl < W::NL1) {
-                    *reinterpret_cast<float4*>(psi_s + it * W::PF + c) = make_float4(pa[0], pa[1], pa[2], pa[3]);
-                    *reinterpret_cast<float4*>(psi_s + (it + 1) * W::PF + c) = make_float4(pb[0], pb[1], pb[2], pb[3]);
+                    *reinterpret_cast<float4*>(psi_s + it * W::PP + c) = make_float4(pa[0], pa[1], pa[2], pa[3]);
+                    *reinterpret_cast<float4*>(psi_s + (it + 1) * W::PP + c) = make_float4(pb[0], pb[1], pb[2], pb[3]);
                 }
             }
         }
@@ -400,11 +415,11 @@ k_edge_forward(const EdgeArgs a) {
             const int row = es.x, pair = es.y;
             const float t = __int_as_float(es.z), chi = __int_as_float(es.w);
             float psi[4];
-            amplitude4<C0, HASR, false, UNI>(a, row, t, pair, c, psi, nullptr, qm + b * kMaxR, nullptr, k2, k3);
+            amplitude4<C0, HASR, false, UNI>(a, row, t, pair, c, psi, nullptr, qm + b * W::PQ, nullptr, k2, k3);
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc0[k] += chi * psi[k];
             if (cl < W::NL1)
-                *reinterpret_cast<float4*>(psi_s + b * W::PF + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
+                *reinterpret_cast<float4*>(psi_s + b * W::PP + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
         }
         __syncwarp();
         // lane = edge: the harmonic weights chi^2 B_lm of the lane's edge, parked next to the amplitudes
@@ -416,28 +431,43 @@ k_edge_forward(const EdgeArgs a) {
             const float chi = __int_as_float(qes[lane].w);
             const float w = chi * chi;
             float* wr = wbs + lane * W::PW;
+            if (W::VECW) {
+                float4* w4 = reinterpret_cast<float4*>(wr);
+                w4[0] = make_float4(w * B1[0], w * B1[1], w * B1[2], w * B2[0]);
+                w4[1] = make_float4(w * B2[1], w * B2[2], w * B2[3], w * B2[4]);
+                if (L >= 3) {
+                    w4[2] = make_float4(w * B3[0], w * B3[1], w * B3[2], w * B3[3]);
+                    w4[3] = make_float4(w * B3[4], w * B3[5], w * B3[6], 0.f);
+                }
+                if (L >= 4) {
+                    w4[4] = make_float4(w * B4[0], w * B4[1], w * B4[2], w * B4[3]);
+                    w4[5] = make_float4(w * B4[4], w * B4[5], w * B4[6], w * B4[7]);
+                    w4[6] = make_float4(w * B4[8], 0.f, 0.f, 0.f);
+                }
+            } else {
 #pragma unroll
-            for (int m = 0; m < 3; ++m) wr[m] = w * B1[m];
+                for (int m = 0; m < 3; ++m) wr[m] = w * B1[m];
 #pragma unroll
-            for (int m = 0; m < 5; ++m) wr[3 + m] = w * B2[m];
-            if (L >= 3) {
+                for (int m = 0; m < 5; ++m) wr[3 + m] = w * B2[m];
+                if (L >= 3) {
 #pragma unroll
-                for (int m = 0; m < 7; ++m) wr[8 + m] = w * B3[m];
-            }
-            if (L >= 4) {
+                    for (int m = 0; m < 7; ++m) wr[8 + m] = w * B3[m];
+                }
+                if (L >= 4) {
 #pragma unroll
-                for (int m = 0; m < 9; ++m) wr[15 + m] = w * B4[m];
+                    for (int m = 0; m < 9; ++m) wr[W::O4 + m] = w * B4[m];
+                }
             }
         }
         __syncwarp();
-        // lane = job: the sums over the batch stay in the lane's registers for the whole row; per edge
-        // a lane reads its four amplitudes and its weight (every lane inside the same two rows)
+        // lane = job: the sums over the batch stay in the lane's registers for the whole row; per edge of
+        // its group a lane reads its vector and its scalar (every lane of a group inside the same two rows)
 #pragma unroll 4
-        for (int e = 0; e < nb; ++e) {
+        for (int e = eg; e < nb; e += W::EG) {
 #pragma unroll
             for (int sl = 0; sl < W::SLOTS; ++sl) {
-                const float4 p4 = *reinterpret_cast<const float4*>(psi_s + e * W::PF + j_psi[sl]);
-                const float wv = wbs[e * W::PW + j_w[sl]];
+                const float4 p4 = *reinterpret_cast<const float4*>(psi_s + e * W::PP + j_v[sl]);
+                const float wv = psi_s[e * W::PW + j_s[sl]];
                 accJ[sl][0] += wv * p4.x; accJ[sl][1] += wv * p4.y; accJ[sl][2] += wv * p4.z; accJ[sl][3] += wv * p4.w;
             }
         }
@@ -482,10 +512,18 @@ k_edge_forward(const EdgeArgs a) {
     if (sub == 0) *reinterpret_cast<float4*>(row_out + c) = make_float4(acc0[0], acc0[1], acc0[2], acc0[3]);
 #pragma unroll
     for (int sl = 0; sl < W::SLOTS; ++sl) {
-        if (j_out[sl] < 0) continue;
+#pragma unroll
+        for (int off = W::JW; off < 32; off <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) accJ[sl][k] += __shfl_xor_sync(kFull, accJ[sl][k], off);
+        }
+        if (eg != 0 || j_n[sl] == 0) continue;
         float* o = row_out + a.d.offA[1] + j_out[sl];
-        if (lane + 32 * sl < W::J1 + W::J2) *reinterpret_cast<float4*>(o) = make_float4(accJ[sl][0], accJ[sl][1], accJ[sl][2], accJ[sl][3]);
-        else o[0] = accJ[sl][0];
+        if (lane + W::JW * sl < W::J1 + W::J2) *reinterpret_cast<float4*>(o) = make_float4(accJ[sl][0], accJ[sl][1], accJ[sl][2], accJ[sl][3]);
+        else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) if (k < j_n[sl]) o[k] = accJ[sl][k];
+        }
     }
     if (lane == 0) {
         const float h0 = (float)s0, h1 = (float)s1;
@@ -550,7 +588,7 @@ k_edge_backward(const EdgeArgs a) {
 
         auto run_batch = [&](const int nb) {     // the first nb queue slots
             if (HASR) {
-                eval_modes<true>(a, qes, nb, lane, qm, qm + 32 * kMaxR);
+                eval_modes<true, kMaxR>(a, qes, nb, lane, qm, qm + 32 * kMaxR);
                 __syncwarp();
             }
             for (int it = 0; it * W::EPI < nb; ++it) {
