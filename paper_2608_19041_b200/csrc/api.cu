@@ -132,8 +132,7 @@ void fill_info(const Dims& d, umlmd_info* o) {
     o->H = d.H; o->H_pair = d.Hp; o->table_rows = d.n_rows;
 }
 
-// the fp32 feature rows and the state of a small single-tile system stay readable after an
-// evaluation (umlmd_get_intermediates); larger systems skip the copy nothing else reads
+// the state of a small single-tile system stays readable after an evaluation (umlmd_get_intermediates)
 constexpr int64_t kIntermediatesMaxAtoms = 65536;
 bool keeps_intermediates(const umlmd_t* h) { return h->nb.N < kIntermediatesMaxAtoms && h->nb.N <= h->node_tile; }
 
@@ -214,13 +213,12 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         { Scope sc(h, kEdgeFwd, 1); API_CUDA(h, launch_edge_forward(ea, h->st)); }
         InvArgs ia;
         ia.d = d; ia.m = h->md; ia.type_s = nb.type_s; ia.a0 = a0; ia.n = n; ia.state = h->state; ia.desc = h->desc;
-        // tensor-core MLP: the invariants kernel writes the first GEMM's operand split itself; the
-        // fp32 feature rows are then only kept where something still reads them (the identity
-        // residual of a first layer as wide as the feature vector, or the intermediates query of a
-        // system smaller than one node tile)
+        // tensor-core MLP: the invariants kernel writes the first GEMM's operand split itself, and the fp32
+        // feature rows only where something still reads them (the identity residual of a first layer as wide
+        // as the feature vector; umlmd_get_intermediates makes its own from the state)
         const bool presplit = mlp_uses_tc(d.F, h->mlp_path);
         ia.desc_hi = presplit ? h->tc_hi : nullptr; ia.desc_lo = presplit ? h->tc_lo : nullptr;
-        ia.write_desc = !presplit || d.D_out == d.F || keeps_intermediates(h);
+        ia.write_desc = !presplit || d.D_out == d.F;
         const bool fold_x0 = presplit && d.D_out != d.F;      // first GEMM skips the per-species constant columns
         ia.skip_x0_split = fold_x0;
         { Scope sc(h, kInvFwd, 1); API_CUDA(h, launch_invariants_forward(ia, h->st)); }
@@ -942,6 +940,12 @@ int umlmd_get_intermediates(umlmd_t* h, float* d_state, float* d_desc) {
     if (!h->have_list) return fail(h, UMLMD_E_NO_NEIGHBORS, "no neighbor list built");
     if (!keeps_intermediates(h)) return fail(h, UMLMD_E_CAPACITY, "intermediates are only kept for systems of one tile and fewer than 65536 atoms");
     if (d_state) API_CUDA(h, launch_unsort_state(h->nb, h->state, h->d.SP, h->d.S + 2, d_state, h->st));
+    if (d_desc && !h->have_edge_grad && h->nb.n_owned > 0) {      // (after a backward pass both buffers hold gradients)
+        InvArgs ia = {};
+        ia.d = h->d; ia.m = h->md; ia.type_s = h->nb.type_s; ia.a0 = 0; ia.n = (int)h->nb.n_owned; ia.state = h->state; ia.desc = h->desc;
+        ia.write_desc = true;
+        API_CUDA(h, launch_invariants_forward(ia, h->st));
+    }
     if (d_desc) API_CUDA(h, launch_unsort_state(h->nb, h->desc, h->d.DP, h->d.D_out, d_desc, h->st));
     API_CUDA(h, cudaStreamSynchronize(h->st));
     return UMLMD_OK;

@@ -4,7 +4,7 @@
 // invariant, assembly and diagonal calibration -- and the matching vector-Jacobian
 // product, which turns dE/dD into dE/d(sums) in place of the saved sums.
 //
-// A block handles 32 atoms with eight warps, lane = atom.  All per-atom tensors live in
+// A block handles 32 atoms with eight or sixteen warps, lane = atom.  All per-atom tensors live in
 // shared memory in an [index][atom] layout with row pitch 33, so a warp that reads or
 // writes one index for its 32 atoms touches 32 distinct banks, and every index computation
 // is uniform over the warp.  The work of a phase is cut into units (an output row, a pair
@@ -32,8 +32,7 @@ namespace umd {
 namespace {
 
 constexpr int AT = 32;               // atoms per block = lanes
-constexpr int NW = 8;                // warps per block
-constexpr int NT = AT * NW;
+// Warps per block (NW): eight; sixteen while the blocks are too few to fill the machine (launchers below).
 constexpr int P = AT + 1;            // row pitch of the [index][atom] layout
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -129,8 +128,9 @@ struct Plan {                                 // widths and the shared-memory pl
 // Shared front of both passes: stage the small matrices and the block's slice of the state
 // array (everything behind the C0 scalar sums), then, one warp per harmonic row, normalise
 // and align it, XT = (X / M_1)(I + W), and project it on the probes, Z = XT A.
-template <int C1, int C2, int L>
+template <int C1, int C2, int L, int NW>
 struct Front {
+    static constexpr int NT = 32 * NW;
     using PL = Plan<C1, C2, L>;
     static constexpr int K1 = C2, K2 = 2;
     float *ST, *XT, *ZZ;
@@ -138,34 +138,41 @@ struct Front {
     const GauntSparse *G123, *G233;
     int nv, b0, lane, warp, C0, TW, o1, o2, o3, o4, oS;
     float iM1;
-    double M1d;
+    // normalisers of the block's atoms and their reciprocals: the double-precision root and division are made
+    // once per atom, not once per warp that needs them (2 to 7 % of either kernel)
+    struct Norms { double M0[AT], M1[AT]; float iM0[AT], iM1[AT]; };
+    const Norms* norms;
 
-    template <int C, int K>
-    __device__ __forceinline__ void align_row(const float* xr, const float* W, const float* A, float* xt, float* z) const {
-        float rr[C];
-#pragma unroll
-        for (int b = 0; b < C; ++b) rr[b] = 0.f;
+    // four columns, from b on, of one aligned row: (X / M_1)(I + W)
+    template <int C>
+    __device__ __forceinline__ void align4(const float* xr, const float* W, int b, float* xt) const {
+        float r[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const float x = xr[c * P] * iM1;
-#pragma unroll
-            for (int b = 0; b < C; b += 4) {
-                const float4 w = *reinterpret_cast<const float4*>(W + c * C + b);
-                rr[b] += x * w.x; rr[b + 1] += x * w.y; rr[b + 2] += x * w.z; rr[b + 3] += x * w.w;
-            }
+            const float4 w = *reinterpret_cast<const float4*>(W + c * C + b);
+            r[0] += x * w.x; r[1] += x * w.y; r[2] += x * w.z; r[3] += x * w.w;
         }
 #pragma unroll
-        for (int b = 0; b < C; ++b) xt[b * P] = rr[b];
+        for (int k = 0; k < 4; ++k) xt[(b + k) * P] = r[k];
+    }
+    // NK probes of one aligned row, from k0 on
+    template <int C, int K, int NK>
+    __device__ __forceinline__ void probe(const float* xt, const float* A, int k0, float* z) const {
+        float r[NK];
 #pragma unroll
-        for (int kk = 0; kk < K; ++kk) {
-            float s = 0.f;
+        for (int k = 0; k < NK; ++k) r[k] = 0.f;
 #pragma unroll
-            for (int c = 0; c < C; ++c) s += rr[c] * A[c * K + kk];
-            z[kk * P] = s;
+        for (int c = 0; c < C; ++c) {
+            const float x = xt[c * P];
+#pragma unroll
+            for (int k = 0; k < NK; ++k) r[k] += x * A[c * K + k0 + k];
         }
+#pragma unroll
+        for (int k = 0; k < NK; ++k) z[(k0 + k) * P] = r[k];
     }
 
-    __device__ __forceinline__ void setup(const InvArgs& a, float* st, float* xt, float* zz, float* mats) {
+    __device__ __forceinline__ void setup(const InvArgs& a, float* st, float* xt, float* zz, float* mats, Norms* nm) {
         const Dims& d = a.d;
         const int tid = threadIdx.x;
         lane = tid & 31; warp = tid >> 5;
@@ -207,26 +214,40 @@ struct Front {
             }
         }
         __syncthreads();
-        M1d = sqrt(0.25 + (double)ST[(oS + 1) * P + lane] + (double)ST[(oS + 3) * P + lane]);
-        iM1 = (float)(1.0 / M1d);
-        for (int u = warp; u < 10; u += NW) {
-            if (u < 3) align_row<C1, K1>(ST + (o1 + u * C1) * P + lane, mW1, mA1, XT + u * C1 * P + lane, ZZ + u * K1 * P + lane);
-            else if (u < 8)
-                align_row<C2, K2>(ST + (o2 + (u - 3) * C2) * P + lane, mW2, mA2, XT + (PL::nX1 + (u - 3) * C2) * P + lane,
-                                  ZZ + (PL::nZ1 + (u - 3) * K2) * P + lane);
-            else if (u == 8 && L >= 3) {
+        if (warp < 2) {
+            const double m = sqrt(0.25 + (double)ST[(oS + warp) * P + lane] + (double)ST[(oS + 2 + warp) * P + lane]);
+            const float im = (float)(1.0 / m);
+            if (warp == 0) { nm->M0[lane] = m; nm->iM0[lane] = im; }
+            else { nm->M1[lane] = m; nm->iM1[lane] = im; }
+        }
+        __syncthreads();
+        norms = nm;
+        iM1 = nm->iM1[lane];
+        // a unit is four columns of a row (a whole row of sixteen on one warp was the longest chain of the phase)
+        constexpr int q1 = C1 / 4, q2 = C2 / 4, n12 = 3 * q1 + 5 * q2;
+        for (int u = warp; u < n12 + 2; u += NW) {
+            if (u < 3 * q1) align4<C1>(ST + (o1 + u / q1 * C1) * P + lane, mW1, u % q1 * 4, XT + u / q1 * C1 * P + lane);
+            else if (u < n12) {
+                const int r = (u - 3 * q1) / q2, b = (u - 3 * q1) % q2 * 4;
+                align4<C2>(ST + (o2 + r * C2) * P + lane, mW2, b, XT + (PL::nX1 + r * C2) * P + lane);
+            } else if (u == n12 && L >= 3) {
 #pragma unroll
                 for (int mm = 0; mm < 7; ++mm) XT[(PL::nX1 + PL::nX2 + mm) * P + lane] = ST[(o3 + mm) * P + lane] * iM1;
-            } else if (u == 9 && L >= 4) {
+            } else if (u == n12 + 1 && L >= 4) {
 #pragma unroll
                 for (int mm = 0; mm < 9; ++mm) XT[(PL::nX1 + PL::nX2 + PL::nX3 + mm) * P + lane] = ST[(o4 + mm) * P + lane] * iM1;
             }
         }
         __syncthreads();
-    }
-    // 1 / M_0 of atom aa (the same value in every lane)
-    __device__ __forceinline__ double M0_of(int aa) const {
-        return sqrt(0.25 + (double)ST[oS * P + aa] + (double)ST[(oS + 2) * P + aa]);
+        constexpr int k1 = K1 / 4;
+        for (int u = warp; u < 3 * k1 + 5; u += NW) {
+            if (u < 3 * k1) probe<C1, K1, 4>(XT + u / k1 * C1 * P + lane, mA1, u % k1 * 4, ZZ + u / k1 * K1 * P + lane);
+            else {
+                const int r = u - 3 * k1;
+                probe<C2, K2, 2>(XT + (PL::nX1 + r * C2) * P + lane, mA2, 0, ZZ + (PL::nZ1 + r * K2) * P + lane);
+            }
+        }
+        __syncthreads();
     }
     // U[m1][e] and Y[m1] of the sparse couplings, one unit per m1
     __device__ __forceinline__ void gaunt_pre(float* PRE, int& uctr) const {
@@ -259,14 +280,19 @@ struct Front {
     }
 };
 
-// one calibrated feature-vector entry: fp32 and / or its half-precision split
-__device__ __forceinline__ void put_feature(const InvArgs& a, size_t off, float v, bool split_ok) {
-    if (a.write_desc) a.desc[off] = v;
-    if (a.desc_hi && split_ok) split_f16(v, a.desc_hi[off], a.desc_lo[off]);
+// two neighbouring calibrated feature-vector entries (even column): fp32 and / or their half-precision split
+__device__ __forceinline__ void put_features(const InvArgs& a, size_t off, float v0, float v1, bool split_ok) {
+    if (a.write_desc) *reinterpret_cast<float2*>(a.desc + off) = make_float2(v0, v1);
+    if (a.desc_hi && split_ok) {
+        const __half2 h = __floats2half2_rn(v0, v1);
+        const float2 f = __half22float2(h);
+        *reinterpret_cast<__half2*>(a.desc_hi + off) = h;
+        *reinterpret_cast<__half2*>(a.desc_lo + off) = __floats2half2_rn(v0 - f.x, v1 - f.y);
+    }
 }
 
-template <int C1, int C2, int L>
-__global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
+template <int C1, int C2, int L, int NW>
+__global__ void __launch_bounds__(32 * NW) k_inv_forward(const InvArgs a) {
     using PL = Plan<C1, C2, L>;
     constexpr int K1 = C2, K2 = 2;
     extern __shared__ float sm[];
@@ -284,10 +310,11 @@ __global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
     float* DS = PRE + PL::nPreF * P;
     float* ST = DS;
     (void)TW;
-    Front<C1, C2, L> f;
-    f.setup(a, ST, XT, ZZ, mats);
+    using FR = Front<C1, C2, L, NW>;
+    __shared__ typename FR::Norms norms;
+    FR f;
+    f.setup(a, ST, XT, ZZ, mats, &norms);
     const int lane = f.lane, warp = f.warp, nv = f.nv, b0 = f.b0;
-    const double M0lane = f.M0_of(lane);           // kept: the state slice is overwritten below
     int uctr = 0;
     int dbase = c_full;                            // first column of the portion in the staging area
 #define TAKE() ((uctr++ % NW) == warp)
@@ -295,43 +322,50 @@ __global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
 
     f.gaunt_pre(PRE, uctr);
 
-    // Columns [0, c_full): the centre's initial features (a gather by species) and the
-    // normalised scalar sums A_0 / M_0.  A warp takes one atom at a time, lane = column.
+    // Columns [0, c_full): the centre's initial features (a gather by species) and the normalised scalar
+    // sums A_0 / M_0.  A warp takes one atom at a time, a lane two columns (every store of the features is
+    // four or eight bytes a lane: with single halves, and a copy in single precision that only a query read, this
+    // block was half of the kernel: 128,000 atoms at C0 = 128 took 0.190 ms, so 0.136).
     {
         const float* st_g = a.state + (size_t)b0 * d.SP;
         float im0[AT / NW];
         int ty[AT / NW];
+        const bool x0_out = a.write_desc || !a.skip_x0_split;
 #pragma unroll
         for (int i = 0; i < AT / NW; ++i) {
             const int aa = warp + i * NW;
-            im0[i] = (float)(1.0 / f.M0_of(aa));
-            ty[i] = aa < nv ? a.type_s[a.a0 + b0 + aa] : 0;
+            im0[i] = norms.iM0[aa];
+            ty[i] = x0_out && aa < nv ? a.type_s[a.a0 + b0 + aa] : 0;
         }
-        for (int cb = 0; cb < c_full; cb += 64) {
-            float v[2][AT / NW];
+        for (int cb = x0_out ? 0 : C0 & ~31; cb < c_full; cb += 128) {
+            float2 v[2][AT / NW];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int col = cb + 32 * h + lane;
+                const int col = cb + 64 * h + 2 * lane;
 #pragma unroll
                 for (int i = 0; i < AT / NW; ++i) {
                     const int aa = warp + i * NW;
-                    v[h][i] = 0.f;
+                    v[h][i] = make_float2(0.f, 0.f);
                     if (aa < nv && col < c_full) {
-                        if (col < C0) { if (a.write_desc || !a.skip_x0_split) v[h][i] = __ldg(m.X0 + ty[i] * C0 + col); }
-                        else v[h][i] = st_g[(size_t)aa * d.SP + (col - C0)] * im0[i];
+                        if (col < C0) { if (x0_out) v[h][i] = __ldg(reinterpret_cast<const float2*>(m.X0 + ty[i] * C0 + col)); }
+                        else {
+                            v[h][i] = *reinterpret_cast<const float2*>(st_g + (size_t)aa * d.SP + (col - C0));
+                            v[h][i].x *= im0[i]; v[h][i].y *= im0[i];
+                        }
                     }
                 }
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int col = cb + 32 * h + lane;
+                const int col = cb + 64 * h + 2 * lane;
                 if (col >= c_full) continue;
-                const float mu_c = __ldg(m.mu + col), is_c = __ldg(m.inv_sigma + col);
+                const float2 mu_c = __ldg(reinterpret_cast<const float2*>(m.mu + col)), is_c = __ldg(reinterpret_cast<const float2*>(m.inv_sigma + col));
                 const bool split_col = !(a.skip_x0_split && col < C0);
 #pragma unroll
                 for (int i = 0; i < AT / NW; ++i) {
                     const int aa = warp + i * NW;
-                    if (aa < nv) put_feature(a, (size_t)(b0 + aa) * d.DP + col, (v[h][i] - mu_c) * is_c, split_col);
+                    if (aa < nv)
+                        put_features(a, (size_t)(b0 + aa) * d.DP + col, (v[h][i].x - mu_c.x) * is_c.x, (v[h][i].y - mu_c.y) * is_c.y, split_col);
                 }
             }
         }
@@ -355,13 +389,13 @@ __global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
         float v = 0.f;
         if (lane < nv) {
             if (c < C0) v = __ldg(m.X0 + a.type_s[a.a0 + b0 + lane] * C0 + c);
-            else v = a.state[(size_t)(b0 + lane) * d.SP + (c - C0)] * (float)(1.0 / M0lane);
+            else v = a.state[(size_t)(b0 + lane) * d.SP + (c - C0)] * norms.iM0[lane];
         }
         DSK(c) = v;
     }
     if (TAKE()) {   // the two normalising scales, calibrated here in double precision
-        DSK(kM0) = (float)((M0lane - (double)__ldg(m.mu + kM0)) * (double)__ldg(m.inv_sigma + kM0));
-        DSK(kM1) = (float)((f.M1d - (double)__ldg(m.mu + kM1)) * (double)__ldg(m.inv_sigma + kM1));
+        DSK(kM0) = (float)((norms.M0[lane] - (double)__ldg(m.mu + kM0)) * (double)__ldg(m.inv_sigma + kM0));
+        DSK(kM1) = (float)((norms.M1[lane] - (double)__ldg(m.mu + kM1)) * (double)__ldg(m.inv_sigma + kM1));
     }
     // Gram blocks, row-major upper triangle, strict off-diagonals times sqrt 2; a unit is
     // rows u and C-1-u, which together hold C+1 entries
@@ -379,19 +413,21 @@ __global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
             }
         }
     }
-    // ---- first portion out: calibrate and write, lane = column ---------------------------
+    // ---- first portion out: calibrate and write, lane = two columns (lo and hi are even) -------
     auto write_out = [&](const int lo, const int hi) {
         __syncthreads();
-        for (int cb = lo; cb < hi; cb += 32) {
-            const int col = cb + lane;
+        for (int cb = lo; cb < hi; cb += 64) {
+            const int col = cb + 2 * lane;
             if (col >= hi) continue;
-            float mu_c = 0.f, is_c = 1.f;
-            if (col < d.D_out && col != kM0 && col != kM1) { mu_c = __ldg(m.mu + col); is_c = __ldg(m.inv_sigma + col); }
+            float2 mu_c = make_float2(0.f, 0.f), is_c = make_float2(1.f, 1.f);
+            if (col < d.D_out && col != kM0) { mu_c.x = __ldg(m.mu + col); is_c.x = __ldg(m.inv_sigma + col); }
+            if (col + 1 < d.D_out && col != kM0) { mu_c.y = __ldg(m.mu + col + 1); is_c.y = __ldg(m.inv_sigma + col + 1); }
             const bool split_col = !(a.skip_x0_split && col < C0);
+            const float* ds = DS + (col - lo) * P;
 #pragma unroll
             for (int i = 0; i < AT / NW; ++i) {
                 const int aa = warp + i * NW;
-                if (aa < nv) put_feature(a, (size_t)(b0 + aa) * d.DP + col, (DS[(col - lo) * P + aa] - mu_c) * is_c, split_col);
+                if (aa < nv) put_features(a, (size_t)(b0 + aa) * d.DP + col, (ds[aa] - mu_c.x) * is_c.x, (ds[P + aa] - mu_c.y) * is_c.y, split_col);
             }
         }
         __syncthreads();
@@ -514,7 +550,9 @@ __global__ void __launch_bounds__(NT) k_inv_forward(const InvArgs a) {
 }
 
 // transpose of the alignment and probe maps for one harmonic row: g = dXt + dZ A^T,
-// dX = g (I + W)^T / M_1; returns the row's share of sum g . Xt
+// dX = g (I + W)^T / M_1; returns the row's share of sum g . Xt  (four channels per unit in two phases, as in
+// the forward kernel, was tried: 8 to 16 warps per block have other units of this phase anyway, and the second
+// barrier cost 1 to 3 %)
 template <int C, int K>
 __device__ __forceinline__ float back_row(const float* dxt, const float* dz, const float* A, const float* W,
                                           const float* xt, float* out, float iM1) {
@@ -543,8 +581,8 @@ __device__ __forceinline__ float back_row(const float* dxt, const float* dz, con
     return dot;
 }
 
-template <int C1, int C2, int L>
-__global__ void __launch_bounds__(NT, 3) k_inv_backward(const InvArgs a) {
+template <int C1, int C2, int L, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 1) k_inv_backward(const InvArgs a) {
     using PL = Plan<C1, C2, L>;
     constexpr int K1 = C2, K2 = 2;
     extern __shared__ float sm[];
@@ -601,10 +639,11 @@ __global__ void __launch_bounds__(NT, 3) k_inv_backward(const InvArgs a) {
             }
         }
     };
-    Front<C1, C2, L> f;
-    f.setup(a, ST, XT, ZZ, mats);
+    using FR = Front<C1, C2, L, NW>;
+    __shared__ typename FR::Norms norms;
+    FR f;
+    f.setup(a, ST, XT, ZZ, mats, &norms);
     const int lane = f.lane, warp = f.warp, nv = f.nv;
-    const double M0lane = f.M0_of(lane);           // kept: the state slice is overwritten next
     __syncthreads();
     stage(d.oG[2], d.DP);
     __syncthreads();
@@ -700,7 +739,7 @@ __global__ void __launch_bounds__(NT, 3) k_inv_backward(const InvArgs a) {
 #pragma unroll
         for (int u = 0; u < UA; ++u) {
             const int aa = warp + u * NW;
-            const float im0 = (float)(1.0 / __shfl_sync(kFull, M0lane, aa));
+            const float im0 = norms.iM0[aa];
             float part = 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -923,7 +962,7 @@ __global__ void __launch_bounds__(NT, 3) k_inv_backward(const InvArgs a) {
         float dot1 = 0.f;
 #pragma unroll
         for (int u = 0; u < 10; ++u) dot1 += AUX[(1 + u) * P + lane];
-        const float iM0 = (float)(1.0 / M0lane);
+        const float iM0 = norms.iM0[lane];
         const float dot0 = AUX[lane];
         ST[f.oS * P + lane] = (dM0 - dot0 * iM0) * 0.5f * iM0;
         ST[(f.oS + 1) * P + lane] = (dM1 - dot1 * f.iM1) * 0.5f * f.iM1;
@@ -958,13 +997,19 @@ cudaError_t dispatch(const InvArgs& a, cudaStream_t st) {
         nDS = na > nb ? na : nb;
         if (TW > nDS) nDS = TW;
     }
+    // While the blocks leave SMs with one or (forward) two of them, nothing but a block's own warps hides the
+    // latency of its phases, and sixteen of them shorten every phase; beyond that more blocks per SM do it
+    // better.  Measured, sixteen against eight warps: forward, 4000 atoms 13.2 / 14.8 us, 8000 atoms 24.6 / 28.2;
+    // backward, 597 atoms of degree three 16.8 / 18.9 us, 8000 atoms 49.7 / 33.2 (registers hold one wide block).
+    const bool wide = blocks <= (FWD ? 2 : 1) * 148;
 #define UMLMD_CASE(c1, c2, l)                                                                   \
     if (C1 == c1 && C2 == c2 && L == l) {                                                       \
         const size_t bytes = Plan<c1, c2, l>::bytes(TW, nDS, !FWD);                             \
-        auto kern = FWD ? k_inv_forward<c1, c2, l> : k_inv_backward<c1, c2, l>;                 \
+        auto kern = wide ? (FWD ? k_inv_forward<c1, c2, l, 16> : k_inv_backward<c1, c2, l, 16>) \
+                         : (FWD ? k_inv_forward<c1, c2, l, 8> : k_inv_backward<c1, c2, l, 8>);  \
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
         if (e != cudaSuccess) return e;                                                         \
-        kern<<<blocks, NT, bytes, st>>>(a);                                                     \
+        kern<<<blocks, wide ? 512 : 256, bytes, st>>>(a);                                       \
         return cudaGetLastError();                                                              \
     }
     UMLMD_CASE(4, 4, 2) UMLMD_CASE(4, 4, 3) UMLMD_CASE(8, 4, 2) UMLMD_CASE(8, 4, 3)
