@@ -63,7 +63,8 @@ typedef struct umlmd_options {
                             pair) for every GEMM; path 2 takes the whole MLP in one kernel per block of atoms where
                             that is faster (small systems, narrow models), and otherwise the kernel of path 4 for
                             the last GEMM of the backward pass; 2, 3 and 4 need F % 8 == 0 and fall back to 1 otherwise */
-    int32_t  pair_table_mb;  /* device memory, MiB, that per-pair amplitude tables may take
+    int32_t  pair_table_mb;  /* device memory, MiB, that per-pair amplitude tables may take, without the
+                                copies for values alone, which add two thirds of it
                                 (see umlmd_build_neighbors); 0 = 192, negative = never build them */
     int32_t  gemm_spin_limit;       /* polls after which a wait inside the tensor-core GEMM's operand
                                        pipeline gives up (the kernel then finishes with garbage, and the
@@ -138,7 +139,7 @@ const char* umlmd_last_error(const umlmd_t* h);
  * is allocated (library plumbing, no counterpart in the paper; the paper's memory-scaling note is
  * the model: a fixed tile workspace plus terms linear in atoms and in edges).  An upper estimate
  * within a few per cent; per-pair amplitude tables, when the species present are few enough for
- * them, add at most umlmd_options.pair_table_mb on top.
+ * them, add at most 5/3 of umlmd_options.pair_table_mb on top.
  */
 int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t* bytes);
 

@@ -42,6 +42,9 @@ struct Dims {
     int CP;                  // table channels C0+R rounded up to 4
     int n_rows;              // table intervals
     float tab_k2, tab_k3;    // steps of the packed quadratic and cubic coefficients of the radial table
+    int v_sub, n_vrows;      // value table (below): intervals per table interval, and in all
+    float vdx, inv_vdx;      // its spacing
+    float tab_v1, tab_v2;    // steps of its packed linear and quadratic coefficients
     float rc, dx, inv_dx;
 };
 
@@ -59,6 +62,7 @@ struct GauntSparseBig {      // the same with room for the degree-4 triples
 // Device-resident constants of one model.
 struct ModelDev {
     float* table;     // [n_rows][3][CP] cubic Hermite pieces of [g, q]: c0, c1 (fp32), packed (c2, c3)
+    float* vtable;    // [n_vrows][2][CP] quadratic pieces of [g, q] for their values alone: a0 (fp32), packed (a1, a2)
     float* pairmod;   // [T*T][2+R][C0]: scale gamma, shift beta, mode mixing U[:, mu]
     float* X0;        // [T][C0]
     float* W1p;       // [C1][C1]  I + W_1
@@ -111,6 +115,18 @@ __host__ __device__ inline unsigned tab_pack(float c2, float c3, float k2, float
 __host__ __device__ inline void tab_unpack(unsigned w, float k2, float k3, float* c2, float* c3) {
     *c2 = k2 * (float)((int)w >> 12);
     *c3 = k3 * (float)((int)(w << 20) >> 20);
+}
+
+// Value table.  A pass that needs no derivative reads two words per channel instead of three: the piece is
+// expanded about the middle of the interval, p(s) = a0 + a1 s + a2 s^2 with |s| <= h = spacing / 2, a0 in
+// single precision and (a1, a2) packed like (c2, c3) above.  The cubic term is folded into a1 (s^3 is within
+// h^3 / 4 of (3/4) h^2 s); what is left of it, and the rounding of a1 and a2 to 20 and 12 bits, add up to less
+// than half of the rounding of a0 at the default spacing (0.07 to 0.4 of 2^-24 of the largest value for the
+// workloads' radial maps).  A coarser table is cut into v_sub intervals of at most 0.0025 Angstrom.
+__host__ __device__ inline void value_piece(double c0, double c1, double c2, double c3, double mid, double h, double* a) {
+    a[0] = ((c3 * mid + c2) * mid + c1) * mid + c0;
+    a[1] = (3 * c3 * mid + 2 * c2) * mid + c1 + 0.75 * h * h * c3;
+    a[2] = 3 * c3 * mid + c2;
 }
 
 // One frame of a batched evaluation (umlmd_compute_batch): its own cell and its slice of the

@@ -39,6 +39,8 @@ struct Geom {
 
 // phase 1: one lane, one edge
 // Hf: cell of the destination's frame in a batched evaluation (rows), null for a single system
+// VALUE: row and offset in the value table, else in the table with derivatives
+template <bool VALUE>
 __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool in_range, double xi, double yi,
                                               double zi, int ti, const double* __restrict__ Hf) {
     Geom g;
@@ -79,16 +81,17 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     const float poly = 1.0f + x * (4.0f + x * (10.0f + x * (20.0f + 35.0f * x)));
     g.chi = t2 * t2 * poly;
     g.dchi = -280.0f * x2 * x2 * t2 * t * inv_rc;
-    int row = (int)(g.rho * a.d.inv_dx);
-    row = row < a.d.n_rows - 1 ? row : a.d.n_rows - 1;
+    const int n_rows = VALUE ? a.d.n_vrows : a.d.n_rows;
+    int row = (int)(g.rho * (VALUE ? a.d.inv_vdx : a.d.inv_dx));
+    row = row < n_rows - 1 ? row : n_rows - 1;
     g.row = row;
-    g.t = g.rho - (float)row * a.d.dx;
+    g.t = VALUE ? fmaf(-((float)row + 0.5f), a.d.vdx, g.rho) : fmaf(-(float)row, a.d.dx, g.rho);
     if (a.table_uni) {
         // per-pair amplitude tables, one after another: the pair selects the table (ti is
         // already the compact index of the centre's species)
         if (a.n_present > 1) {           // with one species there is one table and no lookup
             g.pair = ti * a.n_present + a.species_slot[tj];
-            g.row += g.pair * a.d.n_rows;
+            g.row += g.pair * n_rows;
         }
     } else {
         g.pair = ti * a.d.T + tj;
@@ -164,9 +167,8 @@ __device__ __forceinline__ void harmonics_grad_contract(float x, float y, float 
     *gx = ax; *gy = ay; *gz = az;
 }
 
-// value (and derivative) of four consecutive table channels at offset t in row `row`: three
+// value and derivative of four consecutive table channels at offset t in row `row`: three
 // 16-byte loads, c0, c1 and the packed (c2, c3) words with steps k2, k3 (common.cuh, tab_pack)
-template <bool DERIV>
 __device__ __forceinline__ void table_eval4(const float* __restrict__ table, int CP, int row, int c, float t,
                                             float k2, float k3, float* v, float* dv) {
     const float* p = table + (size_t)row * 3 * CP + c;
@@ -178,21 +180,42 @@ __device__ __forceinline__ void table_eval4(const float* __restrict__ table, int
     {                                                                                                  \
         const float i2 = (float)(w.f >> 12), i3 = (float)((w.f << 20) >> 20);                          \
         v[k] = fmaf(i3, u3, fmaf(i2, u2, fmaf(c1.f, t, c0.f)));                                        \
-        if (DERIV) dv[k] = fmaf(i3, v3, fmaf(i2, v2, c1.f));                                           \
+        dv[k] = fmaf(i3, v3, fmaf(i2, v2, c1.f));                                                      \
     }
     UMLMD_PIECE(0, x) UMLMD_PIECE(1, y) UMLMD_PIECE(2, z) UMLMD_PIECE(3, w)
 #undef UMLMD_PIECE
 }
+// values alone, from the value table (common.cuh, value_piece): two 16-byte loads, t from the middle of the
+// piece, k2 and k3 the steps of its linear and quadratic coefficients.  The forward kernel is bound by what it
+// pulls from L2 and through the L1 data pipe, and a row is 8 bytes per channel instead of the 12 of the table
+// with derivatives: 1,000,000 atoms of 64 species at C0 = 128 11.9 -> 10.3 ms, 128,000 of five species 0.84 ->
+// 0.69, 64,000 of one 1.02 -> 0.84, 216,000 at C0 = 8 0.867 -> 0.807.
+__device__ __forceinline__ void value_eval4(const float* __restrict__ table, int CP, int row, int c, float t,
+                                            float k2, float k3, float* v) {
+    const float* p = table + (size_t)row * 2 * CP + c;
+    const float4 a0 = ldg4(p);
+    const int4 w = __ldg(reinterpret_cast<const int4*>(p + CP));
+    const float u1 = k2 * t, u2 = k3 * t * t;
+#define UMLMD_PIECE(k, f) v[k] = fmaf((float)((w.f << 20) >> 20), u2, fmaf((float)(w.f >> 12), u1, a0.f));
+    UMLMD_PIECE(0, x) UMLMD_PIECE(1, y) UMLMD_PIECE(2, z) UMLMD_PIECE(3, w)
+#undef UMLMD_PIECE
+}
 
+// one channel of either table
 template <bool DERIV>
-__device__ __forceinline__ void table_eval1(const float* __restrict__ table, int CP, int row, int c, float t,
-                                            float k2, float k3, float* v, float* dv) {
-    const float* p = table + (size_t)row * 3 * CP + c;
-    const float c0 = __ldg(p), c1 = __ldg(p + CP);
-    const int w = __ldg(reinterpret_cast<const int*>(p + 2 * CP));
-    const float i2 = (float)(w >> 12), i3 = (float)((w << 20) >> 20);
-    *v = fmaf(i3, k3 * t * t * t, fmaf(i2, k2 * t * t, fmaf(c1, t, c0)));
-    if (DERIV) *dv = fmaf(i3, 3.0f * k3 * t * t, fmaf(i2, 2.0f * k2 * t, c1));
+__device__ __forceinline__ void table_eval1(const EdgeArgs& a, int row, int c, float t, float* v, float* dv) {
+    const int CP = a.d.CP;
+    const float* p = DERIV ? a.table + (size_t)row * 3 * CP + c : a.vtable + (size_t)row * 2 * CP + c;
+    const float c0 = __ldg(p);
+    const int w = __ldg(reinterpret_cast<const int*>(p + (DERIV ? 2 : 1) * CP));
+    const float hi = (float)(w >> 12), lo = (float)((w << 20) >> 20);
+    if (DERIV) {
+        const float c1 = __ldg(p + CP), k2 = a.d.tab_k2, k3 = a.d.tab_k3;
+        *v = fmaf(lo, k3 * t * t * t, fmaf(hi, k2 * t * t, fmaf(c1, t, c0)));
+        *dv = fmaf(lo, 3.0f * k3 * t * t, fmaf(hi, 2.0f * k2 * t, c1));
+    } else {
+        *v = fmaf(lo, a.d.tab_v2 * t * t, fmaf(hi, a.d.tab_v1 * t, c0));
+    }
 }
 
 // Shared radial modes q_mu(rho) (and derivatives) of the first nb queued edges, one (edge, mode)
@@ -205,7 +228,7 @@ __device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, i
         const int b = idx / R, q = idx - b * R;
         const int4 es = qes[b];
         float qv, dqv = 0.f;
-        table_eval1<DERIV>(a.table, a.d.CP, es.x, a.d.C0 + q, __int_as_float(es.z), a.d.tab_k2, a.d.tab_k3, &qv, &dqv);
+        table_eval1<DERIV>(a, es.x, a.d.C0 + q, __int_as_float(es.z), &qv, &dqv);
         qm[b * PQ + q] = qv;
         if (DERIV) dqm[b * PQ + q] = dqv;
     }
@@ -220,11 +243,13 @@ template <int C0, bool HASR, bool DERIV, bool UNI>
 __device__ __forceinline__ void amplitude4(const EdgeArgs& a, int row, float t, int pair, int c, float* psi,
                                            float* dpsi, const float* qm, const float* dqm, float k2, float k3) {
     if (UNI) {
-        table_eval4<DERIV>(a.table_uni, C0, row, c, t, k2, k3, psi, dpsi);
+        if (DERIV) table_eval4(a.table_uni, C0, row, c, t, k2, k3, psi, dpsi);
+        else value_eval4(a.vtable_uni, C0, row, c, t, k2, k3, psi);
         return;
     }
     float g[4], dg[4];
-    table_eval4<DERIV>(a.table, a.d.CP, row, c, t, k2, k3, g, dg);
+    if (DERIV) table_eval4(a.table, a.d.CP, row, c, t, k2, k3, g, dg);
+    else value_eval4(a.vtable, a.d.CP, row, c, t, k2, k3, g);
     const int R = HASR ? a.d.R : 0;
     const float* pm = a.pairmod + (size_t)pair * (2 + R) * C0 + c;
     const float4 ga = ldg4(pm), be = ldg4(pm + C0);
@@ -346,7 +371,7 @@ k_edge_forward(const EdgeArgs a) {
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
     const double xi = a.xs[3 * (size_t)i], yi = a.xs[3 * (size_t)i + 1], zi = a.xs[3 * (size_t)i + 2];
     const int ti = UNI ? a.species_slot[a.type_s[i]] : a.type_s[i];
-    const float k2 = UNI ? tab_step2(__ldg(a.uni_scale)) : a.d.tab_k2, k3 = UNI ? tab_step3(__ldg(a.uni_scale + 1)) : a.d.tab_k3;
+    const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + 2)) : a.d.tab_v1, k3 = UNI ? tab_step3(__ldg(a.uni_scale + 3)) : a.d.tab_v2;
     const eidx_t e0 = a.row_ptr[i];
     const int len = (int)(a.row_ptr[i + 1] - e0);      // edge offsets are 64-bit, offsets inside a row are not
     const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
@@ -476,7 +501,7 @@ k_edge_forward(const EdgeArgs a) {
 
     int qn = 0;
     for (int base = 0; base < len; base += 32) {
-        const Geom g = edge_geometry(a, e0 + base + lane, base + lane < len, xi, yi, zi, ti, Hf);
+        const Geom g = edge_geometry<true>(a, e0 + base + lane, base + lane < len, xi, yi, zi, ti, Hf);
         const unsigned vmask = __ballot_sync(kFull, g.valid);
         const int p = qn + __popc(vmask & lt_mask);       // queue slot of this lane's edge, if it has one
         if (g.valid) { const double c2 = (double)g.chi * (double)g.chi; s0 += c2; s1 += c2 * c2; }
@@ -695,7 +720,7 @@ k_edge_backward(const EdgeArgs a) {
         int qn = 0;
         for (int base = 0; base < len; base += 32) {
             const int e = base + lane;                                // offset inside the row
-            const Geom g = edge_geometry(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
+            const Geom g = edge_geometry<false>(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
             if (g.valid && p < 32) {
@@ -774,15 +799,16 @@ cudaError_t dispatch(const EdgeArgs& a, int blocks, cudaStream_t st) {
 // Tables of psi_c(rho) = gamma_c g_c(rho) + beta_c + sum_mu U_c,mu q_mu(rho) for the ordered
 // pairs (present[a], present[b]), stored as [a * n_present + b][row][3][C0] in the format of the
 // radial table: the cubic coefficients are linear in the tabulated functions, so the same
-// combination of the coefficient rows of [g, q] gives them.  Two passes: the first finds the
-// largest |c2| and |c3| (the scale of the packed words), the second writes the rows.
+// combination of the coefficient rows of [g, q] gives them; and as [..][n_vrows][2][C0] in that of the value
+// table.  Two passes: the first finds the largest magnitudes of the coefficients that are packed (the scale
+// of the words), the second writes the rows.
 template <bool WRITE>
 __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, const float* __restrict__ pairmod,
                                    const int* __restrict__ present, int n_present, float* __restrict__ scale,
-                                   float* __restrict__ out) {
+                                   float* __restrict__ out, float* __restrict__ vout) {
     const int64_t per_pair = (int64_t)d.n_rows * d.C0;
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // over [pair][row][c]
-    float c2 = 0.f, c3 = 0.f;
+    float c2 = 0.f, c3 = 0.f, a1 = 0.f, a2 = 0.f;
     if (idx < per_pair * n_present * n_present) {
         const int pr = (int)(idx / per_pair);
         const int64_t in_pair = idx - pr * per_pair;
@@ -806,6 +832,17 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
             for (int k = 0; k < 4; ++k) v[k] += u * o[k];
         }
         c2 = (float)v[2]; c3 = (float)v[3];
+        const double w = (double)d.dx / d.v_sub;
+        for (int sub = 0; sub < d.v_sub; ++sub) {          // values alone (common.cuh, value_piece)
+            double p[3];
+            value_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, p);
+            a1 = fmaxf(a1, fabsf((float)p[1])); a2 = fmaxf(a2, fabsf((float)p[2]));
+            if (WRITE) {
+                float* vrow = vout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
+                vrow[c] = (float)p[0];
+                vrow[d.C0 + c] = __uint_as_float(tab_pack((float)p[1], (float)p[2], tab_step2(scale[2]), tab_step3(scale[3])));
+            }
+        }
         if (WRITE) {
             float* orow = out + ((size_t)pr * d.n_rows + row) * 3 * d.C0;
             orow[c] = (float)v[0];
@@ -814,15 +851,12 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
         }
     }
     if (!WRITE) {        // non-negative floats order like their bit patterns
-        float a2 = fabsf(c2), a3 = fabsf(c3);
+        float mx[4] = {fabsf(c2), fabsf(c3), a1, a2};
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            a2 = fmaxf(a2, __shfl_xor_sync(0xffffffffu, a2, off));
-            a3 = fmaxf(a3, __shfl_xor_sync(0xffffffffu, a3, off));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(reinterpret_cast<unsigned*>(scale), __float_as_uint(a2));
-            atomicMax(reinterpret_cast<unsigned*>(scale) + 1, __float_as_uint(a3));
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], off));
+            if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(scale) + k, __float_as_uint(mx[k]));
         }
     }
 }
@@ -830,14 +864,14 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
 }  // namespace
 
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
-                                    int n_present, float* scale, float* out, cudaStream_t st) {
+                                    int n_present, float* scale, float* out, float* vout, cudaStream_t st) {
     const int64_t n = (int64_t)d.n_rows * d.C0 * n_present * n_present;
     if (n == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(scale, 0, 2 * sizeof(float), st);
+    cudaError_t e = cudaMemsetAsync(scale, 0, 4 * sizeof(float), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((n + 255) / 256);
-    k_fuse_pair_tables<false><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out);
-    k_fuse_pair_tables<true><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out);
+    k_fuse_pair_tables<false><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout);
+    k_fuse_pair_tables<true><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout);
     return cudaGetLastError();
 }
 

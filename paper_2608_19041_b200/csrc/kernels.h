@@ -68,12 +68,16 @@ struct EdgeArgs {
     const int* frame_of;
     const float* table_uni;
     const float* uni_scale;
+    // the same two tables for values alone (value_piece), read by the forward pass; uni_scale[2..3] = largest
+    // |a1|, |a2| of vtable_uni
+    const float* vtable;
+    const float* vtable_uni;
     const int* species_slot;    // [T] species -> index among the species present
     int n_present;
 };
 // present: device array of the n_present species indices, ascending
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
-                                    int n_present, float* scale, float* out, cudaStream_t st);
+                                    int n_present, float* scale, float* out, float* vout, cudaStream_t st);
 cudaError_t launch_edge_forward(const EdgeArgs& a, cudaStream_t st);
 cudaError_t launch_edge_backward(const EdgeArgs& a, int* n_blocks, cudaStream_t st);
 int edge_backward_blocks(int n_rows_in_tile);

@@ -16,6 +16,7 @@
 //    scaled to unit Frobenius norm, sign -1 (the sign both printed closed forms carry).
 #include "model.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -309,6 +310,46 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                 hi[((size_t)s * NC + c) * 2] = c2; hi[((size_t)s * NC + c) * 2 + 1] = c3;
                 if (std::fabs(c2) > m2) m2 = std::fabs(c2);
                 if (std::fabs(c3) > m3) m3 = std::fabs(c3);
+            }
+        }
+        // values alone: quadratic pieces about the middle of (a fraction of) the interval
+        d.v_sub = 1;
+        while (D1 / d.v_sub > 0.0025) d.v_sub *= 2;
+        std::vector<float> va;
+        double m0 = 0, q1 = 0, q2 = 0, q3 = 0;
+        for (;; d.v_sub *= 2) {
+            const double w = D1 / d.v_sub, hw = 0.5 * w;
+            va.assign((size_t)n_rows * d.v_sub * NC * 3, 0.0f);
+            m0 = q1 = q2 = q3 = 0;
+            float* o = va.data();
+            for (int s = 0; s < n_rows; ++s) {
+                const double* ya = &Y[(size_t)s * 2 * NC];
+                const double* yb = &Y[(size_t)(s + 1) * 2 * NC];
+                for (int sub = 0; sub < d.v_sub; ++sub)
+                    for (int c = 0; c < NC; ++c, o += 3) {
+                        const double del = yb[c] - ya[c], p0 = ya[NC + c], p1 = yb[NC + c];
+                        const double c2 = (3 * del - (2 * p0 + p1) * D1) * (1 / D2), c3 = (-2 * del + (p0 + p1) * D1) * (1 / D3);
+                        double p[3];
+                        value_piece(ya[c], p0, c2, c3, (sub + 0.5) * w, hw, p);
+                        m0 = std::max(m0, std::fabs(p[0])); q1 = std::max(q1, std::fabs(p[1]));
+                        q2 = std::max(q2, std::fabs(p[2])); q3 = std::max(q3, std::fabs(c3));
+                        o[0] = (float)p[0]; o[1] = (float)p[1]; o[2] = (float)p[2];
+                    }
+            }
+            const double off = q3 * hw * hw * hw / 4 + q1 / (2.0 * kTabI2Max) * hw + q2 / (2.0 * kTabI3Max) * hw * hw;
+            if (off <= m0 * 0x1p-24 || n_rows * (int64_t)d.v_sub > 100000) break;    // at most the rounding of a0
+        }
+        d.n_vrows = n_rows * d.v_sub;
+        d.vdx = (float)(D1 / d.v_sub); d.inv_vdx = (float)(d.v_sub / D1);
+        d.tab_v1 = tab_step2((float)q1); d.tab_v2 = tab_step3((float)q2);
+        m->vtable.assign((size_t)d.n_vrows * 2 * CP, 0.0f);
+        const float* v = va.data();
+        for (int s = 0; s < d.n_vrows; ++s) {
+            float* row = &m->vtable[(size_t)s * 2 * CP];
+            for (int c = 0; c < NC; ++c, v += 3) {
+                row[c] = v[0];
+                const unsigned w = tab_pack(v[1], v[2], d.tab_v1, d.tab_v2);
+                std::memcpy(&row[CP + c], &w, sizeof(w));
             }
         }
         d.tab_k2 = tab_step2(m2); d.tab_k3 = tab_step3(m3);
