@@ -40,9 +40,10 @@ struct umlmd {
     int64_t pair_table_budget = 192ll << 20;            // bytes; negative = never build them
     bool pair_tables = false;                           // in use for the current system
     std::vector<int> present;                           // species the tables were built for, ascending
-    float* table_uni = nullptr; size_t table_uni_cap = 0;   // [present^2][n_rows][3][C0], capacity in floats
+    float* table_uni = nullptr; size_t table_uni_cap = 0;   // [present^2][n_rows][3][C0], capacity in floats (C0 < 32)
     float* vtable_uni = nullptr; size_t vtable_uni_cap = 0; // [present^2][n_vrows][2][C0], the same for values alone
-    float* uni_scale = nullptr;                         // [4] largest |c2|, |c3|, |a1|, |a2| of those tables
+    float* dtable_uni = nullptr; size_t dtable_uni_cap = 0; // [present^2][n_vrows][2][C0], envelope products (from C0 = 32 on, instead of table_uni)
+    float* uni_scale = nullptr;                         // [6] largest |c2|, |c3|, |a1|, |a2| and |a1|, |a2| of those tables
     int* d_species = nullptr;                           // [3T]: occurrence flags, species -> slot, present list
     int* h_species = nullptr;                           // pinned [T]
     // MD
@@ -201,8 +202,9 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         const int n = NR - a0 < B ? NR - a0 : B;
         EdgeArgs ea;
         ea.d = d; ea.table = h->md.table; ea.pairmod = h->md.pairmod; ea.xs = nb.xs; ea.rec = nb.rec; ea.type_s = nb.type_s;
-        ea.table_uni = h->pair_tables ? h->table_uni : nullptr;
-        ea.vtable = h->md.vtable; ea.vtable_uni = h->pair_tables ? h->vtable_uni : nullptr;
+        ea.uni = h->pair_tables; ea.table_uni = h->table_uni;
+        ea.vtable = h->md.vtable; ea.vtable_uni = h->vtable_uni;
+        ea.dtable = h->md.dtable; ea.dtable_uni = h->dtable_uni;
         ea.uni_scale = h->uni_scale;
         ea.species_slot = h->d_species + d.T; ea.n_present = (int)h->present.size();
         ea.frames = nb.batch ? nb.frames : nullptr; ea.frame_of = nb.frame_of;
@@ -347,7 +349,7 @@ int ensure_device_model(umlmd_t* h) {
     cudaError_t e = cudaSuccess;
     auto up = [&](const std::vector<float>& v, float** p) { if (e == cudaSuccess) e = upload(h, v, p); };
     auto uph = [&](const std::vector<__half>& v, __half** p) { if (e == cudaSuccess) e = upload(h, v, p); };
-    up(m.table, &md.table); up(m.vtable, &md.vtable); up(m.pairmod, &md.pairmod); up(m.X0, &md.X0); up(m.W1p, &md.W1p); up(m.W2p, &md.W2p);
+    up(m.table, &md.table); up(m.vtable, &md.vtable); up(m.dtable, &md.dtable); up(m.pairmod, &md.pairmod); up(m.X0, &md.X0); up(m.W1p, &md.W1p); up(m.W2p, &md.W2p);
     up(m.A1, &md.A1); up(m.A2, &md.A2); up(m.mu, &md.mu); up(m.inv_sigma, &md.inv_sigma);
     up(m.type_bias, &md.type_bias);
     for (int t = 0; t < h->d.n_hidden; ++t) { up(m.theta[t], &md.theta[t]); up(m.thetaT[t], &md.thetaT[t]); up(m.bias[t], &md.bias[t]);
@@ -417,28 +419,30 @@ int setup_pair_tables(umlmd_t* h) {
     std::vector<int> present;
     for (int t = 0; t < d.T; ++t) if (h->h_species[t]) present.push_back(t);
     const size_t np = present.size();
-    const size_t floats = np * np * (size_t)d.n_rows * 3 * d.C0;
-    const size_t vfloats = np * np * (size_t)d.n_vrows * 2 * d.C0;      // at the usual spacings two thirds as many
-    h->pair_tables = np > 0 && h->pair_table_budget >= 0 && floats * sizeof(float) <= (size_t)h->pair_table_budget &&
-                     3 * (floats + vfloats) * sizeof(float) <= 5 * (size_t)h->pair_table_budget;
+    // the rule counts tables with derivatives; what is kept is 4/3 (products) or 5/3 of that at the usual spacings
+    const size_t full = np * np * (size_t)d.n_rows * 3 * d.C0 * sizeof(float);
+    const bool wide = wide_channels(d.C0);
+    const size_t vfloats = np * np * (size_t)d.n_vrows * 2 * d.C0, dfloats = wide ? vfloats : 0;
+    const size_t floats = wide ? 0 : np * np * (size_t)d.n_rows * 3 * d.C0;
+    h->pair_tables = np > 0 && h->pair_table_budget >= 0 && full <= (size_t)h->pair_table_budget &&
+                     3 * (floats + vfloats + dfloats) * sizeof(float) <= 5 * (size_t)h->pair_table_budget;
     if (!h->pair_tables || present == h->present) return UMLMD_OK;
-    if (floats > h->table_uni_cap) {
-        dev_free(h->table_uni); h->table_uni = nullptr; h->table_uni_cap = 0;
-        void* p = nullptr;
-        API_CUDA(h, dev_malloc(&p, sizeof(float) * floats));
-        h->table_uni = (float*)p; h->table_uni_cap = floats;
-    }
-    if (vfloats > h->vtable_uni_cap) {
-        dev_free(h->vtable_uni); h->vtable_uni = nullptr; h->vtable_uni_cap = 0;
-        void* p = nullptr;
-        API_CUDA(h, dev_malloc(&p, sizeof(float) * vfloats));
-        h->vtable_uni = (float*)p; h->vtable_uni_cap = vfloats;
-    }
+    auto grow = [&](float** p, size_t* cap, size_t need) {
+        if (need <= *cap) return cudaSuccess;
+        dev_free(*p); *p = nullptr; *cap = 0;
+        void* q = nullptr;
+        const cudaError_t e = dev_malloc(&q, sizeof(float) * need);
+        if (e == cudaSuccess) { *p = (float*)q; *cap = need; }
+        return e;
+    };
+    API_CUDA(h, grow(&h->table_uni, &h->table_uni_cap, floats));
+    API_CUDA(h, grow(&h->vtable_uni, &h->vtable_uni_cap, vfloats));
+    API_CUDA(h, grow(&h->dtable_uni, &h->dtable_uni_cap, dfloats));
     std::vector<int> up(2 * (size_t)d.T, 0);          // species -> slot, then the present list
     for (size_t k = 0; k < np; ++k) { up[present[k]] = (int)k; up[d.T + k] = present[k]; }
     API_CUDA(h, cudaMemcpyAsync(h->d_species + d.T, up.data(), sizeof(int) * up.size(), cudaMemcpyHostToDevice, h->st));
-    if (!h->uni_scale) { void* p = nullptr; API_CUDA(h, dev_malloc(&p, 4 * sizeof(float))); h->uni_scale = (float*)p; }
-    API_CUDA(h, launch_fuse_pair_tables(d, h->md.table, h->md.pairmod, h->d_species + 2 * d.T, (int)np, h->uni_scale, h->table_uni, h->vtable_uni, h->st));
+    if (!h->uni_scale) { void* p = nullptr; API_CUDA(h, dev_malloc(&p, 8 * sizeof(float))); h->uni_scale = (float*)p; }
+    API_CUDA(h, launch_fuse_pair_tables(d, h->md.table, h->md.pairmod, h->d_species + 2 * d.T, (int)np, h->uni_scale, h->table_uni, h->vtable_uni, h->dtable_uni, h->st));
     API_CUDA(h, cudaStreamSynchronize(h->st));       // `up` is pageable host memory
     h->launches_total += 2;
     h->present = present;
@@ -491,7 +495,7 @@ int umlmd_destroy(umlmd_t* h) {
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
     void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
-                    h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->table_uni, h->vtable_uni, h->d_species, h->uni_scale};
+                    h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->table_uni, h->vtable_uni, h->dtable_uni, h->d_species, h->uni_scale};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
     for (cudaEvent_t e : h->free_events) cudaEventDestroy(e);
@@ -594,7 +598,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     int64_t t = 0;
     // model constants (uploaded by the first build)
     auto vec = [&](size_t n, size_t elem) { t += (int64_t)(n * elem + 16); };
-    vec(m.table.size(), 4); vec(m.vtable.size(), 4); vec(m.pairmod.size(), 4); vec(m.X0.size(), 4); vec(m.W1p.size(), 4); vec(m.W2p.size(), 4);
+    vec(m.table.size(), 4); vec(m.vtable.size(), 4); vec(m.dtable.size(), 4); vec(m.pairmod.size(), 4); vec(m.X0.size(), 4); vec(m.W1p.size(), 4); vec(m.W2p.size(), 4);
     vec(m.A1.size(), 4); vec(m.A2.size(), 4); vec(m.mu.size(), 4); vec(m.inv_sigma.size(), 4); vec(m.type_bias.size(), 4);
     for (int k = 0; k < d.n_hidden; ++k) {
         vec(m.theta[k].size(), 4); vec(m.thetaT[k].size(), 4); vec(m.bias[k].size(), 4);

@@ -42,9 +42,10 @@ struct Dims {
     int CP;                  // table channels C0+R rounded up to 4
     int n_rows;              // table intervals
     float tab_k2, tab_k3;    // steps of the packed quadratic and cubic coefficients of the radial table
-    int v_sub, n_vrows;      // value table (below): intervals per table interval, and in all
+    int v_sub, v_shift, n_vrows;   // value table (below): intervals per table interval (2^v_shift), and in all
     float vdx, inv_vdx;      // its spacing
     float tab_v1, tab_v2;    // steps of its packed linear and quadratic coefficients
+    float tab_d1, tab_d2;    // the same for the product table
     float rc, dx, inv_dx;
 };
 
@@ -63,6 +64,7 @@ struct GauntSparseBig {      // the same with room for the degree-4 triples
 struct ModelDev {
     float* table;     // [n_rows][3][CP] cubic Hermite pieces of [g, q]: c0, c1 (fp32), packed (c2, c3)
     float* vtable;    // [n_vrows][2][CP] quadratic pieces of [g, q] for their values alone: a0 (fp32), packed (a1, a2)
+    float* dtable;    // [n_vrows][2][CP] the same format: derivative of envelope times g (C0 >= 32)
     float* pairmod;   // [T*T][2+R][C0]: scale gamma, shift beta, mode mixing U[:, mu]
     float* X0;        // [T][C0]
     float* W1p;       // [C1][C1]  I + W_1
@@ -101,7 +103,9 @@ typedef long long eidx_t;      // edge offsets are 64-bit: a list may hold more 
 // own scale (c2 = k2 I2, c3 = k3 I3; k = largest magnitude in the table / largest integer) cost
 // nothing in the value and leave the derivative within a few 1e-7 of its largest entry at the
 // default spacing (the error grows with the spacing like the interpolation error itself).
-// One 32-bit word: I2 in the upper 20 bits, I3 in the lower 12, both two's complement.
+// One 32-bit word: I2 in the upper 20 bits, I3 in the lower 12, both two's complement.  (A word whose parts
+// decode without shifts, the low bits through the mantissa of 2^23, took an addition more and was 3 to 8 %
+// slower in the forward kernel.)
 constexpr int kTabI2Max = (1 << 19) - 1, kTabI3Max = (1 << 11) - 1;
 __host__ __device__ inline float tab_step2(float max_abs_c2) { return max_abs_c2 * (1.0f / (float)kTabI2Max); }
 __host__ __device__ inline float tab_step3(float max_abs_c3) { return max_abs_c3 * (1.0f / (float)kTabI3Max); }
@@ -128,6 +132,32 @@ __host__ __device__ inline void value_piece(double c0, double c1, double c2, dou
     a[1] = (3 * c3 * mid + 2 * c2) * mid + c1 + 0.75 * h * h * c3;
     a[2] = 3 * c3 * mid + c2;
 }
+
+// Product table.  Of the scalar channels the backward pass needs one number per edge, sum_c G_c (chi psi_c)':
+// the derivative of the product of envelope and amplitude is tabulated by itself, in the format and on the
+// grid of the value table (expanded from the cubic piece and the envelope's derivatives, cubic term folded),
+// two words per channel and one dot product instead of three words and two.  The leading C1 channels, which
+// also carry the degrees >= 1, add their amplitude from the value table: (chi^2 psi)' = chi ((chi psi)' + chi' psi).
+// chi = 1 - I_x(5, 4).
+__host__ __device__ inline void product_piece(double c0, double c1, double c2, double c3, double mid, double h, double rho, double rc,
+                                              double* a) {
+    const double x = rho / rc, u = 1 - x, r = 1 / rc;
+    const double e0 = u * u * u * u * (1 + x * (4 + x * (10 + x * (20 + 35 * x))));
+    const double e1 = -280 * r * x * x * x * x * u * u * u;
+    const double e2 = -280 * r * r * x * x * x * u * u * (4 * u - 3 * x);
+    const double e3 = -280 * r * r * r * x * x * u * (12 * u * u - 24 * x * u + 6 * x * x);
+    const double e4 = -280 * r * r * r * r * x * (24 * u * u * u - 108 * x * u * u + 72 * x * x * u - 6 * x * x * x);
+    const double p0 = ((c3 * mid + c2) * mid + c1) * mid + c0, p1 = (3 * c3 * mid + 2 * c2) * mid + c1, p2 = 6 * c3 * mid + 2 * c2, p3 = 6 * c3;
+    const double d3 = (e4 * p0 + 4 * e3 * p1 + 6 * e2 * p2 + 4 * e1 * p3) / 6;
+    a[0] = e1 * p0 + e0 * p1;
+    a[1] = e2 * p0 + 2 * e1 * p1 + e0 * p2 + 0.75 * h * h * d3;
+    a[2] = 0.5 * (e3 * p0 + 3 * e2 * p1 + 3 * e1 * p2 + e0 * p3);
+    a[3] = d3;
+}
+// Models of at least 32 channels without shared modes, or with per-pair tables (which hold the modes), use the
+// product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the channels are leading
+// ones, and with modes their derivatives are needed anyway: there the table with derivatives is less to read.
+__host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }
 
 // One frame of a batched evaluation (umlmd_compute_batch): its own cell and its slice of the
 // concatenated atom arrays.

@@ -86,7 +86,7 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     row = row < n_rows - 1 ? row : n_rows - 1;
     g.row = row;
     g.t = VALUE ? fmaf(-((float)row + 0.5f), a.d.vdx, g.rho) : fmaf(-(float)row, a.d.dx, g.rho);
-    if (a.table_uni) {
+    if (a.uni) {
         // per-pair amplitude tables, one after another: the pair selects the table (ti is
         // already the compact index of the centre's species)
         if (a.n_present > 1) {           // with one species there is one table and no lookup
@@ -278,6 +278,22 @@ __device__ __forceinline__ void amplitude4(const EdgeArgs& a, int row, float t, 
     }
 }
 
+// (chi psi_c)' of this lane's four channels for one edge, from the product table; row and t of the value grid, dchi
+// the envelope's derivative (only without per-pair tables)
+template <int C0, bool UNI>
+__device__ __forceinline__ void product4(const EdgeArgs& a, int row, float t, int pair, int c, float dchi, float d1, float d2, float* d) {
+    if (UNI) {
+        value_eval4(a.dtable_uni, C0, row, c, t, d1, d2, d);
+        return;
+    }
+    float g[4];
+    value_eval4(a.dtable, a.d.CP, row, c, t, d1, d2, g);
+    const float* pm = a.pairmod + (size_t)pair * 2 * C0 + c;
+    const float4 ga = ldg4(pm), be = ldg4(pm + C0);
+    d[0] = fmaf(ga.x, g[0], be.x * dchi); d[1] = fmaf(ga.y, g[1], be.y * dchi);
+    d[2] = fmaf(ga.z, g[2], be.z * dchi); d[3] = fmaf(ga.w, g[3], be.w * dchi);
+}
+
 // G = groups of four channels a lane holds in the channel-parallel phase (group g starts at
 // channel 4 * lane_in_group + g * C0 / G, so every 16-byte load instruction of a group of lanes
 // still covers one contiguous segment)
@@ -316,18 +332,29 @@ template <int C0, int L, int G = 1> struct Widths {
 };
 
 // The channel-parallel phase of the backward pass waits on load latency, and what hides it best
-// depends on the width (all measured on the edge backward kernel).  C0 = 128: four channel groups
-// per lane, that many times the table and pair loads in flight, at 16 resident warps per SM (128
-// registers): 10 % faster than two groups, and than two groups at 24 warps.  C0 = 32 and 64:
-// two groups at 24 warps (85 registers, a few spilled words): 9-13 % faster than 16 warps,
-// four groups being slower again.  C0 <= 16: one group, 24 warps (13 % faster than 16).
-template <int C0> struct BwdGroups { static constexpr int G = C0 >= 128 ? 4 : (C0 >= 32 ? 2 : 1); };
+// depends on the width and on what is read (all measured on the edge backward kernel).  C0 = 128 with shared
+// table and pair cache, or degree three: four channel groups per lane, that many times the loads in flight,
+// at 16 resident warps per SM (128 registers): 64,007 atoms of one species 1.10 ms against 1.19 with two
+// groups at 24 warps (85 registers, spilled words), the 64-species mixture 12.6 against 14.6.  With shared modes,
+// and with per-pair tables at degree two (fewer registers spilled): the latter, 1.62 -> 1.49 ms for 40,009 atoms
+// with four modes, 1.00 -> 0.94 for 128,000 atoms of five species.  C0 = 32 and 64: two groups at 24 warps;
+// C0 <= 16: one group, 24 warps.  FEW: rows for more than 24 but not more than 32 warps per SM (3553 to 4736): 64
+// registers and one wave beat 85 and two (4000 atoms at C0 = 64: 41 -> 35 us; 597 atoms 25 against 21, 32,400
+// atoms 254 against 234).
+template <int C0, int L, bool HASR, bool UNI, bool FEW> struct BwdShape {
+    static constexpr bool two = C0 >= 128 && (HASR || (UNI && L == 2));
+    static constexpr int G = C0 >= 128 ? (two ? 2 : 4) : (C0 >= 32 ? 2 : 1);
+    static constexpr int warps = C0 >= 128 ? (two ? 24 : 16) : (FEW ? 32 : 24);
+    static constexpr bool tight = two || FEW;
+};
 
-template <int C0, int L, bool HASR> struct BwdSmem {          // dynamic shared memory of the backward kernel
-    using W = Widths<C0, L, BwdGroups<C0>::G>;
+template <int C0, int L, bool HASR, bool UNI> struct BwdSmem {          // dynamic shared memory of the backward kernel
+    using W = Widths<C0, L, BwdShape<C0, L, HASR, UNI, false>::G>;
     static constexpr int queue_floats = 32 * 4 + 5 * 32;    // queue of in-range edges: int4 and five scalars per slot
     static constexpr int mode_floats = HASR ? 2 * 32 * kMaxR : 0;   // parked radial modes and their derivatives
-    static constexpr int per_warp = (32 * W::PB + 2 * 32 * (W::LH + 1) + W::NHI + 3) / 4 * 4 + mode_floats + queue_floats;   // floats
+    static constexpr bool products = wide_channels(C0) && !HASR;    // reads the product table (product_piece)
+    static constexpr int n_red = products ? 1 : 2;                  // partial dot products per edge and lane pair
+    static constexpr int per_warp = (32 * W::PB + n_red * 32 * (W::LH + 1) + W::NHI + 3) / 4 * 4 + mode_floats + queue_floats;   // floats
     static constexpr size_t bytes = kWarpsPerBlock * 9 * sizeof(double) + sizeof(float) * kWarpsPerBlock * per_warp;
 };
 
@@ -565,21 +592,23 @@ k_edge_forward(const EdgeArgs a) {
 // the edge's lane then does the whole degree >= 1 contraction by itself against the
 // destination's gradient block held in shared memory, and assembles dE/dr_ij.  Edges in the
 // skin shell get a zero gradient as soon as their geometry is known.
-template <int C0, int L, bool HASR, bool UNI>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 ? 3 : 2) * 8 / kWarpsPerBlock)
+template <int C0, int L, bool HASR, bool UNI, bool FEW>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, BwdShape<C0, L, HASR, UNI, FEW>::warps / kWarpsPerBlock)
 k_edge_backward(const EdgeArgs a) {
-    constexpr int G = BwdGroups<C0>::G;
+    using SM = BwdSmem<C0, L, HASR, UNI>;
+    constexpr int G = BwdShape<C0, L, HASR, UNI, FEW>::G;
+    constexpr bool PR = SM::products;
     using W = Widths<C0, L, G>;
     extern __shared__ __align__(16) unsigned char dsm[];
     double (*vsum)[9] = reinterpret_cast<double (*)[9]>(dsm);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    float* const wbase = reinterpret_cast<float*>(dsm + kWarpsPerBlock * 9 * sizeof(double)) + wid * BwdSmem<C0, L, HASR>::per_warp;
+    float* const wbase = reinterpret_cast<float*>(dsm + kWarpsPerBlock * 9 * sizeof(double)) + wid * SM::per_warp;
     float* const psi_s = wbase;                                  // [32][PB]: psi, dpsi of the leading channels
-    float* const red = psi_s + 32 * W::PB;                       // [2][32][LH+1] partial dot products
-    float* const hi_s = red + 2 * 32 * (W::LH + 1);              // [NHI] gradient of the degree >= 1 sums
+    float* const red = psi_s + 32 * W::PB;                       // [n_red][32][LH+1] partial dot products
+    float* const hi_s = red + SM::n_red * 32 * (W::LH + 1);   // [NHI] gradient of the degree >= 1 sums
     // queue of edges inside the cutoff: (row, pair, t, chi), then dx, dy, dz, dchi, edge index
-    int4* const qes = reinterpret_cast<int4*>(wbase + BwdSmem<C0, L, HASR>::per_warp - BwdSmem<C0, L, HASR>::queue_floats);
-    float* const qm = reinterpret_cast<float*>(qes) - BwdSmem<C0, L, HASR>::mode_floats;   // [2][32][kMaxR]
+    int4* const qes = reinterpret_cast<int4*>(wbase + SM::per_warp - SM::queue_floats);
+    float* const qm = reinterpret_cast<float*>(qes) - SM::mode_floats;   // [2][32][kMaxR]
     float* const qd = reinterpret_cast<float*>(qes + 32);        // [5][32]
     const int i = a.a0 + blockIdx.x * kWarpsPerBlock + wid;
     const bool active = i < a.a1;
@@ -592,7 +621,10 @@ k_edge_backward(const EdgeArgs a) {
     if (active) {
         const double xi = a.xs[3 * (size_t)i], yi = a.xs[3 * (size_t)i + 1], zi = a.xs[3 * (size_t)i + 2];
         const int ti = UNI ? a.species_slot[a.type_s[i]] : a.type_s[i];
-        const float k2 = UNI ? tab_step2(__ldg(a.uni_scale)) : a.d.tab_k2, k3 = UNI ? tab_step3(__ldg(a.uni_scale + 1)) : a.d.tab_k3;
+        // steps of the packed words: of the table with derivatives, or of the value and the product table
+        const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + (PR ? 2 : 0))) : (PR ? a.d.tab_v1 : a.d.tab_k2),
+                    k3 = UNI ? tab_step3(__ldg(a.uni_scale + (PR ? 3 : 1))) : (PR ? a.d.tab_v2 : a.d.tab_k3);
+        const float d1 = UNI ? tab_step2(__ldg(a.uni_scale + 4)) : a.d.tab_d1, d2 = UNI ? tab_step3(__ldg(a.uni_scale + 5)) : a.d.tab_d2;
         const eidx_t e0 = a.row_ptr[i];
         const int len = (int)(a.row_ptr[i + 1] - e0);
         const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
@@ -616,33 +648,70 @@ k_edge_backward(const EdgeArgs a) {
                 eval_modes<true, kMaxR>(a, qes, nb, lane, qm, qm + 32 * kMaxR);
                 __syncwarp();
             }
-            for (int it = 0; it * W::EPI < nb; ++it) {
-                const int b = it * W::EPI + sub;
-                const bool act = b < nb;
-                float pa = 0.f, pb = 0.f;
-                if (act) {
-                    const int4 es = qes[b];
-                    const int row = es.x, pair = es.y;
-                    const float t = __int_as_float(es.z);
-                    float psi[4 * G], dpsi[4 * G];
-#pragma unroll
-                    for (int gq = 0; gq < G; ++gq)
-                        amplitude4<C0, HASR, true, UNI>(a, row, t, pair, c + gq * W::GOFF, psi + 4 * gq, dpsi + 4 * gq,
-                                                        qm + b * kMaxR, qm + (32 + b) * kMaxR, k2, k3);
-#pragma unroll
-                    for (int k = 0; k < 4 * G; ++k) { pa += h0[k] * dpsi[k]; pb += h0[k] * psi[k]; }
-                    if (cl < W::NL1) {       // the leading C1 channels all sit in group 0
-                        *reinterpret_cast<float4*>(psi_s + b * W::PB + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
-                        *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + c) = make_float4(dpsi[0], dpsi[1], dpsi[2], dpsi[3]);
+            if constexpr (PR) {
+                // the leading channels' amplitudes, four channels of an edge per lane
+                constexpr int LE = 32 / W::NL1;             // edges per step
+                for (int b0 = 0; b0 < nb; b0 += LE) {
+                    const int b = b0 + lane / W::NL1, cc = 4 * (lane % W::NL1);
+                    if (b < nb) {
+                        const int4 es = qes[b];
+                        float psi[4];
+                        amplitude4<C0, false, false, UNI>(a, es.x, __int_as_float(es.z), es.y, cc, psi, nullptr, nullptr, nullptr, k2, k3);
+                        *reinterpret_cast<float4*>(psi_s + b * W::PB + cc) = make_float4(psi[0], psi[1], psi[2], psi[3]);
                     }
                 }
-                // neighbouring lanes are paired before the partial sums are parked, which halves
-                // the parking area (it decides how many blocks fit on an SM)
-                pa += __shfl_xor_sync(kFull, pa, 1);
-                pb += __shfl_xor_sync(kFull, pb, 1);
-                if (act && !(cl & 1)) {
-                    red[b * (W::LH + 1) + (cl >> 1)] = pa;
-                    red[(32 + b) * (W::LH + 1) + (cl >> 1)] = pb;
+                // all channels: sum_c G_c (chi psi_c)'
+                for (int it = 0; it * W::EPI < nb; ++it) {
+                    const int b = it * W::EPI + sub;
+                    const bool act = b < nb;
+                    float pa = 0.f;
+                    if (act) {
+                        const int4 es = qes[b];
+                        const float t = __int_as_float(es.z), dchi = UNI ? 0.f : qd[96 + b];
+#pragma unroll
+                        for (int gq = 0; gq < G; ++gq) {
+                            float d[4];
+                            product4<C0, UNI>(a, es.x, t, es.y, c + gq * W::GOFF, dchi, d1, d2, d);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) pa += h0[4 * gq + k] * d[k];
+                            if (gq == 0 && cl < W::NL1)     // the leading C1 channels all sit in group 0
+                                *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + c) = make_float4(d[0], d[1], d[2], d[3]);
+                        }
+                    }
+                    // neighbouring lanes are paired before the partial sums are parked, which halves
+                    // the parking area (it decides how many blocks fit on an SM)
+                    pa += __shfl_xor_sync(kFull, pa, 1);
+                    if (act && !(cl & 1)) red[b * (W::LH + 1) + (cl >> 1)] = pa;
+                }
+            } else {
+                for (int it = 0; it * W::EPI < nb; ++it) {
+                    const int b = it * W::EPI + sub;
+                    const bool act = b < nb;
+                    float pa = 0.f, pb = 0.f;
+                    if (act) {
+                        const int4 es = qes[b];
+                        const int row = es.x, pair = es.y;
+                        const float t = __int_as_float(es.z);
+                        float psi[4 * G], dpsi[4 * G];
+    #pragma unroll
+                        for (int gq = 0; gq < G; ++gq)
+                            amplitude4<C0, HASR, true, UNI>(a, row, t, pair, c + gq * W::GOFF, psi + 4 * gq, dpsi + 4 * gq,
+                                                            qm + b * kMaxR, qm + (32 + b) * kMaxR, k2, k3);
+    #pragma unroll
+                        for (int k = 0; k < 4 * G; ++k) { pa += h0[k] * dpsi[k]; pb += h0[k] * psi[k]; }
+                        if (cl < W::NL1) {       // the leading C1 channels all sit in group 0
+                            *reinterpret_cast<float4*>(psi_s + b * W::PB + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
+                            *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + c) = make_float4(dpsi[0], dpsi[1], dpsi[2], dpsi[3]);
+                        }
+                    }
+                    // neighbouring lanes are paired before the partial sums are parked, which halves
+                    // the parking area (it decides how many blocks fit on an SM)
+                    pa += __shfl_xor_sync(kFull, pa, 1);
+                    pb += __shfl_xor_sync(kFull, pb, 1);
+                    if (act && !(cl & 1)) {
+                        red[b * (W::LH + 1) + (cl >> 1)] = pa;
+                        red[(32 + b) * (W::LH + 1) + (cl >> 1)] = pb;
+                    }
                 }
             }
             __syncwarp();
@@ -654,56 +723,117 @@ k_edge_backward(const EdgeArgs a) {
                 const float gux = gdx * inv_rho, guy = gdy * inv_rho, guz = gdz * inv_rho;
                 float sa = 0.f, sb = 0.f;
 #pragma unroll
-                for (int j = 0; j < W::LH; ++j) { sa += red[lane * (W::LH + 1) + j]; sb += red[(32 + lane) * (W::LH + 1) + j]; }
-                float ps[W::C1], dps[W::C1], ec[W::C1];
-#pragma unroll
-                for (int q = 0; q < W::C1 / 4; ++q) {
-                    const float4 p4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + 4 * q);
-                    const float4 d4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + W::C1 + 4 * q);
-                    ps[4 * q] = p4.x; ps[4 * q + 1] = p4.y; ps[4 * q + 2] = p4.z; ps[4 * q + 3] = p4.w;
-                    dps[4 * q] = d4.x; dps[4 * q + 1] = d4.y; dps[4 * q + 2] = d4.z; dps[4 * q + 3] = d4.w;
+                for (int j = 0; j < W::LH; ++j) {
+                    sa += red[lane * (W::LH + 1) + j];
+                    if (!PR) sb += red[(32 + lane) * (W::LH + 1) + j];
                 }
-#pragma unroll
-                for (int k = 0; k < W::C1; ++k) ec[k] = 0.f;
+                // degrees >= 1: t_lm = sum_c psi_c G_lmc (for the harmonics' gradient), bt = sum_lm B_lm t_lm and
+                // pr1 = sum_lm B_lm sum_c dps_c G_lmc.  By component, all channels in registers; where the registers are
+                // few (BwdShape), by four channels, which keeps the components' sums instead: 0.94 against 1.02 ms for
+                // the 128,000 atoms of five species, but 1.12 against 1.10 at 128 registers.
                 float B1[3], B2[5], B3[7], B4[9], t1[3], t2[5], t3[7], t4[9];
                 harmonics_s1<L>(gux, guy, guz, B1, B2, B3, B4);
-                float bt = 0.f;    // sum_lm B_lm t_lm,  t_lm = sum_c psi_c G_lmc
+                float bt = 0.f, pr1 = 0.f;
+                if constexpr (BwdShape<C0, L, HASR, UNI, FEW>::tight) {
+                    const float* pr = psi_s + lane * W::PB;
 #pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    float tm = 0.f;
+                    for (int m = 0; m < 3; ++m) t1[m] = 0.f;
 #pragma unroll
-                    for (int k = 0; k < W::C1; ++k) { const float hv = H1[m * W::C1 + k]; tm += ps[k] * hv; ec[k] += B1[m] * hv; }
-                    t1[m] = tm; bt += B1[m] * tm;
-                }
+                    for (int m = 0; m < 5; ++m) t2[m] = 0.f;
 #pragma unroll
-                for (int m = 0; m < 5; ++m) {
-                    float tm = 0.f;
+                    for (int m = 0; m < 7; ++m) t3[m] = 0.f;
 #pragma unroll
-                    for (int k = 0; k < W::C2; ++k) { const float hv = H2[m * W::C2 + k]; tm += ps[k] * hv; ec[k] += B2[m] * hv; }
-                    t2[m] = tm; bt += B2[m] * tm;
-                }
+                    for (int m = 0; m < 9; ++m) t4[m] = 0.f;
 #pragma unroll
-                for (int m = 0; m < 7; ++m) {
-                    float tm = 0.f;
-                    if (L >= 3) { const float hv = H3[m]; tm = ps[0] * hv; ec[0] += B3[m] * hv; bt += B3[m] * tm; }
-                    t3[m] = tm;
-                }
+                    for (int q = 0; q < W::C1 / 4; ++q) {
+                        const float4 p = *reinterpret_cast<const float4*>(pr + 4 * q), d = *reinterpret_cast<const float4*>(pr + W::C1 + 4 * q);
 #pragma unroll
-                for (int m = 0; m < 9; ++m) {
-                    float tm = 0.f;
-                    if (L >= 4) { const float hv = H4[m]; tm = ps[0] * hv; ec[0] += B4[m] * hv; bt += B4[m] * tm; }
-                    t4[m] = tm;
+                        for (int m = 0; m < 3; ++m) {
+                            const float4 hv = *reinterpret_cast<const float4*>(H1 + m * W::C1 + 4 * q);
+                            t1[m] += p.x * hv.x + p.y * hv.y + p.z * hv.z + p.w * hv.w;
+                            pr1 += B1[m] * (d.x * hv.x + d.y * hv.y + d.z * hv.z + d.w * hv.w);
+                        }
+                        if (4 * q < W::C2) {
+#pragma unroll
+                            for (int m = 0; m < 5; ++m) {
+                                const float4 hv = *reinterpret_cast<const float4*>(H2 + m * W::C2 + 4 * q);
+                                t2[m] += p.x * hv.x + p.y * hv.y + p.z * hv.z + p.w * hv.w;
+                                pr1 += B2[m] * (d.x * hv.x + d.y * hv.y + d.z * hv.z + d.w * hv.w);
+                            }
+                        }
+                        if (q == 0 && L >= 3) {
+#pragma unroll
+                            for (int m = 0; m < 7; ++m) { const float hv = H3[m]; t3[m] = p.x * hv; pr1 += B3[m] * (d.x * hv); }
+                        }
+                        if (q == 0 && L >= 4) {
+#pragma unroll
+                            for (int m = 0; m < 9; ++m) { const float hv = H4[m]; t4[m] = p.x * hv; pr1 += B4[m] * (d.x * hv); }
+                        }
+                    }
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) bt += B1[m] * t1[m];
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) bt += B2[m] * t2[m];
+                    if (L >= 3) {
+#pragma unroll
+                        for (int m = 0; m < 7; ++m) bt += B3[m] * t3[m];
+                    }
+                    if (L >= 4) {
+#pragma unroll
+                        for (int m = 0; m < 9; ++m) bt += B4[m] * t4[m];
+                    }
+                } else {
+                    float ps[W::C1], dps[W::C1], ec[W::C1];
+#pragma unroll
+                    for (int q = 0; q < W::C1 / 4; ++q) {
+                        const float4 p4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + 4 * q);
+                        const float4 d4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + W::C1 + 4 * q);
+                        ps[4 * q] = p4.x; ps[4 * q + 1] = p4.y; ps[4 * q + 2] = p4.z; ps[4 * q + 3] = p4.w;
+                        dps[4 * q] = d4.x; dps[4 * q + 1] = d4.y; dps[4 * q + 2] = d4.z; dps[4 * q + 3] = d4.w;
+                    }
+#pragma unroll
+                    for (int k = 0; k < W::C1; ++k) ec[k] = 0.f;
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        float tm = 0.f;
+#pragma unroll
+                        for (int k = 0; k < W::C1; ++k) { const float hv = H1[m * W::C1 + k]; tm += ps[k] * hv; ec[k] += B1[m] * hv; }
+                        t1[m] = tm; bt += B1[m] * tm;
+                    }
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) {
+                        float tm = 0.f;
+#pragma unroll
+                        for (int k = 0; k < W::C2; ++k) { const float hv = H2[m * W::C2 + k]; tm += ps[k] * hv; ec[k] += B2[m] * hv; }
+                        t2[m] = tm; bt += B2[m] * tm;
+                    }
+#pragma unroll
+                    for (int m = 0; m < 7; ++m) {
+                        float tm = 0.f;
+                        if (L >= 3) { const float hv = H3[m]; tm = ps[0] * hv; ec[0] += B3[m] * hv; bt += B3[m] * tm; }
+                        t3[m] = tm;
+                    }
+#pragma unroll
+                    for (int m = 0; m < 9; ++m) {
+                        float tm = 0.f;
+                        if (L >= 4) { const float hv = H4[m]; tm = ps[0] * hv; ec[0] += B4[m] * hv; bt += B4[m] * tm; }
+                        t4[m] = tm;
+                    }
+#pragma unroll
+                    for (int k = 0; k < W::C1; ++k) pr1 += ec[k] * dps[k];
                 }
                 const float w = chi * chi;
-                float pr1 = 0.f;
-#pragma unroll
-                for (int k = 0; k < W::C1; ++k) pr1 += ec[k] * dps[k];
                 float ux, uy, uz;
                 harmonics_grad_contract<L>(gux, guy, guz, t1, t2, t3, t4, &ux, &uy, &uz);
                 const float pux = w * ux, puy = w * uy, puz = w * uz;
-                const float p_rho = chi * sa + w * pr1;
-                const float p_chi = sb + 2.0f * chi * bt;
-                const float dEdrho = p_rho + (p_chi + 2.0f * chi * ds0 + 4.0f * w * chi * ds1) * dchi;
+                float dEdrho;
+                if (PR) {        // sa = sum_c G_c (chi psi_c)', dps = (chi psi)'
+                    dEdrho = sa + chi * (pr1 + dchi * bt) + (2.0f * chi * ds0 + 4.0f * w * chi * ds1) * dchi;
+                } else {         // sa = sum_c G_c psi_c', sb = sum_c G_c psi_c, dps = psi'
+                    const float p_rho = chi * sa + w * pr1;
+                    const float p_chi = sb + 2.0f * chi * bt;
+                    dEdrho = p_rho + (p_chi + 2.0f * chi * ds0 + 4.0f * w * chi * ds1) * dchi;
+                }
                 const float dot = pux * gux + puy * guy + puz * guz;
                 const float gx = dEdrho * gux + (pux - dot * gux) * inv_rho;
                 const float gy = dEdrho * guy + (puy - dot * guy) * inv_rho;
@@ -720,7 +850,7 @@ k_edge_backward(const EdgeArgs a) {
         int qn = 0;
         for (int base = 0; base < len; base += 32) {
             const int e = base + lane;                                // offset inside the row
-            const Geom g = edge_geometry<false>(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
+            const Geom g = edge_geometry<PR>(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
             if (g.valid && p < 32) {
@@ -747,14 +877,26 @@ k_edge_backward(const EdgeArgs a) {
         }
         if (qn > 0) run_batch(qn);
     }
-    // block partial of sum_e g (x) r, in double, fixed order
+    // block partial of sum_e g (x) r, in double, fixed order: eight components change lanes in halves, so that
+    // lane 4 k ends with the sum of component k; the ninth goes through every step
+    double v9 = (double)vir[8], v8[8];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        double v = (double)vir[k];
+    for (int k = 0; k < 8; ++k) v8[k] = (double)vir[k];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-        if (lane == 0) vsum[wid][k] = v;
+    for (int n = 4, off = 16; n >= 1; n >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const double send = up ? v8[k] : v8[k + n], mine = up ? v8[k + n] : v8[k];
+            v8[k] = mine + __shfl_xor_sync(kFull, send, off);
+        }
     }
+    v8[0] += __shfl_xor_sync(kFull, v8[0], 2);
+    v8[0] += __shfl_xor_sync(kFull, v8[0], 1);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v9 += __shfl_xor_sync(kFull, v9, off);
+    if ((lane & 3) == 0) vsum[wid][lane >> 2] = v8[0];
+    if (lane == 0) vsum[wid][8] = v9;
     __syncthreads();
     if (threadIdx.x < 9) {
         double v = 0.0;
@@ -767,17 +909,21 @@ k_edge_backward(const EdgeArgs a) {
 // per-pair amplitude tables already hold the modes, so the kernels without them are used
 template <int C0, int L>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    if (a.table_uni) k_edge_forward<C0, L, false, true><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
+    if (a.uni) k_edge_forward<C0, L, false, true><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     else if (a.d.R > 0) k_edge_forward<C0, L, true, false><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     else k_edge_forward<C0, L, false, false><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 template <int C0, int L>
 cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    const bool hasr = a.d.R > 0 && !a.table_uni;
-    const size_t bytes = hasr ? BwdSmem<C0, L, true>::bytes : BwdSmem<C0, L, false>::bytes;
-    auto kern = a.table_uni ? k_edge_backward<C0, L, false, true>
-                            : (hasr ? k_edge_backward<C0, L, true, false> : k_edge_backward<C0, L, false, false>);
+    const bool hasr = a.d.R > 0 && !a.uni;
+    const bool few = a.a1 - a.a0 > 148 * 24 && a.a1 - a.a0 <= 148 * 32;
+    const size_t bytes = a.uni ? BwdSmem<C0, L, false, true>::bytes : (hasr ? BwdSmem<C0, L, true, false>::bytes : BwdSmem<C0, L, false, false>::bytes);
+    constexpr bool FEW = C0 <= 64;           // (wider ones have no such variant)
+    auto kern = few ? (a.uni ? k_edge_backward<C0, L, false, true, FEW>
+                             : (hasr ? k_edge_backward<C0, L, true, false, FEW> : k_edge_backward<C0, L, false, false, FEW>))
+                    : (a.uni ? k_edge_backward<C0, L, false, true, false>
+                             : (hasr ? k_edge_backward<C0, L, true, false, false> : k_edge_backward<C0, L, false, false, false>));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
@@ -797,18 +943,18 @@ cudaError_t dispatch(const EdgeArgs& a, int blocks, cudaStream_t st) {
 }
 
 // Tables of psi_c(rho) = gamma_c g_c(rho) + beta_c + sum_mu U_c,mu q_mu(rho) for the ordered
-// pairs (present[a], present[b]), stored as [a * n_present + b][row][3][C0] in the format of the
+// pairs (present[a], present[b]), stored as [a * n_present + b][row][3][C0] (below C0 = 32) in the format of the
 // radial table: the cubic coefficients are linear in the tabulated functions, so the same
-// combination of the coefficient rows of [g, q] gives them; and as [..][n_vrows][2][C0] in that of the value
-// table.  Two passes: the first finds the largest magnitudes of the coefficients that are packed (the scale
+// combination of the coefficient rows of [g, q] gives them; and as [..][n_vrows][2][C0] in those of the
+// value and product tables.  Two passes: the first finds the largest magnitudes of the coefficients that are packed (the scale
 // of the words), the second writes the rows.
 template <bool WRITE>
 __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, const float* __restrict__ pairmod,
                                    const int* __restrict__ present, int n_present, float* __restrict__ scale,
-                                   float* __restrict__ out, float* __restrict__ vout) {
+                                   float* __restrict__ out, float* __restrict__ vout, float* __restrict__ dout) {
     const int64_t per_pair = (int64_t)d.n_rows * d.C0;
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // over [pair][row][c]
-    float c2 = 0.f, c3 = 0.f, a1 = 0.f, a2 = 0.f;
+    float c2 = 0.f, c3 = 0.f, a1 = 0.f, a2 = 0.f, b1 = 0.f, b2 = 0.f;
     if (idx < per_pair * n_present * n_present) {
         const int pr = (int)(idx / per_pair);
         const int64_t in_pair = idx - pr * per_pair;
@@ -842,8 +988,17 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
                 vrow[c] = (float)p[0];
                 vrow[d.C0 + c] = __uint_as_float(tab_pack((float)p[1], (float)p[2], tab_step2(scale[2]), tab_step3(scale[3])));
             }
+            if (!wide_channels(d.C0)) continue;
+            double q[4];                                   // envelope products (product_piece)
+            product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, (double)row * d.dx + (sub + 0.5) * w, (double)d.rc, q);
+            b1 = fmaxf(b1, fabsf((float)q[1])); b2 = fmaxf(b2, fabsf((float)q[2]));
+            if (WRITE) {
+                float* drow = dout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
+                drow[c] = (float)q[0];
+                drow[d.C0 + c] = __uint_as_float(tab_pack((float)q[1], (float)q[2], tab_step2(scale[4]), tab_step3(scale[5])));
+            }
         }
-        if (WRITE) {
+        if (WRITE && !wide_channels(d.C0)) {
             float* orow = out + ((size_t)pr * d.n_rows + row) * 3 * d.C0;
             orow[c] = (float)v[0];
             orow[d.C0 + c] = (float)v[1];
@@ -851,9 +1006,9 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
         }
     }
     if (!WRITE) {        // non-negative floats order like their bit patterns
-        float mx[4] = {fabsf(c2), fabsf(c3), a1, a2};
+        float mx[6] = {fabsf(c2), fabsf(c3), a1, a2, b1, b2};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 6; ++k) {
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], off));
             if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(scale) + k, __float_as_uint(mx[k]));
@@ -864,14 +1019,14 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
 }  // namespace
 
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
-                                    int n_present, float* scale, float* out, float* vout, cudaStream_t st) {
+                                    int n_present, float* scale, float* out, float* vout, float* dout, cudaStream_t st) {
     const int64_t n = (int64_t)d.n_rows * d.C0 * n_present * n_present;
     if (n == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(scale, 0, 4 * sizeof(float), st);
+    cudaError_t e = cudaMemsetAsync(scale, 0, 6 * sizeof(float), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((n + 255) / 256);
-    k_fuse_pair_tables<false><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout);
-    k_fuse_pair_tables<true><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout);
+    k_fuse_pair_tables<false><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout, dout);
+    k_fuse_pair_tables<true><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout, dout);
     return cudaGetLastError();
 }
 

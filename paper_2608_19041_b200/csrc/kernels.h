@@ -59,7 +59,7 @@ struct EdgeArgs {
     float* state;           // [a1-a0][SP]: forward writes sums; backward reads dE/d(sums)
     float* g;               // [E][3] per-edge gradient (backward)
     double* virial_part;    // [blocks][9] partial virial sums (backward)
-    // non-null when the species present are few enough for per-pair amplitude tables:
+    bool uni;               // the species present are few enough for per-pair amplitude tables:
     // [n_present^2][n_rows][3][C0] cubic pieces of psi_c(rho) of each ordered pair, in the format
     // of the radial table (launch_fuse_pair_tables), read instead of table, pairmod and the radial
     // modes; uni_scale[0..1] = largest |c2|, |c3| of these tables (scale of their packed words)
@@ -72,12 +72,16 @@ struct EdgeArgs {
     // |a1|, |a2| of vtable_uni
     const float* vtable;
     const float* vtable_uni;
+    // product tables (product_piece), read by the backward pass (wide_channels); uni_scale[4..5] = largest |a1|,
+    // |a2| of dtable_uni.  There is no table_uni then.
+    const float* dtable;
+    const float* dtable_uni;
     const int* species_slot;    // [T] species -> index among the species present
     int n_present;
 };
 // present: device array of the n_present species indices, ascending
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
-                                    int n_present, float* scale, float* out, float* vout, cudaStream_t st);
+                                    int n_present, float* scale, float* out, float* vout, float* dout, cudaStream_t st);
 cudaError_t launch_edge_forward(const EdgeArgs& a, cudaStream_t st);
 cudaError_t launch_edge_backward(const EdgeArgs& a, int* n_blocks, cudaStream_t st);
 int edge_backward_blocks(int n_rows_in_tile);

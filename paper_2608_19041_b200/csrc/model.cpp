@@ -315,13 +315,15 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         // values alone: quadratic pieces about the middle of (a fraction of) the interval
         d.v_sub = 1;
         while (D1 / d.v_sub > 0.0025) d.v_sub *= 2;
-        std::vector<float> va;
-        double m0 = 0, q1 = 0, q2 = 0, q3 = 0;
+        std::vector<float> va, da;
+        double m0 = 0, q1 = 0, q2 = 0, q3 = 0, n0 = 0, r1 = 0, r2 = 0, r3 = 0;
+        const bool products = wide_channels(C0) && R == 0;
         for (;; d.v_sub *= 2) {
             const double w = D1 / d.v_sub, hw = 0.5 * w;
             va.assign((size_t)n_rows * d.v_sub * NC * 3, 0.0f);
-            m0 = q1 = q2 = q3 = 0;
-            float* o = va.data();
+            if (products) da.assign(va.size(), 0.0f);
+            m0 = q1 = q2 = q3 = n0 = r1 = r2 = r3 = 0;
+            float *o = va.data(), *od = da.data();
             for (int s = 0; s < n_rows; ++s) {
                 const double* ya = &Y[(size_t)s * 2 * NC];
                 const double* yb = &Y[(size_t)(s + 1) * 2 * NC];
@@ -334,24 +336,39 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                         m0 = std::max(m0, std::fabs(p[0])); q1 = std::max(q1, std::fabs(p[1]));
                         q2 = std::max(q2, std::fabs(p[2])); q3 = std::max(q3, std::fabs(c3));
                         o[0] = (float)p[0]; o[1] = (float)p[1]; o[2] = (float)p[2];
+                        if (!products || c >= C0) continue;        // (the modes' products are formed from their values)
+                        double q[4];
+                        float* t = od + (o - va.data());
+                        product_piece(ya[c], p0, c2, c3, (sub + 0.5) * w, hw, s * D1 + (sub + 0.5) * w, m->rc, q);
+                        n0 = std::max(n0, std::fabs(q[0])); r1 = std::max(r1, std::fabs(q[1]));
+                        r2 = std::max(r2, std::fabs(q[2])); r3 = std::max(r3, std::fabs(q[3]));
+                        t[0] = (float)q[0]; t[1] = (float)q[1]; t[2] = (float)q[2];
                     }
             }
+            const double off_d = r3 * hw * hw * hw / 4 + r1 / (2.0 * kTabI2Max) * hw + r2 / (2.0 * kTabI3Max) * hw * hw;
             const double off = q3 * hw * hw * hw / 4 + q1 / (2.0 * kTabI2Max) * hw + q2 / (2.0 * kTabI3Max) * hw * hw;
-            if (off <= m0 * 0x1p-24 || n_rows * (int64_t)d.v_sub > 100000) break;    // at most the rounding of a0
+            if ((off <= m0 * 0x1p-24 && off_d <= n0 * 0x1p-23) || n_rows * (int64_t)d.v_sub > 100000) break;    // about the rounding of a0
         }
         d.n_vrows = n_rows * d.v_sub;
+        for (d.v_shift = 0; (1 << d.v_shift) < d.v_sub; ++d.v_shift) {}
+        d.tab_d1 = tab_step2((float)r1); d.tab_d2 = tab_step3((float)r2);
         d.vdx = (float)(D1 / d.v_sub); d.inv_vdx = (float)(d.v_sub / D1);
         d.tab_v1 = tab_step2((float)q1); d.tab_v2 = tab_step3((float)q2);
         m->vtable.assign((size_t)d.n_vrows * 2 * CP, 0.0f);
-        const float* v = va.data();
-        for (int s = 0; s < d.n_vrows; ++s) {
-            float* row = &m->vtable[(size_t)s * 2 * CP];
-            for (int c = 0; c < NC; ++c, v += 3) {
-                row[c] = v[0];
-                const unsigned w = tab_pack(v[1], v[2], d.tab_v1, d.tab_v2);
-                std::memcpy(&row[CP + c], &w, sizeof(w));
+        auto pack = [&](const std::vector<float>& pieces, float k1, float k2, std::vector<float>* out) {
+            const float* v = pieces.data();
+            for (int s = 0; s < d.n_vrows; ++s) {
+                float* row = &(*out)[(size_t)s * 2 * CP];
+                for (int c = 0; c < NC; ++c, v += 3) {
+                    row[c] = v[0];
+                    const unsigned w = tab_pack(v[1], v[2], k1, k2);
+                    std::memcpy(&row[CP + c], &w, sizeof(w));
+                }
             }
-        }
+        };
+        pack(va, d.tab_v1, d.tab_v2, &m->vtable);
+        m->dtable.assign(products ? m->vtable.size() : 0, 0.0f);
+        if (products) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
         d.tab_k2 = tab_step2(m2); d.tab_k3 = tab_step3(m3);
         for (int s = 0; s < n_rows; ++s)
             for (int c = 0; c < NC; ++c) {
