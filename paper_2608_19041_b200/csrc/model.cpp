@@ -393,27 +393,39 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                 }
             }
         m->pairmod.assign((size_t)T * T * (2 + R) * C0, 0.0f);
-        std::vector<double> hid(Hp), o(NO);
+        // four neighbours at a time share every row of the output weights (the sums of each keep their order)
+        constexpr int NB = 4;
+        std::vector<double> hid((size_t)Hp * NB), o((size_t)NO * NB);
         for (int a = 0; a < T; ++a)
-            for (int b = 0; b < T; ++b) {
-                for (int k = 0; k < Hp; ++k) {
-                    const double g = top[(size_t)a * 2 * Hp + k] + bot[(size_t)b * 2 * Hp + k];
-                    const double v = top[(size_t)a * 2 * Hp + Hp + k] + bot[(size_t)b * 2 * Hp + Hp + k];
-                    hid[k] = g * sigmoid(g) * v;
-                }
+            for (int b0 = 0; b0 < T; b0 += NB) {
+                const int nb = std::min(NB, T - b0);
+                for (int k = 0; k < Hp; ++k)
+                    for (int i = 0; i < NB; ++i) {
+                        const size_t b = (size_t)(b0 + std::min(i, nb - 1));
+                        const double g = top[(size_t)a * 2 * Hp + k] + bot[b * 2 * Hp + k];
+                        const double v = top[(size_t)a * 2 * Hp + Hp + k] + bot[b * 2 * Hp + Hp + k];
+                        hid[(size_t)k * NB + i] = g * sigmoid(g) * v;
+                    }
                 std::fill(o.begin(), o.end(), 0.0);
+                double *o0 = o.data(), *o1 = o0 + NO, *o2 = o1 + NO, *o3 = o2 + NO;
                 for (int k = 0; k < Hp; ++k) {
-                    const double hk = hid[k];
-                    const double* w = &W_p_out[(size_t)k * NO];
-                    for (int j = 0; j < NO; ++j) o[j] += hk * w[j];
+                    const double *hk = &hid[(size_t)k * NB], *w = &W_p_out[(size_t)k * NO];
+                    const double h0 = hk[0], h1 = hk[1], h2 = hk[2], h3 = hk[3];
+                    for (int j = 0; j < NO; ++j) {
+                        const double wj = w[j];
+                        o0[j] += h0 * wj; o1[j] += h1 * wj; o2[j] += h2 * wj; o3[j] += h3 * wj;
+                    }
                 }
-                float* pm = &m->pairmod[(size_t)(a * T + b) * (2 + R) * C0];
-                for (int c = 0; c < C0; ++c) {
-                    pm[c] = (float)(1.0 + std::tanh(0.1 * o[c]));
-                    pm[C0 + c] = (float)(X0[(size_t)a * C0 + c] + X0[(size_t)b * C0 + c] +
-                                         std::tanh(0.1 * o[C0 + c]));
-                    for (int q = 0; q < R; ++q)  // U[c][q] = tanh(w[c*R + q])
-                        pm[(size_t)(2 + q) * C0 + c] = (float)std::tanh(0.1 * o[2 * C0 + c * R + q]);
+                for (int i = 0; i < nb; ++i) {
+                    const int b = b0 + i;
+                    const double* oi = &o[(size_t)i * NO];
+                    float* pm = &m->pairmod[(size_t)(a * T + b) * (2 + R) * C0];
+                    for (int c = 0; c < C0; ++c) {
+                        pm[c] = (float)(1.0 + std::tanh(0.1 * oi[c]));
+                        pm[C0 + c] = (float)(X0[(size_t)a * C0 + c] + X0[(size_t)b * C0 + c] + std::tanh(0.1 * oi[C0 + c]));
+                        for (int q = 0; q < R; ++q)  // U[c][q] = tanh(w[c*R + q])
+                            pm[(size_t)(2 + q) * C0 + c] = (float)std::tanh(0.1 * oi[2 * C0 + c * R + q]);
+                    }
                 }
             }
     }
