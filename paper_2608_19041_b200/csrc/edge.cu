@@ -26,10 +26,17 @@ namespace {
 // registers and shared memory waiting for it (measured at eight / four / two warps per block, 131072
 // atoms of the 64-species workload: backward 1.535 / 1.487 / 1.479 ms, forward 1.318 / 1.301 / 1.294 ms;
 // four keeps the per-block virial partials at a quarter of the atom count).
-constexpr int kWarpsPerBlock = 4;
+constexpr int kWarpsPerBlock = kEdgeRowsPerBlock;
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+
+// the part of a row of *len edges from *e0 on that warp w takes, where the warps of a block share a row
+__device__ __forceinline__ void quarter_of_row(int w, eidx_t* e0, int* len) {
+    const int first = (int)((int64_t)*len * w / kWarpsPerBlock), last = (int)((int64_t)*len * (w + 1) / kWarpsPerBlock);
+    *e0 += first;
+    *len = last - first;
+}
 
 struct Geom {
     float dx, dy, dz, rho, inv_rho, ux, uy, uz, chi, dchi, t;
@@ -375,10 +382,12 @@ template <int C0, int L, bool HASR, bool UNI> struct BwdSmem {          // dynam
 // Up to C0 = 64 a fourth group of eight resident warps per SM (64 registers, a few spilled words) is worth more
 // than the registers: the channel-parallel phase waits on load latency (measured: 6-10 % on the
 // forward kernel at C0 = 8 .. 64, 2 % the other way at C0 = 128, which stays at 24 warps).
-template <int C0, int L, bool HASR, bool UNI>
+// SPLIT: the warps of a block take a quarter each of one row (edge_rows_split) and add up their sums at the end.
+template <int C0, int L, bool HASR, bool UNI, bool SPLIT>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 ? 4 : 3) * 8 / kWarpsPerBlock)
 k_edge_forward(const EdgeArgs a) {
     using W = Widths<C0, L>;
+    static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");
     // scratch per warp: the parked amplitudes of the batch, first the radial modes and then (once the
     // amplitudes are done) the harmonic weights chi^2 B_lm
     __shared__ __align__(16) float scratch[kWarpsPerBlock][W::SCRATCH];
@@ -387,8 +396,9 @@ k_edge_forward(const EdgeArgs a) {
     // the table reads) and the edge vector
     __shared__ int4 q_es[kWarpsPerBlock][32];
     __shared__ float q_d[kWarpsPerBlock][3 * 32];
+    __shared__ double s_part[SPLIT ? kWarpsPerBlock : 1][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int i = a.a0 + blockIdx.x * kWarpsPerBlock + wid;
+    const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
     if (i >= a.a1) return;
     float* const psi_s = scratch[wid];             // [32][PP]
     float* const qm = scratch[wid] + W::OW;        // [32][PQ] radial modes
@@ -399,8 +409,9 @@ k_edge_forward(const EdgeArgs a) {
     const double xi = a.xs[3 * (size_t)i], yi = a.xs[3 * (size_t)i + 1], zi = a.xs[3 * (size_t)i + 2];
     const int ti = UNI ? a.species_slot[a.type_s[i]] : a.type_s[i];
     const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + 2)) : a.d.tab_v1, k3 = UNI ? tab_step3(__ldg(a.uni_scale + 3)) : a.d.tab_v2;
-    const eidx_t e0 = a.row_ptr[i];
-    const int len = (int)(a.row_ptr[i + 1] - e0);      // edge offsets are 64-bit, offsets inside a row are not
+    eidx_t e0 = a.row_ptr[i];
+    int len = (int)(a.row_ptr[i + 1] - e0);      // edge offsets are 64-bit, offsets inside a row are not
+    if (SPLIT) quarter_of_row(wid, &e0, &len);
     const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
     const unsigned lt_mask = (1u << lane) - 1u;
     float acc0[4] = {0.f, 0.f, 0.f, 0.f};
@@ -560,7 +571,8 @@ k_edge_forward(const EdgeArgs a) {
         s0 += __shfl_xor_sync(kFull, s0, off);
         s1 += __shfl_xor_sync(kFull, s1, off);
     }
-    float* row_out = a.state + (size_t)(i - a.a0) * a.d.SP;
+    float* const row_glob = a.state + (size_t)(i - a.a0) * a.d.SP;
+    float* const row_out = SPLIT ? psi_s : row_glob;        // (the batches are done with the scratch)
     if (sub == 0) *reinterpret_cast<float4*>(row_out + c) = make_float4(acc0[0], acc0[1], acc0[2], acc0[3]);
 #pragma unroll
     for (int sl = 0; sl < W::SLOTS; ++sl) {
@@ -577,10 +589,24 @@ k_edge_forward(const EdgeArgs a) {
             for (int k = 0; k < 4; ++k) if (k < j_n[sl]) o[k] = accJ[sl][k];
         }
     }
-    if (lane == 0) {
+    if (SPLIT) {
+        if (lane == 0) { s_part[wid][0] = s0; s_part[wid][1] = s1; }
+        __syncthreads();
+        for (int v = threadIdx.x; v < C0 + W::NHI; v += kWarpsPerBlock * 32) {      // (S = C0 + NHI)
+            float t = scratch[0][v];
+#pragma unroll
+            for (int w = 1; w < kWarpsPerBlock; ++w) t += scratch[w][v];
+            row_glob[v] = t;
+        }
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int w = 1; w < kWarpsPerBlock; ++w) { s0 += s_part[w][0]; s1 += s_part[w][1]; }
+        }
+    }
+    if (SPLIT ? threadIdx.x == 0 : lane == 0) {
         const float h0 = (float)s0, h1 = (float)s1;
-        row_out[a.d.S] = h0; row_out[a.d.S + 1] = h1;
-        row_out[a.d.S + 2] = (float)(s0 - (double)h0); row_out[a.d.S + 3] = (float)(s1 - (double)h1);
+        row_glob[a.d.S] = h0; row_glob[a.d.S + 1] = h1;
+        row_glob[a.d.S + 2] = (float)(s0 - (double)h0); row_glob[a.d.S + 3] = (float)(s1 - (double)h1);
     }
 }
 
@@ -592,7 +618,7 @@ k_edge_forward(const EdgeArgs a) {
 // the edge's lane then does the whole degree >= 1 contraction by itself against the
 // destination's gradient block held in shared memory, and assembles dE/dr_ij.  Edges in the
 // skin shell get a zero gradient as soon as their geometry is known.
-template <int C0, int L, bool HASR, bool UNI, bool FEW>
+template <int C0, int L, bool HASR, bool UNI, bool FEW, bool SPLIT>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, BwdShape<C0, L, HASR, UNI, FEW>::warps / kWarpsPerBlock)
 k_edge_backward(const EdgeArgs a) {
     using SM = BwdSmem<C0, L, HASR, UNI>;
@@ -610,7 +636,7 @@ k_edge_backward(const EdgeArgs a) {
     int4* const qes = reinterpret_cast<int4*>(wbase + SM::per_warp - SM::queue_floats);
     float* const qm = reinterpret_cast<float*>(qes) - SM::mode_floats;   // [2][32][kMaxR]
     float* const qd = reinterpret_cast<float*>(qes + 32);        // [5][32]
-    const int i = a.a0 + blockIdx.x * kWarpsPerBlock + wid;
+    const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
     const bool active = i < a.a1;
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -625,8 +651,9 @@ k_edge_backward(const EdgeArgs a) {
         const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + (PR ? 2 : 0))) : (PR ? a.d.tab_v1 : a.d.tab_k2),
                     k3 = UNI ? tab_step3(__ldg(a.uni_scale + (PR ? 3 : 1))) : (PR ? a.d.tab_v2 : a.d.tab_k3);
         const float d1 = UNI ? tab_step2(__ldg(a.uni_scale + 4)) : a.d.tab_d1, d2 = UNI ? tab_step3(__ldg(a.uni_scale + 5)) : a.d.tab_d2;
-        const eidx_t e0 = a.row_ptr[i];
-        const int len = (int)(a.row_ptr[i + 1] - e0);
+        eidx_t e0 = a.row_ptr[i];
+        int len = (int)(a.row_ptr[i + 1] - e0);
+        if (SPLIT) quarter_of_row(wid, &e0, &len);
         const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
         const float* grow = a.state + (size_t)(i - a.a0) * a.d.SP;
         float h0[4 * G];
@@ -717,7 +744,7 @@ k_edge_backward(const EdgeArgs a) {
             __syncwarp();
             if (lane < nb) {
                 const float gdx = qd[lane], gdy = qd[32 + lane], gdz = qd[64 + lane], dchi = qd[96 + lane];
-                const int e = __float_as_int(qd[128 + lane]);       // offset inside the row
+                const int e = __float_as_int(qd[128 + lane]);       // offset inside the warp's part of the row
                 const float chi = __int_as_float(qes[lane].w);
                 const float inv_rho = 1.0f / sqrtf(gdx * gdx + gdy * gdy + gdz * gdz + kEpsReg * kEpsReg);
                 const float gux = gdx * inv_rho, guy = gdy * inv_rho, guz = gdz * inv_rho;
@@ -849,7 +876,7 @@ k_edge_backward(const EdgeArgs a) {
 
         int qn = 0;
         for (int base = 0; base < len; base += 32) {
-            const int e = base + lane;                                // offset inside the row
+            const int e = base + lane;
             const Geom g = edge_geometry<PR>(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
@@ -907,34 +934,39 @@ k_edge_backward(const EdgeArgs a) {
 
 
 // per-pair amplitude tables already hold the modes, so the kernels without them are used
-template <int C0, int L>
+template <int C0, int L, bool SPLIT>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    if (a.uni) k_edge_forward<C0, L, false, true><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
-    else if (a.d.R > 0) k_edge_forward<C0, L, true, false><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
-    else k_edge_forward<C0, L, false, false><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
+    if (a.uni) k_edge_forward<C0, L, false, true, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
+    else if (a.d.R > 0) k_edge_forward<C0, L, true, false, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
+    else k_edge_forward<C0, L, false, false, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     return cudaGetLastError();
 }
-template <int C0, int L>
-cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    const bool hasr = a.d.R > 0 && !a.uni;
+template <int C0, int L, bool HASR, bool UNI>
+cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
     const bool few = a.a1 - a.a0 > 148 * 24 && a.a1 - a.a0 <= 148 * 32;
-    const size_t bytes = a.uni ? BwdSmem<C0, L, false, true>::bytes : (hasr ? BwdSmem<C0, L, true, false>::bytes : BwdSmem<C0, L, false, false>::bytes);
+    constexpr size_t bytes = BwdSmem<C0, L, HASR, UNI>::bytes;
     constexpr bool FEW = C0 <= 64;           // (wider ones have no such variant)
-    auto kern = few ? (a.uni ? k_edge_backward<C0, L, false, true, FEW>
-                             : (hasr ? k_edge_backward<C0, L, true, false, FEW> : k_edge_backward<C0, L, false, false, FEW>))
-                    : (a.uni ? k_edge_backward<C0, L, false, true, false>
-                             : (hasr ? k_edge_backward<C0, L, true, false, false> : k_edge_backward<C0, L, false, false, false>));
+    auto kern = split ? k_edge_backward<C0, L, HASR, UNI, false, true>
+                      : (few ? k_edge_backward<C0, L, HASR, UNI, FEW, false> : k_edge_backward<C0, L, HASR, UNI, false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
     return cudaGetLastError();
 }
+template <bool FWD, int C0, int L>
+cudaError_t launch(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
+    if (FWD) return split ? launch_fwd_r<C0, L, true>(a, blocks, st) : launch_fwd_r<C0, L, false>(a, blocks, st);
+    if (a.uni) return launch_bwd_r<C0, L, false, true>(a, blocks, split, st);
+    if (a.d.R > 0) return launch_bwd_r<C0, L, true, false>(a, blocks, split, st);
+    return launch_bwd_r<C0, L, false, false>(a, blocks, split, st);
+}
 
 template <bool FWD>
-cudaError_t dispatch(const EdgeArgs& a, int blocks, cudaStream_t st) {
-#define UMLMD_CASE(C0v, Lv)                                                       \
-    if (a.d.C0 == C0v && a.d.L == Lv)                                             \
-        return FWD ? launch_fwd_r<C0v, Lv>(a, blocks, st) : launch_bwd_r<C0v, Lv>(a, blocks, st);
+cudaError_t dispatch(const EdgeArgs& a, cudaStream_t st) {
+    const int rows = a.a1 - a.a0, blocks = edge_blocks(rows);
+    const bool split = edge_rows_split(rows);
+#define UMLMD_CASE(C0v, Lv) \
+    if (a.d.C0 == C0v && a.d.L == Lv) return launch<FWD, C0v, Lv>(a, blocks, split, st);
     UMLMD_CASE(8, 2) UMLMD_CASE(8, 3) UMLMD_CASE(16, 2) UMLMD_CASE(16, 3) UMLMD_CASE(32, 2)
     UMLMD_CASE(32, 3) UMLMD_CASE(64, 2) UMLMD_CASE(64, 3) UMLMD_CASE(128, 2) UMLMD_CASE(128, 3)
     UMLMD_CASE(8, 4) UMLMD_CASE(16, 4) UMLMD_CASE(32, 4) UMLMD_CASE(64, 4) UMLMD_CASE(128, 4)
@@ -1030,19 +1062,13 @@ cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const flo
     return cudaGetLastError();
 }
 
-int edge_backward_blocks(int n_rows) { return (n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock; }
-
 cudaError_t launch_edge_forward(const EdgeArgs& a, cudaStream_t st) {
-    const int rows = a.a1 - a.a0;
-    if (rows <= 0) return cudaSuccess;
-    return dispatch<true>(a, (rows + kWarpsPerBlock - 1) / kWarpsPerBlock, st);
+    return a.a1 > a.a0 ? dispatch<true>(a, st) : cudaSuccess;
 }
 
 cudaError_t launch_edge_backward(const EdgeArgs& a, int* n_blocks, cudaStream_t st) {
-    const int rows = a.a1 - a.a0;
-    *n_blocks = edge_backward_blocks(rows);
-    if (rows <= 0) return cudaSuccess;
-    return dispatch<false>(a, *n_blocks, st);
+    *n_blocks = edge_blocks(a.a1 - a.a0);
+    return a.a1 > a.a0 ? dispatch<false>(a, st) : cudaSuccess;
 }
 
 }  // namespace umd

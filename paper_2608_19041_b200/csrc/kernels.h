@@ -79,12 +79,26 @@ struct EdgeArgs {
     const int* species_slot;    // [T] species -> index among the species present
     int n_present;
 };
+constexpr int kEdgeRowsPerBlock = 4, kEdgeSplitRows = 1184;
 // present: device array of the n_present species indices, ascending
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
                                     int n_present, float* scale, float* out, float* vout, float* dout, cudaStream_t st);
 cudaError_t launch_edge_forward(const EdgeArgs& a, cudaStream_t st);
 cudaError_t launch_edge_backward(const EdgeArgs& a, int* n_blocks, cudaStream_t st);
-int edge_backward_blocks(int n_rows_in_tile);
+// Few rows: the four warps of a block share a row, a quarter of its edges each.  A warp works through a row as a
+// serial chain of table reads, which a chip with fewer than eight warps per scheduler does not hide: up to 1184 rows
+// (four warps each and every warp resident) the two edge kernels together took, a warp per row against shared, at
+// 108 / 592 / 1184 rows: C0 = 32 28 / 29 / 29 against 21 / 21 / 27 us, C0 = 64 with degree three 44 / 44 / 46 against
+// 26 / 27 / 37, C0 = 128 with 64 species 49 / 52 / 58 against 24 / 32 / 52, with four modes 173 / 191 / 208 against
+// 62 / 78 / 137; at 1776 rows sharing loses (C0 = 32: 31 against 35, C0 = 128: 63 against 63).
+inline bool edge_rows_split(int64_t rows) { return rows <= kEdgeSplitRows; }
+inline int edge_blocks(int rows) { return edge_rows_split(rows) ? rows : (rows + kEdgeRowsPerBlock - 1) / kEdgeRowsPerBlock; }
+// most blocks (partial virials) that the tiles of up to N rows, B at a time, have
+inline int64_t edge_blocks_max(int64_t N, int64_t B) {
+    if (B <= 0) return 0;
+    const int64_t last = edge_blocks((int)B), split = B < kEdgeSplitRows ? B : kEdgeSplitRows;
+    return N / B * last + (last > split ? last : split);
+}
 
 // ---- invariants.cu -------------------------------------------------------------------
 struct InvArgs {
