@@ -20,6 +20,7 @@ static_assert(kReduceBlocks * 10 >= kRedMaxBlocks, "one scratch area serves both
 __global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
                              const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
                              double* __restrict__ out, int* __restrict__ err) {
+    chain_begin();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= N) return;
     const eidx_t e0 = row_ptr[warp];
@@ -113,6 +114,7 @@ __global__ void k_scatter3(int N, const int* __restrict__ perm, const double* __
 
 __global__ void k_scatter1(int N, const int* __restrict__ perm, const double* __restrict__ in,
                            double* __restrict__ out) {
+    chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) out[perm[i]] = in[i];
 }
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(kFrameBlock) k_frame_reduce(const FrameCell* _
                                                               const float* __restrict__ g, const double* __restrict__ xs, bool want_virial,
                                                               double* __restrict__ out, int* __restrict__ err) {
     __shared__ double sh[kFrameBlock / 32 * 10];
+    chain_begin();
     const FrameCell& fc = frames[blockIdx.x];
     const int lane = threadIdx.x & 31;
     double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -219,6 +222,7 @@ __global__ void __launch_bounds__(kRedBlock) k_reduce(const double* __restrict__
                                                       int* __restrict__ err, double* __restrict__ h_out, int* __restrict__ h_err) {
     __shared__ double sh[kRedBlock / 32 * 10];
     __shared__ bool last;
+    chain_begin();
     double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     const int first = blockIdx.x * kRedBlock + threadIdx.x, step = gridDim.x * kRedBlock;
     for (int i = first; i < N; i += step) {
@@ -263,6 +267,7 @@ __global__ void __launch_bounds__(kRedBlock) k_reduce(const double* __restrict__
 __global__ void k_vv(int64_t N, double* __restrict__ pos, double* __restrict__ vel, const double* __restrict__ force,
                      const int* __restrict__ type, const double* __restrict__ inv_mass, double dt, int kicks, bool drift,
                      const double* __restrict__ scale) {
+    chain_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const double c = 0.5 * dt * kAccelUnit * inv_mass[type[i]];
@@ -324,6 +329,7 @@ __global__ void __launch_bounds__(kRedBlock) k_kick_thermostat(int64_t N, double
                                                                double* __restrict__ st, int halves, NhcParams p) {
     __shared__ double sh[kRedBlock / 32];
     __shared__ bool last;
+    chain_begin();
     double v[1] = {0};
     for (int64_t i = (int64_t)blockIdx.x * kRedBlock + threadIdx.x; i < N; i += (int64_t)gridDim.x * kRedBlock) {
         const int t = type[i];
@@ -393,8 +399,7 @@ cudaError_t launch_force_assembly(const NeighborDev& nb, const float* g, double*
                                   int* d_err, cudaStream_t st) {
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
-    k_force_rows<<<(N + 7) / 8, 256, 0, st>>>(N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err);
-    return cudaGetLastError();
+    return launch_chained(k_force_rows, (N + 7) / 8, 256, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err);
 }
 
 cudaError_t launch_atom_virial(const NeighborDev& nb, const float* g, double* d_out, cudaStream_t st) {
@@ -417,24 +422,22 @@ cudaError_t launch_scatter_forces(const NeighborDev& nb, const double* f_sorted,
 cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
                                 double* d_out, int* d_err, cudaStream_t st) {
     if (nb.n_frames <= 0) return cudaSuccess;
-    k_frame_reduce<<<nb.n_frames, kFrameBlock, 0, st>>>(nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial, d_out, d_err);
-    return cudaGetLastError();
+    return launch_chained(k_frame_reduce, nb.n_frames, kFrameBlock, 0, st, nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial,
+                          d_out, d_err);
 }
 
 cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part,
                                         int n_part, double* scratch, unsigned* counter, double* out, int* d_err, double* h_out,
                                         int* h_err, cudaStream_t st) {
     const int N = (int)nb.N, blocks = (N + 4 * kRedBlock - 1) / (4 * kRedBlock);
-    k_reduce<<<blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks), kRedBlock, 0, st>>>(
-        e_atom, N, nb.perm, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
-    return cudaGetLastError();
+    return launch_chained(k_reduce, blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks), kRedBlock, 0, st, e_atom, N,
+                          nb.perm, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
 }
 
 cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out, cudaStream_t st) {
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
-    k_scatter1<<<(N + 255) / 256, 256, 0, st>>>(N, nb.perm, e_sorted, d_out);
-    return cudaGetLastError();
+    return launch_chained(k_scatter1, (N + 255) / 256, 256, 0, st, N, nb.perm, e_sorted, d_out);
 }
 
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width, float* out,
@@ -456,17 +459,15 @@ cudaError_t launch_vv_kick_drift(int64_t N, double* pos, double* vel, const doub
                                  const double* inv_mass, double dt, int kicks, bool drift, const double* d_scale,
                                  cudaStream_t st) {
     if (N == 0) return cudaSuccess;
-    k_vv<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, pos, vel, force, type, inv_mass, dt, kicks, drift, d_scale);
-    return cudaGetLastError();
+    return launch_chained(k_vv, (unsigned)((N + 255) / 256), 256, 0, st, N, pos, vel, force, type, inv_mass, dt, kicks, drift, d_scale);
 }
 
 cudaError_t launch_kick_thermostat(int64_t N, double* vel, const double* force, const int* type, const double* mass,
                                    const double* inv_mass, double dt, bool kick, double* scratch, unsigned* counter, double* d_state,
                                    int halves, const NhcParams& p, cudaStream_t st) {
     const int64_t blocks = (N + 2 * kRedBlock - 1) / (2 * kRedBlock);
-    k_kick_thermostat<<<(unsigned)(blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks)), kRedBlock, 0, st>>>(
-        N, vel, force, type, mass, inv_mass, dt, kick, scratch, counter, d_state, halves, p);
-    return cudaGetLastError();
+    return launch_chained(k_kick_thermostat, (unsigned)(blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks)), kRedBlock, 0, st,
+                          N, vel, force, type, mass, inv_mass, dt, kick, scratch, counter, d_state, halves, p);
 }
 
 cudaError_t launch_kinetic_energy(int64_t N, const double* vel, const int* type, const double* mass,

@@ -397,6 +397,7 @@ k_edge_forward(const EdgeArgs a) {
     __shared__ int4 q_es[kWarpsPerBlock][32];
     __shared__ float q_d[kWarpsPerBlock][3 * 32];
     __shared__ double s_part[SPLIT ? kWarpsPerBlock : 1][2];
+    chain_begin();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
     if (i >= a.a1) return;
@@ -627,6 +628,7 @@ k_edge_backward(const EdgeArgs a) {
     using W = Widths<C0, L, G>;
     extern __shared__ __align__(16) unsigned char dsm[];
     double (*vsum)[9] = reinterpret_cast<double (*)[9]>(dsm);
+    chain_begin();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float* const wbase = reinterpret_cast<float*>(dsm + kWarpsPerBlock * 9 * sizeof(double)) + wid * SM::per_warp;
     float* const psi_s = wbase;                                  // [32][PB]: psi, dpsi of the leading channels
@@ -936,9 +938,9 @@ k_edge_backward(const EdgeArgs a) {
 // per-pair amplitude tables already hold the modes, so the kernels without them are used
 template <int C0, int L, bool SPLIT>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    if (a.uni) k_edge_forward<C0, L, false, true, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
-    else if (a.d.R > 0) k_edge_forward<C0, L, true, false, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
-    else k_edge_forward<C0, L, false, false, SPLIT><<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
+    auto kern = a.uni ? k_edge_forward<C0, L, false, true, SPLIT>
+                      : (a.d.R > 0 ? k_edge_forward<C0, L, true, false, SPLIT> : k_edge_forward<C0, L, false, false, SPLIT>);
+    kern<<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 template <int C0, int L, bool HASR, bool UNI>

@@ -193,6 +193,7 @@ struct Front {
             G123 = reinterpret_cast<const GauntSparse*>(g1);
             G233 = reinterpret_cast<const GauntSparse*>(g2);
         }
+        chain_begin();
         b0 = blockIdx.x * AT;
         nv = a.n - b0 < AT ? a.n - b0 : AT;
         C0 = d.C0; TW = d.SP - C0;
@@ -1009,8 +1010,7 @@ cudaError_t dispatch(const InvArgs& a, cudaStream_t st) {
                          : (FWD ? k_inv_forward<c1, c2, l, 8> : k_inv_backward<c1, c2, l, 8>);  \
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
         if (e != cudaSuccess) return e;                                                         \
-        kern<<<blocks, wide ? 512 : 256, bytes, st>>>(a);                                       \
-        return cudaGetLastError();                                                              \
+        return launch_chained(kern, blocks, wide ? 512 : 256, bytes, st, a);                    \
     }
     UMLMD_CASE(4, 4, 2) UMLMD_CASE(4, 4, 3) UMLMD_CASE(8, 4, 2) UMLMD_CASE(8, 4, 3)
     UMLMD_CASE(16, 8, 2) UMLMD_CASE(16, 8, 3) UMLMD_CASE(4, 4, 4) UMLMD_CASE(8, 4, 4) UMLMD_CASE(16, 8, 4)

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fused(const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    chain_begin();
 
     // The copy and the issue warp run their loops as whole warps, one elected lane issuing: the loop state
     // and the descriptors are then warp-uniform and live in uniform registers, where the copy and MMA
@@ -512,8 +513,7 @@ cudaError_t launch_mlp_fused(const MlpArgs& a, cudaStream_t st) {
     static const cudaError_t attr = cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
     if (attr != cudaSuccess) return attr;
     const int items = (a.n + g.NA - 1) / g.NA;
-    k_mlp_fused<<<items < 148 ? items : 148, THREADS, used + (uint32_t)g.stages * W_BYTES, st>>>(maps, g);
-    return cudaGetLastError();
+    return launch_chained(k_mlp_fused, items < 148 ? items : 148, THREADS, used + (uint32_t)g.stages * W_BYTES, st, maps, g);
 }
 
 }  // namespace umd

@@ -562,6 +562,7 @@ __global__ void k_gather_positions(int N, const int* __restrict__ perm, const in
                                    const double* __restrict__ pos, const double* __restrict__ xs0,
                                    CellRows H, double max_disp2, const int* __restrict__ type_s,
                                    double* __restrict__ xs, float4* __restrict__ rec, int* __restrict__ err) {
+    chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const int o = perm[i];
@@ -1013,8 +1014,8 @@ cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, 
     CellRows H;
     for (int k = 0; k < 9; ++k) H.h[k] = nb.H[k];
     H.tri = nb.tri;
-    k_gather_positions<<<(N + 255) / 256, 256, 0, st>>>(N, nb.perm, nb.img, d_pos, nb.xs0, H, max_disp2, nb.type_s, nb.xs, nb.rec, d_err);
-    return cudaGetLastError();
+    return launch_chained(k_gather_positions, (N + 255) / 256, 256, 0, st, N, nb.perm, nb.img, d_pos, nb.xs0, H, max_disp2, nb.type_s,
+                          nb.xs, nb.rec, d_err);
 }
 
 }  // namespace umd
