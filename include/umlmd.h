@@ -63,8 +63,9 @@ typedef struct umlmd_options {
                             pair) for every GEMM; path 2 takes the whole MLP in one kernel per block of atoms where
                             that is faster (small systems, narrow models), and otherwise the kernel of path 4 for
                             the last GEMM of the backward pass; 2, 3 and 4 need F % 8 == 0 and fall back to 1 otherwise */
-    int32_t  pair_table_mb;  /* device memory, MiB, that per-pair amplitude tables may take, without the
-                                copies for values alone, which add two thirds of it
+    int32_t  pair_table_mb;  /* device memory, MiB, that per-pair amplitude tables may take, counted as table_rows x
+                                3 x C0 words per pair (what is kept is 4/3 of that from C0 = 32 on, else 5/3; more at
+                                table spacings above 0.0025 Angstrom)
                                 (see umlmd_build_neighbors); 0 = 192, negative = never build them */
     int32_t  gemm_spin_limit;       /* polls after which a wait inside the tensor-core GEMM's operand
                                        pipeline gives up (the kernel then finishes with garbage, and the
@@ -139,7 +140,7 @@ const char* umlmd_last_error(const umlmd_t* h);
  * is allocated (library plumbing, no counterpart in the paper; the paper's memory-scaling note is
  * the model: a fixed tile workspace plus terms linear in atoms and in edges).  An upper estimate
  * within a few per cent; per-pair amplitude tables, when the species present are few enough for
- * them, add at most 5/3 of umlmd_options.pair_table_mb on top.
+ * them, add at most 5/3 of umlmd_options.pair_table_mb on top at table spacings up to 0.0025 Angstrom.
  */
 int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t* bytes);
 
@@ -167,9 +168,10 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
  * The call also finds which species occur.  When the P species present are few enough that
  * P^2 tables of table_rows x 3 x C0 words fit in umlmd_options.pair_table_mb, the edge
  * amplitude of every ordered pair (s, s') among them, psi_c(rho) = gamma_c g_c(rho) + beta_c +
- * sum_mu U_c,mu q_mu(rho), is tabulated as a cubic table of its own (the same linear
- * combination of the coefficient rows of the radial table), and umlmd_compute reads one row of
- * that table per edge instead of the radial table, the pair cache and the shared modes.  The
+ * sum_mu U_c,mu q_mu(rho), is tabulated by itself (the same linear
+ * combination of the coefficient rows of the radial table; pieces for values and for
+ * what the backward pass needs), and umlmd_compute reads one row of
+ * these per edge and pass instead of the radial table, the pair cache and the shared modes.  The
  * species are re-examined at every call; the tables are kept while the set does not change.
  */
 int umlmd_build_neighbors(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type,
