@@ -67,6 +67,7 @@ struct umlmd {
         cudaGraphExec_t exec = nullptr;
         const void* key[4] = {nullptr, nullptr, nullptr, nullptr}; double key_dt = 0, key_x0 = 0, key_x1 = 0; int64_t key_serial = -1; int key_flags = 0;
         bool seen = false;                           // the key's sequence has run once as plain launches
+        bool edge_grad = false;                      // it leaves edge gradients (have_edge_grad after it)
         int64_t launches[16] = {0}; int64_t total = 0;   // what one replay launches, per class
     };
     Replay rp_compute, rp_step, rp_nvt;
@@ -318,6 +319,7 @@ int run_replayed(umlmd_t* h, umlmd_t::Replay& r, const void* k0, const void* k1,
         cudaError_t e = cudaStreamBeginCapture(h->cap_st, cudaStreamCaptureModeRelaxed);
         if (e == cudaSuccess) {
             rc = body();
+            r.edge_grad = h->have_edge_grad;
             e = cudaStreamEndCapture(h->cap_st, &graph);
             if (rc == UMLMD_OK && e == cudaSuccess) e = cudaGraphInstantiate(&r.exec, graph, 0);
             if (graph) cudaGraphDestroy(graph);
@@ -337,6 +339,7 @@ int run_replayed(umlmd_t* h, umlmd_t::Replay& r, const void* k0, const void* k1,
     h->launches_total += r.total;
     ++h->graph_replays;
     API_CUDA(h, cudaGraphLaunch(r.exec, h->st));
+    h->have_edge_grad = r.edge_grad;                 // (body, which sets it, has not run)
     return UMLMD_OK;
 }
 

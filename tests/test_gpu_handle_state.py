@@ -1,0 +1,59 @@
+"""What a handle keeps from call to call: flags across replayed sequences, buffers across systems of growing size."""
+
+import numpy as np
+import pytest
+import torch
+
+from workloads import SMALL_PROFILES, make_blob
+
+pytestmark = pytest.mark.gpu
+
+
+def _box(n, n_types, seed=0, a=2.6):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    k = int(np.ceil(n ** (1 / 3)))
+    sites = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * a
+    pos = torch.tensor(sites + rng.uniform(-0.2, 0.2, (n, 3))).cuda()
+    types = torch.tensor(rng.integers(0, n_types, n).astype(np.int32)).cuda()
+    return pos, types, np.eye(3) * a * k
+
+
+@pytest.mark.parametrize("driver", ["nve", "nvt"])
+def test_replayed_evaluations_keep_track_of_what_the_buffers_hold(driver):
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES["p16_2_0"]
+    blob = make_blob(p, seed=3, bias_scale=0.2)
+    start, types, cell = _box(150, p["T"], seed=4)
+    results = []
+    for graphs in (-1, 1):
+        m = binding.Model(blob, launch_graphs=graphs)
+        pos, vel = start.clone(), torch.zeros_like(start)
+        ea, f = torch.empty(150, dtype=torch.float64, device="cuda"), torch.empty_like(pos)
+        m.build_neighbors(pos, types, cell, (1, 1, 1), 1.0)
+        m.set_md_state(pos, vel, [20.0] * p["T"])
+
+        def energy():
+            m.compute(pos, forces=False, virial=False, out_atom_energy=ea)
+
+        def steps(n):
+            return m.step(n, 1e-4) if driver == "nve" else m.step_nvt(n, 1e-4, 300.0, 0.1)
+
+        for _ in range(3):                # plain, recorded, replayed
+            energy()
+        steps(1)                          # its only step runs plain and leaves gradients
+        energy()                          # replayed: forward values again
+        state, desc = m.get_intermediates()
+        with pytest.raises(binding.UmlmdError) as e:
+            m.atom_virial()
+        assert e.value.code == -1
+        # the other way round: the last evaluation with forces is a replayed one
+        steps(4)
+        energy()
+        out = [m.compute(pos, out_forces=f) for _ in range(3)][-1]
+        w = m.atom_virial()
+        assert np.abs(w.sum(dim=0).cpu().numpy() - out["virial"]).max() <= 1e-6 * w.abs().sum().item()
+        results.append((state.clone(), desc.clone(), w.clone(), out["energy"]))
+        assert (m.query()["graph_replays"] > 0) == (graphs == 1)
+        m.close()
+    for a, b in zip(*results):
+        assert torch.equal(a, b) if isinstance(a, torch.Tensor) else a == b
