@@ -47,7 +47,7 @@ struct umlmd {
     int* d_species = nullptr;                           // [3T]: occurrence flags, species -> slot, present list
     int* h_species = nullptr;                           // pinned [T]
     // MD
-    double* md_pos = nullptr; double* md_vel = nullptr; double* md_force = nullptr; int64_t md_cap = 0;
+    double* md_pos = nullptr; double* md_vel = nullptr; double* md_force = nullptr; int64_t md_cap = 0;    // (capacity in doubles)
     double* d_mass = nullptr; double* d_inv_mass = nullptr;
     bool have_md = false, have_force = false;
     bool have_edge_grad = false;     // h->g holds the edge gradients of the positions in nb.xs
@@ -748,7 +748,7 @@ int umlmd_set_md_state(umlmd_t* h, double* d_pos, double* d_vel, const double* m
     API_CUDA(h, cudaMemcpyAsync(h->d_mass, m.data(), sizeof(double) * T, cudaMemcpyHostToDevice, h->st));
     API_CUDA(h, cudaMemcpyAsync(h->d_inv_mass, im.data(), sizeof(double) * T, cudaMemcpyHostToDevice, h->st));
     API_CUDA(h, cudaStreamSynchronize(h->st));
-    if (h->nb.N > h->md_cap || !h->md_force) API_CUDA(h, dev_ensure(&h->md_force, &h->md_cap, h->nb.N * 3));
+    API_CUDA(h, dev_ensure(&h->md_force, &h->md_cap, h->nb.N * 3));
     h->md_pos = d_pos; h->md_vel = d_vel;
     h->have_md = true; h->have_force = false; h->nhc_reset = true;
     ++h->list_serial;                // masses and buffers of the recorded step sequence may have changed

@@ -57,3 +57,33 @@ def test_replayed_evaluations_keep_track_of_what_the_buffers_hold(driver):
         m.close()
     for a, b in zip(*results):
         assert torch.equal(a, b) if isinstance(a, torch.Tensor) else a == b
+
+
+def test_md_state_of_a_larger_system_gets_a_larger_force_buffer():
+    # accounting alone: nothing is launched on the buffer
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES["p16_2_0"]
+    m = binding.Model(make_blob(p, seed=3))
+    for n, grown in ((300, None), (880, 24 * (880 - 300)), (881, 0), (400, 0)):      # (buffers are padded by 16 elements)
+        pos, types, cell = _box(n, p["T"])
+        m.build_neighbors(pos, types, cell, (1, 1, 1), 1.0)
+        held = m.query()["device_bytes"]
+        m.set_md_state(pos, torch.zeros_like(pos), [20.0] * p["T"])
+        assert grown is None or m.query()["device_bytes"] - held == grown, n
+    m.close()
+
+
+def test_md_after_a_smaller_system_on_the_same_handle():
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES["p16_2_0"]
+    blob = make_blob(p, seed=3, bias_scale=0.2)
+    used, results = binding.Model(blob), []
+    for n, m in ((300, used), (880, used), (880, binding.Model(blob))):
+        pos, types, cell = _box(n, p["T"], seed=5)
+        vel = torch.zeros_like(pos)
+        m.build_neighbors(pos, types, cell, (1, 1, 1), 1.0)
+        m.set_md_state(pos, vel, [20.0] * p["T"])
+        e = m.step(12, 1e-4, rebuild_every=5)
+        results.append((e, pos, vel))
+    (ea, pa, va), (eb, pb, vb) = results[1:]
+    assert ea == eb and torch.equal(pa, pb) and torch.equal(va, vb)
