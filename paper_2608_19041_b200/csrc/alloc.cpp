@@ -15,7 +15,11 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) { *p = nullptr; return e; }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();          // reported here: the next launch check must not find it again
+        return e;
+    }
     std::lock_guard<std::mutex> lk(g_mu);
     g_sizes[*p] = bytes;
     g_total += (int64_t)bytes;

@@ -148,8 +148,10 @@ int ensure_workspace(umlmd_t* h) {
     const Dims& d = h->d;
     const int64_t N = h->nb.N, E = h->nb.E;
     const int64_t B = N < h->node_tile ? N : h->node_tile;
-    if (B > h->tile_cap || !h->state) {
+    // (a capacity of several buffers is zero until all of them are there, so that a failed allocation is made up for later)
+    if (B > h->tile_cap) {
         int64_t c;
+        h->tile_cap = 0;
         c = 0; API_CUDA(h, dev_ensure(&h->state, &c, B * d.SP));
         c = 0; API_CUDA(h, dev_ensure(&h->desc, &c, B * d.DP));
         const int64_t wmax = d.DP > d.F ? d.DP : d.F;
@@ -165,8 +167,9 @@ int ensure_workspace(umlmd_t* h) {
         h->tile_cap = B;
     }
     if (E > h->g_cap || !h->g) { API_CUDA(h, dev_ensure(&h->g, &h->g_cap, E * 3, 1.1)); h->g_cap /= 3; }
-    if (N > h->n_cap || !h->e_atom) {
+    if (N > h->n_cap) {
         int64_t c;
+        h->n_cap = 0;
         c = 0; API_CUDA(h, dev_ensure(&h->e_atom, &c, N));
         c = 0; API_CUDA(h, dev_ensure(&h->f_sorted, &c, N * 3));
         c = 0; API_CUDA(h, dev_ensure(&h->type_o, &c, N));
@@ -375,7 +378,17 @@ int ensure_device_model(umlmd_t* h) {
     if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_out, sizeof(double) * 16);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_err, sizeof(int) * 4);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-    if (e != cudaSuccess) return fail(h, UMLMD_E_CUDA, std::string("model upload: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {                    // nothing stays half done: the next call starts over
+        cudaStreamSynchronize(h->st);
+        for (void* q : h->model_allocs) dev_free(q);
+        h->model_allocs.clear();
+        dev_free(h->scratch); dev_free(h->d_out); dev_free(h->d_err);
+        h->scratch = h->d_out = nullptr; h->d_err = nullptr;
+        if (h->h_out) cudaFreeHost(h->h_out);
+        if (h->h_err) cudaFreeHost(h->h_err);
+        h->h_out = nullptr; h->h_err = nullptr;
+        return fail(h, UMLMD_E_CUDA, std::string("model upload: ") + cudaGetErrorString(e));
+    }
     h->on_device = true;
     return UMLMD_OK;
 }
@@ -384,9 +397,9 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
                const int pbc[3], double skin, const BuildFetch* fetch) {
     int rc = ensure_device_model(h);
     if (rc != UMLMD_OK) return rc;
+    h->have_list = false;            // (until it and the workspace for it are complete)
     { Scope sc(h, kNeighbor, 5 + (fetch && N > 0)); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, fetch, h->st, &h->err); }
-    if (rc != UMLMD_OK) { h->have_list = false; return rc; }
-    h->have_list = true;
+    if (rc != UMLMD_OK) return rc;
     h->have_edge_grad = false;       // edges were renumbered
     h->steps_since_build = 0;
     ++h->list_serial;                // recorded launch sequences name the old list
@@ -399,17 +412,20 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
         if (h->nb.E > h->nb.E_owned)
             API_CUDA(h, cudaMemsetAsync(h->g + 3 * (size_t)h->nb.E_owned, 0, sizeof(float) * 3 * (size_t)(h->nb.E - h->nb.E_owned), h->st));
     }
+    h->have_list = true;
     return UMLMD_OK;
 }
 
 int ensure_species_buffers(umlmd_t* h) {
     int rc = ensure_device_model(h);
-    if (rc != UMLMD_OK || h->d_species) return rc;
+    if (rc != UMLMD_OK) return rc;
     const size_t T = (size_t)h->d.T;
-    void* p = nullptr;
-    API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * T));
-    h->d_species = (int*)p;
-    API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * T));
+    if (!h->d_species) {
+        void* p = nullptr;
+        API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * T));
+        h->d_species = (int*)p;
+    }
+    if (!h->h_species) API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * T));
     return UMLMD_OK;
 }
 
@@ -426,9 +442,11 @@ int setup_pair_tables(umlmd_t* h) {
     const bool wide = wide_channels(d.C0);
     const size_t vfloats = np * np * (size_t)d.n_vrows * 2 * d.C0, dfloats = wide ? vfloats : 0;
     const size_t floats = wide ? 0 : np * np * (size_t)d.n_rows * 3 * d.C0;
-    h->pair_tables = np > 0 && h->pair_table_budget >= 0 && full <= (size_t)h->pair_table_budget &&
+    const bool use = np > 0 && h->pair_table_budget >= 0 && full <= (size_t)h->pair_table_budget &&
                      3 * (floats + vfloats + dfloats) * sizeof(float) <= 5 * (size_t)h->pair_table_budget;
-    if (!h->pair_tables || present == h->present) return UMLMD_OK;
+    h->pair_tables = use && present == h->present;
+    if (!use || h->pair_tables) return UMLMD_OK;
+    h->present.clear();                               // no tables until all of them are made
     auto grow = [&](float** p, size_t* cap, size_t need) {
         if (need <= *cap) return cudaSuccess;
         dev_free(*p); *p = nullptr; *cap = 0;
@@ -448,6 +466,7 @@ int setup_pair_tables(umlmd_t* h) {
     API_CUDA(h, cudaStreamSynchronize(h->st));       // `up` is pageable host memory
     h->launches_total += 2;
     h->present = present;
+    h->pair_tables = true;
     return UMLMD_OK;
 }
 
@@ -553,10 +572,13 @@ int umlmd_build_neighbors(umlmd_t* h, int64_t N, const double* d_pos, const int3
     const BuildFetch fetch = {h->d.T, h->d_species, h->h_species, h->h_err};
     rc = build_list(h, N, d_pos, d_type, cell, pbc, skin, &fetch);
     if (rc != UMLMD_OK) return rc;
+    h->have_list = false;                        // (until the rest has worked as well)
     rc = decode_device_errors(h, *h->h_err);
-    if (rc != UMLMD_OK) { h->have_list = false; return rc; }
+    if (rc != UMLMD_OK) return rc;
     if (N > 0) API_CUDA(h, cudaMemcpyAsync(h->type_o, d_type, sizeof(int) * N, cudaMemcpyDeviceToDevice, h->st));
-    return setup_pair_tables(h);
+    rc = setup_pair_tables(h);
+    h->have_list = rc == UMLMD_OK;
+    return rc;
 }
 
 int umlmd_get_neighbors(umlmd_t* h, int32_t* d_row_ptr, int32_t* d_src, int8_t* d_shift, int64_t cap,
@@ -743,8 +765,11 @@ int umlmd_set_md_state(umlmd_t* h, double* d_pos, double* d_vel, const double* m
         if (!(mass_per_type[t] > 0) || !std::isfinite(mass_per_type[t])) return fail(h, UMLMD_E_INVALID_ARG, "masses must be positive");
         m[t] = mass_per_type[t]; im[t] = 1.0 / mass_per_type[t];
     }
-    int64_t c;
-    if (!h->d_mass) { c = 0; API_CUDA(h, dev_ensure(&h->d_mass, &c, T)); c = 0; API_CUDA(h, dev_ensure(&h->d_inv_mass, &c, T)); }
+    h->have_md = false;                          // (until the buffers are there)
+    int64_t c = 0;
+    if (!h->d_mass) API_CUDA(h, dev_ensure(&h->d_mass, &c, T));
+    c = 0;
+    if (!h->d_inv_mass) API_CUDA(h, dev_ensure(&h->d_inv_mass, &c, T));
     API_CUDA(h, cudaMemcpyAsync(h->d_mass, m.data(), sizeof(double) * T, cudaMemcpyHostToDevice, h->st));
     API_CUDA(h, cudaMemcpyAsync(h->d_inv_mass, im.data(), sizeof(double) * T, cudaMemcpyHostToDevice, h->st));
     API_CUDA(h, cudaStreamSynchronize(h->st));

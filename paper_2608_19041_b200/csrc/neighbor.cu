@@ -689,6 +689,7 @@ static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, i
     nb->E_owned = n_owned < N ? nb->h_totals[1] : total;
     if (total > nb->E_cap) {
         int64_t c;
+        nb->E_cap = 0;                           // (until all of them are there)
         c = 0; NB_CHECK(dev_ensure(&nb->nbr, &c, total, 1.1));
         c = 0; NB_CHECK(dev_ensure(&nb->rev, &c, total, 1.1));
         nb->E_cap = c;
@@ -801,9 +802,10 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     if (N == 0) { nb->E = 0; return UMLMD_OK; }
 
     // per-atom arrays (all sized from one capacity)
-    if (N > nb->N_cap || !nb->wpos) {
+    if (N > nb->N_cap) {
         const int64_t need = N + 1;
         int64_t c;
+        nb->N_cap = 0;
         c = 0; NB_CHECK(dev_ensure(&nb->wpos, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs0, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs, &c, need * 3));
@@ -931,9 +933,10 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
     for (int k = 0; k < 9; ++k) nb->H[k] = 0;
     nb->E = 0;
     if (N == 0) return UMLMD_OK;
-    if (N > nb->N_cap || !nb->xs) {
+    if (N > nb->N_cap) {
         const int64_t need = N + 1;
         int64_t c;
+        nb->N_cap = 0;
         // the same per-atom arrays as the cell-list build sizes (the two builds may alternate on one handle)
         c = 0; NB_CHECK(dev_ensure(&nb->wpos, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs0, &c, need * 3));

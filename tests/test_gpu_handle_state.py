@@ -87,3 +87,44 @@ def test_md_after_a_smaller_system_on_the_same_handle():
         results.append((e, pos, vel))
     (ea, pa, va), (eb, pb, vb) = results[1:]
     assert ea == eb and torch.equal(pa, pb) and torch.equal(va, vb)
+
+
+def test_a_failed_allocation_leaves_no_list_and_is_made_up_for():
+    """Builds of a large system with less and less device memory to spare fail wherever the memory runs out; after each
+    the handle refuses to evaluate, and evaluates a small system as before."""
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES["p128_2_0"]
+    small, big = _box(600, p["T"], seed=6), _box(60000, p["T"], seed=7)
+    blob = make_blob(p, seed=3, bias_scale=0.2)
+
+    def evaluate(m):
+        m.build_neighbors(*small, (1, 1, 1), 1.0)
+        out = m.compute(small[0], atom_energy=True)
+        return out["forces"], out["atom_energy"]
+
+    m = binding.Model(blob)
+    ref = evaluate(m)
+    m.close()
+    failed = 0
+    for spare_mb in (24, 64, 100, 140, 180, 240, 300, 380, 460, 560, 700):
+        m = binding.Model(blob)
+        if spare_mb % 100:                               # on a handle in use, and on one whose first build it is
+            evaluate(m)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = torch.empty(max(torch.cuda.mem_get_info()[0] - (spare_mb << 20), 1), dtype=torch.uint8, device="cuda")
+        try:
+            m.build_neighbors(*big, (1, 1, 1), 1.0)
+        except binding.UmlmdError as e:
+            assert e.code == -8
+            failed += 1
+            lib = binding.lib()
+            assert lib.umlmd_compute(m._h, big[0].data_ptr(), None, None, None, None) == -5
+            assert lib.umlmd_step(m._h, 1, 0.001, 0, None, None) == -5
+            assert lib.umlmd_atom_virial(m._h, big[0].data_ptr()) == -5
+        del hog
+        torch.cuda.empty_cache()
+        for a, b in zip(evaluate(m), ref):
+            assert torch.equal(a, b), spare_mb
+        m.close()
+    assert failed >= 6
