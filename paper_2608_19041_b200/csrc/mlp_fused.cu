@@ -244,9 +244,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_mlp_fused(const __grid_constant_
                             }
                         }
                     }
-                    if (go) if (elect_one()) umma_commit(acc_full + 8 * buf);
-                    // (by_tile: that phase is complete or about to be; a later wait must not find it still open)
+                    // by_tile: the phase of the epilogue before is complete or about to be.  It is waited for ahead of the
+                    // commit: once that is out, the next epilogue may complete a phase of the same parity as the one before
                     if (by_tile) go = go && wait_all(acc_free, (use - 1) & 1);
+                    if (go) if (elect_one()) umma_commit(acc_full + 8 * buf);
                 }
                 if (q > 0) ++uses;
             }

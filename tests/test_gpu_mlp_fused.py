@@ -48,3 +48,24 @@ def test_matches_the_cuda_core_path(name, sizes):
         assert (ref["atom_energy"] - out["atom_energy"]).abs().max().item() <= de, n
         assert (ref["atom_energy"] - alone["atom_energy"]).abs().max().item() <= de, n
         assert (ref["forces"] - out["forces"]).abs().max().item() <= df, n
+
+
+@pytest.mark.parametrize("name,n", [("cfg2_cu4000", 14209), ("cfg4_hea128k", 11840), ("cfg4_hea128k", 8000)])
+def test_one_accumulator_set_never_waits_for_a_phase_that_is_over(name, n):
+    # blocks so large that tensor memory holds one set of accumulators: every pass but the first of a block then waits for
+    # the epilogue before it, many times over, with a limit that an ordinary wait stays far below
+    from paper_2608_19041_b200 import binding
+    blob = make_blob(CONFIGS[name]["profile"], seed=51, bias_scale=0.2)
+    m = binding.Model(blob, gemm_spin_limit=200000, launch_graphs=1)
+    k = int(np.ceil(n ** (1 / 3)))
+    sites = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * 6.5      # no neighbours: the MLP is the call
+    pos, types = torch.tensor(sites).cuda(), torch.zeros(n, dtype=torch.int32, device="cuda")
+    m.build_neighbors(pos, types, np.eye(3) * 6.5 * k, (0, 0, 0), 0.0)
+    f, e = torch.empty_like(pos), torch.empty(n, dtype=torch.float64, device="cuda")
+    first = None
+    for _ in range(300):
+        m.compute(pos, out_forces=f, out_atom_energy=e)
+        m.compute(pos, forces=False, virial=False, out_atom_energy=e)
+        first = e.clone() if first is None else first
+        assert torch.equal(e, first)
+    m.close()
