@@ -511,7 +511,8 @@ cudaError_t launch_mlp_fused(const MlpArgs& a, cudaStream_t st) {
         }
     }
     if (!ok) return cudaErrorInvalidValue;
-    static const cudaError_t attr = cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    // (per launch, as a kernel's attributes belong to one device and a process may have handles on several)
+    const cudaError_t attr = cudaFuncSetAttribute(k_mlp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
     if (attr != cudaSuccess) return attr;
     const int items = (a.n + g.NA - 1) / g.NA;
     return launch_chained(k_mlp_fused, items < 148 ? items : 148, THREADS, used + (uint32_t)g.stages * W_BYTES, st, maps, g);

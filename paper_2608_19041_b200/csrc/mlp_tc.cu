@@ -31,6 +31,7 @@
 // tensor memory is always released.
 #include <cuda.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "common.cuh"
@@ -769,24 +770,12 @@ bool gemm_tc_available() { return encode_fn() != nullptr; }
 // that the one-tile-per-CTA kernel, with twice as many and half as long CTAs, finishes sooner.
 int gemm_tc_pick_variant(int M, int N, int requested) {
     if (requested == 4) {      // two-CTA kernel where there is enough work for the pairs, else one tile per CTA
-        static int n_sm4 = 0;
-        if (n_sm4 == 0) {
-            int dev = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm4, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                n_sm4 = 148;
-        }
         const int items1 = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-        return items1 <= n_sm4 ? 3 : 4;
+        return items1 <= sm_count() ? 3 : 4;
     }
     if (requested != 2) return requested;
-    static int n_sm = 0;
-    if (n_sm == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            n_sm = 148;
-    }
     const int items = ((N + BN - 1) / BN) * ((M + 2 * BM - 1) / (2 * BM));
-    return 2 * items <= n_sm ? 3 : 2;
+    return 2 * items <= sm_count() ? 3 : 2;
 }
 
 bool gemm_tc_supported(const GemmArgs& g) {
@@ -812,21 +801,24 @@ int gemm_tc2_tile(int N, bool head) {
 template <int MODE>
 cudaError_t launch_tc2(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUtensorMap& mBh, const CUtensorMap& mBl,
                        const GemmArgs& g, int NT, cudaStream_t st) {
-    static int max_clusters = 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(P_THREADS); cfg.dynamicSmemBytes = C2_SMEM_BYTES; cfg.stream = st; cfg.attrs = at; cfg.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc2<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C2_SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    // pairs of SMs that can hold a cluster at once, by device (the query is not one for every launch)
+    static std::atomic<int> clusters_of[64];
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    int max_clusters = dev < 64 ? clusters_of[dev].load(std::memory_order_relaxed) : 0;
     if (max_clusters == 0) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_tc2<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C2_SMEM_BYTES);
-        if (e != cudaSuccess) return e;
         cfg.gridDim = dim3(2 * 74);
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k_gemm_tc2<MODE>, &cfg);      // pairs of SMs that can hold a cluster at once
+        e = cudaOccupancyMaxActiveClusters(&max_clusters, k_gemm_tc2<MODE>, &cfg);
         if (e != cudaSuccess) return e;
-        if (n < 1) return cudaErrorInvalidConfiguration;
-        max_clusters = n;
+        if (max_clusters < 1) return cudaErrorInvalidConfiguration;
+        if (dev < 64) clusters_of[dev].store(max_clusters, std::memory_order_relaxed);
     }
     const int items = ((g.N + NT - 1) / NT) * ((g.M + 2 * BM - 1) / (2 * BM));
     const int ncl = items < max_clusters ? items : max_clusters;
@@ -835,21 +827,6 @@ cudaError_t launch_tc2(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUt
 }
 
 cudaError_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st) {
-    static bool attr_set = false;
-    static int n_sm = 0;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tcp<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tcp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gemm_tcp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES);
-        int dev = 0;
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     if (!g.a_presplit) {
         const size_t total = (size_t)g.M * (g.K >> 2);
         int blocks = (int)((total + 255) / 256);
@@ -870,18 +847,16 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, cudaStream_t st) {
         if (mode == 2) return launch_tc2<2>(mAh, mAl, mBh, mBl, g, NT, st);
         return launch_tc2<0>(mAh, mAl, mBh, mBl, g, NT, st);
     }
-    if (g.variant == 3) {                                  // one 128 x 128 tile per CTA, two CTAs per SM
-        dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-        if (mode == 1) k_gemm_tc<1><<<grid, 192, SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-        else if (mode == 2) k_gemm_tc<2><<<grid, 192, SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-        else k_gemm_tc<0><<<grid, 192, SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-    } else {                                               // persistent, 256 x 128 items
-        const int items = ((g.N + BN - 1) / BN) * ((g.M + 2 * BM - 1) / (2 * BM));
-        const int grid = items < n_sm ? items : n_sm;
-        if (mode == 1) k_gemm_tcp<1><<<grid, P_THREADS, P_SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-        else if (mode == 2) k_gemm_tcp<2><<<grid, P_THREADS, P_SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-        else k_gemm_tcp<0><<<grid, P_THREADS, P_SMEM_BYTES, st>>>(mAh, mAl, mBh, mBl, g);
-    }
+    // the shared-memory attribute is set per launch: it belongs to one device, and a process may have handles on several
+    const bool persistent = g.variant != 3;                // 256 x 128 items; else one 128 x 128 tile per CTA, two CTAs per SM
+    auto kern = persistent ? (mode == 1 ? k_gemm_tcp<1> : (mode == 2 ? k_gemm_tcp<2> : k_gemm_tcp<0>))
+                           : (mode == 1 ? k_gemm_tc<1> : (mode == 2 ? k_gemm_tc<2> : k_gemm_tc<0>));
+    const int smem = persistent ? P_SMEM_BYTES : SMEM_BYTES, n_sm = sm_count();
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int items = ((g.N + BN - 1) / BN) * ((g.M + 2 * BM - 1) / (2 * BM));
+    const dim3 grid = persistent ? dim3(items < n_sm ? items : n_sm) : dim3((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
+    kern<<<grid, persistent ? P_THREADS : 192, smem, st>>>(mAh, mAl, mBh, mBl, g);
     return cudaGetLastError();
 }
 

@@ -99,6 +99,13 @@ inline EncodeFn encode_fn() {
     return fn;
 }
 
+// SMs of the current device
+inline int sm_count() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 148;
+    return n;
+}
+
 // 2-D map over a row-major [rows][cols] half-precision matrix with row pitch ld (elements); box =
 // 32 cols x box_rows rows
 inline bool make_map(CUtensorMap* map, const __half* ptr, int rows, int cols, int ld, int box_rows = 128) {
