@@ -359,11 +359,28 @@ int umlmd_get_intermediates(umlmd_t* h, float* d_state, float* d_desc);
 
 /*
  * Evaluate the tabulated radial map at n distances (host arrays): out_g [n, C0+R] holds
- * g(rho) then q(rho), out_dg their derivatives, from the same cubic polynomials the
- * kernels use (evaluated on the host from the device table's float32 coefficients).
+ * g(rho) then q(rho), out_dg their derivatives, from the cubic Hermite pieces that every table of
+ * the edge kernels is derived from (evaluated on the host from the device table's float32
+ * coefficients).
  */
 int umlmd_eval_radial_table(const umlmd_t* h, int64_t n, const double* rho, double* out_g,
                             double* out_dg);
+
+/*
+ * What the edge kernels read for centre species type_i and neighbour species type_j at n distances
+ * (host arrays): out_psi [n, C0] the amplitudes psi_c of the forward pass (quadratic pieces), and
+ * out_dchipsi [n, C0] (may be NULL) the derivative of envelope times amplitude that the backward
+ * pass works with -- from C0 = 32 on, without shared modes or from per-pair tables, quadratic pieces
+ * of that product, otherwise formed from the cubic pieces.  per_pair = 0: shared table and pair
+ * cache; 1: the tables that umlmd_build_neighbors makes for a system of just these two species.
+ * Pieces are at most 0.0025 Angstrom long, and cut finer until those of g, q and of the envelope's
+ * products follow the cubic pieces within 2^-24 (psi) and 2^-23 (product) of their largest magnitude,
+ * besides the rounding of the leading coefficient; a table of more than 100,000 pieces is cut no
+ * further, whether that is met or not.  Energy and force agree to that rounding, not exactly: psi
+ * jumps by it from one piece to the next.
+ */
+int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int32_t per_pair, int64_t n, const double* rho,
+                           double* out_psi, double* out_dchipsi);
 
 /*
  * Per-kernel-class accounting.  The handle always counts the kernels it launches; with

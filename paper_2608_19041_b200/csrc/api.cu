@@ -1014,6 +1014,91 @@ int umlmd_eval_radial_table(const umlmd_t* h, int64_t n, const double* rho, doub
     return UMLMD_OK;
 }
 
+int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int32_t per_pair, int64_t n, const double* rho,
+                           double* out_psi, double* out_dchipsi) {
+    if (!h || n < 0 || (n > 0 && (!rho || !out_psi))) return UMLMD_E_INVALID_ARG;
+    const Dims& d = h->d;
+    if (type_i < 0 || type_j < 0 || type_i >= d.T || type_j >= d.T) return UMLMD_E_INVALID_ARG;
+    const HostModel& m = h->hm;
+    const int C0 = d.C0, R = d.R;
+    const double dx = h->hm.dx, w = dx / d.v_sub;
+    const bool products = wide_channels(C0) && (per_pair || R == 0);      // what the backward pass reads: else rows with derivatives
+    auto pair_row = [&](int a, int b) { return &m.pairmod[(size_t)(a * d.T + b) * (2 + R) * C0]; };
+    auto word = [](const float* p) { unsigned u; std::memcpy(&u, p, sizeof(u)); return u; };
+    // steps of the packed words of tables made for a system of these two species
+    double big[6] = {0, 0, 0, 0, 0, 0};
+    const int two[2] = {type_i, type_j};
+    for (int s = 0; per_pair && s < d.n_rows; ++s)
+        for (int ab = 0; ab < 4; ++ab)
+            for (int c = 0; c < C0; ++c) {
+                double v[4], q[4];
+                pair_cubic(d, &m.table[(size_t)s * 3 * d.CP], pair_row(two[ab >> 1], two[ab & 1]) + c, c, v);
+                auto grow = [&](int k, double x) { big[k] = std::fmax(big[k], std::fabs((double)(float)x)); };
+                grow(0, v[2]); grow(1, v[3]);
+                for (int sub = 0; sub < d.v_sub; ++sub) {
+                    value_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, q);
+                    grow(2, q[1]); grow(3, q[2]);
+                    if (!products) continue;
+                    product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, s * dx + (sub + 0.5) * w, (double)d.rc, q);
+                    grow(4, q[1]); grow(5, q[2]);
+                }
+            }
+    const float step[6] = {per_pair ? tab_step2((float)big[0]) : d.tab_k2, per_pair ? tab_step3((float)big[1]) : d.tab_k3,
+                           per_pair ? tab_step2((float)big[2]) : d.tab_v1, per_pair ? tab_step3((float)big[3]) : d.tab_v2,
+                           per_pair ? tab_step2((float)big[4]) : d.tab_d1, per_pair ? tab_step3((float)big[5]) : d.tab_d2};
+    const float* pm = pair_row(type_i, type_j);
+    for (int64_t i = 0; i < n; ++i) {
+        const double r = rho[i], x = r / (double)d.rc, u = 1 - x;
+        const double chi = u * u * u * u * (1 + x * (4 + x * (10 + x * (20 + 35 * x)))), dchi = -280 * x * x * x * x * u * u * u / (double)d.rc;
+        auto at = [&](double spacing, int rows) {
+            const int row = (int)std::floor(r / spacing);
+            return row < 0 ? 0 : (row > rows - 1 ? rows - 1 : row);
+        };
+        const int vrow = at(w, d.n_vrows), row = at(dx, d.n_rows), crow = vrow / d.v_sub;
+        const double t = r - (vrow + 0.5) * w, tc = r - row * dx, mid = (vrow % d.v_sub + 0.5) * w, rho_mid = (vrow + 0.5) * w;
+        // one piece: from the stored word, or rounded and packed as the tables of a pair are
+        auto stored = [&](const std::vector<float>& tab, int c, const float* st) {
+            const float* p = &tab[(size_t)vrow * 2 * d.CP + c];
+            float a1, a2;
+            tab_unpack(word(p + d.CP), st[0], st[1], &a1, &a2);
+            return ((double)a2 * t + (double)a1) * t + (double)p[0];
+        };
+        auto packed = [&](const double* a, const float* st) {
+            float a1, a2;
+            tab_unpack(tab_pack((float)a[1], (float)a[2], st[0], st[1]), st[0], st[1], &a1, &a2);
+            return ((double)a2 * t + (double)a1) * t + (double)(float)a[0];
+        };
+        for (int c = 0; c < C0; ++c) {
+            double v[4], q[4], psi, out;
+            if (per_pair) {
+                pair_cubic(d, &m.table[(size_t)crow * 3 * d.CP], pm + c, c, v);
+                value_piece(v[0], v[1], v[2], v[3], mid, 0.5 * w, q);
+                psi = packed(q, step + 2);
+            } else {
+                psi = (double)pm[c] * stored(m.vtable, c, step + 2) + (double)pm[C0 + c];
+                for (int k = 0; k < R; ++k) psi += (double)pm[(size_t)(2 + k) * C0 + c] * stored(m.vtable, C0 + k, step + 2);
+            }
+            if (products && per_pair) {
+                product_piece(v[0], v[1], v[2], v[3], mid, 0.5 * w, rho_mid, (double)d.rc, q);
+                out = packed(q, step + 4);
+            } else if (products) {
+                out = (double)pm[c] * stored(m.dtable, c, step + 4) + (double)pm[C0 + c] * dchi;
+            } else {
+                pair_cubic(d, &m.table[(size_t)row * 3 * d.CP], pm + c, c, v);
+                float c2 = (float)v[2], c3 = (float)v[3];
+                if (per_pair) {
+                    tab_unpack(tab_pack(c2, c3, step[0], step[1]), step[0], step[1], &c2, &c3);
+                    v[0] = (float)v[0]; v[1] = (float)v[1]; v[2] = c2; v[3] = c3;
+                }
+                out = chi * ((3 * v[3] * tc + 2 * v[2]) * tc + v[1]) + dchi * (((v[3] * tc + v[2]) * tc + v[1]) * tc + v[0]);
+            }
+            out_psi[i * C0 + c] = psi;
+            if (out_dchipsi) out_dchipsi[i * C0 + c] = out;
+        }
+    }
+    return UMLMD_OK;
+}
+
 int umlmd_set_profiling(umlmd_t* h, int enabled) {
     if (!h) return UMLMD_E_INVALID_ARG;
     h->prof_on = enabled != 0;

@@ -126,7 +126,9 @@ __host__ __device__ inline void tab_unpack(unsigned w, float k2, float k3, float
 // single precision and (a1, a2) packed like (c2, c3) above.  The cubic term is folded into a1 (s^3 is within
 // h^3 / 4 of (3/4) h^2 s); what is left of it, and the rounding of a1 and a2 to 20 and 12 bits, add up to less
 // than half of the rounding of a0 at the default spacing (0.07 to 0.4 of 2^-24 of the largest value for the
-// workloads' radial maps).  A coarser table is cut into v_sub intervals of at most 0.0025 Angstrom.
+// workloads' radial maps).  An interval is cut into v_sub pieces of at most 0.0025 Angstrom, and into more until
+// they add up to no more than that rounding for g and q, and for their products (below, from C0 = 32 on, whichever
+// table holds them) to no more than 2^-23 of the largest; once there are more than 100,000 pieces the table is cut no further.
 __host__ __device__ inline void value_piece(double c0, double c1, double c2, double c3, double mid, double h, double* a) {
     a[0] = ((c3 * mid + c2) * mid + c1) * mid + c0;
     a[1] = (3 * c3 * mid + 2 * c2) * mid + c1 + 0.75 * h * h * c3;
@@ -153,6 +155,21 @@ __host__ __device__ inline void product_piece(double c0, double c1, double c2, d
     a[1] = e2 * p0 + 2 * e1 * p1 + e0 * p2 + 0.75 * h * h * d3;
     a[2] = 0.5 * (e3 * p0 + 3 * e2 * p1 + 3 * e1 * p2 + e0 * p3);
     a[3] = d3;
+}
+// The cubic piece of the amplitude psi_c = gamma_c g_c + beta_c + sum_mu U_c,mu q_mu of one species pair in one row of
+// the radial table (linear in the tabulated functions): `row` that row, `pm` channel c of the pair's row in the cache.
+__host__ __device__ inline void pair_cubic(const Dims& d, const float* row, const float* pm, int c, double* v) {
+    for (int q = -1; q < d.R; ++q) {
+        const int col = q < 0 ? c : d.C0 + q;
+        unsigned w;
+        memcpy(&w, row + 2 * d.CP + col, sizeof(w));
+        float c2, c3;
+        tab_unpack(w, d.tab_k2, d.tab_k3, &c2, &c3);
+        const double o[4] = {(double)row[col], (double)row[d.CP + col], (double)c2, (double)c3};
+        const double u = (double)pm[(size_t)(q < 0 ? 0 : 2 + q) * d.C0];
+        for (int k = 0; k < 4; ++k) v[k] = q < 0 ? u * o[k] : v[k] + u * o[k];
+        if (q < 0) v[0] += (double)pm[d.C0];
+    }
 }
 // Models of at least 32 channels without shared modes, or with per-pair tables (which hold the modes), use the
 // product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the channels are leading

@@ -997,20 +997,8 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
         const int si = present[pr / n_present], sj = present[pr % n_present];
         const float* pm = pairmod + (size_t)(si * d.T + sj) * (2 + d.R) * d.C0 + c;
         const float* tr = table + (size_t)row * 3 * d.CP;
-        auto coef = [&](int col, double* o) {     // the four coefficients of column col of the radial table
-            float h2, h3;
-            tab_unpack(__float_as_uint(tr[2 * d.CP + col]), d.tab_k2, d.tab_k3, &h2, &h3);
-            o[0] = (double)tr[col]; o[1] = (double)tr[d.CP + col]; o[2] = (double)h2; o[3] = (double)h3;
-        };
-        double v[4], o[4];
-        coef(c, o);
-        for (int k = 0; k < 4; ++k) v[k] = (double)pm[0] * o[k];
-        v[0] += (double)pm[d.C0];
-        for (int q = 0; q < d.R; ++q) {
-            coef(d.C0 + q, o);
-            const double u = (double)pm[(size_t)(2 + q) * d.C0];
-            for (int k = 0; k < 4; ++k) v[k] += u * o[k];
-        }
+        double v[4];
+        pair_cubic(d, tr, pm, c, v);
         c2 = (float)v[2]; c3 = (float)v[3];
         const double w = (double)d.dx / d.v_sub;
         for (int sub = 0; sub < d.v_sub; ++sub) {          // values alone (common.cuh, value_piece)

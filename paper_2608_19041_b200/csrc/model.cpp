@@ -317,12 +317,15 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         while (D1 / d.v_sub > 0.0025) d.v_sub *= 2;
         std::vector<float> va, da;
         double m0 = 0, q1 = 0, q2 = 0, q3 = 0, n0 = 0, r1 = 0, r2 = 0, r3 = 0;
-        const bool products = wide_channels(C0) && R == 0;
+        // the product table of the radial map is kept without shared modes only, but with them the per-pair tables hold the
+        // same products of gamma g + beta + U q: their bound is checked on the columns of g and q and on a constant
+        const bool wide = wide_channels(C0), products = wide && R == 0;
         for (;; d.v_sub *= 2) {
             const double w = D1 / d.v_sub, hw = 0.5 * w;
             va.assign((size_t)n_rows * d.v_sub * NC * 3, 0.0f);
             if (products) da.assign(va.size(), 0.0f);
             m0 = q1 = q2 = q3 = n0 = r1 = r2 = r3 = 0;
+            double k0 = 0, k1 = 0, k2 = 0, k3 = 0;         // of the constant
             float *o = va.data(), *od = da.data();
             for (int s = 0; s < n_rows; ++s) {
                 const double* ya = &Y[(size_t)s * 2 * NC];
@@ -336,18 +339,29 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                         m0 = std::max(m0, std::fabs(p[0])); q1 = std::max(q1, std::fabs(p[1]));
                         q2 = std::max(q2, std::fabs(p[2])); q3 = std::max(q3, std::fabs(c3));
                         o[0] = (float)p[0]; o[1] = (float)p[1]; o[2] = (float)p[2];
-                        if (!products || c >= C0) continue;        // (the modes' products are formed from their values)
+                        if (!wide) continue;
                         double q[4];
-                        float* t = od + (o - va.data());
                         product_piece(ya[c], p0, c2, c3, (sub + 0.5) * w, hw, s * D1 + (sub + 0.5) * w, m->rc, q);
                         n0 = std::max(n0, std::fabs(q[0])); r1 = std::max(r1, std::fabs(q[1]));
                         r2 = std::max(r2, std::fabs(q[2])); r3 = std::max(r3, std::fabs(q[3]));
+                        if (!products) continue;
+                        float* t = od + (o - va.data());
                         t[0] = (float)q[0]; t[1] = (float)q[1]; t[2] = (float)q[2];
                     }
+                for (int sub = 0; wide && sub < d.v_sub; ++sub) {
+                    double q[4];
+                    product_piece(1, 0, 0, 0, (sub + 0.5) * w, hw, s * D1 + (sub + 0.5) * w, m->rc, q);
+                    k0 = std::max(k0, std::fabs(q[0])); k1 = std::max(k1, std::fabs(q[1]));
+                    k2 = std::max(k2, std::fabs(q[2])); k3 = std::max(k3, std::fabs(q[3]));
+                }
             }
-            const double off_d = r3 * hw * hw * hw / 4 + r1 / (2.0 * kTabI2Max) * hw + r2 / (2.0 * kTabI3Max) * hw * hw;
-            const double off = q3 * hw * hw * hw / 4 + q1 / (2.0 * kTabI2Max) * hw + q2 / (2.0 * kTabI3Max) * hw * hw;
-            if ((off <= m0 * 0x1p-24 && off_d <= n0 * 0x1p-23) || n_rows * (int64_t)d.v_sub > 100000) break;    // about the rounding of a0
+            auto off = [&](double a1, double a2, double a3) {
+                return a3 * hw * hw * hw / 4 + a1 / (2.0 * kTabI2Max) * hw + a2 / (2.0 * kTabI3Max) * hw * hw;
+            };
+            // about the rounding of a0; not refined beyond 100000 intervals, met or not
+            if ((off(q1, q2, q3) <= m0 * 0x1p-24 && off(r1, r2, r3) <= n0 * 0x1p-23 && off(k1, k2, k3) <= k0 * 0x1p-23) ||
+                n_rows * (int64_t)d.v_sub > 100000)
+                break;
         }
         d.n_vrows = n_rows * d.v_sub;
         for (d.v_shift = 0; (1 << d.v_shift) < d.v_sub; ++d.v_shift) {}

@@ -1,0 +1,92 @@
+"""The tables that the edge kernels read (quadratic pieces of the amplitudes, and of envelope times amplitude) against the
+cubic pieces they are derived from, on the host."""
+
+import numpy as np
+import pytest
+
+from paper_2608_19041_b200 import binding
+from workloads import SMALL_PROFILES, make_blob
+from workloads.weights import HEADER_BYTES, blob_array_shapes
+
+U24 = 2.0 ** -24
+
+
+def _envelope(rho, rc):
+    x = rho / rc
+    u = 1 - x
+    return u ** 4 * (1 + x * (4 + x * (10 + x * (20 + 35 * x)))), -280 * x ** 4 * u ** 3 / rc
+
+
+def _cubic(m, p, a, b, rho):
+    """psi and (chi psi)' of the pair from the cubic pieces and the pair cache."""
+    g, dg = m.eval_radial_table(rho)
+    pm = m.eval_pair_cache(a, b)
+    C0 = p["C0"]
+    psi, dpsi = pm[0] * g[:, :C0] + pm[1], pm[0] * dg[:, :C0]
+    for q in range(p["R"]):
+        psi = psi + pm[2 + q] * g[:, C0 + q:C0 + q + 1]
+        dpsi = dpsi + pm[2 + q] * dg[:, C0 + q:C0 + q + 1]
+    chi, dchi = _envelope(rho, p["rc"])
+    return psi, chi[:, None] * dpsi + dchi[:, None] * psi
+
+
+def _radii(p, dx):
+    rho = np.random.default_rng(0).uniform(0.0, p["rc"], 4000)
+    k = np.arange(1, 400) * (dx / 4)                    # joints of whole, halved and quartered intervals
+    return np.concatenate([rho, [0.0, 1e-9, p["rc"] - 1e-9], k - 1e-12, k + 1e-12])
+
+
+def _distance(m, p, per_pair, dx):
+    """Largest distances from the cubic pieces, in units of 2^-24 of the largest magnitude."""
+    rho, worst = _radii(p, dx), [0.0, 0.0]
+    for a in range(p["T"]):
+        for b in range(p["T"]):
+            got, ref = m.eval_edge_tables(a, b, rho, per_pair), _cubic(m, p, a, b, rho)
+            for k in range(2):
+                worst[k] = max(worst[k], np.abs(got[k] - ref[k]).max() / (U24 * np.abs(ref[k]).max()))
+    return worst
+
+
+def _steep_blob(p, seed, small, top):
+    """A radial map of a large smooth part and a small one of high frequency, and pairs that add nothing to it."""
+    blob, at = bytearray(make_blob(p, seed)), HEADER_BYTES
+    for name, shape in blob_array_shapes(p):
+        n = 4 * int(np.prod(shape))
+        w = np.frombuffer(bytes(blob[at:at + n]), dtype="<f4").reshape(shape).copy()
+        if name == "X0":
+            w[:] = 0.0
+        if name == "omega":
+            w[-1] = top
+        if name == "W_in":
+            w[1:-1] = 0.0
+            w[-1] *= small
+        blob[at:at + n] = w.astype("<f4").tobytes()
+        at += n
+    return bytes(blob)
+
+
+# Pieces are cut until psi is within 1 and the product within 2 units of 2^-24 of their largest magnitude; the leading
+# coefficient's rounding adds half a unit, and where gamma g, beta and U q cancel, the sum of the parts' errors
+# meets a smaller magnitude.  Against the shared tables, which come from the map itself, the cubic pieces' own packed words
+# add up to a unit of value and two of derivative at the default spacing (their share grows with the spacing).
+PSI, PRODUCT = 3.0, 5.0
+
+
+@pytest.mark.parametrize("basis", ["bessel", "gaussian"])
+@pytest.mark.parametrize("name,dx,per_pair", [
+    ("p8_2_0", 0.002, 0), ("p8_2_0", 0.002, 1), ("p16_3_2", 0.002, 0), ("p16_3_2", 0.002, 1), ("p32_2_0_res", 0.002, 0),
+    ("p32_2_0_res", 0.002, 1), ("p32_2_4", 0.002, 0), ("p32_2_4", 0.002, 1), ("p32_2_4", 0.05, 1), ("p64_3_8", 0.002, 1),
+    ("p128_2_0", 0.002, 0), ("p128_2_0", 0.002, 1), ("p128_2_0", 0.01, 1)])
+def test_edge_tables_follow_the_cubic_pieces(name, dx, per_pair, basis):
+    p = SMALL_PROFILES[name]
+    m = binding.Model(make_blob(p, seed=5, basis=basis), table_dx=dx)
+    psi, product = _distance(m, p, per_pair, dx)
+    assert psi <= PSI and product <= PRODUCT
+
+
+def test_a_steep_map_with_shared_modes_is_cut_for_the_products_too():
+    # a large smooth part and a small one of high frequency: the values are within their bound long before the products
+    p = SMALL_PROFILES["p32_2_4"]
+    m = binding.Model(_steep_blob(p, 3, 3e-6, 250))
+    psi, product = _distance(m, p, 1, 0.002)
+    assert psi <= PSI and product <= PRODUCT
