@@ -236,8 +236,12 @@ __device__ __forceinline__ double image_shift(const Grid& g, int nx, int ny, int
 // lane idle.  FILL = false: count the neighbours.  FILL = true: write them, in the order of the walk.
 // Bound by instruction issue: nine instructions per centre and 32 candidates in the count pass,
 // about twenty in the fill pass.
-template <bool FILL, int G>
-__global__ void __launch_bounds__(128) k_scan_cells(Grid g, Near nr, const int* __restrict__ cell_start, const float4* __restrict__ rec,
+// SPREAD = false: the warps of a few blocks share a cell, and with it the candidates in L1.  SPREAD = true: a cell's atoms
+// are cut into groups of G from its first atom on, and a warp takes the groups that start among `span` consecutive
+// atoms of the internal order, so that there are N / span warps however the atoms are spread over the cells.
+template <bool FILL, int G, bool SPREAD>
+__global__ void __launch_bounds__(128) k_scan_cells(int N, int span, Grid g, Near nr, const int* __restrict__ skey,
+                                                    const int* __restrict__ cell_start, const float4* __restrict__ rec,
                                                     const double* __restrict__ xs0, int* __restrict__ deg,
                                                     const eidx_t* __restrict__ row_ptr, int2* __restrict__ nbr, int* __restrict__ err) {
     struct Run { int end, first, code; float sx, sy, sz; };   // candidates before its end; atom of candidate 0; image
@@ -247,9 +251,30 @@ __global__ void __launch_bounds__(128) k_scan_cells(Grid g, Near nr, const int* 
     const unsigned lt_mask = (1u << lane) - 1u;
     const int wz = 2 * g.m[2] + 1, wy = 2 * g.m[1] + 1, wx = 2 * g.m[0] + 1;
     const int n_keys = g.halves * g.ncell;
-    for (int key0 = blockIdx.x; key0 < n_keys; key0 += gridDim.x) {
-    const int c_end = cell_start[key0 + 1], first_i = cell_start[key0] + G * (warp + n_warps * blockIdx.y);
-    if (first_i >= c_end) continue;
+    const int64_t span0 = SPREAD ? ((int64_t)blockIdx.x * n_warps + warp) * span : 0;
+    int key_l = 0;
+    unsigned todo = 0;                           // SPREAD: lanes whose atom starts a group
+    if (SPREAD) {
+        bool lead = false;
+        if (lane < span && span0 + lane < N) {
+            key_l = skey[span0 + lane];
+            lead = ((int)span0 + lane - cell_start[key_l]) % G == 0;
+        }
+        todo = __ballot_sync(0xffffffffu, lead);
+    }
+    for (int key0 = blockIdx.x; SPREAD ? todo != 0 : key0 < n_keys; key0 += gridDim.x) {
+    int first_i = 0;
+    if (SPREAD) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1;
+        first_i = (int)span0 + l;
+        key0 = __shfl_sync(0xffffffffu, key_l, l);
+    }
+    const int c_end = cell_start[key0 + 1];
+    if (!SPREAD) {
+        first_i = cell_start[key0] + G * (warp + n_warps * blockIdx.y);
+        if (first_i >= c_end) continue;
+    }
     const int key = key0 < g.ncell ? key0 : key0 - g.ncell;         // a ghost's own bin
     const int cx = key % g.nc[0], cy = (key / g.nc[0]) % g.nc[1], cz = key / (g.nc[0] * g.nc[1]);
     const int sz0 = walk_start(cz, g.m[2], g.nc[2], g.pbc[2], g.sorted);
@@ -271,7 +296,7 @@ __global__ void __launch_bounds__(128) k_scan_cells(Grid g, Near nr, const int* 
     int per_line = 0;
     for (int tx = 0, xc, nx; tx < wx; ++per_line) tx += x_run(tx, &xc, &nx);
     const int n_runs = wz * wy * per_line;
-    for (int i0 = first_i; i0 < c_end; i0 += G * n_warps * gridDim.y) {
+    for (int i0 = first_i; SPREAD ? i0 == first_i : i0 < c_end; i0 += G * n_warps * gridDim.y) {
     const int gn = min(G, c_end - i0);
     // lane k < G keeps centre k in double precision; every lane has all of them in single precision
     double xi = 0, yi = 0, zi = 0;
@@ -750,10 +775,13 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
         }
     }
     int64_t ncell = 1;
+    bool coarse = false;                        // fewer bins than the list radius allows: two list radii wide or more
     const double rl_pad = r_list * (1.0 + 1e-9) + 1e-12;
     for (int k = 0; k < 3; ++k) {
         g.L[k] = L[k]; g.lo[k] = lo[k]; g.pbc[k] = pbc[k] ? 1 : 0;
-        int nc = (int)std::floor(ext[k] * unit[k] / rl_pad);
+        const double whole = std::floor(ext[k] * unit[k] / rl_pad);
+        if (whole > 1024) coarse = true;
+        int nc = whole > 1024 ? 1024 : (int)whole;
         // a periodic box of less than three list radii: bins of a half, third or quarter of the list
         // radius still give 2 m + 1 distinct bins (from 2.5, 2.33 and 2.25 list radii on), and with them
         // rows sorted by neighbour index
@@ -763,7 +791,6 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
                 if (fine >= 2 * q + 1) { nc = fine; break; }
             }
         if (nc < 1) nc = 1;
-        if (nc > 1024) nc = 1024;
         g.nc[k] = nc;
     }
     // keep the cell table modest relative to the atom count
@@ -772,6 +799,7 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
         for (int k = 1; k < 3; ++k) if (g.nc[k] > g.nc[kmax]) kmax = k;
         if (g.nc[kmax] == 1) break;
         g.nc[kmax] = (g.nc[kmax] + 1) / 2;
+        coarse = true;
     }
     for (int k = 0; k < 3; ++k) {
         const double cw = ext[k] / g.nc[k];
@@ -853,19 +881,29 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     // 125 cells: count and fill 19 + 24 us; with one block per cell they took 34 + 45).
     // Both are bound by instruction issue.  With one warp per centre and every test in double precision
     // 216,000 atoms with 273 neighbours took 1.21 + 1.49 ms, so 0.32 + 0.52.
-    const bool few = N < 16384;
-    const dim3 scan_blocks((unsigned)(nkeys < 148 * 64 ? nkeys : 148 * 64), few ? 4 : 1);
-    const int scan_threads = 128;
-    auto scan = few ? k_scan_cells<false, 2> : k_scan_cells<false, 8>;
-    scan<<<scan_blocks, scan_threads, 0, st>>>(g, nr, nb->cell_start, nb->rec, nb->xs0, nb->deg, nullptr, nullptr, d_err);
+    // Where cells hold more than their own warps take at a time, the groups of centres are spread over warps atom by
+    // atom instead: in cells two list radii wide and more (coarse: a box mostly empty, in which a cluster of atoms
+    // falls into a few cells; 200,000 atoms in a box of 5000 Angstrom build in 20 ms, by the cells' own warps in 604; 2000
+    // in 400 Angstrom in 149 us, so 425), and in small systems of more than 32 atoms per cell (108 atoms in one cell 146 us,
+    // so 265; 4000 of dense carbon 154, so 212, and 194, so 393, without periodicity).  Elsewhere the shared candidates win
+    // (9000 atoms of water 194 us, spread 200), also in larger dense systems, whose cells are many (30,000 atoms of
+    // carbon 287 us, spread 330).  Spans of eight atoms for eight centres, of one for two (no warp then has two groups).
+    const bool few = N < 16384, apart = coarse || (few && N > 32 * nkeys);
+    const int span = few ? 1 : 8;
+    const dim3 scan_blocks(apart ? (unsigned)((N64 + span - 1) / span) : (unsigned)(nkeys < 148 * 64 ? nkeys : 148 * 64), !apart && few ? 4 : 1);
+    const int scan_threads = apart ? 32 : 128;
+    auto scan = apart ? (few ? k_scan_cells<false, 2, true> : k_scan_cells<false, 8, true>)
+                       : (few ? k_scan_cells<false, 2, false> : k_scan_cells<false, 8, false>);
+    scan<<<scan_blocks, scan_threads, 0, st>>>(N, span, g, nr, nb->key2, nb->cell_start, nb->rec, nb->xs0, nb->deg, nullptr, nullptr, d_err);
     NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
     tmp_bytes = nb->cub_bytes;
     NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, N + 1, st));
     int code = read_totals(nb, N, n_owned, d_type, d_err, fetch, st, err);
     if (code != UMLMD_OK) return code;
     if (nb->E > 0) {
-        auto fill = few ? k_scan_cells<true, 2> : k_scan_cells<true, 8>;
-        fill<<<scan_blocks, scan_threads, 0, st>>>(g, nr, nb->cell_start, nb->rec, nb->xs0, nullptr, nb->row_ptr, nb->nbr, d_err);
+        auto fill = apart ? (few ? k_scan_cells<true, 2, true> : k_scan_cells<true, 8, true>)
+                           : (few ? k_scan_cells<true, 2, false> : k_scan_cells<true, 8, false>);
+        fill<<<scan_blocks, scan_threads, 0, st>>>(N, span, g, nr, nb->key2, nb->cell_start, nb->rec, nb->xs0, nullptr, nb->row_ptr, nb->nbr, d_err);
         NB_CHECK(cudaMemsetAsync(nb->rev, 0xff, sizeof(eidx_t) * (size_t)nb->E, st));
         auto reverse = g.sorted ? k_reverse_map<kByIndex> : k_reverse_map<kByBin>;
         reverse<<<(N + TB / 32 - 1) / (TB / 32), TB, 0, st>>>(N, g, nb->key2, nb->row_ptr, nb->nbr, nb->rev);

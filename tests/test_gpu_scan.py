@@ -67,3 +67,52 @@ def test_pairs_at_the_list_radius(origin):
         pos += [a, a + RC * (1.0 + (-1.0) ** k * 10.0 ** -rng.integers(3, 14)) * u]
     pos = np.array(pos)
     _run(pos, np.eye(3) * 400.0, (0, 0, 0), 0.0, np.arange(len(pos)))
+
+
+def _cluster(n, seed, a=2.32):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    k = int(np.ceil(n ** (1 / 3)))
+    sites = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n] * a
+    return sites + rng.uniform(-0.26, 0.26, (n, 3))
+
+
+@pytest.mark.parametrize("pbc", [(1, 1, 1), (0, 0, 0)])
+@pytest.mark.parametrize("n", [1500, 16500])
+def test_rows_of_a_cluster_in_a_large_box(n, pbc):
+    # bins far wider than the list radius hold most of the atoms; a few atoms elsewhere keep the box open that large
+    rng = np.random.Generator(np.random.PCG64(9))
+    L = 60.0 * np.cbrt(n)
+    pos = np.concatenate([0.4 * L + _cluster(n, 8), rng.random((40, 3)) * L])
+    _run(pos, np.eye(3) * L, pbc, 1.0, np.sort(rng.choice(len(pos), 48, replace=False)))
+
+
+@pytest.mark.parametrize("pbc", [(1, 1, 1), (0, 1, 0)])
+@pytest.mark.parametrize("n", [64, 513, 2197])
+def test_rows_of_full_cells(n, pbc):
+    # more than 32 atoms per cell: 64 in a single one, 2197 of them in 27
+    pos = _cluster(n, 7, a=1.8)
+    L = 1.8 * np.ceil(n ** (1 / 3) - 1e-9)
+    _run(pos, np.eye(3) * L, pbc, 1.0, np.arange(0, n, max(1, n // 60)))
+
+
+def test_a_cluster_is_shared_among_the_whole_machine():
+    # 200,000 atoms in some fifty bins: about 30 times the candidates per atom of a filled box.  Shared evenly the build takes
+    # some 25 times as long; left to a few warps of each bin it took 750 times as long
+    import time
+    from paper_2608_19041_b200 import binding
+    n = 200000
+    pos = torch.tensor(_cluster(n, 8)).cuda()
+    types = torch.zeros(n, dtype=torch.int32, device="cuda")
+    m = binding.Model(make_blob(SMALL_PROFILES["p8_2_0"], 3))
+    best = []
+    for edge in (2.32 * 59, 5000.0):
+        ts = []
+        for _ in range(4):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            m.build_neighbors(pos, types, np.eye(3) * edge, (1, 1, 1), 1.0)
+            torch.cuda.synchronize()
+            ts.append(time.perf_counter() - t)
+        best.append(min(ts))
+    m.close()
+    assert best[1] <= 150 * best[0], best
