@@ -1,4 +1,5 @@
 // extern "C" entry points of libumlmd (see include/umlmd.h for the contract).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -27,25 +28,28 @@ struct umlmd {
     // workspace
     float* state = nullptr; float* desc = nullptr; float* pre = nullptr; float* hbuf = nullptr;
     __half* tc_hi = nullptr; __half* tc_lo = nullptr;   // half-precision split of the current GEMM's activations
-    float* fused_scratch = nullptr;      // per-CTA areas of the one-kernel MLP
+    float* fused_scratch = nullptr; int64_t fused_cap = 0;      // per-CTA areas of the one-kernel MLP
     int64_t tile_cap = 0;
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
     double* virial_part = nullptr; int64_t vpart_cap = 0;
     double* frame_out = nullptr; int64_t frame_out_cap = 0;     // batched evaluation: [n_frames][10] energy, virial
-    double* h_frame = nullptr; int64_t h_frame_cap = 0;         // pinned copy of it
+    double* h_frame = nullptr; int64_t h_frame_cap = 0;         // pinned copy of it: part of `pinned`, or frame_pinned for many frames
+    void* frame_pinned = nullptr;
     double* scratch = nullptr; double* d_out = nullptr; int* d_err = nullptr;
-    double* h_out = nullptr; int* h_err = nullptr;      // pinned
+    void* pinned = nullptr;                             // one allocation for h_out, h_frame, h_err, h_species and the list's h_totals
+    double* h_out = nullptr; int* h_err = nullptr;
     // per-pair amplitude tables of the species present (set up by umlmd_build_neighbors)
     int64_t pair_table_budget = 192ll << 20;            // bytes; negative = never build them
     bool pair_tables = false;                           // in use for the current system
     std::vector<int> present;                           // species the tables were built for, ascending
-    float* table_uni = nullptr; size_t table_uni_cap = 0;   // [present^2][n_rows][3][C0], capacity in floats (C0 < 32)
-    float* vtable_uni = nullptr; size_t vtable_uni_cap = 0; // [present^2][n_vrows][2][C0], the same for values alone
-    float* dtable_uni = nullptr; size_t dtable_uni_cap = 0; // [present^2][n_vrows][2][C0], envelope products (from C0 = 32 on, instead of table_uni)
+    float* uni = nullptr; int64_t uni_cap = 0;              // one allocation for the four below
     float* uni_scale = nullptr;                         // [6] largest |c2|, |c3|, |a1|, |a2| and |a1|, |a2| of those tables
+    float* table_uni = nullptr;                         // [present^2][n_rows][3][C0] (C0 < 32)
+    float* vtable_uni = nullptr;                        // [present^2][n_vrows][2][C0], the same for values alone
+    float* dtable_uni = nullptr;                        // [present^2][n_vrows][2][C0], envelope products (from C0 = 32 on, instead of table_uni)
     int* d_species = nullptr;                           // [3T]: occurrence flags, species -> slot, present list
-    int* h_species = nullptr;                           // pinned [T]
+    int* h_species = nullptr;                           // [T]
     // MD
     double* md_pos = nullptr; double* md_vel = nullptr; double* md_force = nullptr; int64_t md_cap = 0;    // (capacity in doubles)
     double* d_mass = nullptr; double* d_inv_mass = nullptr;
@@ -125,7 +129,7 @@ cudaError_t upload(umlmd_t* h, const std::vector<T>& v, T** out) {
     if (e != cudaSuccess) return e;
     h->model_allocs.push_back(p);
     if (!v.empty()) e = cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, h->st);
-    *out = static_cast<T*>(p);
+    if (e == cudaSuccess) *out = static_cast<T*>(p);
     return e;
 }
 
@@ -142,6 +146,15 @@ bool keeps_intermediates(const umlmd_t* h) { return h->nb.N < kIntermediatesMaxA
 // whether some evaluation of up to B rows runs its MLP as a chain of GEMMs
 bool mlp_needs_chain(const umlmd_t* h, int64_t B) {
     return !(mlp_fused_pick(h->d, h->mlp_path, B, true) && mlp_fused_pick(h->d, h->mlp_path, B, false));
+}
+
+// floats that the one-kernel MLP needs for the tiles of `rows` rows, B at a time (none where the rule takes the chain
+// for all of them; it takes it for an energy alone wherever it does with a gradient)
+int64_t fused_floats(const umlmd_t* h, int64_t rows, int64_t B) {
+    int64_t need = 0;
+    for (const int64_t n : {rows < B ? rows : B, B > 0 ? rows % B : 0})
+        if (n > 0 && mlp_fused_pick(h->d, h->mlp_path, n, true)) need = std::max(need, mlp_fused_scratch_floats(h->d, n));
+    return need;
 }
 
 int ensure_workspace(umlmd_t* h) {
@@ -163,9 +176,9 @@ int ensure_workspace(umlmd_t* h) {
         const int64_t split = chain ? 2 * B * wmax : B * d.DP;      // the one-kernel MLP only reads the feature split
         c = 0; API_CUDA(h, dev_ensure(&h->tc_hi, &c, split));
         c = 0; API_CUDA(h, dev_ensure(&h->tc_lo, &c, split));
-        if (mlp_fused_pick(d, h->mlp_path, 1, true)) { c = 0; API_CUDA(h, dev_ensure(&h->fused_scratch, &c, mlp_fused_scratch_floats(d, B))); }
         h->tile_cap = B;
     }
+    if (const int64_t need = fused_floats(h, h->nb.n_owned, B)) API_CUDA(h, dev_ensure(&h->fused_scratch, &h->fused_cap, need));
     if (E > h->g_cap || !h->g) { API_CUDA(h, dev_ensure(&h->g, &h->g_cap, E * 3, 1.1)); h->g_cap /= 3; }
     if (N > h->n_cap) {
         int64_t c;
@@ -346,6 +359,8 @@ int run_replayed(umlmd_t* h, umlmd_t::Replay& r, const void* k0, const void* k1,
     return UMLMD_OK;
 }
 
+constexpr int64_t kFrameDoubles = 256 * 10;      // results of 256 frames have a place from the start
+
 // first use on a device: upload the model constants and allocate the small result buffers
 int ensure_device_model(umlmd_t* h) {
     if (h->on_device) return UMLMD_OK;
@@ -354,7 +369,7 @@ int ensure_device_model(umlmd_t* h) {
     cudaError_t e = cudaSuccess;
     auto up = [&](const std::vector<float>& v, float** p) { if (e == cudaSuccess) e = upload(h, v, p); };
     auto uph = [&](const std::vector<__half>& v, __half** p) { if (e == cudaSuccess) e = upload(h, v, p); };
-    up(m.table, &md.table); up(m.vtable, &md.vtable); up(m.dtable, &md.dtable); up(m.pairmod, &md.pairmod); up(m.X0, &md.X0); up(m.W1p, &md.W1p); up(m.W2p, &md.W2p);
+    up(m.pairmod, &md.pairmod); up(m.X0, &md.X0); up(m.W1p, &md.W1p); up(m.W2p, &md.W2p);
     up(m.A1, &md.A1); up(m.A2, &md.A2); up(m.mu, &md.mu); up(m.inv_sigma, &md.inv_sigma);
     up(m.type_bias, &md.type_bias);
     for (int t = 0; t < h->d.n_hidden; ++t) { up(m.theta[t], &md.theta[t]); up(m.thetaT[t], &md.thetaT[t]); up(m.bias[t], &md.bias[t]);
@@ -375,21 +390,37 @@ int ensure_device_model(umlmd_t* h) {
     if (e == cudaSuccess) { e = dev_malloc(&p, sizeof(double) * 16); h->d_out = (double*)p; }
     if (e == cudaSuccess) { e = dev_malloc(&p, sizeof(int) * 4); h->d_err = (int*)p; }
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_err, 0, sizeof(int) * 4, h->st);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_out, sizeof(double) * 16);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_err, sizeof(int) * 4);
+    if (e == cudaSuccess) { e = dev_malloc(&p, sizeof(int) * 3 * (size_t)h->d.T); h->d_species = (int*)p; }
+    if (e == cudaSuccess) e = cudaMallocHost(&h->pinned, sizeof(double) * (16 + kFrameDoubles) + sizeof(eidx_t) * 2 + sizeof(int) * (4 + (size_t)h->d.T));
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     if (e != cudaSuccess) {                    // nothing stays half done: the next call starts over
         cudaStreamSynchronize(h->st);
         for (void* q : h->model_allocs) dev_free(q);
         h->model_allocs.clear();
-        dev_free(h->scratch); dev_free(h->d_out); dev_free(h->d_err);
-        h->scratch = h->d_out = nullptr; h->d_err = nullptr;
-        if (h->h_out) cudaFreeHost(h->h_out);
-        if (h->h_err) cudaFreeHost(h->h_err);
-        h->h_out = nullptr; h->h_err = nullptr;
+        dev_free(h->scratch); dev_free(h->d_out); dev_free(h->d_err); dev_free(h->d_species);
+        h->scratch = h->d_out = nullptr; h->d_err = h->d_species = nullptr;
+        if (h->pinned) cudaFreeHost(h->pinned);
+        h->pinned = nullptr;
         return fail(h, UMLMD_E_CUDA, std::string("model upload: ") + cudaGetErrorString(e));
     }
+    h->h_out = (double*)h->pinned;
+    h->h_frame = h->h_out + 16;
+    h->h_frame_cap = kFrameDoubles;
+    h->nb.h_totals = (eidx_t*)(h->h_frame + kFrameDoubles);
+    h->h_err = (int*)(h->nb.h_totals + 2);
+    h->h_species = h->h_err + 4;
     h->on_device = true;
+    return UMLMD_OK;
+}
+
+// The radial tables that the kernels of the current system read (a list of species with per-pair tables needs the cubic
+// pieces to make them, others the value table and, for the backward pass, products or cubic pieces).  The first build
+// of a handle waits for these copies: all three took 1 to 1.8 ms more than the one that is needed.
+int ensure_radial_tables(umlmd_t* h, bool pair_tables) {
+    const bool products = !h->hm.dtable.empty();
+    if ((pair_tables || !products) && !h->md.table) API_CUDA(h, upload(h, h->hm.table, &h->md.table));
+    if (!pair_tables && !h->md.vtable) API_CUDA(h, upload(h, h->hm.vtable, &h->md.vtable));
+    if (!pair_tables && products && !h->md.dtable) API_CUDA(h, upload(h, h->hm.dtable, &h->md.dtable));
     return UMLMD_OK;
 }
 
@@ -416,19 +447,6 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     return UMLMD_OK;
 }
 
-int ensure_species_buffers(umlmd_t* h) {
-    int rc = ensure_device_model(h);
-    if (rc != UMLMD_OK) return rc;
-    const size_t T = (size_t)h->d.T;
-    if (!h->d_species) {
-        void* p = nullptr;
-        API_CUDA(h, dev_malloc(&p, sizeof(int) * 3 * T));
-        h->d_species = (int*)p;
-    }
-    if (!h->h_species) API_CUDA(h, cudaMallocHost((void**)&h->h_species, sizeof(int) * T));
-    return UMLMD_OK;
-}
-
 // With few species present, psi_c(rho) of every ordered pair among them is tabulated by itself,
 // so that the edge kernels read one table row per edge and neither pair rows nor shared modes.
 // The tables depend on the model and the set of species only, so they are kept across builds.
@@ -445,23 +463,19 @@ int setup_pair_tables(umlmd_t* h) {
     const bool use = np > 0 && h->pair_table_budget >= 0 && full <= (size_t)h->pair_table_budget &&
                      3 * (floats + vfloats + dfloats) * sizeof(float) <= 5 * (size_t)h->pair_table_budget;
     h->pair_tables = use && present == h->present;
-    if (!use || h->pair_tables) return UMLMD_OK;
+    if (h->pair_tables) return UMLMD_OK;
+    const int rc = ensure_radial_tables(h, use);
+    if (rc != UMLMD_OK || !use) return rc;
     h->present.clear();                               // no tables until all of them are made
-    auto grow = [&](float** p, size_t* cap, size_t need) {
-        if (need <= *cap) return cudaSuccess;
-        dev_free(*p); *p = nullptr; *cap = 0;
-        void* q = nullptr;
-        const cudaError_t e = dev_malloc(&q, sizeof(float) * need);
-        if (e == cudaSuccess) { *p = (float*)q; *cap = need; }
-        return e;
-    };
-    API_CUDA(h, grow(&h->table_uni, &h->table_uni_cap, floats));
-    API_CUDA(h, grow(&h->vtable_uni, &h->vtable_uni_cap, vfloats));
-    API_CUDA(h, grow(&h->dtable_uni, &h->dtable_uni_cap, dfloats));
+    constexpr size_t head = 32;                       // floats; the tables behind start on 128 bytes
+    API_CUDA(h, dev_ensure(&h->uni, &h->uni_cap, (int64_t)(head + floats + vfloats + dfloats)));
+    h->uni_scale = h->uni;
+    h->table_uni = h->uni + head;
+    h->vtable_uni = h->table_uni + floats;
+    h->dtable_uni = h->vtable_uni + vfloats;
     std::vector<int> up(2 * (size_t)d.T, 0);          // species -> slot, then the present list
     for (size_t k = 0; k < np; ++k) { up[present[k]] = (int)k; up[d.T + k] = present[k]; }
     API_CUDA(h, cudaMemcpyAsync(h->d_species + d.T, up.data(), sizeof(int) * up.size(), cudaMemcpyHostToDevice, h->st));
-    if (!h->uni_scale) { void* p = nullptr; API_CUDA(h, dev_malloc(&p, 8 * sizeof(float))); h->uni_scale = (float*)p; }
     API_CUDA(h, launch_fuse_pair_tables(d, h->md.table, h->md.pairmod, h->d_species + 2 * d.T, (int)np, h->uni_scale, h->table_uni, h->vtable_uni, h->dtable_uni, h->st));
     API_CUDA(h, cudaStreamSynchronize(h->st));       // `up` is pageable host memory
     h->launches_total += 2;
@@ -516,7 +530,7 @@ int umlmd_destroy(umlmd_t* h) {
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
     void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
-                    h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->table_uni, h->vtable_uni, h->dtable_uni, h->d_species, h->uni_scale};
+                    h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->uni, h->d_species};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
     for (cudaEvent_t e : h->free_events) cudaEventDestroy(e);
@@ -524,10 +538,8 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->rp_step.exec) cudaGraphExecDestroy(h->rp_step.exec);
     if (h->rp_nvt.exec) cudaGraphExecDestroy(h->rp_nvt.exec);
     if (h->cap_st) cudaStreamDestroy(h->cap_st);
-    if (h->h_out) cudaFreeHost(h->h_out);
-    if (h->h_err) cudaFreeHost(h->h_err);
-    if (h->h_species) cudaFreeHost(h->h_species);
-    if (h->h_frame) cudaFreeHost(h->h_frame);
+    if (h->pinned) cudaFreeHost(h->pinned);
+    if (h->frame_pinned) cudaFreeHost(h->frame_pinned);
     delete h;
     return UMLMD_OK;
 }
@@ -565,7 +577,7 @@ int umlmd_build_neighbors(umlmd_t* h, int64_t N, const double* d_pos, const int3
     h->have_md = false;
     // which species occur: few enough of them get per-pair amplitude tables (see below); comes back with
     // the edge count, and with what the device found wrong (non-finite positions, image range, species)
-    int rc = ensure_species_buffers(h);
+    int rc = ensure_device_model(h);
     if (rc != UMLMD_OK) return rc;
     *h->h_err = 0;
     for (int t = 0; t < h->d.T; ++t) h->h_species[t] = 0;
@@ -642,7 +654,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t Bt = N < h->node_tile ? N : h->node_tile;
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
-    if (mlp_fused_pick(d, h->mlp_path, 1, true)) t += buf(mlp_fused_scratch_floats(d, Bt), 4);
+    if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
     t += grown(3 * n_edges, 4);
@@ -717,7 +729,7 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
     const int64_t N = frame_offsets[n_frames];
     if (N > 0x7fff0000LL) return fail(h, UMLMD_E_INVALID_ARG, "too many atoms for 32-bit indices");
     if (N > 0 && (!d_pos || !d_type)) return fail(h, UMLMD_E_INVALID_ARG, "null positions or species");
-    int rc = ensure_species_buffers(h);
+    int rc = ensure_device_model(h);
     if (rc != UMLMD_OK) return rc;
     h->have_list = false; h->have_md = false; h->have_edge_grad = false;     // the handle's list is replaced
     ++h->list_serial;
@@ -734,9 +746,10 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
     const int64_t n_out = (int64_t)n_frames * 10;
     API_CUDA(h, dev_ensure(&h->frame_out, &h->frame_out_cap, n_out));
     if (n_out > h->h_frame_cap) {
-        if (h->h_frame) cudaFreeHost(h->h_frame);
-        h->h_frame = nullptr; h->h_frame_cap = 0;
-        API_CUDA(h, cudaMallocHost((void**)&h->h_frame, sizeof(double) * (size_t)n_out));
+        if (h->frame_pinned) cudaFreeHost(h->frame_pinned);
+        h->frame_pinned = nullptr; h->h_frame_cap = 0;
+        API_CUDA(h, cudaMallocHost(&h->frame_pinned, sizeof(double) * (size_t)n_out));
+        h->h_frame = (double*)h->frame_pinned;
         h->h_frame_cap = n_out;
     }
     if (N > 0) {

@@ -218,7 +218,7 @@ struct NeighborDev {
     int* key = nullptr; int* key2 = nullptr; int* idx = nullptr; int* idx2 = nullptr;
     int* cell_start = nullptr; int64_t ncell_cap = 0;
     int* deg = nullptr;
-    eidx_t* h_totals = nullptr;  // pinned [2]: edges in all, edges of owned atoms
+    eidx_t* h_totals = nullptr;  // pinned [2], the caller's: edges in all, edges of owned atoms
     void* cub_tmp = nullptr; size_t cub_bytes = 0;
 };
 

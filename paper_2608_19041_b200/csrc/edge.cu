@@ -981,54 +981,55 @@ cudaError_t dispatch(const EdgeArgs& a, cudaStream_t st) {
 // radial table: the cubic coefficients are linear in the tabulated functions, so the same
 // combination of the coefficient rows of [g, q] gives them; and as [..][n_vrows][2][C0] in those of the
 // value and product tables.  Two passes: the first finds the largest magnitudes of the coefficients that are packed (the scale
-// of the words), the second writes the rows.
+// of the words), the second writes the rows.  A thread takes one channel of one row for kPairsPerThread pairs: the six
+// maxima then meet in memory once per warp and that many pairs (with a thread per pair 25 pairs at C0 = 128 took 1.46 ms,
+// most of it in atomics on six addresses, so 0.32).
+constexpr int kPairsPerThread = 32;
 template <bool WRITE>
 __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, const float* __restrict__ pairmod,
                                    const int* __restrict__ present, int n_present, float* __restrict__ scale,
                                    float* __restrict__ out, float* __restrict__ vout, float* __restrict__ dout) {
-    const int64_t per_pair = (int64_t)d.n_rows * d.C0;
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // over [pair][row][c]
-    float c2 = 0.f, c3 = 0.f, a1 = 0.f, a2 = 0.f, b1 = 0.f, b2 = 0.f;
-    if (idx < per_pair * n_present * n_present) {
-        const int pr = (int)(idx / per_pair);
-        const int64_t in_pair = idx - pr * per_pair;
-        const int c = (int)(in_pair % d.C0);
-        const int64_t row = in_pair / d.C0;
-        const int si = present[pr / n_present], sj = present[pr % n_present];
-        const float* pm = pairmod + (size_t)(si * d.T + sj) * (2 + d.R) * d.C0 + c;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;                // over [row][c]
+    const int first = blockIdx.y * kPairsPerThread, last = min(first + kPairsPerThread, n_present * n_present);
+    float mx[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};       // |c2|, |c3|, |a1|, |a2| of the values, |a1|, |a2| of the products
+    if (idx < d.n_rows * d.C0) {
+        const int row = idx / d.C0, c = idx - row * d.C0;
         const float* tr = table + (size_t)row * 3 * d.CP;
-        double v[4];
-        pair_cubic(d, tr, pm, c, v);
-        c2 = (float)v[2]; c3 = (float)v[3];
         const double w = (double)d.dx / d.v_sub;
-        for (int sub = 0; sub < d.v_sub; ++sub) {          // values alone (common.cuh, value_piece)
-            double p[3];
-            value_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, p);
-            a1 = fmaxf(a1, fabsf((float)p[1])); a2 = fmaxf(a2, fabsf((float)p[2]));
-            if (WRITE) {
-                float* vrow = vout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
-                vrow[c] = (float)p[0];
-                vrow[d.C0 + c] = __uint_as_float(tab_pack((float)p[1], (float)p[2], tab_step2(scale[2]), tab_step3(scale[3])));
+        for (int pr = first; pr < last; ++pr) {
+            const int si = present[pr / n_present], sj = present[pr % n_present];
+            double v[4];
+            pair_cubic(d, tr, pairmod + (size_t)(si * d.T + sj) * (2 + d.R) * d.C0 + c, c, v);
+            const float c2 = (float)v[2], c3 = (float)v[3];
+            mx[0] = fmaxf(mx[0], fabsf(c2)); mx[1] = fmaxf(mx[1], fabsf(c3));
+            for (int sub = 0; sub < d.v_sub; ++sub) {          // values alone (common.cuh, value_piece)
+                double p[3];
+                value_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, p);
+                mx[2] = fmaxf(mx[2], fabsf((float)p[1])); mx[3] = fmaxf(mx[3], fabsf((float)p[2]));
+                if (WRITE) {
+                    float* vrow = vout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
+                    vrow[c] = (float)p[0];
+                    vrow[d.C0 + c] = __uint_as_float(tab_pack((float)p[1], (float)p[2], tab_step2(scale[2]), tab_step3(scale[3])));
+                }
+                if (!wide_channels(d.C0)) continue;
+                double q[4];                                   // envelope products (product_piece)
+                product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, (double)row * d.dx + (sub + 0.5) * w, (double)d.rc, q);
+                mx[4] = fmaxf(mx[4], fabsf((float)q[1])); mx[5] = fmaxf(mx[5], fabsf((float)q[2]));
+                if (WRITE) {
+                    float* drow = dout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
+                    drow[c] = (float)q[0];
+                    drow[d.C0 + c] = __uint_as_float(tab_pack((float)q[1], (float)q[2], tab_step2(scale[4]), tab_step3(scale[5])));
+                }
             }
-            if (!wide_channels(d.C0)) continue;
-            double q[4];                                   // envelope products (product_piece)
-            product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, (double)row * d.dx + (sub + 0.5) * w, (double)d.rc, q);
-            b1 = fmaxf(b1, fabsf((float)q[1])); b2 = fmaxf(b2, fabsf((float)q[2]));
-            if (WRITE) {
-                float* drow = dout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;
-                drow[c] = (float)q[0];
-                drow[d.C0 + c] = __uint_as_float(tab_pack((float)q[1], (float)q[2], tab_step2(scale[4]), tab_step3(scale[5])));
+            if (WRITE && !wide_channels(d.C0)) {
+                float* orow = out + ((size_t)pr * d.n_rows + row) * 3 * d.C0;
+                orow[c] = (float)v[0];
+                orow[d.C0 + c] = (float)v[1];
+                orow[2 * d.C0 + c] = __uint_as_float(tab_pack(c2, c3, tab_step2(scale[0]), tab_step3(scale[1])));
             }
-        }
-        if (WRITE && !wide_channels(d.C0)) {
-            float* orow = out + ((size_t)pr * d.n_rows + row) * 3 * d.C0;
-            orow[c] = (float)v[0];
-            orow[d.C0 + c] = (float)v[1];
-            orow[2 * d.C0 + c] = __uint_as_float(tab_pack(c2, c3, tab_step2(scale[0]), tab_step3(scale[1])));
         }
     }
     if (!WRITE) {        // non-negative floats order like their bit patterns
-        float mx[6] = {fabsf(c2), fabsf(c3), a1, a2, b1, b2};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
 #pragma unroll
@@ -1042,11 +1043,11 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
 
 cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const float* pairmod, const int* present,
                                     int n_present, float* scale, float* out, float* vout, float* dout, cudaStream_t st) {
-    const int64_t n = (int64_t)d.n_rows * d.C0 * n_present * n_present;
-    if (n == 0) return cudaSuccess;
+    const int n = d.n_rows * d.C0, pairs = n_present * n_present;
+    if (n == 0 || pairs == 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(scale, 0, 6 * sizeof(float), st);
     if (e != cudaSuccess) return e;
-    const unsigned blocks = (unsigned)((n + 255) / 256);
+    const dim3 blocks((unsigned)((n + 255) / 256), (unsigned)((pairs + kPairsPerThread - 1) / kPairsPerThread));
     k_fuse_pair_tables<false><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout, dout);
     k_fuse_pair_tables<true><<<blocks, 256, 0, st>>>(d, table, pairmod, present, n_present, scale, out, vout, dout);
     return cudaGetLastError();

@@ -712,7 +712,6 @@ void neighbor_free(NeighborDev* nb) {
                     nb->cub_tmp, nb->bounds};
     for (void* p : ptrs)
         dev_free(p);
-    if (nb->h_totals) cudaFreeHost(nb->h_totals);
     *nb = NeighborDev();
 }
 
@@ -720,7 +719,6 @@ void neighbor_free(NeighborDev* nb) {
 // know by then, and the edge arrays grow to hold the list.
 static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, int* d_err, const BuildFetch* fetch, cudaStream_t st,
                        std::string* err) {
-    if (!nb->h_totals) NB_CHECK(cudaMallocHost((void**)&nb->h_totals, 2 * sizeof(eidx_t)));
     NB_CHECK(cudaMemcpyAsync(nb->h_totals, nb->row_ptr + N, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
     if (n_owned < N) NB_CHECK(cudaMemcpyAsync(nb->h_totals + 1, nb->row_ptr + n_owned, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
     if (fetch) {

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from workloads import SMALL_PROFILES, make_blob
+from workloads import CONFIGS, SMALL_PROFILES, make_blob
 
 pytestmark = pytest.mark.gpu
 
@@ -128,3 +128,30 @@ def test_a_failed_allocation_leaves_no_list_and_is_made_up_for():
             assert torch.equal(a, b), spare_mb
         m.close()
     assert failed >= 6
+
+
+def _held(blob, box, **kw):
+    """Device memory that a handle takes for its first build."""
+    from paper_2608_19041_b200 import binding
+    m = binding.Model(blob, **kw)
+    before = m.query()["device_bytes"]
+    m.build_neighbors(*box, (0, 0, 0), 0.0)
+    held = m.query()["device_bytes"] - before
+    m.close()
+    return held
+
+
+def test_the_first_build_allocates_what_the_system_uses():
+    # the one-kernel MLP's areas only where the rule takes it: 24,000 atoms at F = 384 go through the chain of GEMMs
+    p = CONFIGS["cfg4_hea128k"]["profile"]
+    blob = make_blob(p, seed=3)
+    box = _box(24000, p["T"], a=6.5)
+    assert _held(blob, box) == _held(blob, box, mlp_path=3)
+    # the cubic pieces where per-pair tables are made from them, the value and product tables where they are read themselves
+    p = SMALL_PROFILES["p128_2_0"]
+    blob = make_blob(p, seed=3)
+    box = _box(64, p["T"])
+    rows, pad = 3000, 16
+    cubic, quadratic = 12 * rows * 128 + pad, 8 * rows * 128 + pad
+    tables = 4 * (32 + p["T"] ** 2 * 2 * rows * 2 * 128 + pad)
+    assert _held(blob, box) - _held(blob, box, pair_table_mb=-1) == tables + cubic - 2 * quadratic
