@@ -1052,7 +1052,9 @@ int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int
                     value_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, q);
                     grow(2, q[1]); grow(3, q[2]);
                     if (!products) continue;
-                    product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, s * dx + (sub + 0.5) * w, (double)d.rc, q);
+                    double e[5];
+                    envelope_derivatives(s * dx + (sub + 0.5) * w, (double)d.rc, e);
+                    product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, e, q);
                     grow(4, q[1]); grow(5, q[2]);
                 }
             }
@@ -1092,7 +1094,9 @@ int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int
                 for (int k = 0; k < R; ++k) psi += (double)pm[(size_t)(2 + k) * C0 + c] * stored(m.vtable, C0 + k, step + 2);
             }
             if (products && per_pair) {
-                product_piece(v[0], v[1], v[2], v[3], mid, 0.5 * w, rho_mid, (double)d.rc, q);
+                double e[5];
+                envelope_derivatives(rho_mid, (double)d.rc, e);
+                product_piece(v[0], v[1], v[2], v[3], mid, 0.5 * w, e, q);
                 out = packed(q, step + 4);
             } else if (products) {
                 out = (double)pm[c] * stored(m.dtable, c, step + 4) + (double)pm[C0 + c] * dchi;

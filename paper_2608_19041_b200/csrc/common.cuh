@@ -110,10 +110,11 @@ constexpr int kTabI2Max = (1 << 19) - 1, kTabI3Max = (1 << 11) - 1;
 __host__ __device__ inline float tab_step2(float max_abs_c2) { return max_abs_c2 * (1.0f / (float)kTabI2Max); }
 __host__ __device__ inline float tab_step3(float max_abs_c3) { return max_abs_c3 * (1.0f / (float)kTabI3Max); }
 __host__ __device__ inline unsigned tab_pack(float c2, float c3, float k2, float k3) {
-    float q2 = k2 > 0.f ? c2 / k2 : 0.f, q3 = k3 > 0.f ? c3 / k3 : 0.f;
-    q2 = q2 > (float)kTabI2Max ? (float)kTabI2Max : (q2 < -(float)kTabI2Max ? -(float)kTabI2Max : q2);
-    q3 = q3 > (float)kTabI3Max ? (float)kTabI3Max : (q3 < -(float)kTabI3Max ? -(float)kTabI3Max : q3);
-    const int i2 = (int)(q2 < 0.f ? q2 - 0.5f : q2 + 0.5f), i3 = (int)(q3 < 0.f ? q3 - 0.5f : q3 + 0.5f);
+    // (no branch in it: the host packs rows of channels, several at a time)
+    float q2 = c2 / (k2 > 0.f ? k2 : 1.f), q3 = c3 / (k3 > 0.f ? k3 : 1.f);      // (a step of zero has zeros to pack)
+    q2 = q2 < (float)kTabI2Max ? q2 : (float)kTabI2Max; q2 = q2 > -(float)kTabI2Max ? q2 : -(float)kTabI2Max;
+    q3 = q3 < (float)kTabI3Max ? q3 : (float)kTabI3Max; q3 = q3 > -(float)kTabI3Max ? q3 : -(float)kTabI3Max;
+    const int i2 = (int)(q2 + copysignf(0.5f, q2)), i3 = (int)(q3 + copysignf(0.5f, q3));
     return ((unsigned)i2 << 12) | ((unsigned)i3 & 0xfffu);
 }
 __host__ __device__ inline void tab_unpack(unsigned w, float k2, float k3, float* c2, float* c3) {
@@ -140,20 +141,22 @@ __host__ __device__ inline void value_piece(double c0, double c1, double c2, dou
 // grid of the value table (expanded from the cubic piece and the envelope's derivatives, cubic term folded),
 // two words per channel and one dot product instead of three words and two.  The leading C1 channels, which
 // also carry the degrees >= 1, add their amplitude from the value table: (chi^2 psi)' = chi ((chi psi)' + chi' psi).
-// chi = 1 - I_x(5, 4).
-__host__ __device__ inline void product_piece(double c0, double c1, double c2, double c3, double mid, double h, double rho, double rc,
-                                              double* a) {
+// chi = 1 - I_x(5, 4); e: its value and derivatives of order 1 .. 4 at rho.
+__host__ __device__ inline void envelope_derivatives(double rho, double rc, double* e) {
     const double x = rho / rc, u = 1 - x, r = 1 / rc;
-    const double e0 = u * u * u * u * (1 + x * (4 + x * (10 + x * (20 + 35 * x))));
-    const double e1 = -280 * r * x * x * x * x * u * u * u;
-    const double e2 = -280 * r * r * x * x * x * u * u * (4 * u - 3 * x);
-    const double e3 = -280 * r * r * r * x * x * u * (12 * u * u - 24 * x * u + 6 * x * x);
-    const double e4 = -280 * r * r * r * r * x * (24 * u * u * u - 108 * x * u * u + 72 * x * x * u - 6 * x * x * x);
+    e[0] = u * u * u * u * (1 + x * (4 + x * (10 + x * (20 + 35 * x))));
+    e[1] = -280 * r * x * x * x * x * u * u * u;
+    e[2] = -280 * r * r * x * x * x * u * u * (4 * u - 3 * x);
+    e[3] = -280 * r * r * r * x * x * u * (12 * u * u - 24 * x * u + 6 * x * x);
+    e[4] = -280 * r * r * r * r * x * (24 * u * u * u - 108 * x * u * u + 72 * x * x * u - 6 * x * x * x);
+}
+// e: at the middle of the piece
+__host__ __device__ inline void product_piece(double c0, double c1, double c2, double c3, double mid, double h, const double* e, double* a) {
     const double p0 = ((c3 * mid + c2) * mid + c1) * mid + c0, p1 = (3 * c3 * mid + 2 * c2) * mid + c1, p2 = 6 * c3 * mid + 2 * c2, p3 = 6 * c3;
-    const double d3 = (e4 * p0 + 4 * e3 * p1 + 6 * e2 * p2 + 4 * e1 * p3) / 6;
-    a[0] = e1 * p0 + e0 * p1;
-    a[1] = e2 * p0 + 2 * e1 * p1 + e0 * p2 + 0.75 * h * h * d3;
-    a[2] = 0.5 * (e3 * p0 + 3 * e2 * p1 + 3 * e1 * p2 + e0 * p3);
+    const double d3 = (e[4] * p0 + 4 * e[3] * p1 + 6 * e[2] * p2 + 4 * e[1] * p3) / 6;
+    a[0] = e[1] * p0 + e[0] * p1;
+    a[1] = e[2] * p0 + 2 * e[1] * p1 + e[0] * p2 + 0.75 * h * h * d3;
+    a[2] = 0.5 * (e[3] * p0 + 3 * e[2] * p1 + 3 * e[1] * p2 + e[0] * p3);
     a[3] = d3;
 }
 // The cubic piece of the amplitude psi_c = gamma_c g_c + beta_c + sum_mu U_c,mu q_mu of one species pair in one row of

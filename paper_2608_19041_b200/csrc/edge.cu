@@ -1013,7 +1013,9 @@ __global__ void k_fuse_pair_tables(Dims d, const float* __restrict__ table, cons
                 }
                 if (!wide_channels(d.C0)) continue;
                 double q[4];                                   // envelope products (product_piece)
-                product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, (double)row * d.dx + (sub + 0.5) * w, (double)d.rc, q);
+                double e[5];
+                envelope_derivatives((double)row * d.dx + (sub + 0.5) * w, (double)d.rc, e);
+                product_piece(v[0], v[1], v[2], v[3], (sub + 0.5) * w, 0.5 * w, e, q);
                 mx[4] = fmaxf(mx[4], fabsf((float)q[1])); mx[5] = fmaxf(mx[5], fabsf((float)q[2]));
                 if (WRITE) {
                     float* drow = dout + ((size_t)pr * d.n_vrows + (size_t)row * d.v_sub + sub) * 2 * d.C0;

@@ -264,13 +264,13 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                 j0_derivs(w * rho, &j, &j1);
                 f[n] = w * j; f1[n] = w * w * j1;
             }
-            for (int k = 0; k < 2 * H; ++k) {
-                double s0 = 0, s1 = 0;
-                for (int n = 0; n < N_rbf; ++n) {
-                    const double w = W_in[(size_t)n * 2 * H + k];
-                    s0 += f[n] * w; s1 += f1[n] * w;
-                }
-                a[k] = s0; a1[k] = s1;
+            // (rows of the weights in turn: contiguous, and every sum keeps its order)
+            std::fill(a.begin(), a.end(), 0.0);
+            std::fill(a1.begin(), a1.end(), 0.0);
+            for (int n = 0; n < N_rbf; ++n) {
+                const double* w = &W_in[(size_t)n * 2 * H];
+                const double fn = f[n], fn1 = f1[n];
+                for (int k = 0; k < 2 * H; ++k) { a[k] += fn * w[k]; a1[k] += fn1 * w[k]; }
             }
             for (int k = 0; k < H; ++k) {  // h = SiLU(gate) * value, gate = first H columns
                 const double g = a[k], g1 = a1[k], v = a[H + k], v1 = a1[H + k];
@@ -279,116 +279,124 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                 h[k] = S0 * v;
                 h1[k] = S1 * g1 * v + S0 * v1;
             }
-            double* y = &Y[(size_t)s * 2 * NC];
-            for (int c = 0; c < NC; ++c) {
-                double s0 = 0, s1 = 0;
-                for (int k = 0; k < H; ++k) {
-                    const double w = c < C0 ? W_out[(size_t)k * C0 + c] : W_mode[(size_t)k * R + (c - C0)];
-                    s0 += h[k] * w; s1 += h1[k] * w;
-                }
-                y[c] = s0; y[NC + c] = s1;
+            double* y = &Y[(size_t)s * 2 * NC];       // (zeros)
+            double *y0 = y, *y1 = y + NC;
+            for (int k = 0; k < H; ++k) {
+                const double *w = &W_out[(size_t)k * C0], *wm = R ? &W_mode[(size_t)k * R] : nullptr;
+                const double hk = h[k], hk1 = h1[k];
+                for (int c = 0; c < C0; ++c) { y0[c] += hk * w[c]; y1[c] += hk1 * w[c]; }
+                for (int q = 0; q < R; ++q) { y0[C0 + q] += hk * wm[q]; y1[C0 + q] += hk1 * wm[q]; }
             }
         }
     }
     m->table.assign((size_t)n_rows * 3 * CP, 0.0f);
     {
-        // p(t) = c0 + c1 t + c2 t^2 + c3 t^3, t = rho - rho_s, matching value and slope at both knots;
-        // c2 and c3 are stored packed on the table's own scale (common.cuh, tab_pack)
+        // p(t) = c0 + c1 t + c2 t^2 + c3 t^3, t = rho - rho_s, matching value and slope at both knots; what is packed is kept
+        // packed on the table's own scale (common.cuh, tab_pack).  Coefficients are kept by planes, [row][coefficient][channel],
+        // and the largest magnitudes are taken from the rounded ones.
         const double D1 = m->dx, D2 = D1 * D1, D3 = D2 * D1;
-        std::vector<float> hi((size_t)n_rows * 2 * NC);
+        auto largest = [&](const float* v, float* mx) {
+            int bits, best;                                // (non-negative floats order like their bit patterns)
+            std::memcpy(&best, mx, sizeof(best));
+            for (int c = 0; c < NC; ++c) {
+                std::memcpy(&bits, v + c, sizeof(bits));
+                bits &= 0x7fffffff;
+                best = bits > best ? bits : best;
+            }
+            std::memcpy(mx, &best, sizeof(best));
+        };
+        std::vector<unsigned> words(NC);
+        auto pack_row = [&](const float* hi, const float* lo, float k_hi, float k_lo, float* out) {
+            for (int c = 0; c < NC; ++c) words[c] = tab_pack(hi[c], lo[c], k_hi, k_lo);
+            std::memcpy(out, words.data(), sizeof(unsigned) * (size_t)NC);
+        };
+        std::vector<double> C((size_t)n_rows * 2 * NC);    // c2, c3
+        std::vector<float> cf((size_t)n_rows * 2 * NC);
         float m2 = 0.f, m3 = 0.f;
         for (int s = 0; s < n_rows; ++s) {
-            const double* ya = &Y[(size_t)s * 2 * NC];
-            const double* yb = &Y[(size_t)(s + 1) * 2 * NC];
-            float* row = &m->table[(size_t)s * 3 * CP];
+            const double *ya = &Y[(size_t)s * 2 * NC], *yb = &Y[(size_t)(s + 1) * 2 * NC];
+            double *c2 = &C[(size_t)s * 2 * NC], *c3 = c2 + NC;
+            float *f2 = &cf[(size_t)s * 2 * NC], *f3 = f2 + NC, *row = &m->table[(size_t)s * 3 * CP];
             for (int c = 0; c < NC; ++c) {
-                const double y0 = ya[c], p0 = ya[NC + c], y1 = yb[c], p1 = yb[NC + c];
-                const double del = y1 - y0;
-                row[0 * CP + c] = (float)y0;
-                row[1 * CP + c] = (float)p0;
-                const float c2 = (float)((3 * del - (2 * p0 + p1) * D1) / D2), c3 = (float)((-2 * del + (p0 + p1) * D1) / D3);
-                hi[((size_t)s * NC + c) * 2] = c2; hi[((size_t)s * NC + c) * 2 + 1] = c3;
-                if (std::fabs(c2) > m2) m2 = std::fabs(c2);
-                if (std::fabs(c3) > m3) m3 = std::fabs(c3);
+                const double p0 = ya[NC + c], p1 = yb[NC + c], del = yb[c] - ya[c];
+                const double t2 = 3 * del - (2 * p0 + p1) * D1, t3 = -2 * del + (p0 + p1) * D1;
+                row[c] = (float)ya[c];
+                row[CP + c] = (float)p0;
+                f2[c] = (float)(t2 / D2); f3[c] = (float)(t3 / D3);
+                c2[c] = t2 * (1 / D2); c3[c] = t3 * (1 / D3);
             }
+            largest(f2, &m2); largest(f3, &m3);
         }
+        d.tab_k2 = tab_step2(m2); d.tab_k3 = tab_step3(m3);
+        for (int s = 0; s < n_rows; ++s)
+            pack_row(&cf[(size_t)s * 2 * NC], &cf[(size_t)s * 2 * NC + NC], d.tab_k2, d.tab_k3, &m->table[(size_t)s * 3 * CP + 2 * CP]);
+
         // values alone: quadratic pieces about the middle of (a fraction of) the interval
         d.v_sub = 1;
         while (D1 / d.v_sub > 0.0025) d.v_sub *= 2;
-        std::vector<float> va, da;
-        double m0 = 0, q1 = 0, q2 = 0, q3 = 0, n0 = 0, r1 = 0, r2 = 0, r3 = 0;
         // the product table of the radial map is kept without shared modes only, but with them the per-pair tables hold the
         // same products of gamma g + beta + U q: their bound is checked on the columns of g and q and on a constant
         const bool wide = wide_channels(C0), products = wide && R == 0;
+        std::vector<float> va, da;
+        float v[4], q[4];                                  // largest a0, a1, a2 and cubic term: of the values, of the products
         for (;; d.v_sub *= 2) {
             const double w = D1 / d.v_sub, hw = 0.5 * w;
-            va.assign((size_t)n_rows * d.v_sub * NC * 3, 0.0f);
-            if (products) da.assign(va.size(), 0.0f);
-            m0 = q1 = q2 = q3 = n0 = r1 = r2 = r3 = 0;
-            double k0 = 0, k1 = 0, k2 = 0, k3 = 0;         // of the constant
-            float *o = va.data(), *od = da.data();
+            const size_t rows = (size_t)n_rows * d.v_sub;
+            va.resize(rows * 3 * NC);
+            da.resize((products ? rows : 1) * 3 * NC);
+            std::vector<float> cubic(NC);
+            double k[4] = {0, 0, 0, 0};                    // of the constant
+            for (int i = 0; i < 4; ++i) v[i] = q[i] = 0.f;
             for (int s = 0; s < n_rows; ++s) {
-                const double* ya = &Y[(size_t)s * 2 * NC];
-                const double* yb = &Y[(size_t)(s + 1) * 2 * NC];
-                for (int sub = 0; sub < d.v_sub; ++sub)
-                    for (int c = 0; c < NC; ++c, o += 3) {
-                        const double del = yb[c] - ya[c], p0 = ya[NC + c], p1 = yb[NC + c];
-                        const double c2 = (3 * del - (2 * p0 + p1) * D1) * (1 / D2), c3 = (-2 * del + (p0 + p1) * D1) * (1 / D3);
+                const double *ya = &Y[(size_t)s * 2 * NC], *c2 = &C[(size_t)s * 2 * NC], *c3 = c2 + NC;
+                for (int sub = 0; sub < d.v_sub; ++sub) {
+                    const double mid = (sub + 0.5) * w;
+                    const size_t vrow = (size_t)s * d.v_sub + sub;
+                    float *o = &va[vrow * 3 * NC], *x = cubic.data();
+                    for (int c = 0; c < NC; ++c) {
                         double p[3];
-                        value_piece(ya[c], p0, c2, c3, (sub + 0.5) * w, hw, p);
-                        m0 = std::max(m0, std::fabs(p[0])); q1 = std::max(q1, std::fabs(p[1]));
-                        q2 = std::max(q2, std::fabs(p[2])); q3 = std::max(q3, std::fabs(c3));
-                        o[0] = (float)p[0]; o[1] = (float)p[1]; o[2] = (float)p[2];
-                        if (!wide) continue;
-                        double q[4];
-                        product_piece(ya[c], p0, c2, c3, (sub + 0.5) * w, hw, s * D1 + (sub + 0.5) * w, m->rc, q);
-                        n0 = std::max(n0, std::fabs(q[0])); r1 = std::max(r1, std::fabs(q[1]));
-                        r2 = std::max(r2, std::fabs(q[2])); r3 = std::max(r3, std::fabs(q[3]));
-                        if (!products) continue;
-                        float* t = od + (o - va.data());
-                        t[0] = (float)q[0]; t[1] = (float)q[1]; t[2] = (float)q[2];
+                        value_piece(ya[c], ya[NC + c], c2[c], c3[c], mid, hw, p);
+                        o[c] = (float)p[0]; o[NC + c] = (float)p[1]; o[2 * NC + c] = (float)p[2]; x[c] = (float)c3[c];
                     }
-                for (int sub = 0; wide && sub < d.v_sub; ++sub) {
-                    double q[4];
-                    product_piece(1, 0, 0, 0, (sub + 0.5) * w, hw, s * D1 + (sub + 0.5) * w, m->rc, q);
-                    k0 = std::max(k0, std::fabs(q[0])); k1 = std::max(k1, std::fabs(q[1]));
-                    k2 = std::max(k2, std::fabs(q[2])); k3 = std::max(k3, std::fabs(q[3]));
+                    for (int i = 0; i < 4; ++i) largest(i < 3 ? o + i * NC : x, &v[i]);
+                    if (!wide) continue;
+                    double e[5], p[4];                     // (the envelope is the row's, not the channel's)
+                    envelope_derivatives(s * D1 + mid, m->rc, e);
+                    product_piece(1, 0, 0, 0, mid, hw, e, p);
+                    for (int i = 0; i < 4; ++i) k[i] = std::max(k[i], std::fabs(p[i]));
+                    float* t = &da[(products ? vrow : 0) * 3 * NC];
+                    for (int c = 0; c < NC; ++c) {
+                        product_piece(ya[c], ya[NC + c], c2[c], c3[c], mid, hw, e, p);
+                        t[c] = (float)p[0]; t[NC + c] = (float)p[1]; t[2 * NC + c] = (float)p[2]; x[c] = (float)p[3];
+                    }
+                    for (int i = 0; i < 4; ++i) largest(i < 3 ? t + i * NC : x, &q[i]);
                 }
             }
             auto off = [&](double a1, double a2, double a3) {
                 return a3 * hw * hw * hw / 4 + a1 / (2.0 * kTabI2Max) * hw + a2 / (2.0 * kTabI3Max) * hw * hw;
             };
             // about the rounding of a0; not refined beyond 100000 intervals, met or not
-            if ((off(q1, q2, q3) <= m0 * 0x1p-24 && off(r1, r2, r3) <= n0 * 0x1p-23 && off(k1, k2, k3) <= k0 * 0x1p-23) ||
+            if ((off(v[1], v[2], v[3]) <= v[0] * 0x1p-24 && off(q[1], q[2], q[3]) <= q[0] * 0x1p-23 && off(k[1], k[2], k[3]) <= k[0] * 0x1p-23) ||
                 n_rows * (int64_t)d.v_sub > 100000)
                 break;
         }
         d.n_vrows = n_rows * d.v_sub;
         for (d.v_shift = 0; (1 << d.v_shift) < d.v_sub; ++d.v_shift) {}
-        d.tab_d1 = tab_step2((float)r1); d.tab_d2 = tab_step3((float)r2);
         d.vdx = (float)(D1 / d.v_sub); d.inv_vdx = (float)(d.v_sub / D1);
-        d.tab_v1 = tab_step2((float)q1); d.tab_v2 = tab_step3((float)q2);
-        m->vtable.assign((size_t)d.n_vrows * 2 * CP, 0.0f);
+        d.tab_v1 = tab_step2(v[1]); d.tab_v2 = tab_step3(v[2]);
+        d.tab_d1 = tab_step2(q[1]); d.tab_d2 = tab_step3(q[2]);
         auto pack = [&](const std::vector<float>& pieces, float k1, float k2, std::vector<float>* out) {
-            const float* v = pieces.data();
+            out->assign((size_t)d.n_vrows * 2 * CP, 0.0f);
             for (int s = 0; s < d.n_vrows; ++s) {
+                const float* p = &pieces[(size_t)s * 3 * NC];
                 float* row = &(*out)[(size_t)s * 2 * CP];
-                for (int c = 0; c < NC; ++c, v += 3) {
-                    row[c] = v[0];
-                    const unsigned w = tab_pack(v[1], v[2], k1, k2);
-                    std::memcpy(&row[CP + c], &w, sizeof(w));
-                }
+                std::memcpy(row, p, sizeof(float) * (size_t)NC);
+                pack_row(p + NC, p + 2 * NC, k1, k2, row + CP);
             }
         };
         pack(va, d.tab_v1, d.tab_v2, &m->vtable);
-        m->dtable.assign(products ? m->vtable.size() : 0, 0.0f);
+        m->dtable.clear();
         if (products) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
-        d.tab_k2 = tab_step2(m2); d.tab_k3 = tab_step3(m3);
-        for (int s = 0; s < n_rows; ++s)
-            for (int c = 0; c < NC; ++c) {
-                const unsigned w = tab_pack(hi[((size_t)s * NC + c) * 2], hi[((size_t)s * NC + c) * 2 + 1], d.tab_k2, d.tab_k3);
-                std::memcpy(&m->table[(size_t)s * 3 * CP + 2 * CP + c], &w, sizeof(w));
-            }
     }
 
     // ---- ordered type-pair cache -----------------------------------------------------
