@@ -63,10 +63,9 @@ typedef struct umlmd_options {
                             pair) for every GEMM; path 2 takes the whole MLP in one kernel per block of atoms where
                             that is faster (small systems, narrow models), and otherwise the kernel of path 4 for
                             the last GEMM of the backward pass; 2, 3 and 4 need F % 8 == 0 and fall back to 1 otherwise */
-    int32_t  pair_table_mb;  /* device memory, MiB, that per-pair amplitude tables may take, counted as table_rows x
-                                3 x C0 words per pair (what is kept is 4/3 of that from C0 = 32 on, else 5/3; more at
-                                table spacings above 0.0025 Angstrom)
-                                (see umlmd_build_neighbors); 0 = 192, negative = never build them */
+    int32_t  pair_table_mb;  /* most device memory, MiB, that per-pair amplitude tables may take (see
+                                umlmd_build_neighbors); negative = never build them, 0 = the default: tables are built while
+                                species pairs x table_rows x 3 x C0 words fit in 192 MiB, and take at most 320 */
     int32_t  gemm_spin_limit;       /* polls after which a wait inside the tensor-core GEMM's operand
                                        pipeline gives up (the kernel then finishes with garbage, and the
                                        call returns UMLMD_E_CUDA "pipeline wait expired"); 0 = 4,000,000 */
@@ -140,7 +139,7 @@ const char* umlmd_last_error(const umlmd_t* h);
  * is allocated (library plumbing, no counterpart in the paper; the paper's memory-scaling note is
  * the model: a fixed tile workspace plus terms linear in atoms and in edges).  An upper estimate
  * within a few per cent; per-pair amplitude tables, when the species present are few enough for
- * them, add at most 5/3 of umlmd_options.pair_table_mb on top at table spacings up to 0.0025 Angstrom.
+ * them, add at most umlmd_options.pair_table_mb on top (320 MiB where that is 0).
  */
 int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t* bytes);
 
@@ -166,7 +165,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
  * reproducible bit for bit.  Atoms are renumbered internally in cell order; all outputs
  * of this library are in the caller's numbering.
  * The call also finds which species occur.  When the P species present are few enough that
- * P^2 tables of table_rows x 3 x C0 words fit in umlmd_options.pair_table_mb, the edge
+ * the tables of their P^2 ordered pairs fit in umlmd_options.pair_table_mb, the edge
  * amplitude of every ordered pair (s, s') among them, psi_c(rho) = gamma_c g_c(rho) + beta_c +
  * sum_mu U_c,mu q_mu(rho), is tabulated by itself (the same linear
  * combination of the coefficient rows of the radial table; pieces for values and for

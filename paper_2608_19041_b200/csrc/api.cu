@@ -40,7 +40,7 @@ struct umlmd {
     void* pinned = nullptr;                             // one allocation for h_out, h_frame, h_err, h_species and the list's h_totals
     double* h_out = nullptr; int* h_err = nullptr;
     // per-pair amplitude tables of the species present (set up by umlmd_build_neighbors)
-    int64_t pair_table_budget = 192ll << 20;            // bytes; negative = never build them
+    int64_t pair_table_budget = 0;                      // bytes; 0 = the default rule, negative = never build them
     bool pair_tables = false;                           // in use for the current system
     std::vector<int> present;                           // species the tables were built for, ascending
     float* uni = nullptr; int64_t uni_cap = 0;              // one allocation for the four below
@@ -447,6 +447,8 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     return UMLMD_OK;
 }
 
+constexpr int64_t kPairTablesFull = 192ll << 20, kPairTablesMost = 320ll << 20;
+
 // With few species present, psi_c(rho) of every ordered pair among them is tabulated by itself,
 // so that the edge kernels read one table row per edge and neither pair rows nor shared modes.
 // The tables depend on the model and the set of species only, so they are kept across builds.
@@ -455,19 +457,21 @@ int setup_pair_tables(umlmd_t* h) {
     std::vector<int> present;
     for (int t = 0; t < d.T; ++t) if (h->h_species[t]) present.push_back(t);
     const size_t np = present.size();
-    // the rule counts tables with derivatives; what is kept is 4/3 (products) or 5/3 of that at the usual spacings
-    const size_t full = np * np * (size_t)d.n_rows * 3 * d.C0 * sizeof(float);
+    // By default the rule counts tables of three words per channel, of which 4/3 (values and products, from C0 = 32 on) or 5/3
+    // (cubic pieces and values) is kept at the usual spacings; a limit that the caller has set bounds what is kept.
     const bool wide = wide_channels(d.C0);
+    const int64_t full = (int64_t)(np * np) * d.n_rows * 3 * d.C0 * (int64_t)sizeof(float);
     const size_t vfloats = np * np * (size_t)d.n_vrows * 2 * d.C0, dfloats = wide ? vfloats : 0;
     const size_t floats = wide ? 0 : np * np * (size_t)d.n_rows * 3 * d.C0;
-    const bool use = np > 0 && h->pair_table_budget >= 0 && full <= (size_t)h->pair_table_budget &&
-                     3 * (floats + vfloats + dfloats) * sizeof(float) <= 5 * (size_t)h->pair_table_budget;
+    constexpr size_t head = 32;                       // floats for the scales; the tables behind start on 128 bytes
+    const int64_t kept = (int64_t)((head + floats + vfloats + dfloats + 16) * sizeof(float));       // (as dev_ensure pads it)
+    const bool fits = h->pair_table_budget > 0 ? kept <= h->pair_table_budget : full <= kPairTablesFull && kept <= kPairTablesMost;
+    const bool use = np > 0 && h->pair_table_budget >= 0 && fits;
     h->pair_tables = use && present == h->present;
     if (h->pair_tables) return UMLMD_OK;
     const int rc = ensure_radial_tables(h, use);
     if (rc != UMLMD_OK || !use) return rc;
     h->present.clear();                               // no tables until all of them are made
-    constexpr size_t head = 32;                       // floats; the tables behind start on 128 bytes
     API_CUDA(h, dev_ensure(&h->uni, &h->uni_cap, (int64_t)(head + floats + vfloats + dfloats)));
     h->uni_scale = h->uni;
     h->table_uni = h->uni + head;

@@ -155,3 +155,15 @@ def test_the_first_build_allocates_what_the_system_uses():
     cubic, quadratic = 12 * rows * 128 + pad, 8 * rows * 128 + pad
     tables = 4 * (32 + p["T"] ** 2 * 2 * rows * 2 * 128 + pad)
     assert _held(blob, box) - _held(blob, box, pair_table_mb=-1) == tables + cubic - 2 * quadratic
+
+
+def test_a_limit_on_pair_tables_bounds_their_memory():
+    # three species at C0 = 128: nine pairs of 5.9 MiB, 52.8 in all (39.6 if only the cubic pieces are counted)
+    p = SMALL_PROFILES["p128_2_0"]
+    blob = make_blob(p, seed=3)
+    box = _box(64, p["T"])
+    without = _held(blob, box, pair_table_mb=-1)
+    for limit, built in ((1, False), (45, False), (52, False), (53, True), (400, True), (0, True)):
+        held = _held(blob, box, pair_table_mb=limit) - without
+        assert (held > 0) == built, limit
+        assert held <= (limit or 320) << 20, limit
