@@ -42,7 +42,7 @@ struct Dims {
     int CP;                  // table channels C0+R rounded up to 4
     int n_rows;              // table intervals
     float tab_k2, tab_k3;    // steps of the packed quadratic and cubic coefficients of the radial table
-    int v_sub, v_shift, n_vrows;   // value table (below): intervals per table interval (2^v_shift), and in all
+    int v_sub, n_vrows;      // value table (below): intervals per table interval (a power of two), and in all
     float vdx, inv_vdx;      // its spacing
     float tab_v1, tab_v2;    // steps of its packed linear and quadratic coefficients
     float tab_d1, tab_d2;    // the same for the product table
@@ -176,7 +176,9 @@ __host__ __device__ inline void pair_cubic(const Dims& d, const float* row, cons
 }
 // Models of at least 32 channels without shared modes, or with per-pair tables (which hold the modes), use the
 // product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the channels are leading
-// ones, and with modes their derivatives are needed anyway: there the table with derivatives is less to read.
+// ones, which need both: there the table with derivatives is less to read.  With shared modes and the pair cache the
+// backward pass still forms psi and psi' from the table with derivatives; products with modes, which would take the
+// modes' own products per edge, have not been tried.
 __host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }
 
 // One frame of a batched evaluation (umlmd_compute_batch): its own cell and its slice of the

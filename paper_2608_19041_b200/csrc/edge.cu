@@ -10,9 +10,11 @@
 // loads that a group issues as contiguous segments -- followed by a lane-per-edge phase for
 // the degree >= 1 blocks.  The S+2 sums live in registers and are written once per
 // destination; nothing per-edge is stored in the forward pass.  The backward pass recomputes
-// the same per-edge quantities from the same cubic polynomial (so the force is the exact
-// derivative of the interpolated energy), contracts them with dE/d(sums) and writes one
-// 3-vector per edge; the virial is accumulated in the same pass.
+// the per-edge quantities, contracts them with dE/d(sums) and writes one 3-vector per edge; the
+// virial is accumulated in the same pass.  The two passes read different tables of one cubic
+// interpolant (the forward pass quadratic pieces of its values, the backward pass its own pieces with
+// derivatives or, from C0 = 32 on, quadratic pieces of the derivative of envelope times
+// amplitude): energy and force agree to the tables' rounding (common.cuh, value_piece), not exactly.
 //
 // Harmonics are evaluated with |u|^2 set to one; the regularised direction differs from a
 // unit vector by eps^2/rho^2, far below single precision.

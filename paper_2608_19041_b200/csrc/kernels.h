@@ -87,11 +87,14 @@ cudaError_t launch_fuse_pair_tables(const Dims& d, const float* table, const flo
 cudaError_t launch_edge_forward(const EdgeArgs& a, cudaStream_t st);
 cudaError_t launch_edge_backward(const EdgeArgs& a, int* n_blocks, cudaStream_t st);
 // Few rows: the four warps of a block share a row, a quarter of its edges each.  A warp works through a row as a
-// serial chain of table reads, which a chip with fewer than eight warps per scheduler does not hide: up to 1184 rows
-// (four warps each and every warp resident) the two edge kernels together took, a warp per row against shared, at
+// serial chain of table reads, which a chip with few warps per scheduler does not hide.  One line for both kernels and all
+// widths, drawn where the two together were measured: 1184 rows are the 32 warps per SM of the forward kernel up to C0 = 64
+// (at C0 = 128 it holds 24, the backward kernel 16 to 24, so that rows then come in more than one wave).  The two kernels
+// together took, a warp per row against shared, at
 // 108 / 592 / 1184 rows: C0 = 32 28 / 29 / 29 against 21 / 21 / 27 us, C0 = 64 with degree three 44 / 44 / 46 against
 // 26 / 27 / 37, C0 = 128 with 64 species 49 / 52 / 58 against 24 / 32 / 52, with four modes 173 / 191 / 208 against
-// 62 / 78 / 137; at 1776 rows sharing loses (C0 = 32: 31 against 35, C0 = 128: 63 against 63).
+// 62 / 78 / 137; at 1776 rows sharing loses or gains nothing (C0 = 32: 31 against 35, C0 = 128: 63 against 63; with modes not
+// measured there).
 inline bool edge_rows_split(int64_t rows) { return rows <= kEdgeSplitRows; }
 inline int edge_blocks(int rows) { return edge_rows_split(rows) ? rows : (rows + kEdgeRowsPerBlock - 1) / kEdgeRowsPerBlock; }
 // most blocks (partial virials) that the tiles of up to N rows, B at a time, have

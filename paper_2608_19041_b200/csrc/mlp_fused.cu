@@ -459,6 +459,7 @@ int pick_atoms(const Dims& d, int n) {
 //   23600    62 / 42  108 /  56    109 / 68  171 /  92    126 / 72  188 /  96     87 / 52  118 / 66    220 / 122   246 / 111
 //   47000   111 / 70  157 /  86    199 /121  254 / 123    226 /129  280 / 131    152 / 93  166 / 86    427 / 235   414 / 189
 //  150000   299 /183  340 / 161    551 /334  637 / 306    625 /358  681 / 321    416 /255  387 /199   1345 / 729  1142 / 505
+// (F = 96, forward alone: the line lies below 47,000 atoms, where this kernel is still the faster one; drawn by turns, not by width.)
 bool mlp_fused_pick(const Dims& d, int path, int64_t n, bool grad) {
     const bool applies = path == 2 && d.D_out != d.F && (d.F & 7) == 0 && d.F <= MAX_F && d.n_hidden <= kMaxLayers && a_blocks_of(d) <= MAX_KB &&
                          gemm_tc_available();

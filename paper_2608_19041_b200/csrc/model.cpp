@@ -8,8 +8,9 @@
 //    kernels are bound by exactly that traffic, so the table keeps four coefficients: at the
 //    paper's spacing of 0.002 A the cubic's error, dx^4 |g^(4)| / 384 in the value and about
 //    dx^3 |g^(4)| / 72 in the derivative, is below single-precision rounding of the
-//    amplitude, and the interpolant stays continuously differentiable, so the force is
-//    still the exact derivative of a continuous energy;
+//    amplitude, and the interpolant is continuously differentiable.  The quadratic pieces of values and
+//    of envelope products that the edge kernels read are expanded from it and follow it within the rounding
+//    of single precision: neighbouring pieces join, and the force is the derivative of the energy, to that rounding;
 //  * ordered type-pair cache: scale gamma, shift beta and mode mixing U of the pair
 //    modulation network for all T*T ordered species pairs;
 //  * Gaunt couplings of the generic degree triples, by exact quadrature on the sphere,
@@ -381,7 +382,6 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                 break;
         }
         d.n_vrows = n_rows * d.v_sub;
-        for (d.v_shift = 0; (1 << d.v_shift) < d.v_sub; ++d.v_shift) {}
         d.vdx = (float)(D1 / d.v_sub); d.inv_vdx = (float)(d.v_sub / D1);
         d.tab_v1 = tab_step2(v[1]); d.tab_v2 = tab_step3(v[2]);
         d.tab_d1 = tab_step2(q[1]); d.tab_d2 = tab_step3(q[2]);
