@@ -203,30 +203,34 @@ int decode_device_errors(umlmd_t* h, int word) {
     return UMLMD_OK;
 }
 
+// what the records of the edge kernels hold in place of the species, null for the species itself
+const int* record_slots(const umlmd_t* h) { return h->pair_tables ? h->d_species + h->d.T : nullptr; }
+
 // enqueue one full evaluation; results stay on the device (d_out[0] energy, d_out[1..9] virial)
-// (to_host: results and error word also go to h_out and h_err, and the word is cleared)
-int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_force, double* d_atom_energy, bool to_host = false) {
+// (to_host: results and error word also go to h_out and h_err, and the word is cleared; tail: an MD step, whose rest comes
+// in the launch that assembles the forces, and whose positions have been gathered)
+int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_force, double* d_atom_energy, bool to_host = false,
+                    const StepTail* tail = nullptr) {
     const Dims& d = h->d;
     NeighborDev& nb = h->nb;
     const int N = (int)nb.N;
     const int NR = (int)nb.n_owned;      // rows that are evaluated: the owned atoms, first in the internal order
     // (a batched list was built from these very positions: nothing to gather)
-    if (!nb.batch) { Scope sc(h, kGather, 1); API_CUDA(h, launch_gather_positions(nb, d_pos, h->d_err, h->st)); }
+    if (!nb.batch && !tail) { Scope sc(h, kGather, 1); API_CUDA(h, launch_gather_positions(nb, d_pos, record_slots(h), h->d_err, h->st)); }
     const int B = N < h->node_tile ? N : h->node_tile;
     int vpart_used = 0;
     for (int a0 = 0; a0 < NR; a0 += B) {
         const int n = NR - a0 < B ? NR - a0 : B;
         EdgeArgs ea;
-        ea.d = d; ea.table = h->md.table; ea.pairmod = h->md.pairmod; ea.xs = nb.xs; ea.rec = nb.rec; ea.type_s = nb.type_s;
+        ea.d = d; ea.table = h->md.table; ea.pairmod = h->md.pairmod; ea.fix = nb.fix; ea.quantum = (float)nb.quantum;
         ea.uni = h->pair_tables; ea.table_uni = h->table_uni;
         ea.vtable = h->md.vtable; ea.vtable_uni = h->vtable_uni;
         ea.dtable = h->md.dtable; ea.dtable_uni = h->dtable_uni;
         ea.uni_scale = h->uni_scale;
-        ea.species_slot = h->d_species + d.T; ea.n_present = (int)h->present.size();
+        ea.species_slot = nb.batch ? h->d_species + d.T : nullptr; ea.n_present = (int)h->present.size();
         ea.frames = nb.batch ? nb.frames : nullptr; ea.frame_of = nb.frame_of;
         ea.row_ptr = nb.row_ptr; ea.nbr = nb.nbr;
-        ea.Lx = nb.L[0]; ea.Ly = nb.L[1]; ea.Lz = nb.L[2];
-        for (int k = 0; k < 9; ++k) ea.H[k] = nb.H[k];
+        for (int k = 0; k < 9; ++k) ea.Hq[k] = to_quanta(nb.H[k], 1.0 / nb.quantum);
         ea.tri = nb.tri;
         ea.a0 = a0; ea.a1 = a0 + n; ea.state = h->state; ea.g = h->g;
         ea.virial_part = h->virial_part + (size_t)vpart_used * 9;
@@ -260,17 +264,26 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         }
     }
     h->have_edge_grad = want_grad;
-    if (want_grad) {
-        Scope sc(h, kForce, 1);
-        API_CUDA(h, launch_force_assembly(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, h->d_err, h->st));
-    }
     if (nb.batch) {                   // frames are reduced one by one
+        if (want_grad) {
+            Scope sc(h, kForce, 1);
+            API_CUDA(h, launch_force_assembly(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, h->d_err, h->st));
+        }
         if (d_atom_energy) { Scope sc(h, kReduce, 1); API_CUDA(h, launch_scatter_atom_energy(nb, h->e_atom, d_atom_energy, h->st)); }
         return UMLMD_OK;
     }
-    Scope sc(h, kReduce, 1);
-    API_CUDA(h, launch_reduce_energy_virial(nb, h->e_atom, d_atom_energy, h->virial_part, vpart_used, h->scratch, (unsigned*)h->d_err + 1,
-                                            h->d_out, h->d_err, to_host ? h->h_out : nullptr, to_host ? h->h_err : nullptr, h->st));
+    double* const ho = to_host ? h->h_out : nullptr;
+    int* const he = to_host ? h->h_err : nullptr;
+    unsigned* const counter = (unsigned*)h->d_err + 1;
+    if (want_grad) {
+        Scope sc(h, kForce, assemble_launches(N));
+        API_CUDA(h, launch_assemble(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, tail ? *tail : StepTail{}, h->e_atom, d_atom_energy,
+                                    h->virial_part, vpart_used, h->scratch, counter, h->d_out, h->d_err, ho, he, h->st));
+    } else {
+        Scope sc(h, kReduce, 1);
+        API_CUDA(h, launch_reduce_energy_virial(nb, h->e_atom, d_atom_energy, h->virial_part, vpart_used, h->scratch, counter, h->d_out,
+                                                h->d_err, ho, he, h->st));
+    }
     return UMLMD_OK;
 }
 
@@ -805,7 +818,7 @@ static int maybe_rebuild(umlmd_t* h, int rebuild_every) {
     if (rebuild_every < 0) {
         // displacement-triggered: the gather pass flags any atom that has moved more than half
         // the skin since the build; read the flag (one host synchronisation per step)
-        API_CUDA(h, launch_gather_positions(h->nb, h->md_pos, h->d_err, h->st));
+        API_CUDA(h, launch_gather_positions(h->nb, h->md_pos, record_slots(h), h->d_err, h->st));
         API_CUDA(h, cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
         API_CUDA(h, cudaStreamSynchronize(h->st));
         const int word = *h->h_err;
@@ -859,23 +872,25 @@ int umlmd_step(umlmd_t* h, int nsteps, double dt_ps, int rebuild_every, double* 
         if ((rc = enqueue_compute(h, h->md_pos, true, h->md_force, nullptr)) != UMLMD_OK) return rc;
         h->have_force = true;
     }
+    bool gathered = false;           // the records of the positions to evaluate are there
     for (int s = 0; s < nsteps; ++s) {
-        // opening half kick and drift; from the second step on they were fused with the previous
-        // step's closing half kick
+        // opening half kick and drift; from the second step on they come with the forces of the step before
         if (s == 0) { Scope sc(h, kIntegrate, 1); API_CUDA(h, launch_vv_kick_drift(N, h->md_pos, h->md_vel, h->md_force, h->type_o, h->d_inv_mass, dt_ps, 1, true, nullptr, h->st)); }
         ++h->steps_since_build;
+        const int64_t serial = h->list_serial;
         if ((rc = maybe_rebuild(h, rebuild_every)) != UMLMD_OK) return stop_run(h, rc);
+        if (h->list_serial != serial) gathered = false;
+        else if (rebuild_every < 0) gathered = true;         // (by the test for displacements)
+        if (!gathered) { Scope sc(h, kGather, 1); API_CUDA(h, launch_gather_positions(h->nb, h->md_pos, record_slots(h), h->d_err, h->st)); }
         const bool last = s + 1 == nsteps;
         auto body = [&]() {
-            int r = enqueue_compute(h, h->md_pos, true, h->md_force, nullptr);
-            if (r != UMLMD_OK) return r;
-            Scope sc(h, kIntegrate, 1);
-            API_CUDA(h, launch_vv_kick_drift(N, h->md_pos, h->md_vel, h->md_force, h->type_o, h->d_inv_mass, dt_ps, last ? 1 : 2, !last, nullptr, h->st));
-            return (int)UMLMD_OK;
+            StepTail t = {h->md_pos, h->md_vel, h->d_inv_mass, dt_ps, last ? 1 : 2, !last, gather_args(h->nb, record_slots(h))};
+            return enqueue_compute(h, h->md_pos, true, h->md_force, nullptr, false, &t);
         };
         // a middle step between two list builds launches the same sequence as the one before it
         rc = last ? body() : run_replayed(h, h->rp_step, h->md_pos, h->md_vel, h->md_force, nullptr, dt_ps, 0, body);
         if (rc != UMLMD_OK) return stop_run(h, rc);
+        gathered = !last;
     }
     { Scope sc(h, kIntegrate, 2); API_CUDA(h, launch_kinetic_energy(N, h->md_vel, h->type_o, h->d_mass, h->scratch, h->d_out + 10, h->st)); }
     rc = fetch_results(h, 11);

@@ -16,15 +16,48 @@ constexpr int kRedMaxBlocks = 1024;
 constexpr int kReduceBlocks = 296;        // two per SM
 static_assert(kReduceBlocks * 10 >= kRedMaxBlocks, "one scratch area serves both kinds of reduction");
 
-// out (caller numbering, through perm) and / or f (sorted numbering) may be null
-__global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
-                             const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
-                             double* __restrict__ out, int* __restrict__ err) {
-    chain_begin();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= N) return;
-    const eidx_t e0 = row_ptr[warp];
-    const int len = (int)(row_ptr[warp + 1] - e0);
+// kicks = 0: none; 1: v += (dt/2) a; 2: the closing half kick of one step and the opening half kick of the next, one
+// after the other exactly as two launches would
+__device__ __forceinline__ double vv_kicks(double v, double c, double f, int kicks) {
+    if (kicks >= 1) v = v + c * f;
+    if (kicks == 2) v = v + c * f;
+    return v;
+}
+
+// Current position of sorted atom i, given that of its caller's atom: minus the image offset found at the build, in double
+// (a.xs) and as the edge kernels' record (a.fix); false for a position that is not finite.
+__device__ __forceinline__ bool gather_position(const GatherArgs& a, int i, double x0, double x1, double x2) {
+    const double pos[3] = {x0, x1, x2};
+    const double n0 = (double)a.img[3 * (size_t)i], n1 = (double)a.img[3 * (size_t)i + 1], n2 = (double)a.img[3 * (size_t)i + 2];
+    const double n[3] = {n0, n1, n2};
+    bool finite = true;
+    int fx[3];
+    for (int k = 0; k < 3; ++k) {
+        const double x = a.tri ? pos[k] - ((n0 * a.h[k] + n1 * a.h[3 + k]) + n2 * a.h[6 + k]) : pos[k] - n[k] * a.h[4 * k];
+        if (!isfinite(x)) finite = false;
+        a.xs[3 * (size_t)i + k] = x;
+        fx[k] = to_quanta(x, a.inv_q);
+    }
+    const int t = a.type_s[i];
+    a.fix[i] = make_int4(fx[0], fx[1], fx[2], a.species_slot ? a.species_slot[t] : t);
+    return finite;
+}
+// whether sorted atom i has moved more than half the skin since the build
+__device__ __forceinline__ bool moved_too_far(const GatherArgs& a, int i) {
+    double d2 = 0;
+    for (int k = 0; k < 3; ++k) {
+        const double d = a.xs[3 * (size_t)i + k] - a.xs0[3 * (size_t)i + k];
+        d2 += d * d;
+    }
+    return d2 > a.max_disp2;
+}
+
+// Force on the atom of one row, by a whole warp: every lane ends with all three components.
+__device__ __forceinline__ void force_of_row(int row, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
+                                             const float* __restrict__ g, double* f) {
+    const int lane = threadIdx.x & 31;
+    const eidx_t e0 = row_ptr[row];
+    const int len = (int)(row_ptr[row + 1] - e0);
     double fx = 0, fy = 0, fz = 0;
     for (int k = lane; k < len; k += 32) {
         const eidx_t e = e0 + k;
@@ -42,12 +75,24 @@ __global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const ei
         fy += __shfl_xor_sync(0xffffffffu, fy, off);
         fz += __shfl_xor_sync(0xffffffffu, fz, off);
     }
+    f[0] = fx; f[1] = fy; f[2] = fz;
+}
+
+// out (caller numbering, through perm) and / or f (sorted numbering) may be null
+__global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
+                             const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
+                             double* __restrict__ out, int* __restrict__ err) {
+    chain_begin();
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (warp >= N) return;
+    double v[3];
+    force_of_row(warp, row_ptr, rev, g, v);
     if (lane == 0) {
-        if (f) { f[3 * (size_t)warp] = fx; f[3 * (size_t)warp + 1] = fy; f[3 * (size_t)warp + 2] = fz; }
+        if (f) { f[3 * (size_t)warp] = v[0]; f[3 * (size_t)warp + 1] = v[1]; f[3 * (size_t)warp + 2] = v[2]; }
         if (out) {
             const size_t o = 3 * (size_t)perm[warp];
-            out[o] = fx; out[o + 1] = fy; out[o + 2] = fz;
-            if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(err, kErrNonFinite);
+            out[o] = v[0]; out[o + 1] = v[1]; out[o + 2] = v[2];
+            if (!isfinite(v[0]) || !isfinite(v[1]) || !isfinite(v[2])) atomicOr(err, kErrNonFinite);
         }
     }
 }
@@ -210,60 +255,129 @@ __global__ void __launch_bounds__(kFrameBlock) k_frame_reduce(const FrameCell* _
 
 // Energy and virial of an evaluation: out[0] = sum of the atomic energies, out[1 + k] = -sum of the k-th
 // component of the virial partials; e_out (may be null) receives the atomic energies in the caller's
-// numbering on the way.  Each block sums a strided share of both arrays; the last block to finish adds up
-// the blocks' sums in their order, so the result does not depend on which one it is.  h_out / h_err
+// numbering on the way.  Each of n_blocks blocks sums a strided share of both arrays; the last block of the grid
+// to finish adds up their sums in order, so the result does not depend on which one it is.  h_out / h_err
 // (pinned host memory, may be null) get the results and the error word, which is then cleared: a caller
 // that waits for this call needs no copies.
-// Bound by latency (128,000 atoms, 32,000 partials of 72 bytes: 9.6 us; 108 atoms: 8.3 us.  One block per
-// component behind a pass over the energies took 28 and 11 us, and a copy of the energies 2.5 more).
-__global__ void __launch_bounds__(kRedBlock) k_reduce(const double* __restrict__ e_atom, int N, const int* __restrict__ perm,
-                                                      double* __restrict__ e_out, const double* __restrict__ vpart, int n_vpart,
-                                                      double* __restrict__ part, unsigned* __restrict__ done, double* __restrict__ out,
-                                                      int* __restrict__ err, double* __restrict__ h_out, int* __restrict__ h_err) {
-    __shared__ double sh[kRedBlock / 32 * 10];
-    __shared__ bool last;
-    chain_begin();
+struct ReduceArgs {
+    const double* e_atom; int N; const int* perm; double* e_out;
+    const double* vpart; int n_vpart;
+    double* part; unsigned* done; double* out; int* err; double* h_out; int* h_err;
+    int n_blocks;
+};
+__device__ __forceinline__ void reduce_share(const ReduceArgs& a, int block, double* sh) {
     double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    const int first = blockIdx.x * kRedBlock + threadIdx.x, step = gridDim.x * kRedBlock;
-    for (int i = first; i < N; i += step) {
-        const double e = e_atom[i];
+    const int first = block * kRedBlock + threadIdx.x, step = a.n_blocks * kRedBlock;
+    for (int i = first; i < a.N; i += step) {
+        const double e = a.e_atom[i];
         v[0] += e;
-        if (e_out) e_out[perm[i]] = e;
+        if (a.e_out) a.e_out[a.perm[i]] = e;
     }
-    for (int i = first; i < n_vpart; i += step) {
+    for (int i = first; i < a.n_vpart; i += step) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) v[1 + k] += vpart[(size_t)i * 9 + k];
+        for (int k = 0; k < 9; ++k) v[1 + k] += a.vpart[(size_t)i * 9 + k];
     }
     const double s = block_sums<10>(v, sh);
-    if (threadIdx.x < 10) part[(size_t)blockIdx.x * 10 + threadIdx.x] = s;
+    if (threadIdx.x < 10) a.part[(size_t)block * 10 + threadIdx.x] = s;
+}
+__device__ __forceinline__ void reduce_finish(const ReduceArgs& a, double* sh, bool* last) {
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) *last = atomicAdd(a.done, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!last) return;
+    if (!*last) return;
     __threadfence();
+    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int i = threadIdx.x; i < a.n_blocks; i += kRedBlock) {
 #pragma unroll
-    for (int k = 0; k < 10; ++k) v[k] = 0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedBlock) {
-#pragma unroll
-        for (int k = 0; k < 10; ++k) v[k] += __ldcg(part + (size_t)i * 10 + k);
+        for (int k = 0; k < 10; ++k) v[k] += __ldcg(a.part + (size_t)i * 10 + k);
     }
     const double t = block_sums<10>(v, sh);
-    if (threadIdx.x == 0 && !isfinite(t)) atomicOr(err, kErrNonFinite);
+    if (threadIdx.x == 0 && !isfinite(t)) atomicOr(a.err, kErrNonFinite);
     if (threadIdx.x < 10) {
         const double r = threadIdx.x ? -t : t;
-        out[threadIdx.x] = r;
-        if (h_out) h_out[threadIdx.x] = r;
+        a.out[threadIdx.x] = r;
+        if (a.h_out) a.h_out[threadIdx.x] = r;
     }
     if (threadIdx.x == 0) {
-        *done = 0;
-        if (h_err) *h_err = atomicExch(err, 0);
+        *a.done = 0;
+        if (a.h_err) *a.h_err = atomicExch(a.err, 0);
     }
 }
 
-// kicks = 0: none; kicks = 1: v += (dt/2) a; kicks = 2: the closing half kick of one step and the
-// opening half kick of the next, applied one after the other exactly as two launches would; drift:
-// x += dt v after them; scale (may be null): the thermostat's velocity factor, applied first
+// Energies alone, and larger systems.  Bound by latency (128,000 atoms, 32,000 partials of 72 bytes: 9.6 us; 108 atoms: 8.3 us.  One block per
+// component behind a pass over the energies took 28 and 11 us, and a copy of the energies 2.5 more).
+__global__ void __launch_bounds__(kRedBlock) k_reduce(const ReduceArgs a) {
+    __shared__ double sh[kRedBlock / 32 * 10];
+    __shared__ bool last;
+    chain_begin();
+    reduce_share(a, blockIdx.x, sh);
+    reduce_finish(a, sh, &last);
+}
+
+// The forces of eight rows per block; REDUCE: the first n_blocks blocks of the grid reduce energy and virial instead.  In an
+// MD run (t.pos given) the row's warp goes on with what is local to its atom: the kicks and the drift of velocity Verlet, with
+// the arithmetic of k_vv, and after a drift the records of the next evaluation, with that of the gather.  As launches of
+// their own the reduction took 8 us, kick and drift 4.4 and the gather 3.6 of the 135 us that a step of 4000 atoms took.
+// REDUCE up to kReduceTogether atoms: it costs every block a fence and an atomic, which from there on is more than a launch
+// (40,009 atoms 45.5 us together, 31 + 14 apart; 64,000 of dense carbon 145, 116 + 14).
+constexpr int kReduceTogether = 32768;
+template <bool REDUCE>
+__global__ void __launch_bounds__(kRedBlock) k_assemble(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
+                                                        const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
+                                                        double* __restrict__ out, int* __restrict__ err, const ReduceArgs a, const StepTail t) {
+    __shared__ double sh[kRedBlock / 32 * 10];
+    __shared__ bool last;
+    chain_begin();
+    if (REDUCE && (int)blockIdx.x < a.n_blocks) {
+        reduce_share(a, blockIdx.x, sh);
+    } else {
+        const int row = (int)(blockIdx.x - (REDUCE ? a.n_blocks : 0)) * (kRedBlock / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (row < N) {
+            double v[3];
+            force_of_row(row, row_ptr, rev, g, v);
+            const int o = perm[row];
+            const double mine = lane == 0 ? v[0] : (lane == 1 ? v[1] : v[2]);
+            if (lane < 3) {
+                if (f) f[3 * (size_t)row + lane] = mine;
+                if (out) {
+                    out[3 * (size_t)o + lane] = mine;
+                    if (!isfinite(mine)) atomicOr(err, kErrNonFinite);
+                }
+            }
+            if (t.pos) {
+                // (of the positions that this step has evaluated: the next ones may be binned anew first)
+                if (lane == 0 && moved_too_far(t.gather, row)) atomicOr(err, kErrStale);
+                const int type = t.gather.type_s[row];
+                double x = 0;
+                if (lane < 3) {
+                    const size_t at = 3 * (size_t)o + lane;
+                    x = t.pos[at];
+                    double u = t.vel[at];
+                    u = vv_kicks(u, 0.5 * t.dt * kAccelUnit * t.inv_mass[type], mine, t.kicks);
+                    t.vel[at] = u;
+                    if (t.drift) { x += t.dt * u; t.pos[at] = x; }
+                }
+                if (t.drift) {
+                    const double x0 = __shfl_sync(0xffffffffu, x, 0), x1 = __shfl_sync(0xffffffffu, x, 1), x2 = __shfl_sync(0xffffffffu, x, 2);
+                    if (lane == 0 && !gather_position(t.gather, row, x0, x1, x2)) atomicOr(err, kErrNonFinite);
+                }
+            }
+        }
+    }
+    if (REDUCE) reduce_finish(a, sh, &last);
+}
+
+__global__ void k_gather_positions(int N, const int* __restrict__ perm, const double* __restrict__ pos, const GatherArgs a, int* __restrict__ err) {
+    chain_begin();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const size_t o = 3 * (size_t)perm[i];
+    if (!gather_position(a, i, pos[o], pos[o + 1], pos[o + 2])) atomicOr(err, kErrNonFinite);
+    else if (moved_too_far(a, i)) atomicOr(err, kErrStale);
+}
+
+// kicks: see vv_kicks; drift: x += dt v after them; scale (may be null): the thermostat's velocity factor, applied first
 __global__ void k_vv(int64_t N, double* __restrict__ pos, double* __restrict__ vel, const double* __restrict__ force,
                      const int* __restrict__ type, const double* __restrict__ inv_mass, double dt, int kicks, bool drift,
                      const double* __restrict__ scale) {
@@ -276,8 +390,7 @@ __global__ void k_vv(int64_t N, double* __restrict__ pos, double* __restrict__ v
         const double f = force[3 * i + k];
         double v = vel[3 * i + k];
         if (scale) v *= sc;
-        if (kicks >= 1) v = v + c * f;
-        if (kicks == 2) v = v + c * f;
+        v = vv_kicks(v, c, f, kicks);
         vel[3 * i + k] = v;
         if (drift) pos[3 * i + k] += dt * v;
     }
@@ -426,12 +539,48 @@ cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, con
                           d_out, d_err);
 }
 
+static ReduceArgs reduce_args(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part,
+                              double* scratch, unsigned* counter, double* out, int* d_err, double* h_out, int* h_err) {
+    const int N = (int)nb.N, blocks = (N + 4 * kRedBlock - 1) / (4 * kRedBlock);
+    return {e_atom, N, nb.perm, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err,
+            blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks)};
+}
+
 cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part,
                                         int n_part, double* scratch, unsigned* counter, double* out, int* d_err, double* h_out,
                                         int* h_err, cudaStream_t st) {
-    const int N = (int)nb.N, blocks = (N + 4 * kRedBlock - 1) / (4 * kRedBlock);
-    return launch_chained(k_reduce, blocks < 1 ? 1 : (blocks < kReduceBlocks ? blocks : kReduceBlocks), kRedBlock, 0, st, e_atom, N,
-                          nb.perm, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
+    const ReduceArgs a = reduce_args(nb, e_atom, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
+    return launch_chained(k_reduce, a.n_blocks, kRedBlock, 0, st, a);
+}
+
+int assemble_launches(int64_t N) { return N <= kReduceTogether ? 1 : 2; }
+cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* f_sorted, double* d_force, const StepTail& tail,
+                            const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part, double* scratch,
+                            unsigned* counter, double* out, int* d_err, double* h_out, int* h_err, cudaStream_t st) {
+    const int N = (int)nb.N;
+    const ReduceArgs a = reduce_args(nb, e_atom, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
+    const int rows = (N + kRedBlock / 32 - 1) / (kRedBlock / 32);
+    if (N <= kReduceTogether)
+        return launch_chained(k_assemble<true>, a.n_blocks + rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err, a, tail);
+    const cudaError_t e = launch_chained(k_assemble<false>, rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err, a, tail);
+    return e != cudaSuccess ? e : launch_chained(k_reduce, a.n_blocks, kRedBlock, 0, st, a);
+}
+
+GatherArgs gather_args(const NeighborDev& nb, const int* species_slot) {
+    const double half = 0.5 * nb.skin;
+    GatherArgs a;
+    a.img = nb.img; a.xs0 = nb.xs0; a.type_s = nb.type_s; a.species_slot = species_slot; a.xs = nb.xs; a.fix = nb.fix;
+    for (int k = 0; k < 9; ++k) a.h[k] = nb.H[k];
+    a.tri = nb.tri; a.inv_q = 1.0 / nb.quantum;
+    // a tiny slack keeps a fresh build with zero skin from tripping on its own rounding
+    a.max_disp2 = half * half + 1e-20;
+    return a;
+}
+
+cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, const int* species_slot, int* d_err, cudaStream_t st) {
+    const int N = (int)nb.N;
+    if (N == 0) return cudaSuccess;
+    return launch_chained(k_gather_positions, (N + 255) / 256, 256, 0, st, N, nb.perm, d_pos, gather_args(nb, species_slot), d_err);
 }
 
 cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out, cudaStream_t st) {

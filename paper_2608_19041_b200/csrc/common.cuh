@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <string>
@@ -183,12 +184,31 @@ __host__ __device__ inline void pair_cubic(const Dims& d, const float* row, cons
 // modes' own products per edge, have not been tried.
 __host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }
 
+// Positions for the edge kernels are whole multiples of a power of two q, kept modulo 2^32: an edge vector is an exact
+// difference of integers (image offsets are whole multiples too), rounded once when it becomes single precision.  With R = 2^31 q
+// beyond the list radius rc + skin a component up to that wraps to itself; the longest edge of a list that is not stale is rc + 2 skin,
+// and what lies beyond R comes out as at least 2 R - (rc + 2 skin) > rc, outside the cutoff as it is.  Half a quantum is 1.9e-9 at
+// a list radius of 6 or 7 Angstrom, where the rounding of a component between 1 and 8 to single precision is 6e-8 to 2.4e-7.
+inline double position_quantum(double r_list) {
+    int e;
+    std::frexp(r_list, &e);
+    return std::ldexp(1.0, e - 31);
+}
+__host__ __device__ inline int to_quanta(double x, double inv_q) {
+#ifdef __CUDA_ARCH__
+    return (int)__double2ll_rn(x * inv_q);
+#else
+    return (int)std::llrint(x * inv_q);
+#endif
+}
+
 // One frame of a batched evaluation (umlmd_compute_batch): its own cell and its slice of the
 // concatenated atom arrays.
 struct FrameCell {
     double H[9];      // cell vectors as rows
     double Hinv[9];   // inverse (fractional coordinates f = r Hinv)
     double reach[3];  // cutoff in fractional coordinates along each cell vector, rounded up
+    int Hq[9];        // cell vectors in position quanta (position_quantum), as rows
     float near_tol;   // band around the squared cutoff inside which the scan decides in double precision
     int m[3];         // periodic images to visit along each cell vector (0 for an open direction)
     int pbc[3];
@@ -210,10 +230,11 @@ struct NeighborDev {
     int* type_s = nullptr;       // [N] species, sorted order
     double* xs0 = nullptr;       // [N][3] folded positions at build time, sorted order
     double* xs = nullptr;        // [N][3] current positions minus img*L, sorted order
-    // [N][2] the same positions and the species as one 32-byte record per atom for the edge kernels'
-    // neighbour gathers (one sector and two 16-byte loads instead of four scattered loads):
-    // (x_hi, y_hi, z_hi, species bits), (x_lo, y_lo, z_lo, 0) with x = (double)x_hi + (double)x_lo
-    float4* rec = nullptr;
+    float4* rec = nullptr;       // [N] positions in single precision, what the list search reads
+    // [N] current positions in quanta and the species, one 16-byte load per neighbour of the edge kernels.  x = q llrint(x / q)
+    // modulo 2^32: differences of two coordinates wrap to the true one, whatever the size of the box (position_quantum)
+    int4* fix = nullptr;
+    double quantum = 1;
     eidx_t* row_ptr = nullptr;   // [N+1]
     int2* nbr = nullptr;         // [E] x: sorted index of the neighbour, y: its image n, packed int8 x3
     eidx_t* rev = nullptr;       // [E] index of the reverse edge, -1 if absent

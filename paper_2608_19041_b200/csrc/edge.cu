@@ -2,7 +2,7 @@
 // the recomputing edge backward pass that returns dE/dr_ij for every edge.
 //
 // One warp owns one destination atom and walks its contiguous CSR interval, 32 listed edges
-// at a time: each lane computes the geometry of one edge (displacement from double-precision
+// at a time: each lane computes the geometry of one edge (displacement from fixed-point
 // positions, regularised length, direction, cutoff envelope, table row) and the edges inside
 // the cutoff are queued in shared memory.  Full batches of queued edges are then processed
 // with lanes split over channels -- a group of lanes handles one edge, each lane holding one
@@ -47,11 +47,14 @@ struct Geom {
 };
 
 // phase 1: one lane, one edge
-// Hf: cell of the destination's frame in a batched evaluation (rows), null for a single system
+// c: record of the destination; Hf: cell of its frame in a batched evaluation (rows, in quanta), null for a single system.
+// The edge vector is a difference of integers (common.cuh, position_quantum).  With float pairs, two 16-byte loads and an
+// addition in double per component, this phase was half of what the narrow kernels sent through the L1 data pipe (32 scattered
+// 16-byte loads are 32 of its wavefronts) and a quarter of their instructions.
 // VALUE: row and offset in the value table, else in the table with derivatives
 template <bool VALUE>
-__device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool in_range, double xi, double yi,
-                                              double zi, int ti, const double* __restrict__ Hf) {
+__device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool in_range, const int4& c, int ti,
+                                              const int* __restrict__ Hf) {
     Geom g;
     g.valid = false;
     g.dx = g.dy = g.dz = 0.f; g.rho = 1.f; g.inv_rho = 1.f; g.ux = g.uy = g.uz = 0.f;
@@ -61,23 +64,21 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     const int j = js.x, s = js.y;
     const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff),
               nz = (int)(signed char)((s >> 16) & 0xff);
-    // the neighbour's record: position as float pairs (exact to 2^-48 of the coordinate) and species
-    const float4 r0 = __ldg(a.rec + 2 * (size_t)j), r1 = __ldg(a.rec + 2 * (size_t)j + 1);
-    const double xj[3] = {(double)r0.x + (double)r1.x, (double)r0.y + (double)r1.y, (double)r0.z + (double)r1.z};
-    const int tj = __float_as_int(r0.w);
+    const int4 r = __ldg(a.fix + j);
+    const int tj = r.w;
+    unsigned ix = (unsigned)r.x - (unsigned)c.x, iy = (unsigned)r.y - (unsigned)c.y, iz = (unsigned)r.z - (unsigned)c.z;   // (wraps)
     if (Hf) {
-        g.dx = (float)((xj[0] + ((nx * __ldg(Hf + 0) + ny * __ldg(Hf + 3)) + nz * __ldg(Hf + 6))) - xi);
-        g.dy = (float)((xj[1] + ((nx * __ldg(Hf + 1) + ny * __ldg(Hf + 4)) + nz * __ldg(Hf + 7))) - yi);
-        g.dz = (float)((xj[2] + ((nx * __ldg(Hf + 2) + ny * __ldg(Hf + 5)) + nz * __ldg(Hf + 8))) - zi);
+        ix += nx * (unsigned)__ldg(Hf + 0) + ny * (unsigned)__ldg(Hf + 3) + nz * (unsigned)__ldg(Hf + 6);
+        iy += nx * (unsigned)__ldg(Hf + 1) + ny * (unsigned)__ldg(Hf + 4) + nz * (unsigned)__ldg(Hf + 7);
+        iz += nx * (unsigned)__ldg(Hf + 2) + ny * (unsigned)__ldg(Hf + 5) + nz * (unsigned)__ldg(Hf + 8);
     } else if (a.tri) {        // general cell: the image offset is n . H
-        g.dx = (float)((xj[0] + ((nx * a.H[0] + ny * a.H[3]) + nz * a.H[6])) - xi);
-        g.dy = (float)((xj[1] + ((nx * a.H[1] + ny * a.H[4]) + nz * a.H[7])) - yi);
-        g.dz = (float)((xj[2] + ((nx * a.H[2] + ny * a.H[5]) + nz * a.H[8])) - zi);
+        ix += nx * (unsigned)a.Hq[0] + ny * (unsigned)a.Hq[3] + nz * (unsigned)a.Hq[6];
+        iy += nx * (unsigned)a.Hq[1] + ny * (unsigned)a.Hq[4] + nz * (unsigned)a.Hq[7];
+        iz += nx * (unsigned)a.Hq[2] + ny * (unsigned)a.Hq[5] + nz * (unsigned)a.Hq[8];
     } else {
-        g.dx = (float)((xj[0] + nx * a.Lx) - xi);
-        g.dy = (float)((xj[1] + ny * a.Ly) - yi);
-        g.dz = (float)((xj[2] + nz * a.Lz) - zi);
+        ix += nx * (unsigned)a.Hq[0]; iy += ny * (unsigned)a.Hq[4]; iz += nz * (unsigned)a.Hq[8];
     }
+    g.dx = a.quantum * (float)(int)ix; g.dy = a.quantum * (float)(int)iy; g.dz = a.quantum * (float)(int)iz;
     const float r2 = g.dx * g.dx + g.dy * g.dy + g.dz * g.dz + kEpsReg * kEpsReg;
     g.rho = sqrtf(r2);
     if (!(g.rho < a.d.rc)) return g;       // skin-shell edge: zero weight
@@ -99,7 +100,7 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
         // per-pair amplitude tables, one after another: the pair selects the table (ti is
         // already the compact index of the centre's species)
         if (a.n_present > 1) {           // with one species there is one table and no lookup
-            g.pair = ti * a.n_present + a.species_slot[tj];
+            g.pair = ti * a.n_present + (a.species_slot ? a.species_slot[tj] : tj);
             g.row += g.pair * n_rows;
         }
     } else {
@@ -409,13 +410,13 @@ k_edge_forward(const EdgeArgs a) {
     int4* const qes = q_es[wid];
     float* const qd = q_d[wid];
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
-    const double xi = a.xs[3 * (size_t)i], yi = a.xs[3 * (size_t)i + 1], zi = a.xs[3 * (size_t)i + 2];
-    const int ti = UNI ? a.species_slot[a.type_s[i]] : a.type_s[i];
+    const int4 ci = __ldg(a.fix + i);
+    const int ti = UNI && a.species_slot ? a.species_slot[ci.w] : ci.w;
     const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + 2)) : a.d.tab_v1, k3 = UNI ? tab_step3(__ldg(a.uni_scale + 3)) : a.d.tab_v2;
     eidx_t e0 = a.row_ptr[i];
     int len = (int)(a.row_ptr[i + 1] - e0);      // edge offsets are 64-bit, offsets inside a row are not
     if (SPLIT) quarter_of_row(wid, &e0, &len);
-    const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
+    const int* Hf = a.frames ? a.frames[a.frame_of[i]].Hq : nullptr;
     const unsigned lt_mask = (1u << lane) - 1u;
     float acc0[4] = {0.f, 0.f, 0.f, 0.f};
     // this lane's jobs of the degree >= 1 sums: where its vector and its scalar are in the rows of edge 0, offset
@@ -542,7 +543,7 @@ k_edge_forward(const EdgeArgs a) {
 
     int qn = 0;
     for (int base = 0; base < len; base += 32) {
-        const Geom g = edge_geometry<true>(a, e0 + base + lane, base + lane < len, xi, yi, zi, ti, Hf);
+        const Geom g = edge_geometry<true>(a, e0 + base + lane, base + lane < len, ci, ti, Hf);
         const unsigned vmask = __ballot_sync(kFull, g.valid);
         const int p = qn + __popc(vmask & lt_mask);       // queue slot of this lane's edge, if it has one
         if (g.valid) { const double c2 = (double)g.chi * (double)g.chi; s0 += c2; s1 += c2 * c2; }
@@ -649,8 +650,8 @@ k_edge_backward(const EdgeArgs a) {
     for (int k = 0; k < 9; ++k) vir[k] = 0.f;
 
     if (active) {
-        const double xi = a.xs[3 * (size_t)i], yi = a.xs[3 * (size_t)i + 1], zi = a.xs[3 * (size_t)i + 2];
-        const int ti = UNI ? a.species_slot[a.type_s[i]] : a.type_s[i];
+        const int4 ci = __ldg(a.fix + i);
+        const int ti = UNI && a.species_slot ? a.species_slot[ci.w] : ci.w;
         // steps of the packed words: of the table with derivatives, or of the value and the product table
         const float k2 = UNI ? tab_step2(__ldg(a.uni_scale + (PR ? 2 : 0))) : (PR ? a.d.tab_v1 : a.d.tab_k2),
                     k3 = UNI ? tab_step3(__ldg(a.uni_scale + (PR ? 3 : 1))) : (PR ? a.d.tab_v2 : a.d.tab_k3);
@@ -658,7 +659,7 @@ k_edge_backward(const EdgeArgs a) {
         eidx_t e0 = a.row_ptr[i];
         int len = (int)(a.row_ptr[i + 1] - e0);
         if (SPLIT) quarter_of_row(wid, &e0, &len);
-        const double* Hf = a.frames ? a.frames[a.frame_of[i]].H : nullptr;
+        const int* Hf = a.frames ? a.frames[a.frame_of[i]].Hq : nullptr;
         const float* grow = a.state + (size_t)(i - a.a0) * a.d.SP;
         float h0[4 * G];
 #pragma unroll
@@ -881,7 +882,7 @@ k_edge_backward(const EdgeArgs a) {
         int qn = 0;
         for (int base = 0; base < len; base += 32) {
             const int e = base + lane;
-            const Geom g = edge_geometry<PR>(a, e0 + e, e < len, xi, yi, zi, ti, Hf);
+            const Geom g = edge_geometry<PR>(a, e0 + e, e < len, ci, ti, Hf);
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
             if (g.valid && p < 32) {

@@ -39,23 +39,17 @@ cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, con
 // always filled; edges are copied while they fit `cap` (cap = 0 or null buffers: offsets only).
 int neighbor_export_rows(NeighborDev* nb, int64_t first, int64_t n, int64_t* d_row_ptr, int32_t* d_src,
                          int8_t* d_shift, int64_t cap, cudaStream_t st, std::string* err);
-// xs[i] = pos[perm[i]] - img[i]*L; flags stale / non-finite atoms in *d_err.
-cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, int* d_err,
-                                    cudaStream_t st);
-
 // ---- edge.cu ---------------------------------------------------------------------------
 struct EdgeArgs {
     Dims d;
     const float* table;
     const float* pairmod;
-    const double* xs;       // [N][3] sorted positions
-    const float4* rec;      // [N][2] positions (as float pairs) and species, one record per atom
-    const int* type_s;
+    const int4* fix;        // [N] positions in quanta and species (or its slot, see species_slot), one record per atom
     const eidx_t* row_ptr;
     const int2* nbr;        // [E] neighbour (sorted index) and its image
-    double Lx, Ly, Lz;
-    double H[9];            // cell vectors as rows, used instead of Lx, Ly, Lz when tri
+    int Hq[9];              // cell vectors as rows, in quanta; only the diagonal is read unless tri
     int tri;
+    float quantum;
     int a0, a1;             // destination range [a0, a1) of this tile
     float* state;           // [a1-a0][SP]: forward writes sums; backward reads dE/d(sums)
     float* g;               // [E][3] per-edge gradient (backward)
@@ -77,7 +71,7 @@ struct EdgeArgs {
     // |a2| of dtable_uni.  There is no table_uni then.
     const float* dtable;
     const float* dtable_uni;
-    const int* species_slot;    // [T] species -> index among the species present
+    const int* species_slot;    // [T] species -> index among the species present; null: the records hold that index
     int n_present;
 };
 constexpr int kEdgeRowsPerBlock = 4, kEdgeSplitRows = 1184;
@@ -181,6 +175,24 @@ cudaError_t launch_mlp_forward(const MlpArgs& a, cudaStream_t st);   // layers +
 cudaError_t launch_mlp_backward(const MlpArgs& a, cudaStream_t st);  // needs a forward with want_grad
 
 // ---- assemble.cu ---------------------------------------------------------------------
+// Current positions of the sorted atoms, from the caller's: see gather_position
+struct GatherArgs {
+    const int* img; const double* xs0; const int* type_s;
+    const int* species_slot;    // what the records hold in place of the species (null: the species itself)
+    double* xs; int4* fix;
+    double h[9]; int tri;
+    double inv_q, max_disp2;
+};
+GatherArgs gather_args(const NeighborDev& nb, const int* species_slot);
+// xs[i] = pos[perm[i]] - img[i]*L and the records of the edge kernels; flags stale / non-finite atoms in *d_err
+cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, const int* species_slot, int* d_err, cudaStream_t st);
+// What an MD step does with the forces of an atom once they are there (pos null: nothing): kicks and, if drift, the drift and
+// the records of the next evaluation
+struct StepTail {
+    double* pos; double* vel; const double* inv_mass;
+    double dt; int kicks; int drift;
+    GatherArgs gather;
+};
 // d_flags[t] = 1 for every species t in [0, T) that occurs among the N atoms, 0 otherwise;
 // kErrSpecies is or-ed into *d_err when an index lies outside [0, T)
 cudaError_t launch_species_present(int64_t N, const int* type, int T, int* d_flags, int* d_err, cudaStream_t st);
@@ -200,6 +212,11 @@ cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_a
                                         int n_part, double* scratch, unsigned* counter, double* out, int* d_err, double* h_out,
                                         int* h_err, cudaStream_t st);
 int reduce_scratch_doubles(int64_t N);
+// the same and the force assembly (in one launch, where few atoms make that the better one), with the rest of an MD step (tail)
+int assemble_launches(int64_t N);
+cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* d_force_sorted, double* d_force, const StepTail& tail,
+                            const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part, double* scratch,
+                            unsigned* counter, double* out, int* d_err, double* h_out, int* h_err, cudaStream_t st);
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width,
                                 float* out, cudaStream_t st);
 // velocity Verlet pieces (caller order, double)

@@ -62,8 +62,6 @@ __device__ __forceinline__ int pack_shift(int nx, int ny, int nz) {
     return (nx & 0xff) | ((ny & 0xff) << 8) | ((nz & 0xff) << 16);
 }
 
-struct CellRows { double h[9]; int tri; };
-
 // order-preserving map of a double onto an unsigned integer, for atomicMin / atomicMax
 __device__ __forceinline__ unsigned long long ordered_key(double x) {
     const long long b = __double_as_longlong(x);
@@ -195,7 +193,7 @@ __global__ void k_gather_sorted(int N, int nkeys, const int* __restrict__ skey, 
         img[3 * (size_t)i + k] = img_o[3 * (size_t)o + k];
         hi[k] = (float)w;
     }
-    rec[2 * (size_t)i] = make_float4(hi[0], hi[1], hi[2], 0.f);   // what the scans read; the evaluation rewrites the records
+    rec[i] = make_float4(hi[0], hi[1], hi[2], 0.f);   // what the scans read
 }
 
 // Squared list radius, its single-precision value, and a band around that outside of which a squared
@@ -359,7 +357,7 @@ __global__ void __launch_bounds__(128) k_scan_cells(int N, int span, Grid g, Nea
                 while (f >= runs[r].end) ++r;
                 j_next = runs[r].first + f;
                 code_next = runs[r].code;
-                p_next = __ldg(rec + 2 * (size_t)j_next);
+                p_next = __ldg(rec + j_next);
             }
         };
         fetch(lane);
@@ -492,8 +490,8 @@ __global__ void k_reverse_map(int N, Grid g, const int* __restrict__ skey, const
 // direction the magnitude of the coordinates, and with it the band of the scans, is known only here (without a band
 // every candidate was decided twice)
 __global__ void k_batch_fold(FrameCell* __restrict__ frames, const double* __restrict__ pos,
-                             const int* __restrict__ type, int T, double rc, double* __restrict__ xs, float4* __restrict__ rec,
-                             int* __restrict__ type_s, int* __restrict__ frame_of, int* __restrict__ perm,
+                             const int* __restrict__ type, int T, double rc, double inv_q, double* __restrict__ xs, float4* __restrict__ rec,
+                             int4* __restrict__ fix, int* __restrict__ type_s, int* __restrict__ frame_of, int* __restrict__ perm,
                              int* __restrict__ err) {
     __shared__ double far_s[32];
     FrameCell& fc = frames[blockIdx.x];
@@ -507,20 +505,21 @@ __global__ void k_batch_fold(FrameCell* __restrict__ frames, const double* __res
             fl[k] = fc.pbc[k] ? floor(f) : 0.0;
             if (!(fabs(fl[k]) <= 1.0e6)) { bad = true; fl[k] = 0.0; }
         }
-        float hi[3], lo[3];
+        float hi[3];
+        int fx[3];
         for (int k = 0; k < 3; ++k) {
             const double r = k == 0 ? x : (k == 1 ? y : z);
             const double w = bad ? 0.0 : r - ((fl[0] * fc.H[k] + fl[1] * fc.H[3 + k]) + fl[2] * fc.H[6 + k]);
             xs[3 * (size_t)i + k] = w;
             X = fmax(X, fabs(w));
             hi[k] = (float)w;
-            lo[k] = (float)(w - (double)hi[k]);
+            fx[k] = to_quanta(w, inv_q);
         }
         int t = type[i];
         if (t < 0 || t >= T) { atomicOr(err, kErrSpecies); t = 0; }
         if (bad) atomicOr(err, kErrNonFinite);
-        rec[2 * (size_t)i] = make_float4(hi[0], hi[1], hi[2], __int_as_float(t));
-        rec[2 * (size_t)i + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        rec[i] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        fix[i] = make_int4(fx[0], fx[1], fx[2], t);
         type_s[i] = t;
         frame_of[i] = blockIdx.x;
         perm[i] = i;
@@ -582,7 +581,7 @@ __global__ void k_batch_scan(int N, const FrameCell* __restrict__ frames, const 
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int j = b + 32 * h + lane;
-                        p[h] = j < fc.a1 ? __ldg(rec + 2 * (size_t)j) : make_float4(1.0e18f, 0.f, 0.f, 0.f);
+                        p[h] = j < fc.a1 ? __ldg(rec + j) : make_float4(1.0e18f, 0.f, 0.f, 0.f);
                     }
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -602,34 +601,6 @@ __global__ void k_batch_scan(int N, const FrameCell* __restrict__ frames, const 
         }
     }
     if (!FILL && lane == 0) deg[i] = count;
-}
-
-__global__ void k_gather_positions(int N, const int* __restrict__ perm, const int* __restrict__ img,
-                                   const double* __restrict__ pos, const double* __restrict__ xs0,
-                                   CellRows H, double max_disp2, const int* __restrict__ type_s,
-                                   double* __restrict__ xs, float4* __restrict__ rec, int* __restrict__ err) {
-    chain_begin();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int o = perm[i];
-    const double n0 = (double)img[3 * (size_t)i], n1 = (double)img[3 * (size_t)i + 1], n2 = (double)img[3 * (size_t)i + 2];
-    double d2 = 0;
-    bool bad = false;
-    float hi[3], lo[3];
-    for (int k = 0; k < 3; ++k) {
-        const double x = H.tri ? pos[3 * (size_t)o + k] - ((n0 * H.h[k] + n1 * H.h[3 + k]) + n2 * H.h[6 + k])
-                               : pos[3 * (size_t)o + k] - (double)img[3 * (size_t)i + k] * H.h[4 * k];
-        if (!isfinite(x)) bad = true;
-        xs[3 * (size_t)i + k] = x;
-        hi[k] = (float)x;
-        lo[k] = (float)(x - (double)hi[k]);
-        const double d = x - xs0[3 * (size_t)i + k];
-        d2 += d * d;
-    }
-    rec[2 * (size_t)i] = make_float4(hi[0], hi[1], hi[2], __int_as_float(type_s[i]));
-    rec[2 * (size_t)i + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
-    if (bad) atomicOr(err, kErrNonFinite);
-    else if (d2 > max_disp2) atomicOr(err, kErrStale);
 }
 
 // ---- export in caller numbering ------------------------------------------------------
@@ -708,7 +679,7 @@ struct WidenDeg {
 }  // namespace
 
 void neighbor_free(NeighborDev* nb) {
-    void* ptrs[] = {nb->frames, nb->rec, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->nbr, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
+    void* ptrs[] = {nb->frames, nb->rec, nb->fix, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->nbr, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
                     nb->cub_tmp, nb->bounds};
     for (void* p : ptrs)
         dev_free(p);
@@ -842,7 +813,7 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     g.ncell = (int)ncell; g.n_owned = n_owned; g.halves = n_owned < N ? 2 : 1;
     const int64_t nkeys = (int64_t)g.halves * ncell;
 
-    nb->N = N; nb->skin = skin; nb->r_list = r_list; nb->n_owned = n_owned; nb->E_owned = 0;
+    nb->N = N; nb->skin = skin; nb->r_list = r_list; nb->quantum = position_quantum(r_list); nb->n_owned = n_owned; nb->E_owned = 0;
     for (int k = 0; k < 3; ++k) { nb->L[k] = L[k]; nb->pbc[k] = pbc[k] ? 1 : 0; }
     for (int k = 0; k < 9; ++k) nb->H[k] = cell[k];
     nb->tri = g.tri;
@@ -856,7 +827,8 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
         c = 0; NB_CHECK(dev_ensure(&nb->wpos, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs0, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs, &c, need * 3));
-        c = 0; NB_CHECK(dev_ensure(&nb->rec, &c, need * 2));
+        c = 0; NB_CHECK(dev_ensure(&nb->rec, &c, need));
+        c = 0; NB_CHECK(dev_ensure(&nb->fix, &c, need));
         c = 0; NB_CHECK(dev_ensure(&nb->img, &c, need * 6));   // sorted-order and caller-order halves
         c = 0; NB_CHECK(dev_ensure(&nb->perm, &c, need));
         c = 0; NB_CHECK(dev_ensure(&nb->type_s, &c, need));
@@ -961,6 +933,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
         for (int k = 0; k < 9; ++k) {
             if (!std::isfinite(H[k])) { *err = "non-finite cell in a frame"; return UMLMD_E_UNSUPPORTED_CELL; }
             c.H[k] = H[k];
+            c.Hq[k] = to_quanta(H[k], 1.0 / position_quantum(rc));
         }
         const double cx[3] = {H[4] * H[8] - H[5] * H[7], H[5] * H[6] - H[3] * H[8], H[3] * H[7] - H[4] * H[6]};   // b x c
         const double cy[3] = {H[7] * H[2] - H[8] * H[1], H[8] * H[0] - H[6] * H[2], H[6] * H[1] - H[7] * H[0]};   // c x a
@@ -985,7 +958,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
         c.near_tol = pbc[0] && pbc[1] && pbc[2] ? near_band(rc, 3.0 * X).tol : 1.0e30f;
         c.a0 = (int)offsets[f]; c.a1 = (int)offsets[f + 1];
     }
-    nb->N = N; nb->skin = 0; nb->r_list = rc; nb->tri = 1; nb->batch = true; nb->n_frames = n_frames;
+    nb->N = N; nb->skin = 0; nb->r_list = rc; nb->quantum = position_quantum(rc); nb->tri = 1; nb->batch = true; nb->n_frames = n_frames;
     for (int k = 0; k < 3; ++k) { nb->pbc[k] = pbc[k] ? 1 : 0; nb->L[k] = 0; }
     for (int k = 0; k < 9; ++k) nb->H[k] = 0;
     nb->E = 0;
@@ -998,7 +971,8 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
         c = 0; NB_CHECK(dev_ensure(&nb->wpos, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs0, &c, need * 3));
         c = 0; NB_CHECK(dev_ensure(&nb->xs, &c, need * 3));
-        c = 0; NB_CHECK(dev_ensure(&nb->rec, &c, need * 2));
+        c = 0; NB_CHECK(dev_ensure(&nb->rec, &c, need));
+        c = 0; NB_CHECK(dev_ensure(&nb->fix, &c, need));
         c = 0; NB_CHECK(dev_ensure(&nb->img, &c, need * 6));
         c = 0; NB_CHECK(dev_ensure(&nb->perm, &c, need));
         c = 0; NB_CHECK(dev_ensure(&nb->type_s, &c, need));
@@ -1024,7 +998,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
         nb->cub_bytes = need_scan + 256;
     }
     const int TB = 256;
-    k_batch_fold<<<n_frames, TB, 0, st>>>(nb->frames, d_pos, d_type, T, rc, nb->xs, nb->rec, nb->type_s, nb->frame_of, nb->perm, d_err);
+    k_batch_fold<<<n_frames, TB, 0, st>>>(nb->frames, d_pos, d_type, T, rc, 1.0 / nb->quantum, nb->xs, nb->rec, nb->fix, nb->type_s, nb->frame_of, nb->perm, d_err);
     const int wb = (int)((N + TB / 32 - 1) / (TB / 32));
     k_batch_scan<false><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rc, nb->xs, nb->rec, nb->deg, nullptr, nullptr);
     NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
@@ -1063,19 +1037,6 @@ int neighbor_export_rows(NeighborDev* nb, int64_t first, int64_t n, int64_t* d_r
     }
     NB_CHECK(cudaGetLastError());
     return UMLMD_OK;
-}
-
-cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, int* d_err, cudaStream_t st) {
-    const int N = (int)nb.N;
-    if (N == 0) return cudaSuccess;
-    const double half = 0.5 * nb.skin;
-    // a tiny slack keeps a fresh build with zero skin from tripping on its own rounding
-    const double max_disp2 = half * half + 1e-20;
-    CellRows H;
-    for (int k = 0; k < 9; ++k) H.h[k] = nb.H[k];
-    H.tri = nb.tri;
-    return launch_chained(k_gather_positions, (N + 255) / 256, 256, 0, st, N, nb.perm, nb.img, d_pos, nb.xs0, H, max_disp2, nb.type_s,
-                          nb.xs, nb.rec, d_err);
 }
 
 }  // namespace umd
