@@ -30,6 +30,11 @@ struct umlmd {
     __half* tc_hi = nullptr; __half* tc_lo = nullptr;   // half-precision split of the current GEMM's activations
     float* fused_scratch = nullptr; int64_t fused_cap = 0;      // per-CTA areas of the one-kernel MLP
     int64_t tile_cap = 0;
+    // shared radial modes without per-pair tables (moments.cu): moments of a tile's rows, rows of every tile by species
+    float* moments = nullptr; int64_t moments_cap = 0;
+    int* moment_order = nullptr; int64_t order_cap = 0;
+    int* moment_scratch = nullptr;
+    bool have_groups = false;                        // moment_order belongs to the current list
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
     double* virial_part = nullptr; int64_t vpart_cap = 0;
@@ -233,8 +238,15 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         for (int k = 0; k < 9; ++k) ea.Hq[k] = to_quanta(nb.H[k], 1.0 / nb.quantum);
         ea.tri = nb.tri;
         ea.a0 = a0; ea.a1 = a0 + n; ea.state = h->state; ea.g = h->g;
+        const bool by_moments = h->have_groups && !h->pair_tables && moments_pick(d, n);
+        ea.moments = by_moments ? h->moments : nullptr; ea.n_moments = moment_pitch(d);
+        const MomentArgs mo = {d, h->md.pairmod, nb.type_s, h->moment_order + (a0 / B) * moment_order_ints(d, B), a0, n, h->state, h->moments};
         ea.virial_part = h->virial_part + (size_t)vpart_used * 9;
-        { Scope sc(h, kEdgeFwd, 1); API_CUDA(h, launch_edge_forward(ea, h->st)); }
+        {
+            Scope sc(h, kEdgeFwd, 1 + by_moments);
+            API_CUDA(h, launch_edge_forward(ea, h->st));
+            if (by_moments) API_CUDA(h, launch_moments_forward(mo, h->st));
+        }
         InvArgs ia;
         ia.d = d; ia.m = h->md; ia.type_s = nb.type_s; ia.a0 = a0; ia.n = n; ia.state = h->state; ia.desc = h->desc;
         // tensor-core MLP: the invariants kernel writes the first GEMM's operand split itself, and the fp32
@@ -259,7 +271,11 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
             if (!ma.fused_scratch) { Scope sc(h, kMlpBwd, d.n_hidden); API_CUDA(h, launch_mlp_backward(ma, h->st)); }
             { Scope sc(h, kInvBwd, 1); API_CUDA(h, launch_invariants_backward(ia, h->st)); }
             int blocks = 0;
-            { Scope sc(h, kEdgeBwd, 1); API_CUDA(h, launch_edge_backward(ea, &blocks, h->st)); }
+            {
+                Scope sc(h, kEdgeBwd, 1 + by_moments);
+                if (by_moments) API_CUDA(h, launch_moments_backward(mo, h->st));
+                API_CUDA(h, launch_edge_backward(ea, &blocks, h->st));
+            }
             vpart_used += blocks;
         }
     }
@@ -445,6 +461,7 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     { Scope sc(h, kNeighbor, 5 + (fetch && N > 0)); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, fetch, h->st, &h->err); }
     if (rc != UMLMD_OK) return rc;
     h->have_edge_grad = false;       // edges were renumbered
+    h->have_groups = false;          // rows as well
     h->steps_since_build = 0;
     ++h->list_serial;                // recorded launch sequences name the old list
     rc = ensure_workspace(h);
@@ -457,6 +474,26 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
             API_CUDA(h, cudaMemsetAsync(h->g + 3 * (size_t)h->nb.E_owned, 0, sizeof(float) * 3 * (size_t)(h->nb.E - h->nb.E_owned), h->st));
     }
     h->have_list = true;
+    return UMLMD_OK;
+}
+
+// Groups the rows of the current list by species and makes room for their moments, where its kernels take that way.
+int setup_moments(umlmd_t* h) {
+    const Dims& d = h->d;
+    const int64_t NR = h->nb.n_owned, B = h->nb.N < h->node_tile ? h->nb.N : h->node_tile, rows = NR < B ? NR : B;
+    h->have_groups = false;
+    if (h->pair_tables || !moments_pick(d, rows)) return UMLMD_OK;
+    const int64_t per_tile = moment_order_ints(d, B);
+    int64_t c = 0;
+    if (!h->moment_scratch) API_CUDA(h, dev_ensure(&h->moment_scratch, &c, 2 * d.T));
+    if (rows * moment_pitch(d) > h->moments_cap) API_CUDA(h, dev_ensure(&h->moments, &h->moments_cap, rows * moment_pitch(d)));
+    if ((NR + B - 1) / B * per_tile > h->order_cap) API_CUDA(h, dev_ensure(&h->moment_order, &h->order_cap, (NR + B - 1) / B * per_tile));
+    for (int64_t a0 = 0; a0 < NR; a0 += B) {
+        const int n = (int)(NR - a0 < B ? NR - a0 : B);
+        Scope sc(h, kNeighbor, 2);
+        API_CUDA(h, launch_moment_groups(d, h->nb.type_s + a0, n, h->moment_scratch, h->moment_order + a0 / B * per_tile, h->st));
+    }
+    h->have_groups = true;
     return UMLMD_OK;
 }
 
@@ -546,7 +583,7 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->on_device) cudaStreamSynchronize(h->st);
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
-    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
+    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->moments, h->moment_order, h->moment_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
                     h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->uni, h->d_species};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
@@ -606,6 +643,7 @@ int umlmd_build_neighbors(umlmd_t* h, int64_t N, const double* d_pos, const int3
     if (rc != UMLMD_OK) return rc;
     if (N > 0) API_CUDA(h, cudaMemcpyAsync(h->type_o, d_type, sizeof(int) * N, cudaMemcpyDeviceToDevice, h->st));
     rc = setup_pair_tables(h);
+    if (rc == UMLMD_OK) rc = setup_moments(h);
     h->have_list = rc == UMLMD_OK;
     return rc;
 }
@@ -672,6 +710,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
     if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
+    if (moments_pick(d, Bt)) t += buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
     t += grown(3 * n_edges, 4);
@@ -757,7 +796,7 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
     if (N > 0) {
         if ((rc = decode_device_errors(h, *h->h_err)) != UMLMD_OK) return rc;
         if ((rc = ensure_workspace(h)) != UMLMD_OK) return rc;
-        if ((rc = setup_pair_tables(h)) != UMLMD_OK) return rc;
+        if ((rc = setup_pair_tables(h)) != UMLMD_OK || (rc = setup_moments(h)) != UMLMD_OK) return rc;
         if ((rc = enqueue_compute(h, d_pos, want_grad, d_force, d_atom_energy)) != UMLMD_OK) return rc;
     }
     const int64_t n_out = (int64_t)n_frames * 10;
@@ -847,6 +886,7 @@ static int maybe_rebuild(umlmd_t* h, int rebuild_every) {
             API_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
             return decode_device_errors(h, word);
         }
+        if ((rc = setup_moments(h)) != UMLMD_OK) return rc;
     }
     return UMLMD_OK;
 }
@@ -1054,7 +1094,7 @@ int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int
     const HostModel& m = h->hm;
     const int C0 = d.C0, R = d.R;
     const double dx = h->hm.dx, w = dx / d.v_sub;
-    const bool products = wide_channels(C0) && (per_pair || R == 0);      // what the backward pass reads: else rows with derivatives
+    const bool products = wide_channels(C0);             // what the backward pass reads: else rows with derivatives
     auto pair_row = [&](int a, int b) { return &m.pairmod[(size_t)(a * d.T + b) * (2 + R) * C0]; };
     auto word = [](const float* p) { unsigned u; std::memcpy(&u, p, sizeof(u)); return u; };
     // steps of the packed words of tables made for a system of these two species
@@ -1119,6 +1159,7 @@ int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int
                 out = packed(q, step + 4);
             } else if (products) {
                 out = (double)pm[c] * stored(m.dtable, c, step + 4) + (double)pm[C0 + c] * dchi;
+                for (int k = 0; k < R; ++k) out += (double)pm[(size_t)(2 + k) * C0 + c] * stored(m.dtable, C0 + k, step + 4);
             } else {
                 pair_cubic(d, &m.table[(size_t)row * 3 * d.CP], pm + c, c, v);
                 float c2 = (float)v[2], c3 = (float)v[3];

@@ -177,11 +177,8 @@ __host__ __device__ inline void pair_cubic(const Dims& d, const float* row, cons
         if (q < 0) v[0] += (double)pm[d.C0];
     }
 }
-// Models of at least 32 channels without shared modes, or with per-pair tables (which hold the modes), use the
-// product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the channels are leading
-// ones, which need both: there the table with derivatives is less to read.  With shared modes and the pair cache the
-// backward pass still forms psi and psi' from the table with derivatives; products with modes, which would take the
-// modes' own products per edge, have not been tried.
+// Models of at least 32 channels use the product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the
+// channels are leading ones, which need both: there the table with derivatives is less to read.
 __host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }
 
 // Positions for the edge kernels are whole multiples of a power of two q, kept modulo 2^32: an edge vector is an exact
@@ -201,6 +198,16 @@ __host__ __device__ inline int to_quanta(double x, double inv_q) {
     return (int)std::llrint(x * inv_q);
 #endif
 }
+
+#ifdef __CUDACC__
+// two multiply-adds in one instruction (the pipe takes as long as for two; the issue slot is one)
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 r;
+    asm("{.reg .b64 x, y, z, w; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mov.b64 z, {%6, %7}; fma.rn.f32x2 w, x, y, z; mov.b64 {%0, %1}, w;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+#endif
 
 // One frame of a batched evaluation (umlmd_compute_batch): its own cell and its slice of the
 // concatenated atom arrays.

@@ -211,36 +211,42 @@ __device__ __forceinline__ void value_eval4(const float* __restrict__ table, int
 #undef UMLMD_PIECE
 }
 
-// one channel of either table
-template <bool DERIV>
-__device__ __forceinline__ void table_eval1(const EdgeArgs& a, int row, int c, float t, float* v, float* dv) {
-    const int CP = a.d.CP;
-    const float* p = DERIV ? a.table + (size_t)row * 3 * CP + c : a.vtable + (size_t)row * 2 * CP + c;
-    const float c0 = __ldg(p);
-    const int w = __ldg(reinterpret_cast<const int*>(p + (DERIV ? 2 : 1) * CP));
-    const float hi = (float)(w >> 12), lo = (float)((w << 20) >> 20);
-    if (DERIV) {
-        const float c1 = __ldg(p + CP), k2 = a.d.tab_k2, k3 = a.d.tab_k3;
-        *v = fmaf(lo, k3 * t * t * t, fmaf(hi, k2 * t * t, fmaf(c1, t, c0)));
-        *dv = fmaf(lo, 3.0f * k3 * t * t, fmaf(hi, 2.0f * k2 * t, c1));
-    } else {
-        *v = fmaf(lo, a.d.tab_v2 * t * t, fmaf(hi, a.d.tab_v1 * t, c0));
+// Shared radial modes q_mu(rho) of the first nb queued edges, an edge per lane, parked as qm[edge * PQ + mu]: evaluated once
+// per edge here instead of once per lane in the channel-parallel phase.  (Rows are padded to whole fours of columns.)
+// DQ: what comes with them in dqm: nothing, their derivatives, or the products (chi q)' (product table).
+enum : int { kValuesOnly = 0, kDerivatives = 1, kProducts = 2 };
+template <int DQ, int PQ>
+__device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, int nb, int lane, float* qm, float* dqm) {
+    if (lane >= nb) return;
+    const int4 es = qes[lane];
+    const float t = __int_as_float(es.z);
+    for (int q = 0; q < a.d.R; q += 4) {
+        float v[4], dv[4];
+        if (DQ == kDerivatives) table_eval4(a.table, a.d.CP, es.x, a.d.C0 + q, t, a.d.tab_k2, a.d.tab_k3, v, dv);
+        else value_eval4(a.vtable, a.d.CP, es.x, a.d.C0 + q, t, a.d.tab_v1, a.d.tab_v2, v);
+        if (DQ == kProducts) value_eval4(a.dtable, a.d.CP, es.x, a.d.C0 + q, t, a.d.tab_d1, a.d.tab_d2, dv);
+        *reinterpret_cast<float4*>(qm + lane * PQ + q) = make_float4(v[0], v[1], v[2], v[3]);
+        if (DQ) *reinterpret_cast<float4*>(dqm + lane * PQ + q) = make_float4(dv[0], dv[1], dv[2], dv[3]);
     }
 }
 
-// Shared radial modes q_mu(rho) (and derivatives) of the first nb queued edges, one (edge, mode)
-// pair per lane, parked as qm[edge * PQ + mu]: evaluated once per edge here instead of once
-// per lane in the channel-parallel phase.
-template <bool DERIV, int PQ>
-__device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, int nb, int lane, float* qm, float* dqm) {
+// What a kernel does about shared radial modes (without per-pair tables): there are none; every edge reads its pair's mixing
+// rows; or the scalar channels get them, and beta, from the row's moments (moments.cu)
+enum : int { kNoModes = 0, kModesPerEdge = 1, kMoments = 2 };
+
+// adds sum_mu U_c,mu q_mu of four channels; pm: the pair's rows at the channel
+template <int C0>
+__device__ __forceinline__ void add_modes4(const EdgeArgs& a, const float* pm, const float* qm, float* v) {
     const int R = a.d.R;
-    for (int idx = lane; idx < nb * R; idx += 32) {
-        const int b = idx / R, q = idx - b * R;
-        const int4 es = qes[b];
-        float qv, dqv = 0.f;
-        table_eval1<DERIV>(a, es.x, a.d.C0 + q, __int_as_float(es.z), &qv, &dqv);
-        qm[b * PQ + q] = qv;
-        if (DERIV) dqm[b * PQ + q] = dqv;
+    float q[kMaxR];
+    const float4 v0 = *reinterpret_cast<const float4*>(qm);
+    q[0] = v0.x; q[1] = v0.y; q[2] = v0.z; q[3] = v0.w;
+    if (R > 4) { const float4 v1 = *reinterpret_cast<const float4*>(qm + 4); q[4] = v1.x; q[5] = v1.y; q[6] = v1.z; q[7] = v1.w; }
+#pragma unroll
+    for (int m = 0; m < kMaxR; ++m) {
+        if (m >= R) break;
+        const float4 U = ldg4(pm + (size_t)(2 + m) * C0);
+        v[0] += U.x * q[m]; v[1] += U.y * q[m]; v[2] += U.z * q[m]; v[3] += U.w * q[m];
     }
 }
 
@@ -289,21 +295,28 @@ __device__ __forceinline__ void amplitude4(const EdgeArgs& a, int row, float t, 
 }
 
 // (chi psi_c)' of this lane's four channels for one edge, from the product table; row and t of the value grid, dchi
-// the envelope's derivative (only without per-pair tables)
-template <int C0, bool UNI>
-__device__ __forceinline__ void product4(const EdgeArgs& a, int row, float t, int pair, int c, float dchi, float d1, float d2, float* d) {
+// the envelope's derivative (only without per-pair tables), dqm the edge's parked (chi q)' (MODES).  With moments
+// the beta and mode parts are left out.
+template <int C0, int MODES, bool UNI>
+__device__ __forceinline__ void product4(const EdgeArgs& a, int row, float t, int pair, int c, float dchi, const float* dqm, float d1, float d2,
+                                         float* d) {
     if (UNI) {
         value_eval4(a.dtable_uni, C0, row, c, t, d1, d2, d);
         return;
     }
     float g[4];
     value_eval4(a.dtable, a.d.CP, row, c, t, d1, d2, g);
-    const float* pm = a.pairmod + (size_t)pair * 2 * C0 + c;
-    const float4 ga = ldg4(pm), be = ldg4(pm + C0);
+    const float* pm = a.pairmod + (size_t)pair * (MODES ? 2 + a.d.R : 2) * C0 + c;
+    const float4 ga = ldg4(pm);
+    if (MODES == kMoments) {
+        d[0] = ga.x * g[0]; d[1] = ga.y * g[1]; d[2] = ga.z * g[2]; d[3] = ga.w * g[3];
+        return;
+    }
+    const float4 be = ldg4(pm + C0);
     d[0] = fmaf(ga.x, g[0], be.x * dchi); d[1] = fmaf(ga.y, g[1], be.y * dchi);
     d[2] = fmaf(ga.z, g[2], be.z * dchi); d[3] = fmaf(ga.w, g[3], be.w * dchi);
+    if (MODES) add_modes4<C0>(a, pm, dqm, d);
 }
-
 // G = groups of four channels a lane holds in the channel-parallel phase (group g starts at
 // channel 4 * lane_in_group + g * C0 / G, so every 16-byte load instruction of a group of lanes
 // still covers one contiguous segment)
@@ -351,18 +364,18 @@ template <int C0, int L, int G = 1> struct Widths {
 // C0 <= 16: one group, 24 warps.  FEW: rows for more than 24 but not more than 32 warps per SM (3553 to 4736): 64
 // registers and one wave beat 85 and two (4000 atoms at C0 = 64: 41 -> 35 us; 597 atoms 25 against 21, 32,400
 // atoms 254 against 234).
-template <int C0, int L, bool HASR, bool UNI, bool FEW> struct BwdShape {
-    static constexpr bool two = C0 >= 128 && (HASR || (UNI && L == 2));
+template <int C0, int L, int MODES, bool UNI, bool FEW> struct BwdShape {
+    static constexpr bool two = C0 >= 128 && (MODES == kModesPerEdge || (UNI && L == 2));
     static constexpr int G = C0 >= 128 ? (two ? 2 : 4) : (C0 >= 32 ? 2 : 1);
-    static constexpr int warps = C0 >= 128 ? (two ? 24 : 16) : (FEW ? 32 : 24);
+    static constexpr int warps = C0 >= 128 ? (two ? 24 : 16) : (MODES == kMoments ? 16 : (FEW ? 32 : 24));
     static constexpr bool tight = two || FEW;
 };
 
-template <int C0, int L, bool HASR, bool UNI> struct BwdSmem {          // dynamic shared memory of the backward kernel
-    using W = Widths<C0, L, BwdShape<C0, L, HASR, UNI, false>::G>;
+template <int C0, int L, int MODES, bool UNI> struct BwdSmem {          // dynamic shared memory of the backward kernel
+    using W = Widths<C0, L, BwdShape<C0, L, MODES, UNI, false>::G>;
     static constexpr int queue_floats = 32 * 4 + 5 * 32;    // queue of in-range edges: int4 and five scalars per slot
-    static constexpr int mode_floats = HASR ? 2 * 32 * kMaxR : 0;   // parked radial modes and their derivatives
-    static constexpr bool products = wide_channels(C0) && !HASR;    // reads the product table (product_piece)
+    static constexpr int mode_floats = MODES ? 2 * 32 * kMaxR : 0;   // parked radial modes and their derivatives or products
+    static constexpr bool products = wide_channels(C0);             // reads the product table (product_piece)
     static constexpr int n_red = products ? 1 : 2;                  // partial dot products per edge and lane pair
     static constexpr int per_warp = (32 * W::PB + n_red * 32 * (W::LH + 1) + W::NHI + 3) / 4 * 4 + mode_floats + queue_floats;   // floats
     static constexpr size_t bytes = kWarpsPerBlock * 9 * sizeof(double) + sizeof(float) * kWarpsPerBlock * per_warp;
@@ -386,10 +399,14 @@ template <int C0, int L, bool HASR, bool UNI> struct BwdSmem {          // dynam
 // than the registers: the channel-parallel phase waits on load latency (measured: 6-10 % on the
 // forward kernel at C0 = 8 .. 64, 2 % the other way at C0 = 128, which stays at 24 warps).
 // SPLIT: the warps of a block take a quarter each of one row (edge_rows_split) and add up their sums at the end.
-template <int C0, int L, bool HASR, bool UNI, bool SPLIT>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 ? 4 : 3) * 8 / kWarpsPerBlock)
+// MODES == kMoments: the scalar channels' sums get gamma g alone from the edges; the row's moments, for every species t of the
+// neighbours sum chi and sum chi q_mu, are left for moments.cu, which adds beta and U times them.  40,009 atoms of 64 species
+// with four modes: 1168 us with the 2.5 KB of these rows read per edge.
+template <int C0, int L, int MODES, bool UNI, bool SPLIT>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 && MODES != kMoments ? 4 : 3) * 8 / kWarpsPerBlock)
 k_edge_forward(const EdgeArgs a) {
     using W = Widths<C0, L>;
+    constexpr bool HASR = MODES != kNoModes;
     static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");
     // scratch per warp: the parked amplitudes of the batch, first the radial modes and then (once the
     // amplitudes are done) the harmonic weights chi^2 B_lm
@@ -400,6 +417,7 @@ k_edge_forward(const EdgeArgs a) {
     __shared__ int4 q_es[kWarpsPerBlock][32];
     __shared__ float q_d[kWarpsPerBlock][3 * 32];
     __shared__ double s_part[SPLIT ? kWarpsPerBlock : 1][2];
+    extern __shared__ __align__(16) float moments_s[];         // [warp][a.n_moments]
     chain_begin();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
@@ -448,14 +466,76 @@ k_edge_forward(const EdgeArgs a) {
             }
         }
     }
+    float* const mom = moments_s + (MODES == kMoments ? wid * a.n_moments : 0);
+    if (MODES == kMoments) {
+        for (int v = lane; v < a.n_moments; v += 32) mom[v] = 0.f;
+        __syncwarp();
+    }
     double s0 = 0.0, s1 = 0.0;   // normaliser sums in double: the calibration subtracts their mean
 
     auto run_batch = [&](const int nb) {     // the first nb queue slots
         if (HASR) {
-            eval_modes<false, W::PQ>(a, qes, nb, lane, qm, nullptr);
+            eval_modes<kValuesOnly, W::PQ>(a, qes, nb, lane, qm, nullptr);
             __syncwarp();
         }
         int it = 0;
+        if constexpr (MODES == kMoments) {
+            // moments: the edges of a species are added up by the first of them
+            const int tj = lane < nb ? qes[lane].y - ti * a.d.T : -1;
+            const unsigned same = __match_any_sync(kFull, tj);
+            if (tj >= 0 && (same & lt_mask) == 0) {
+                float v[1 + kMaxR];
+#pragma unroll
+                for (int q = 0; q <= kMaxR; ++q) v[q] = 0.f;
+                for (unsigned m = same; m; m &= m - 1) {
+                    const int b = __ffs(m) - 1;
+                    const float chi = __int_as_float(qes[b].w);
+                    v[0] += chi;
+#pragma unroll
+                    for (int q = 0; q < kMaxR; ++q) if (q < a.d.R) v[1 + q] += chi * qm[b * W::PQ + q];
+                }
+                float* const p = mom + tj * (1 + a.d.R);
+#pragma unroll
+                for (int q = 0; q <= kMaxR; ++q) if (q <= a.d.R) p[q] += v[q];
+            }
+            // the leading channels' whole amplitudes, four channels of an edge per lane
+            constexpr int LE = 32 / W::NL1;
+            for (int b0 = 0; b0 < nb; b0 += LE) {
+                const int b = b0 + lane / W::NL1, cc = 4 * (lane % W::NL1);
+                if (b < nb) {
+                    const int4 es = qes[b];
+                    float psi[4];
+                    amplitude4<C0, true, false, false>(a, es.x, __int_as_float(es.z), es.y, cc, psi, nullptr, qm + b * W::PQ, nullptr, k2, k3);
+                    *reinterpret_cast<float4*>(psi_s + b * W::PP + cc) = make_float4(psi[0], psi[1], psi[2], psi[3]);
+                }
+            }
+            // all channels: chi gamma g, two edges per step of a group of lanes
+            const size_t pitch = (size_t)(2 + a.d.R) * C0;
+            for (; it * W::EPI < nb; it += 2) {
+                float v[2][4];
+                float4 ga[2];
+                float chi[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int b = (it + h) * W::EPI + sub;
+                    chi[h] = 0.f;
+                    if (b < nb) {
+                        const int4 es = qes[b];
+                        chi[h] = __int_as_float(es.w);
+                        value_eval4(a.vtable, a.d.CP, es.x, c, __int_as_float(es.z), k2, k3, v[h]);
+                        ga[h] = ldg4(a.pairmod + (size_t)es.y * pitch + c);
+                    } else {
+                        v[h][0] = v[h][1] = v[h][2] = v[h][3] = 0.f;
+                        ga[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    acc0[0] += chi[h] * (ga[h].x * v[h][0]); acc0[1] += chi[h] * (ga[h].y * v[h][1]);
+                    acc0[2] += chi[h] * (ga[h].z * v[h][2]); acc0[3] += chi[h] * (ga[h].w * v[h][3]);
+                }
+            }
+        }
         if (W::EPI == 1 && !HASR) {
             // whole warp per edge: two edges per step, so that twelve 16-byte table and pair
             // loads are in flight per lane instead of six (the phase waits on their latency)
@@ -475,7 +555,7 @@ k_edge_forward(const EdgeArgs a) {
                 }
             }
         }
-        for (; it * W::EPI < nb; ++it) {
+        for (; MODES != kMoments && it * W::EPI < nb; ++it) {
             const int b = it * W::EPI + sub;
             if (b >= nb) continue;
             const int4 es = qes[b];
@@ -593,6 +673,10 @@ k_edge_forward(const EdgeArgs a) {
             for (int k = 0; k < 4; ++k) if (k < j_n[sl]) o[k] = accJ[sl][k];
         }
     }
+    if (MODES == kMoments) {
+        float* const out = a.moments + (size_t)(i - a.a0) * a.n_moments;
+        for (int v = lane; v < a.n_moments; v += 32) out[v] = mom[v];
+    }
     if (SPLIT) {
         if (lane == 0) { s_part[wid][0] = s0; s_part[wid][1] = s1; }
         __syncthreads();
@@ -622,12 +706,13 @@ k_edge_forward(const EdgeArgs a) {
 // the edge's lane then does the whole degree >= 1 contraction by itself against the
 // destination's gradient block held in shared memory, and assembles dE/dr_ij.  Edges in the
 // skin shell get a zero gradient as soon as their geometry is known.
-template <int C0, int L, bool HASR, bool UNI, bool FEW, bool SPLIT>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, BwdShape<C0, L, HASR, UNI, FEW>::warps / kWarpsPerBlock)
+// MODES == kMoments: beta and the modes enter the scalar channels through the row's H = (beta | U) G_0 (moments.cu).
+template <int C0, int L, int MODES, bool UNI, bool FEW, bool SPLIT>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, BwdShape<C0, L, MODES, UNI, FEW>::warps / kWarpsPerBlock)
 k_edge_backward(const EdgeArgs a) {
-    using SM = BwdSmem<C0, L, HASR, UNI>;
-    constexpr int G = BwdShape<C0, L, HASR, UNI, FEW>::G;
-    constexpr bool PR = SM::products;
+    using SM = BwdSmem<C0, L, MODES, UNI>;
+    constexpr int G = BwdShape<C0, L, MODES, UNI, FEW>::G;
+    constexpr bool PR = SM::products, HASR = MODES != kNoModes;
     using W = Widths<C0, L, G>;
     extern __shared__ __align__(16) unsigned char dsm[];
     double (*vsum)[9] = reinterpret_cast<double (*)[9]>(dsm);
@@ -641,6 +726,7 @@ k_edge_backward(const EdgeArgs a) {
     int4* const qes = reinterpret_cast<int4*>(wbase + SM::per_warp - SM::queue_floats);
     float* const qm = reinterpret_cast<float*>(qes) - SM::mode_floats;   // [2][32][kMaxR]
     float* const qd = reinterpret_cast<float*>(qes + 32);        // [5][32]
+    float* const mom = reinterpret_cast<float*>(dsm + SM::bytes) + (MODES == kMoments ? wid * a.n_moments : 0);   // [n_moments]
     const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
     const bool active = i < a.a1;
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
@@ -668,6 +754,8 @@ k_edge_backward(const EdgeArgs a) {
             h0[4 * gq] = v.x; h0[4 * gq + 1] = v.y; h0[4 * gq + 2] = v.z; h0[4 * gq + 3] = v.w;
         }
         for (int v = lane; v < W::NHI; v += 32) hi_s[v] = grow[a.d.offA[1] + v];
+        if (MODES == kMoments)
+            for (int v = lane; v < a.n_moments; v += 32) mom[v] = a.moments[(size_t)(i - a.a0) * a.n_moments + v];
         const float ds0 = grow[a.d.S], ds1 = grow[a.d.S + 1];
         __syncwarp();
         const float* H1 = hi_s;
@@ -677,7 +765,7 @@ k_edge_backward(const EdgeArgs a) {
 
         auto run_batch = [&](const int nb) {     // the first nb queue slots
             if (HASR) {
-                eval_modes<true, kMaxR>(a, qes, nb, lane, qm, qm + 32 * kMaxR);
+                eval_modes<PR ? kProducts : kDerivatives, kMaxR>(a, qes, nb, lane, qm, qm + 32 * kMaxR);
                 __syncwarp();
             }
             if constexpr (PR) {
@@ -687,8 +775,31 @@ k_edge_backward(const EdgeArgs a) {
                     const int b = b0 + lane / W::NL1, cc = 4 * (lane % W::NL1);
                     if (b < nb) {
                         const int4 es = qes[b];
+                        const float t = __int_as_float(es.z);
                         float psi[4];
-                        amplitude4<C0, false, false, UNI>(a, es.x, __int_as_float(es.z), es.y, cc, psi, nullptr, nullptr, nullptr, k2, k3);
+                        if constexpr (MODES == kMoments) {         // their products as well, from the same pair rows
+                            float d[4];
+                            const float* pm = a.pairmod + (size_t)es.y * (2 + a.d.R) * C0 + cc;
+                            const float dchi = qd[96 + b];
+                            value_eval4(a.vtable, a.d.CP, es.x, cc, t, k2, k3, psi);
+                            value_eval4(a.dtable, a.d.CP, es.x, cc, t, d1, d2, d);
+                            const float4 ga = ldg4(pm), be = ldg4(pm + C0);
+                            psi[0] = fmaf(ga.x, psi[0], be.x); psi[1] = fmaf(ga.y, psi[1], be.y);
+                            psi[2] = fmaf(ga.z, psi[2], be.z); psi[3] = fmaf(ga.w, psi[3], be.w);
+                            d[0] = fmaf(ga.x, d[0], be.x * dchi); d[1] = fmaf(ga.y, d[1], be.y * dchi);
+                            d[2] = fmaf(ga.z, d[2], be.z * dchi); d[3] = fmaf(ga.w, d[3], be.w * dchi);
+                            const float *qv = qm + b * kMaxR, *dq = qm + (32 + b) * kMaxR;
+#pragma unroll
+                            for (int m = 0; m < kMaxR; ++m) {
+                                if (m >= a.d.R) break;
+                                const float4 U = ldg4(pm + (size_t)(2 + m) * C0);
+                                psi[0] += U.x * qv[m]; psi[1] += U.y * qv[m]; psi[2] += U.z * qv[m]; psi[3] += U.w * qv[m];
+                                d[0] += U.x * dq[m]; d[1] += U.y * dq[m]; d[2] += U.z * dq[m]; d[3] += U.w * dq[m];
+                            }
+                            *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + cc) = make_float4(d[0], d[1], d[2], d[3]);
+                        } else {
+                            amplitude4<C0, HASR, false, UNI>(a, es.x, t, es.y, cc, psi, nullptr, qm + b * kMaxR, nullptr, k2, k3);
+                        }
                         *reinterpret_cast<float4*>(psi_s + b * W::PB + cc) = make_float4(psi[0], psi[1], psi[2], psi[3]);
                     }
                 }
@@ -703,10 +814,11 @@ k_edge_backward(const EdgeArgs a) {
 #pragma unroll
                         for (int gq = 0; gq < G; ++gq) {
                             float d[4];
-                            product4<C0, UNI>(a, es.x, t, es.y, c + gq * W::GOFF, dchi, d1, d2, d);
+                            product4<C0, MODES, UNI>(a, es.x, t, es.y, c + gq * W::GOFF, dchi, qm + (32 + b) * kMaxR, d1, d2, d);
 #pragma unroll
                             for (int k = 0; k < 4; ++k) pa += h0[4 * gq + k] * d[k];
-                            if (gq == 0 && cl < W::NL1)     // the leading C1 channels all sit in group 0
+                            // the leading C1 channels all sit in group 0
+                            if (MODES != kMoments && gq == 0 && cl < W::NL1)
                                 *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + c) = make_float4(d[0], d[1], d[2], d[3]);
                         }
                     }
@@ -763,10 +875,16 @@ k_edge_backward(const EdgeArgs a) {
                 // pr1 = sum_lm B_lm sum_c dps_c G_lmc.  By component, all channels in registers; where the registers are
                 // few (BwdShape), by four channels, which keeps the components' sums instead: 0.94 against 1.02 ms for
                 // the 128,000 atoms of five species, but 1.12 against 1.10 at 128 registers.
+                if (MODES == kMoments) {
+                    const float* hr = mom + (qes[lane].y - ti * a.d.T) * (1 + a.d.R);
+                    sa += dchi * hr[0];
+#pragma unroll
+                    for (int q = 0; q < kMaxR; ++q) if (q < a.d.R) sa += qm[(32 + lane) * kMaxR + q] * hr[1 + q];
+                }
                 float B1[3], B2[5], B3[7], B4[9], t1[3], t2[5], t3[7], t4[9];
                 harmonics_s1<L>(gux, guy, guz, B1, B2, B3, B4);
                 float bt = 0.f, pr1 = 0.f;
-                if constexpr (BwdShape<C0, L, HASR, UNI, FEW>::tight) {
+                if constexpr (BwdShape<C0, L, MODES, UNI, FEW>::tight) {
                     const float* pr = psi_s + lane * W::PB;
 #pragma unroll
                     for (int m = 0; m < 3; ++m) t1[m] = 0.f;
@@ -941,18 +1059,29 @@ k_edge_backward(const EdgeArgs a) {
 // per-pair amplitude tables already hold the modes, so the kernels without them are used
 template <int C0, int L, bool SPLIT>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
-    auto kern = a.uni ? k_edge_forward<C0, L, false, true, SPLIT>
-                      : (a.d.R > 0 ? k_edge_forward<C0, L, true, false, SPLIT> : k_edge_forward<C0, L, false, false, SPLIT>);
+    auto kern = a.uni ? k_edge_forward<C0, L, kNoModes, true, SPLIT>
+                      : (a.d.R > 0 ? k_edge_forward<C0, L, kModesPerEdge, false, SPLIT> : k_edge_forward<C0, L, kNoModes, false, SPLIT>);
+    if constexpr (wide_channels(C0) && !SPLIT) {
+        if (a.moments) {
+            kern = k_edge_forward<C0, L, kMoments, false, false>;
+            const size_t bytes = sizeof(float) * kWarpsPerBlock * a.n_moments;
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            if (e != cudaSuccess) return e;
+            kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
     kern<<<blocks, kWarpsPerBlock * 32, 0, st>>>(a);
     return cudaGetLastError();
 }
-template <int C0, int L, bool HASR, bool UNI>
+template <int C0, int L, int MODES, bool UNI>
 cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
     const bool few = a.a1 - a.a0 > 148 * 24 && a.a1 - a.a0 <= 148 * 32;
-    constexpr size_t bytes = BwdSmem<C0, L, HASR, UNI>::bytes;
-    constexpr bool FEW = C0 <= 64;           // (wider ones have no such variant)
-    auto kern = split ? k_edge_backward<C0, L, HASR, UNI, false, true>
-                      : (few ? k_edge_backward<C0, L, HASR, UNI, FEW, false> : k_edge_backward<C0, L, HASR, UNI, false, false>);
+    constexpr bool FEW = C0 <= 64 && MODES != kMoments;           // (the others have no such variant)
+    size_t bytes = BwdSmem<C0, L, MODES, UNI>::bytes;
+    auto kern = few ? k_edge_backward<C0, L, MODES, UNI, FEW, false> : k_edge_backward<C0, L, MODES, UNI, false, false>;
+    if constexpr (MODES == kMoments) bytes += sizeof(float) * kWarpsPerBlock * a.n_moments;
+    else if (split) kern = k_edge_backward<C0, L, MODES, UNI, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
@@ -961,9 +1090,12 @@ cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t
 template <bool FWD, int C0, int L>
 cudaError_t launch(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
     if (FWD) return split ? launch_fwd_r<C0, L, true>(a, blocks, st) : launch_fwd_r<C0, L, false>(a, blocks, st);
-    if (a.uni) return launch_bwd_r<C0, L, false, true>(a, blocks, split, st);
-    if (a.d.R > 0) return launch_bwd_r<C0, L, true, false>(a, blocks, split, st);
-    return launch_bwd_r<C0, L, false, false>(a, blocks, split, st);
+    if (a.uni) return launch_bwd_r<C0, L, kNoModes, true>(a, blocks, split, st);
+    if constexpr (wide_channels(C0)) {
+        if (a.moments) return launch_bwd_r<C0, L, kMoments, false>(a, blocks, false, st);
+    }
+    if (a.d.R > 0) return launch_bwd_r<C0, L, kModesPerEdge, false>(a, blocks, split, st);
+    return launch_bwd_r<C0, L, kNoModes, false>(a, blocks, split, st);
 }
 
 template <bool FWD>

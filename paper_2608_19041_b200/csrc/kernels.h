@@ -73,6 +73,10 @@ struct EdgeArgs {
     const float* dtable_uni;
     const int* species_slot;    // [T] species -> index among the species present; null: the records hold that index
     int n_present;
+    // shared radial modes without per-pair tables, from enough rows on: [a1 - a0][n_moments] moments of the rows (forward)
+    // or gradients of them (backward), see moments.cu; null: every edge reads its pair's mode mixing
+    float* moments;
+    int n_moments;
 };
 constexpr int kEdgeRowsPerBlock = 4, kEdgeSplitRows = 1184;
 // present: device array of the n_present species indices, ascending
@@ -124,6 +128,29 @@ cudaError_t launch_chained(void (*kern)(P...), unsigned blocks, unsigned threads
     c.attrs = &at; c.numAttrs = capturing == cudaStreamCaptureStatusNone ? 1 : 0;
     return cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);
 }
+
+// ---- moments.cu ----------------------------------------------------------------------
+struct MomentArgs {
+    Dims d;
+    const float* pairmod;
+    const int* type_s;
+    const int* order;       // rows of the tile by species (launch_moment_groups)
+    int a0, n;              // tile start (sorted index) and row count
+    float* state;           // [n][SP]
+    float* moments;         // [n][moment_pitch]
+};
+// From 2048 rows on (the two edge kernels and the products, C0 = 128 with 64 species and four modes, by moments against every
+// edge reading its pair's rows: 2100 rows 150 against 211 us, 4000 235 against 406, 40,009 1510 against 2638); below, whole
+// blocks of 64 rows of a species are mostly padding.  640 moments (2.5 KB a row) keep the blocks that fit on an SM.
+constexpr int kMaxMoments = 640, kMomentRows = 2048;
+int moment_pitch(const Dims& d);
+// whether a tile of so many rows, without per-pair tables, takes the way over moments (true for n implies true for more)
+bool moments_pick(const Dims& d, int64_t rows);
+int64_t moment_order_ints(const Dims& d, int64_t rows);
+// type_s: of the tile; scratch: 2 T ints
+cudaError_t launch_moment_groups(const Dims& d, const int* type_s, int n, int* scratch, int* order, cudaStream_t st);
+cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st);    // state += (beta | U)^T moments
+cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st);   // moments = (beta | U) state
 
 // ---- invariants.cu -------------------------------------------------------------------
 struct InvArgs {

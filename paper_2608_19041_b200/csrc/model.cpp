@@ -335,16 +335,15 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         // values alone: quadratic pieces about the middle of (a fraction of) the interval
         d.v_sub = 1;
         while (D1 / d.v_sub > 0.0025) d.v_sub *= 2;
-        // the product table of the radial map is kept without shared modes only, but with them the per-pair tables hold the
-        // same products of gamma g + beta + U q: their bound is checked on the columns of g and q and on a constant
-        const bool wide = wide_channels(C0), products = wide && R == 0;
+        // (the bound of products of gamma g + beta + U q is checked on the columns of g and q and on a constant)
+        const bool wide = wide_channels(C0);
         std::vector<float> va, da;
         float v[4], q[4];                                  // largest a0, a1, a2 and cubic term: of the values, of the products
         for (;; d.v_sub *= 2) {
             const double w = D1 / d.v_sub, hw = 0.5 * w;
             const size_t rows = (size_t)n_rows * d.v_sub;
             va.resize(rows * 3 * NC);
-            da.resize((products ? rows : 1) * 3 * NC);
+            if (wide) da.resize(rows * 3 * NC);
             std::vector<float> cubic(NC);
             double k[4] = {0, 0, 0, 0};                    // of the constant
             for (int i = 0; i < 4; ++i) v[i] = q[i] = 0.f;
@@ -365,7 +364,7 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
                     envelope_derivatives(s * D1 + mid, m->rc, e);
                     product_piece(1, 0, 0, 0, mid, hw, e, p);
                     for (int i = 0; i < 4; ++i) k[i] = std::max(k[i], std::fabs(p[i]));
-                    float* t = &da[(products ? vrow : 0) * 3 * NC];
+                    float* t = &da[vrow * 3 * NC];
                     for (int c = 0; c < NC; ++c) {
                         product_piece(ya[c], ya[NC + c], c2[c], c3[c], mid, hw, e, p);
                         t[c] = (float)p[0]; t[NC + c] = (float)p[1]; t[2 * NC + c] = (float)p[2]; x[c] = (float)p[3];
@@ -396,7 +395,7 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         };
         pack(va, d.tab_v1, d.tab_v2, &m->vtable);
         m->dtable.clear();
-        if (products) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
+        if (wide) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
     }
 
     // ---- ordered type-pair cache -----------------------------------------------------
