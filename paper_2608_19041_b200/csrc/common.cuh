@@ -106,23 +106,30 @@ typedef long long eidx_t;      // edge offsets are 64-bit: a list may hold more 
 // own scale (c2 = k2 I2, c3 = k3 I3; k = largest magnitude in the table / largest integer) cost
 // nothing in the value and leave the derivative within a few 1e-7 of its largest entry at the
 // default spacing (the error grows with the spacing like the interpolation error itself).
-// One 32-bit word: I2 in the upper 20 bits, I3 in the lower 12, both two's complement.  (A word whose parts
-// decode without shifts, the low bits through the mantissa of 2^23, took an addition more and was 3 to 8 %
-// slower in the forward kernel.)
-constexpr int kTabI2Max = (1 << 19) - 1, kTabI3Max = (1 << 11) - 1;
+// One 32-bit word: 4096 I2 + I3, two's complement.  The word as a whole, as a number, is 4096 times I2 + I3 / 4096, and I2 is
+// rounded so that this is what represents c2: one conversion gives it (scale k2 / 4096), a shift and another one I3 (the
+// lower 12 bits at the top of a word, scale k3 / 2^20), where the two parts as bit fields took two shifts more per channel.
+// (A word whose parts decode without conversions, the low bits through the mantissa of 2^23, took an addition more and
+// was 3 to 8 % slower in the forward kernel.)
+constexpr int kTabI2Max = (1 << 19) - 2, kTabI3Max = (1 << 11) - 1;
+constexpr float kTabHi = 1.0f / 4096.0f, kTabLo = 1.0f / 1048576.0f;     // scales of the two converted numbers, in units of k2 and k3
 __host__ __device__ inline float tab_step2(float max_abs_c2) { return max_abs_c2 * (1.0f / (float)kTabI2Max); }
 __host__ __device__ inline float tab_step3(float max_abs_c3) { return max_abs_c3 * (1.0f / (float)kTabI3Max); }
 __host__ __device__ inline unsigned tab_pack(float c2, float c3, float k2, float k3) {
     // (no branch in it: the host packs rows of channels, several at a time)
     float q2 = c2 / (k2 > 0.f ? k2 : 1.f), q3 = c3 / (k3 > 0.f ? k3 : 1.f);      // (a step of zero has zeros to pack)
-    q2 = q2 < (float)kTabI2Max ? q2 : (float)kTabI2Max; q2 = q2 > -(float)kTabI2Max ? q2 : -(float)kTabI2Max;
     q3 = q3 < (float)kTabI3Max ? q3 : (float)kTabI3Max; q3 = q3 > -(float)kTabI3Max ? q3 : -(float)kTabI3Max;
-    const int i2 = (int)(q2 + copysignf(0.5f, q2)), i3 = (int)(q3 + copysignf(0.5f, q3));
-    return ((unsigned)i2 << 12) | ((unsigned)i3 & 0xfffu);
+    const int i3 = (int)(q3 + copysignf(0.5f, q3));
+    q2 -= (float)i3 * kTabHi;
+    q2 = q2 < (float)kTabI2Max ? q2 : (float)kTabI2Max; q2 = q2 > -(float)kTabI2Max ? q2 : -(float)kTabI2Max;
+    const int i2 = (int)(q2 + copysignf(0.5f, q2));
+    return ((unsigned)i2 << 12) + (unsigned)i3;
 }
+__host__ __device__ inline float tab_hi(unsigned w) { return (float)(int)w; }
+__host__ __device__ inline float tab_lo(unsigned w) { return (float)(int)(w << 20); }
 __host__ __device__ inline void tab_unpack(unsigned w, float k2, float k3, float* c2, float* c3) {
-    *c2 = k2 * (float)((int)w >> 12);
-    *c3 = k3 * (float)((int)(w << 20) >> 20);
+    *c2 = (k2 * kTabHi) * tab_hi(w);
+    *c3 = (k3 * kTabLo) * tab_lo(w);
 }
 
 // Value table.  A pass that needs no derivative reads two words per channel instead of three: the piece is

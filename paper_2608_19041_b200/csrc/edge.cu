@@ -177,39 +177,66 @@ __device__ __forceinline__ void harmonics_grad_contract(float x, float y, float 
     *gx = ax; *gy = ay; *gz = az;
 }
 
+// a b + c of two channels: in one instruction (PAIR), which saves issue slots, or in two, which leaves the registers where they
+// are: the forward kernel at C0 = 128 with the pair cache takes 378 us with single multiply-adds and 443 with pairs (40,009 atoms of
+// 64 species, 80 registers), the backward kernel 449 with pairs and 466 without; C0 = 64, 32,400 atoms, forward 160 and 164.
+template <bool PAIR>
+__device__ __forceinline__ float2 axpy2(float2 a, float2 b, float2 c) {
+    return PAIR ? ffma2(a, b, c) : make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4& v) { return make_float2(v.z, v.w); }
+// the two numbers of a packed word of two channels (common.cuh, tab_pack)
+__device__ __forceinline__ float2 word_hi2(int a, int b) { return make_float2(tab_hi(a), tab_hi(b)); }
+__device__ __forceinline__ float2 word_lo2(int a, int b) { return make_float2(tab_lo(a), tab_lo(b)); }
+
 // value and derivative of four consecutive table channels at offset t in row `row`: three
-// 16-byte loads, c0, c1 and the packed (c2, c3) words with steps k2, k3 (common.cuh, tab_pack)
+// 16-byte loads, c0, c1 and the packed (c2, c3) words with steps k2, k3
 __device__ __forceinline__ void table_eval4(const float* __restrict__ table, int CP, int row, int c, float t,
                                             float k2, float k3, float* v, float* dv) {
     const float* p = table + (size_t)row * 3 * CP + c;
     const float4 c0 = ldg4(p), c1 = ldg4(p + CP);
     const int4 w = __ldg(reinterpret_cast<const int4*>(p + 2 * CP));
-    const float u2 = k2 * t * t, u3 = k3 * t * t * t;           // c2 t^2 = I2 u2, c3 t^3 = I3 u3
-    const float v2 = 2.0f * k2 * t, v3 = 3.0f * k3 * t * t;
-#define UMLMD_PIECE(k, f)                                                                              \
-    {                                                                                                  \
-        const float i2 = (float)(w.f >> 12), i3 = (float)((w.f << 20) >> 20);                          \
-        v[k] = fmaf(i3, u3, fmaf(i2, u2, fmaf(c1.f, t, c0.f)));                                        \
-        dv[k] = fmaf(i3, v3, fmaf(i2, v2, c1.f));                                                      \
-    }
-    UMLMD_PIECE(0, x) UMLMD_PIECE(1, y) UMLMD_PIECE(2, z) UMLMD_PIECE(3, w)
-#undef UMLMD_PIECE
+    const float s2 = k2 * kTabHi * t, s3 = k3 * kTabLo * t * t;
+    const float2 tt = both(t), u2 = both(s2 * t), u3 = both(s3 * t), v2 = both(2.0f * s2), v3 = both(3.0f * s3);
+    const float2 ha = word_hi2(w.x, w.y), hb = word_hi2(w.z, w.w), la = word_lo2(w.x, w.y), lb = word_lo2(w.z, w.w);
+    const float2 a = ffma2(la, u3, ffma2(ha, u2, ffma2(lo2(c1), tt, lo2(c0)))), b = ffma2(lb, u3, ffma2(hb, u2, ffma2(hi2(c1), tt, hi2(c0))));
+    const float2 da = ffma2(la, v3, ffma2(ha, v2, lo2(c1))), db = ffma2(lb, v3, ffma2(hb, v2, hi2(c1)));
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    dv[0] = da.x; dv[1] = da.y; dv[2] = db.x; dv[3] = db.y;
 }
 // values alone, from the value table (common.cuh, value_piece): two 16-byte loads, t from the middle of the
 // piece, k2 and k3 the steps of its linear and quadratic coefficients.  The forward kernel is bound by what it
 // pulls from L2 and through the L1 data pipe, and a row is 8 bytes per channel instead of the 12 of the table
 // with derivatives: 1,000,000 atoms of 64 species at C0 = 128 11.9 -> 10.3 ms, 128,000 of five species 0.84 ->
 // 0.69, 64,000 of one 1.02 -> 0.84, 216,000 at C0 = 8 0.867 -> 0.807.
+template <bool PAIR = true>
 __device__ __forceinline__ void value_eval4(const float* __restrict__ table, int CP, int row, int c, float t,
                                             float k2, float k3, float* v) {
     const float* p = table + (size_t)row * 2 * CP + c;
     const float4 a0 = ldg4(p);
     const int4 w = __ldg(reinterpret_cast<const int4*>(p + CP));
-    const float u1 = k2 * t, u2 = k3 * t * t;
-#define UMLMD_PIECE(k, f) v[k] = fmaf((float)((w.f << 20) >> 20), u2, fmaf((float)(w.f >> 12), u1, a0.f));
-    UMLMD_PIECE(0, x) UMLMD_PIECE(1, y) UMLMD_PIECE(2, z) UMLMD_PIECE(3, w)
-#undef UMLMD_PIECE
+    const float2 u1 = both(k2 * kTabHi * t), u2 = both(k3 * kTabLo * t * t);
+    const float2 a = axpy2<PAIR>(word_lo2(w.x, w.y), u2, axpy2<PAIR>(word_hi2(w.x, w.y), u1, lo2(a0)));
+    const float2 b = axpy2<PAIR>(word_lo2(w.z, w.w), u2, axpy2<PAIR>(word_hi2(w.z, w.w), u1, hi2(a0)));
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
+// v += s u, four channels
+template <bool PAIR = true>
+__device__ __forceinline__ void axpy4(float s, const float4& u, float* v) {
+    const float2 a = axpy2<PAIR>(both(s), lo2(u), make_float2(v[0], v[1])), b = axpy2<PAIR>(both(s), hi2(u), make_float2(v[2], v[3]));
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+template <bool PAIR = true>
+__device__ __forceinline__ void axpy4(float s, const float* u, float* v) { axpy4<PAIR>(s, make_float4(u[0], u[1], u[2], u[3]), v); }
+// v = u v + w, four channels
+template <bool PAIR = true>
+__device__ __forceinline__ void affine4(const float4& u, const float4& w, float* v) {
+    const float2 a = axpy2<PAIR>(lo2(u), make_float2(v[0], v[1]), lo2(w)), b = axpy2<PAIR>(hi2(u), make_float2(v[2], v[3]), hi2(w));
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ float4 scaled(float s, const float4& u) { return make_float4(s * u.x, s * u.y, s * u.z, s * u.w); }
 
 // Shared radial modes q_mu(rho) of the first nb queued edges, an edge per lane, parked as qm[edge * PQ + mu]: evaluated once
 // per edge here instead of once per lane in the channel-parallel phase.  (Rows are padded to whole fours of columns.)
@@ -235,7 +262,7 @@ __device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, i
 enum : int { kNoModes = 0, kModesPerEdge = 1, kMoments = 2 };
 
 // adds sum_mu U_c,mu q_mu of four channels; pm: the pair's rows at the channel
-template <int C0>
+template <int C0, bool PAIR = true>
 __device__ __forceinline__ void add_modes4(const EdgeArgs& a, const float* pm, const float* qm, float* v) {
     const int R = a.d.R;
     float q[kMaxR];
@@ -245,8 +272,7 @@ __device__ __forceinline__ void add_modes4(const EdgeArgs& a, const float* pm, c
 #pragma unroll
     for (int m = 0; m < kMaxR; ++m) {
         if (m >= R) break;
-        const float4 U = ldg4(pm + (size_t)(2 + m) * C0);
-        v[0] += U.x * q[m]; v[1] += U.y * q[m]; v[2] += U.z * q[m]; v[3] += U.w * q[m];
+        axpy4<PAIR>(q[m], ldg4(pm + (size_t)(2 + m) * C0), v);
     }
 }
 
@@ -255,42 +281,23 @@ __device__ __forceinline__ void add_modes4(const EdgeArgs& a, const float* pm, c
 // species present is tabulated by itself (a.table_uni, row pitch C0; `row` already points into
 // the edge's pair), so neither pair rows nor modes are read.  k2, k3: steps of the packed
 // coefficients of the table that is read
-template <int C0, bool HASR, bool DERIV, bool UNI>
+template <int C0, bool HASR, bool DERIV, bool UNI, bool PAIR = true>
 __device__ __forceinline__ void amplitude4(const EdgeArgs& a, int row, float t, int pair, int c, float* psi,
                                            float* dpsi, const float* qm, const float* dqm, float k2, float k3) {
     if (UNI) {
         if (DERIV) table_eval4(a.table_uni, C0, row, c, t, k2, k3, psi, dpsi);
-        else value_eval4(a.vtable_uni, C0, row, c, t, k2, k3, psi);
+        else value_eval4<PAIR>(a.vtable_uni, C0, row, c, t, k2, k3, psi);
         return;
     }
-    float g[4], dg[4];
-    if (DERIV) table_eval4(a.table, a.d.CP, row, c, t, k2, k3, g, dg);
-    else value_eval4(a.vtable, a.d.CP, row, c, t, k2, k3, g);
-    const int R = HASR ? a.d.R : 0;
-    const float* pm = a.pairmod + (size_t)pair * (2 + R) * C0 + c;
+    if (DERIV) table_eval4(a.table, a.d.CP, row, c, t, k2, k3, psi, dpsi);
+    else value_eval4<PAIR>(a.vtable, a.d.CP, row, c, t, k2, k3, psi);
+    const float* pm = a.pairmod + (size_t)pair * (2 + (HASR ? a.d.R : 0)) * C0 + c;
     const float4 ga = ldg4(pm), be = ldg4(pm + C0);
-    psi[0] = ga.x * g[0] + be.x; psi[1] = ga.y * g[1] + be.y;
-    psi[2] = ga.z * g[2] + be.z; psi[3] = ga.w * g[3] + be.w;
-    if (DERIV) { dpsi[0] = ga.x * dg[0]; dpsi[1] = ga.y * dg[1]; dpsi[2] = ga.z * dg[2]; dpsi[3] = ga.w * dg[3]; }
+    affine4<PAIR>(ga, be, psi);
+    if (DERIV) { dpsi[0] *= ga.x; dpsi[1] *= ga.y; dpsi[2] *= ga.z; dpsi[3] *= ga.w; }
     if (HASR) {
-        float qv[kMaxR], dqv[kMaxR];
-        {
-            const float4 v0 = *reinterpret_cast<const float4*>(qm);
-            qv[0] = v0.x; qv[1] = v0.y; qv[2] = v0.z; qv[3] = v0.w;
-            if (R > 4) { const float4 v1 = *reinterpret_cast<const float4*>(qm + 4); qv[4] = v1.x; qv[5] = v1.y; qv[6] = v1.z; qv[7] = v1.w; }
-            if (DERIV) {
-                const float4 d0 = *reinterpret_cast<const float4*>(dqm);
-                dqv[0] = d0.x; dqv[1] = d0.y; dqv[2] = d0.z; dqv[3] = d0.w;
-                if (R > 4) { const float4 d1 = *reinterpret_cast<const float4*>(dqm + 4); dqv[4] = d1.x; dqv[5] = d1.y; dqv[6] = d1.z; dqv[7] = d1.w; }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < kMaxR; ++q) {
-            if (q >= R) break;
-            const float4 U = ldg4(pm + (size_t)(2 + q) * C0);
-            psi[0] += U.x * qv[q]; psi[1] += U.y * qv[q]; psi[2] += U.z * qv[q]; psi[3] += U.w * qv[q];
-            if (DERIV) { dpsi[0] += U.x * dqv[q]; dpsi[1] += U.y * dqv[q]; dpsi[2] += U.z * dqv[q]; dpsi[3] += U.w * dqv[q]; }
-        }
+        add_modes4<C0, PAIR>(a, pm, qm, psi);
+        if (DERIV) add_modes4<C0>(a, pm, dqm, dpsi);
     }
 }
 
@@ -304,23 +311,21 @@ __device__ __forceinline__ void product4(const EdgeArgs& a, int row, float t, in
         value_eval4(a.dtable_uni, C0, row, c, t, d1, d2, d);
         return;
     }
-    float g[4];
-    value_eval4(a.dtable, a.d.CP, row, c, t, d1, d2, g);
+    value_eval4(a.dtable, a.d.CP, row, c, t, d1, d2, d);
     const float* pm = a.pairmod + (size_t)pair * (MODES ? 2 + a.d.R : 2) * C0 + c;
     const float4 ga = ldg4(pm);
     if (MODES == kMoments) {
-        d[0] = ga.x * g[0]; d[1] = ga.y * g[1]; d[2] = ga.z * g[2]; d[3] = ga.w * g[3];
+        d[0] *= ga.x; d[1] *= ga.y; d[2] *= ga.z; d[3] *= ga.w;
         return;
     }
-    const float4 be = ldg4(pm + C0);
-    d[0] = fmaf(ga.x, g[0], be.x * dchi); d[1] = fmaf(ga.y, g[1], be.y * dchi);
-    d[2] = fmaf(ga.z, g[2], be.z * dchi); d[3] = fmaf(ga.w, g[3], be.w * dchi);
+    affine4(ga, scaled(dchi, ldg4(pm + C0)), d);
     if (MODES) add_modes4<C0>(a, pm, dqm, d);
 }
 // G = groups of four channels a lane holds in the channel-parallel phase (group g starts at
 // channel 4 * lane_in_group + g * C0 / G, so every 16-byte load instruction of a group of lanes
 // still covers one contiguous segment)
-template <int C0, int L, int G = 1> struct Widths {
+// ROWS: amplitudes and weights of an edge in one row at C0 = 128 too (see VECW)
+template <int C0, int L, int G = 1, bool ROWS = false> struct Widths {
     static constexpr int C1 = C0 <= 16 ? 4 : (C0 <= 64 ? 8 : 16);
     static constexpr int C2 = C1 / 2 > 4 ? C1 / 2 : 4;
     static constexpr int LPE = C0 / (4 * G);    // lanes per edge in the channel-parallel phase
@@ -330,25 +335,24 @@ template <int C0, int L, int G = 1> struct Widths {
     static constexpr int NL1 = C1 / 4;          // lanes of a group that hold degree-1 channels
     static constexpr int NHI = 3 * C1 + 5 * C2 + (L >= 3 ? 7 : 0) + (L >= 4 ? 9 : 0);   // sums of degree >= 1
     static constexpr int PB = ((2 * C1 / 4 + 1) & 1) ? 2 * C1 + 4 : 2 * C1 + 8;   // backward: psi, dpsi
-    // Forward, sums of degree >= 1: a job is four multiply-adds per edge, a vector times a scalar.  Degrees 1
-    // and 2: four consecutive channels (vector) of one harmonic component (scalar).  Degrees 3 and 4 have
-    // one channel: where VECW, four components (vector) of it, else one component.  Below C0 = 128 the jobs
-    // are at most sixteen, so that EG groups of JW lanes take every EG-th edge each (with one group, 8 to 18
-    // lanes of 32 worked, over all edges: the forward kernel of 216,000 atoms with 158 neighbours at C0 = 8
-    // took 1.109 ms, so 0.867; C0 = 64: 4000 atoms 31.4 -> 29.1 us, 32,400 atoms with degree three 201 -> 198).
-    static constexpr bool VECW = C0 <= 64;
-    static constexpr int J1 = 3 * (C1 / 4), J2 = 5 * (C2 / 4), J3 = L >= 3 ? (VECW ? 2 : 7) : 0, J4 = L >= 4 ? (VECW ? 3 : 9) : 0;
-    static constexpr int NJ = J1 + J2 + J3 + J4;
-    static constexpr int JW = NJ <= 8 ? 8 : (NJ <= 16 ? 16 : 32), EG = 32 / JW;
-    static constexpr int SLOTS = (NJ + JW - 1) / JW;
-    // the parked row of an edge: leading C1 amplitudes, harmonic weights (degree 3 from 8 on, degree 4 from
-    // 15, or 16 where VECW).  VECW: one row, pitch / 4 odd, so that 16-byte accesses of eight consecutive
-    // lanes fall on distinct banks.  C0 = 128: a whole warp works on one edge, amplitude rows need no padding,
-    // and the weights sit behind them with an odd pitch, which takes less room (L1 is what is left over).
-    static constexpr int O4 = VECW ? 16 : 15;
-    static constexpr int NM = L >= 4 ? O4 + (VECW ? 12 : 9) : (L >= 3 ? (VECW ? 16 : 15) : 8);
+    // Forward, sums of degree >= 1: a job is four consecutive channels (vector) of two components of degrees 1 and 2, in their
+    // order (scalars; PAIRS): two reads of the parked row for eight multiply-adds.  (The L1 data pipe takes a cycle for every word
+    // that a lane reads, broadcast or not: a job of one component reads five words for four multiply-adds.  C0 = 64, 32,400 atoms,
+    // 170 -> 160 us; at C0 = 8, whose eight jobs of one component fill a group, 234 -> 244 for 64,000 atoms with 158 neighbours.)
+    // The channels that only degree 1 has get two pairs for its three components.  Degrees 3 and 4 have one channel: four
+    // components of them (vector) times that (scalar).  EG groups of JW lanes take every EG-th edge each.
+    static constexpr bool PAIRS = C0 >= 32;
+    static constexpr int JFULL = C2 / 4 * (PAIRS ? 4 : 8), JLOW = (C1 - C2) / 4 * (PAIRS ? 2 : 3), J3 = L >= 3 ? 2 : 0, J4 = L >= 4 ? 3 : 0;
+    static constexpr int NJ = JFULL + JLOW + J3 + J4;
+    static constexpr int JW = NJ <= 4 ? 4 : (NJ <= 8 ? 8 : (NJ <= 16 ? 16 : 32)), EG = 32 / JW;
+    // the parked row of an edge: leading C1 amplitudes, harmonic weights (degree 3 from 8 on, degree 4 from 16).  VECW: one
+    // row, pitch / 4 odd, so that 16-byte accesses of eight consecutive lanes fall on distinct banks.  C0 = 128 with per-pair
+    // tables: amplitude rows need no padding, and the weights sit behind them (40,009 atoms of five species 197 us, 214 in one
+    // row; with the pair cache the other way, 410 and 378 for 64 species).
+    static constexpr bool VECW = C0 <= 64 || ROWS;
+    static constexpr int NM = L >= 4 ? 28 : (L >= 3 ? 16 : 8);
     static constexpr int PP = VECW ? (((C1 + NM) / 4) & 1 ? C1 + NM : C1 + NM + 4) : C1;      // pitch of the amplitudes
-    static constexpr int PW = VECW ? PP : (NM | 1);                                           // pitch of the weights
+    static constexpr int PW = VECW ? PP : ((NM / 4) & 1 ? NM : NM + 4);                       // pitch of the weights
     static constexpr int OW = VECW ? C1 : 32 * C1;                                            // offset of the weights
     static constexpr int PQ = VECW ? PP : kMaxR;     // the radial modes sit where the weights come later
     static constexpr int SCRATCH = VECW ? 32 * PP : 32 * C1 + (32 * PW > 32 * kMaxR ? 32 * PW : 32 * kMaxR);
@@ -395,17 +399,27 @@ template <int C0, int L, int MODES, bool UNI> struct BwdSmem {          // dynam
 //      components of a one-channel degree) for the whole row, and for every edge of its group of
 //      edges adds vector x scalar from the parked row: two shared-memory reads per edge and group of
 //      lanes, where summing per-edge products by transposition took six.
-// Up to C0 = 64 a fourth group of eight resident warps per SM (64 registers, a few spilled words) is worth more
-// than the registers: the channel-parallel phase waits on load latency (measured: 6-10 % on the
-// forward kernel at C0 = 8 .. 64, 2 % the other way at C0 = 128, which stays at 24 warps).
+// What hides the load latency of the channel-parallel phase best depends on the width and on what is read.  Up to C0 = 64, 32
+// warps per SM (64 registers, a few spilled words; 24 were 6 to 10 % slower).  C0 = 128: with per-pair tables an edge per half
+// warp, two channel groups per lane, at 24 warps (40,009 atoms of five species 196 us; two at 16 warps 242, four at 20 warps
+// 194); with shared table and pair cache four groups at 16 warps (131,072 atoms of 64 species 1184 us, 8000 93; two groups 1232
+// and 95, one at 24 warps 1212 and 100); the same by moments two groups at 20 warps (688 us, one at 24 700, four at 16 723,
+// 40,009 atoms with four modes).
+template <int C0, int MODES, bool UNI> struct FwdShape {
+    static constexpr bool cache = !UNI && MODES == kNoModes;
+    static constexpr int G = C0 < 128 || MODES == kModesPerEdge ? 1 : (cache ? 4 : 2);
+    static constexpr int warps = C0 < 128 ? (MODES < kMoments ? 32 : 24) : (cache ? 16 : (MODES == kMoments ? 20 : 24));
+};
 // SPLIT: the warps of a block take a quarter each of one row (edge_rows_split) and add up their sums at the end.
 // MODES == kMoments: the scalar channels' sums get gamma g alone from the edges; the row's moments, for every species t of the
 // neighbours sum chi and sum chi q_mu, are left for moments.cu, which adds beta and U times them.  40,009 atoms of 64 species
 // with four modes: 1168 us with the 2.5 KB of these rows read per edge.
 template <int C0, int L, int MODES, bool UNI, bool SPLIT>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, (C0 <= 64 && MODES != kMoments ? 4 : 3) * 8 / kWarpsPerBlock)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, FwdShape<C0, MODES, UNI>::warps / kWarpsPerBlock)
 k_edge_forward(const EdgeArgs a) {
-    using W = Widths<C0, L>;
+    constexpr int G = FwdShape<C0, MODES, UNI>::G;          // channel groups of a lane
+    constexpr bool PAIR = C0 < 128 || UNI;                  // see axpy2
+    using W = Widths<C0, L, G, !UNI>;
     constexpr bool HASR = MODES != kNoModes;
     static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");
     // scratch per warp: the parked amplitudes of the batch, first the radial modes and then (once the
@@ -436,36 +450,36 @@ k_edge_forward(const EdgeArgs a) {
     if (SPLIT) quarter_of_row(wid, &e0, &len);
     const int* Hf = a.frames ? a.frames[a.frame_of[i]].Hq : nullptr;
     const unsigned lt_mask = (1u << lane) - 1u;
-    float acc0[4] = {0.f, 0.f, 0.f, 0.f};
-    // this lane's jobs of the degree >= 1 sums: where its vector and its scalar are in the rows of edge 0, offset
-    // of the result in the output block, number of results (0: no job)
-    float accJ[W::SLOTS][4];
-    int j_v[W::SLOTS], j_s[W::SLOTS], j_out[W::SLOTS], j_n[W::SLOTS];
-    const int eg = lane / W::JW;
+    float acc0[4 * G];
 #pragma unroll
-    for (int sl = 0; sl < W::SLOTS; ++sl) {
-        accJ[sl][0] = accJ[sl][1] = accJ[sl][2] = accJ[sl][3] = 0.f;
-        const int j = lane % W::JW + W::JW * sl;
-        j_v[sl] = 0; j_s[sl] = W::OW; j_out[sl] = 0; j_n[sl] = 0;
-        if (j < W::J1) {
-            const int m = j / (W::C1 / 4), cb = j % (W::C1 / 4);
-            j_v[sl] = 4 * cb; j_s[sl] += m; j_out[sl] = m * W::C1 + 4 * cb; j_n[sl] = 4;
-        } else if (j < W::J1 + W::J2) {
-            const int jj = j - W::J1, m = jj / (W::C2 / 4), cb = jj % (W::C2 / 4);
-            j_v[sl] = 4 * cb; j_s[sl] += 3 + m; j_out[sl] = 3 * W::C1 + m * W::C2 + 4 * cb; j_n[sl] = 4;
-        } else if (j < W::NJ) {
-            const int jj = j - W::J1 - W::J2;
-            const bool deg3 = jj < W::J3;
-            const int first = W::VECW ? (deg3 ? 4 * jj : 4 * (jj - W::J3)) : (deg3 ? jj : jj - W::J3);   // component
-            j_out[sl] = 3 * W::C1 + 5 * W::C2 + (deg3 ? 0 : 7) + first;
-            if (W::VECW) {                  // vector: the weights, scalar: the channel's amplitude
-                j_v[sl] = W::OW + (deg3 ? 8 : W::O4) + first; j_s[sl] = 0;      // (one pitch for both)
-                j_n[sl] = min(4, (deg3 ? 7 : 9) - first);
-            } else {
-                j_s[sl] += (deg3 ? 8 : W::O4) + first; j_n[sl] = 1;
-            }
+    for (int k = 0; k < 4 * G; ++k) acc0[k] = 0.f;
+    // this lane's job of the degree >= 1 sums: where its vector and its scalars are in the rows of edge 0, offset of the
+    // results in the output block and their number, for each of its components
+    float2 accJ[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) accJ[k] = make_float2(0.f, 0.f);
+    int j_v = 0, j_s = W::OW, j_out[2] = {0, 0}, j_n[2] = {0, 0};
+    const int eg = lane / W::JW, job = lane % W::JW;
+    if (job < W::JFULL + W::JLOW) {
+        constexpr int NF = W::PAIRS ? 4 : 8, NL = W::PAIRS ? 2 : 3, NC = W::PAIRS ? 2 : 1;      // jobs of a run of channels, components of a job
+        const int cb = job < W::JFULL ? job / NF : W::C2 / 4 + (job - W::JFULL) / NL, part = job < W::JFULL ? job % NF : (job - W::JFULL) % NL;
+        j_v = 4 * cb; j_s += NC * part;
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+            const int m = NC * part + h;
+            if (m < 3) { j_out[h] = m * W::C1 + 4 * cb; j_n[h] = 4; }
+            else if (4 * cb < W::C2) { j_out[h] = 3 * W::C1 + (m - 3) * W::C2 + 4 * cb; j_n[h] = 4; }
         }
+    } else if (job < W::NJ) {
+        const int jj = job - W::JFULL - W::JLOW;
+        const bool deg3 = jj < W::J3;
+        const int first = deg3 ? 4 * jj : 4 * (jj - W::J3);      // component
+        j_v = W::OW + (deg3 ? 8 : 16) + first; j_s = 0;
+        j_out[0] = 3 * W::C1 + 5 * W::C2 + (deg3 ? 0 : 7) + first;
+        j_n[0] = min(4, (deg3 ? 7 : 9) - first);
     }
+    const bool swapped = job >= W::JFULL + W::JLOW && job < W::NJ;      // (weights and amplitudes change places in the jobs of one channel)
+    const int pitch_v = swapped ? W::PW : W::PP, pitch_s = swapped ? W::PP : W::PW;
     float* const mom = moments_s + (MODES == kMoments ? wid * a.n_moments : 0);
     if (MODES == kMoments) {
         for (int v = lane; v < a.n_moments; v += 32) mom[v] = 0.f;
@@ -478,7 +492,6 @@ k_edge_forward(const EdgeArgs a) {
             eval_modes<kValuesOnly, W::PQ>(a, qes, nb, lane, qm, nullptr);
             __syncwarp();
         }
-        int it = 0;
         if constexpr (MODES == kMoments) {
             // moments: the edges of a species are added up by the first of them
             const int tj = lane < nb ? qes[lane].y - ti * a.d.T : -1;
@@ -505,68 +518,35 @@ k_edge_forward(const EdgeArgs a) {
                 if (b < nb) {
                     const int4 es = qes[b];
                     float psi[4];
-                    amplitude4<C0, true, false, false>(a, es.x, __int_as_float(es.z), es.y, cc, psi, nullptr, qm + b * W::PQ, nullptr, k2, k3);
+                    amplitude4<C0, true, false, false, PAIR>(a, es.x, __int_as_float(es.z), es.y, cc, psi, nullptr, qm + b * W::PQ, nullptr, k2, k3);
                     *reinterpret_cast<float4*>(psi_s + b * W::PP + cc) = make_float4(psi[0], psi[1], psi[2], psi[3]);
                 }
             }
-            // all channels: chi gamma g, two edges per step of a group of lanes
-            const size_t pitch = (size_t)(2 + a.d.R) * C0;
-            for (; it * W::EPI < nb; it += 2) {
-                float v[2][4];
-                float4 ga[2];
-                float chi[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int b = (it + h) * W::EPI + sub;
-                    chi[h] = 0.f;
-                    if (b < nb) {
-                        const int4 es = qes[b];
-                        chi[h] = __int_as_float(es.w);
-                        value_eval4(a.vtable, a.d.CP, es.x, c, __int_as_float(es.z), k2, k3, v[h]);
-                        ga[h] = ldg4(a.pairmod + (size_t)es.y * pitch + c);
-                    } else {
-                        v[h][0] = v[h][1] = v[h][2] = v[h][3] = 0.f;
-                        ga[h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    acc0[0] += chi[h] * (ga[h].x * v[h][0]); acc0[1] += chi[h] * (ga[h].y * v[h][1]);
-                    acc0[2] += chi[h] * (ga[h].z * v[h][2]); acc0[3] += chi[h] * (ga[h].w * v[h][3]);
-                }
-            }
         }
-        if (W::EPI == 1 && !HASR) {
-            // whole warp per edge: two edges per step, so that twelve 16-byte table and pair
-            // loads are in flight per lane instead of six (the phase waits on their latency)
-            for (; it + 1 < nb; it += 2) {
-                const int4 ea = qes[it], eb = qes[it + 1];
-                float pa[4], pb[4];
-                amplitude4<C0, HASR, false, UNI>(a, ea.x, __int_as_float(ea.z), ea.y, c, pa, nullptr, nullptr, nullptr, k2, k3);
-                amplitude4<C0, HASR, false, UNI>(a, eb.x, __int_as_float(eb.z), eb.y, c, pb, nullptr, nullptr, nullptr, k2, k3);
-                const float ca = __int_as_float(ea.w), cb = __int_as_float(eb.w);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc0[k] += ca * pa[k];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc0[k] += cb * pb[k];
-                if (cl < W::NL1) {
-                    *reinterpret_cast<float4*>(psi_s + it * W::PP + c) = make_float4(pa[0], pa[1], pa[2], pa[3]);
-                    *reinterpret_cast<float4*>(psi_s + (it + 1) * W::PP + c) = make_float4(pb[0], pb[1], pb[2], pb[3]);
-                }
-            }
-        }
-        for (; MODES != kMoments && it * W::EPI < nb; ++it) {
+        // lanes = channels, a group of lanes per edge
+        constexpr int UNR = C0 >= 32 ? 1 : 2;     // (unrolled as the compiler would: C0 = 64, 32,400 atoms 185 us, so 160)
+#pragma unroll UNR
+        for (int it = 0; it * W::EPI < nb; ++it) {
             const int b = it * W::EPI + sub;
             if (b >= nb) continue;
             const int4 es = qes[b];
-            const int row = es.x, pair = es.y;
             const float t = __int_as_float(es.z), chi = __int_as_float(es.w);
-            float psi[4];
-            amplitude4<C0, HASR, false, UNI>(a, row, t, pair, c, psi, nullptr, qm + b * W::PQ, nullptr, k2, k3);
+            float psi[4 * G];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc0[k] += chi * psi[k];
-            if (cl < W::NL1)
-                *reinterpret_cast<float4*>(psi_s + b * W::PP + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
+            for (int gq = 0; gq < G; ++gq) {
+                const int cc = c + gq * W::GOFF;
+                if (MODES == kMoments) {
+                    value_eval4<PAIR>(a.vtable, a.d.CP, es.x, cc, t, k2, k3, psi + 4 * gq);
+                    const float4 ga = scaled(chi, ldg4(a.pairmod + (size_t)es.y * (2 + a.d.R) * C0 + cc));
+                    acc0[4 * gq] += ga.x * psi[4 * gq]; acc0[4 * gq + 1] += ga.y * psi[4 * gq + 1];
+                    acc0[4 * gq + 2] += ga.z * psi[4 * gq + 2]; acc0[4 * gq + 3] += ga.w * psi[4 * gq + 3];
+                } else {
+                    amplitude4<C0, HASR, false, UNI, PAIR>(a, es.x, t, es.y, cc, psi + 4 * gq, nullptr, qm + b * W::PQ, nullptr, k2, k3);
+                    axpy4<PAIR>(chi, psi + 4 * gq, acc0 + 4 * gq);
+                }
+            }
+            // (the leading C1 channels all sit in group 0)
+            if (MODES != kMoments && cl < W::NL1) *reinterpret_cast<float4*>(psi_s + b * W::PP + c) = make_float4(psi[0], psi[1], psi[2], psi[3]);
         }
         __syncwarp();
         // lane = edge: the harmonic weights chi^2 B_lm of the lane's edge, parked next to the amplitudes
@@ -578,44 +558,32 @@ k_edge_forward(const EdgeArgs a) {
             const float chi = __int_as_float(qes[lane].w);
             const float w = chi * chi;
             float* wr = wbs + lane * W::PW;
-            if (W::VECW) {
-                float4* w4 = reinterpret_cast<float4*>(wr);
-                w4[0] = make_float4(w * B1[0], w * B1[1], w * B1[2], w * B2[0]);
-                w4[1] = make_float4(w * B2[1], w * B2[2], w * B2[3], w * B2[4]);
-                if (L >= 3) {
-                    w4[2] = make_float4(w * B3[0], w * B3[1], w * B3[2], w * B3[3]);
-                    w4[3] = make_float4(w * B3[4], w * B3[5], w * B3[6], 0.f);
-                }
-                if (L >= 4) {
-                    w4[4] = make_float4(w * B4[0], w * B4[1], w * B4[2], w * B4[3]);
-                    w4[5] = make_float4(w * B4[4], w * B4[5], w * B4[6], w * B4[7]);
-                    w4[6] = make_float4(w * B4[8], 0.f, 0.f, 0.f);
-                }
-            } else {
-#pragma unroll
-                for (int m = 0; m < 3; ++m) wr[m] = w * B1[m];
-#pragma unroll
-                for (int m = 0; m < 5; ++m) wr[3 + m] = w * B2[m];
-                if (L >= 3) {
-#pragma unroll
-                    for (int m = 0; m < 7; ++m) wr[8 + m] = w * B3[m];
-                }
-                if (L >= 4) {
-#pragma unroll
-                    for (int m = 0; m < 9; ++m) wr[W::O4 + m] = w * B4[m];
-                }
+            float4* w4 = reinterpret_cast<float4*>(wr);
+            w4[0] = make_float4(w * B1[0], w * B1[1], w * B1[2], w * B2[0]);
+            w4[1] = make_float4(w * B2[1], w * B2[2], w * B2[3], w * B2[4]);
+            if (L >= 3) {
+                w4[2] = make_float4(w * B3[0], w * B3[1], w * B3[2], w * B3[3]);
+                w4[3] = make_float4(w * B3[4], w * B3[5], w * B3[6], 0.f);
+            }
+            if (L >= 4) {
+                w4[4] = make_float4(w * B4[0], w * B4[1], w * B4[2], w * B4[3]);
+                w4[5] = make_float4(w * B4[4], w * B4[5], w * B4[6], w * B4[7]);
+                w4[6] = make_float4(w * B4[8], 0.f, 0.f, 0.f);
             }
         }
         __syncwarp();
         // lane = job: the sums over the batch stay in the lane's registers for the whole row; per edge of
-        // its group a lane reads its vector and its scalar (every lane of a group inside the same two rows)
-#pragma unroll 4
+        // its group a lane reads its vector and its scalars (every lane of a group inside the same two rows)
+#pragma unroll 2
         for (int e = eg; e < nb; e += W::EG) {
-#pragma unroll
-            for (int sl = 0; sl < W::SLOTS; ++sl) {
-                const float4 p4 = *reinterpret_cast<const float4*>(psi_s + e * W::PP + j_v[sl]);
-                const float wv = psi_s[e * W::PW + j_s[sl]];
-                accJ[sl][0] += wv * p4.x; accJ[sl][1] += wv * p4.y; accJ[sl][2] += wv * p4.z; accJ[sl][3] += wv * p4.w;
+            const float4 p4 = *reinterpret_cast<const float4*>(psi_s + e * pitch_v + j_v);
+            if constexpr (W::PAIRS) {
+                const float2 w2 = *reinterpret_cast<const float2*>(psi_s + e * pitch_s + j_s);
+                accJ[0] = axpy2<PAIR>(both(w2.x), lo2(p4), accJ[0]); accJ[1] = axpy2<PAIR>(both(w2.x), hi2(p4), accJ[1]);
+                accJ[2] = axpy2<PAIR>(both(w2.y), lo2(p4), accJ[2]); accJ[3] = axpy2<PAIR>(both(w2.y), hi2(p4), accJ[3]);
+            } else {
+                const float wv = psi_s[e * pitch_s + j_s];
+                accJ[0] = axpy2<PAIR>(both(wv), lo2(p4), accJ[0]); accJ[1] = axpy2<PAIR>(both(wv), hi2(p4), accJ[1]);
             }
         }
         __syncwarp();                           // the next batch overwrites both
@@ -648,7 +616,7 @@ k_edge_forward(const EdgeArgs a) {
 #pragma unroll
     for (int off = W::LPE; off < 32; off <<= 1) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc0[k] += __shfl_xor_sync(kFull, acc0[k], off);
+        for (int k = 0; k < 4 * G; ++k) acc0[k] += __shfl_xor_sync(kFull, acc0[k], off);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -657,20 +625,29 @@ k_edge_forward(const EdgeArgs a) {
     }
     float* const row_glob = a.state + (size_t)(i - a.a0) * a.d.SP;
     float* const row_out = SPLIT ? psi_s : row_glob;        // (the batches are done with the scratch)
-    if (sub == 0) *reinterpret_cast<float4*>(row_out + c) = make_float4(acc0[0], acc0[1], acc0[2], acc0[3]);
+    if (sub == 0) {
 #pragma unroll
-    for (int sl = 0; sl < W::SLOTS; ++sl) {
+        for (int gq = 0; gq < G; ++gq)
+            *reinterpret_cast<float4*>(row_out + c + gq * W::GOFF) = make_float4(acc0[4 * gq], acc0[4 * gq + 1], acc0[4 * gq + 2], acc0[4 * gq + 3]);
+    }
 #pragma unroll
-        for (int off = W::JW; off < 32; off <<= 1) {
+    for (int off = W::JW; off < 32; off <<= 1) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) accJ[sl][k] += __shfl_xor_sync(kFull, accJ[sl][k], off);
+        for (int k = 0; k < 4; ++k) {
+            accJ[k].x += __shfl_xor_sync(kFull, accJ[k].x, off);
+            accJ[k].y += __shfl_xor_sync(kFull, accJ[k].y, off);
         }
-        if (eg != 0 || j_n[sl] == 0) continue;
-        float* o = row_out + a.d.offA[1] + j_out[sl];
-        if (lane + W::JW * sl < W::J1 + W::J2) *reinterpret_cast<float4*>(o) = make_float4(accJ[sl][0], accJ[sl][1], accJ[sl][2], accJ[sl][3]);
-        else {
+    }
+    if (eg == 0) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) if (k < j_n[sl]) o[k] = accJ[sl][k];
+        for (int h = 0; h < 2; ++h) {
+            float* o = row_out + a.d.offA[1] + j_out[h];
+            const float v[4] = {accJ[2 * h].x, accJ[2 * h].y, accJ[2 * h + 1].x, accJ[2 * h + 1].y};
+            if (j_n[h] == 4 && !swapped) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+            else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) if (k < j_n[h]) o[k] = v[k];
+            }
         }
     }
     if (MODES == kMoments) {
@@ -784,17 +761,15 @@ k_edge_backward(const EdgeArgs a) {
                             value_eval4(a.vtable, a.d.CP, es.x, cc, t, k2, k3, psi);
                             value_eval4(a.dtable, a.d.CP, es.x, cc, t, d1, d2, d);
                             const float4 ga = ldg4(pm), be = ldg4(pm + C0);
-                            psi[0] = fmaf(ga.x, psi[0], be.x); psi[1] = fmaf(ga.y, psi[1], be.y);
-                            psi[2] = fmaf(ga.z, psi[2], be.z); psi[3] = fmaf(ga.w, psi[3], be.w);
-                            d[0] = fmaf(ga.x, d[0], be.x * dchi); d[1] = fmaf(ga.y, d[1], be.y * dchi);
-                            d[2] = fmaf(ga.z, d[2], be.z * dchi); d[3] = fmaf(ga.w, d[3], be.w * dchi);
+                            affine4(ga, be, psi);
+                            affine4(ga, scaled(dchi, be), d);
                             const float *qv = qm + b * kMaxR, *dq = qm + (32 + b) * kMaxR;
 #pragma unroll
                             for (int m = 0; m < kMaxR; ++m) {
                                 if (m >= a.d.R) break;
                                 const float4 U = ldg4(pm + (size_t)(2 + m) * C0);
-                                psi[0] += U.x * qv[m]; psi[1] += U.y * qv[m]; psi[2] += U.z * qv[m]; psi[3] += U.w * qv[m];
-                                d[0] += U.x * dq[m]; d[1] += U.y * dq[m]; d[2] += U.z * dq[m]; d[3] += U.w * dq[m];
+                                axpy4(qv[m], U, psi);
+                                axpy4(dq[m], U, d);
                             }
                             *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + cc) = make_float4(d[0], d[1], d[2], d[3]);
                         } else {
@@ -807,7 +782,7 @@ k_edge_backward(const EdgeArgs a) {
                 for (int it = 0; it * W::EPI < nb; ++it) {
                     const int b = it * W::EPI + sub;
                     const bool act = b < nb;
-                    float pa = 0.f;
+                    float2 p2 = make_float2(0.f, 0.f);
                     if (act) {
                         const int4 es = qes[b];
                         const float t = __int_as_float(es.z), dchi = UNI ? 0.f : qd[96 + b];
@@ -815,8 +790,8 @@ k_edge_backward(const EdgeArgs a) {
                         for (int gq = 0; gq < G; ++gq) {
                             float d[4];
                             product4<C0, MODES, UNI>(a, es.x, t, es.y, c + gq * W::GOFF, dchi, qm + (32 + b) * kMaxR, d1, d2, d);
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) pa += h0[4 * gq + k] * d[k];
+                            p2 = ffma2(make_float2(h0[4 * gq], h0[4 * gq + 1]), make_float2(d[0], d[1]), p2);
+                            p2 = ffma2(make_float2(h0[4 * gq + 2], h0[4 * gq + 3]), make_float2(d[2], d[3]), p2);
                             // the leading C1 channels all sit in group 0
                             if (MODES != kMoments && gq == 0 && cl < W::NL1)
                                 *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + c) = make_float4(d[0], d[1], d[2], d[3]);
@@ -824,6 +799,7 @@ k_edge_backward(const EdgeArgs a) {
                     }
                     // neighbouring lanes are paired before the partial sums are parked, which halves
                     // the parking area (it decides how many blocks fit on an SM)
+                    float pa = p2.x + p2.y;
                     pa += __shfl_xor_sync(kFull, pa, 1);
                     if (act && !(cl & 1)) red[b * (W::LH + 1) + (cl >> 1)] = pa;
                 }
@@ -932,6 +908,52 @@ k_edge_backward(const EdgeArgs a) {
 #pragma unroll
                         for (int m = 0; m < 9; ++m) bt += B4[m] * t4[m];
                     }
+                } else if constexpr (C0 >= 128) {      // pairs of channels (narrower ones were 1 % slower that way)
+                    float2 ps[W::C1 / 2], dps[W::C1 / 2], ec[W::C1 / 2], pr2 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int q = 0; q < W::C1 / 4; ++q) {
+                        const float4 p4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + 4 * q);
+                        const float4 d4 = *reinterpret_cast<const float4*>(psi_s + lane * W::PB + W::C1 + 4 * q);
+                        ps[2 * q] = lo2(p4); ps[2 * q + 1] = hi2(p4);
+                        dps[2 * q] = lo2(d4); dps[2 * q + 1] = hi2(d4);
+                    }
+#pragma unroll
+                    for (int k = 0; k < W::C1 / 2; ++k) ec[k] = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        float2 tm = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int k = 0; k < W::C1 / 2; ++k) {
+                            const float2 hv = *reinterpret_cast<const float2*>(H1 + m * W::C1 + 2 * k);
+                            tm = ffma2(ps[k], hv, tm); ec[k] = ffma2(both(B1[m]), hv, ec[k]);
+                        }
+                        t1[m] = tm.x + tm.y; bt += B1[m] * t1[m];
+                    }
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) {
+                        float2 tm = make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int k = 0; k < W::C2 / 2; ++k) {
+                            const float2 hv = *reinterpret_cast<const float2*>(H2 + m * W::C2 + 2 * k);
+                            tm = ffma2(ps[k], hv, tm); ec[k] = ffma2(both(B2[m]), hv, ec[k]);
+                        }
+                        t2[m] = tm.x + tm.y; bt += B2[m] * t2[m];
+                    }
+#pragma unroll
+                    for (int m = 0; m < 7; ++m) {
+                        float tm = 0.f;
+                        if (L >= 3) { const float hv = H3[m]; tm = ps[0].x * hv; ec[0].x += B3[m] * hv; bt += B3[m] * tm; }
+                        t3[m] = tm;
+                    }
+#pragma unroll
+                    for (int m = 0; m < 9; ++m) {
+                        float tm = 0.f;
+                        if (L >= 4) { const float hv = H4[m]; tm = ps[0].x * hv; ec[0].x += B4[m] * hv; bt += B4[m] * tm; }
+                        t4[m] = tm;
+                    }
+#pragma unroll
+                    for (int k = 0; k < W::C1 / 2; ++k) pr2 = ffma2(ec[k], dps[k], pr2);
+                    pr1 = pr2.x + pr2.y;
                 } else {
                     float ps[W::C1], dps[W::C1], ec[W::C1];
 #pragma unroll
