@@ -34,6 +34,11 @@ struct umlmd {
     float* moments = nullptr; int64_t moments_cap = 0;
     int* moment_order = nullptr; int64_t order_cap = 0;
     int* moment_scratch = nullptr;
+    // scalar channels by splines (moments.cu): coefficients of the pair of spline_species, intervals
+    float* spline = nullptr; int64_t spline_cap = 0;
+    int spline_n = 0, spline_species = -1;
+    bool spline_failed = false;                      // the radial map takes more intervals than are worth it
+    std::vector<double> spline_coef;                 // of the radial map and modes
     bool have_groups = false;                        // moment_order belongs to the current list
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
@@ -208,6 +213,13 @@ int decode_device_errors(umlmd_t* h, int word) {
     return UMLMD_OK;
 }
 
+double mean_row(const umlmd_t* h) { return h->nb.N > 0 ? (double)h->nb.E / (double)h->nb.N : 0.0; }      // listed neighbours
+// rows of spline coefficients, padded to whole 16-byte pieces
+int spline_pitch(const umlmd_t* h) { return (h->spline_n + 7 + 3) / 4 * 4; }
+bool use_splines(const umlmd_t* h, int64_t rows) {
+    return h->pair_tables && h->present.size() == 1 && h->spline_n > 0 && h->spline_species == h->present[0] && splines_pick(h->d, rows, mean_row(h));
+}
+
 // what the records of the edge kernels hold in place of the species, null for the species itself
 const int* record_slots(const umlmd_t* h) { return h->pair_tables ? h->d_species + h->d.T : nullptr; }
 
@@ -238,9 +250,11 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         for (int k = 0; k < 9; ++k) ea.Hq[k] = to_quanta(nb.H[k], 1.0 / nb.quantum);
         ea.tri = nb.tri;
         ea.a0 = a0; ea.a1 = a0 + n; ea.state = h->state; ea.g = h->g;
-        const bool by_moments = h->have_groups && !h->pair_tables && moments_pick(d, n);
-        ea.moments = by_moments ? h->moments : nullptr; ea.n_moments = moment_pitch(d);
-        const MomentArgs mo = {d, h->md.pairmod, nb.type_s, h->moment_order + (a0 / B) * moment_order_ints(d, B), a0, n, h->state, h->moments};
+        const bool by_splines = use_splines(h, n), by_moments = by_splines || (h->have_groups && !h->pair_tables && moments_pick(d, n));
+        ea.moments = by_moments ? h->moments : nullptr; ea.n_moments = by_splines ? spline_pitch(h) : moment_pitch(d);
+        ea.spline_n = by_splines ? h->spline_n : 0; ea.spline_inv_h = (float)(h->spline_n / h->hm.rc);
+        const int* order = by_splines || !by_moments ? nullptr : h->moment_order + (a0 / B) * moment_order_ints(d, B);
+        const MomentArgs mo = {d, h->md.pairmod, nb.type_s, order, a0, n, h->state, h->moments, ea.n_moments, by_splines ? h->spline : nullptr};
         ea.virial_part = h->virial_part + (size_t)vpart_used * 9;
         {
             Scope sc(h, kEdgeFwd, 1 + by_moments);
@@ -477,11 +491,44 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     return UMLMD_OK;
 }
 
-// Groups the rows of the current list by species and makes room for their moments, where its kernels take that way.
+// Spline coefficients of the one pair of a system of one species; the fit (2 to 5 ms) is made once per model, by the first system
+// that uses it.
+int setup_splines(umlmd_t* h) {
+    const Dims& d = h->d;
+    const int t = h->present[0], NC = d.C0 + d.R;
+    if (h->spline_failed || h->spline_species == t) return UMLMD_OK;
+    if (h->spline_n == 0) h->spline_n = fit_radial_splines(h->hm, &h->spline_coef);
+    h->spline_failed = h->spline_n == 0;
+    if (h->spline_failed) return UMLMD_OK;
+    std::vector<float> S((size_t)spline_pitch(h) * d.C0, 0.0f);
+    const float* pm = &h->hm.pairmod[(size_t)(t * d.T + t) * (2 + d.R) * d.C0];
+    for (int k = 0; k < h->spline_n + 7; ++k) {
+        const double* g = &h->spline_coef[(size_t)k * NC];
+        for (int c = 0; c < d.C0; ++c) {
+            double v = (double)pm[c] * g[c] + (double)pm[d.C0 + c];          // (the basis functions add up to one)
+            for (int q = 0; q < d.R; ++q) v += (double)pm[(size_t)(2 + q) * d.C0 + c] * g[d.C0 + q];
+            S[(size_t)k * d.C0 + c] = (float)v;
+        }
+    }
+    h->spline_species = -1;
+    if ((int64_t)S.size() > h->spline_cap) API_CUDA(h, dev_ensure(&h->spline, &h->spline_cap, (int64_t)S.size()));
+    API_CUDA(h, cudaMemcpyAsync(h->spline, S.data(), sizeof(float) * S.size(), cudaMemcpyHostToDevice, h->st));
+    API_CUDA(h, cudaStreamSynchronize(h->st));       // (S is pageable host memory)
+    h->spline_species = t;
+    return UMLMD_OK;
+}
+
+// Makes room for the moments of a tile's rows, and groups the rows of the current list by species, where its kernels take that way.
 int setup_moments(umlmd_t* h) {
     const Dims& d = h->d;
     const int64_t NR = h->nb.n_owned, B = h->nb.N < h->node_tile ? h->nb.N : h->node_tile, rows = NR < B ? NR : B;
     h->have_groups = false;
+    if (h->pair_tables && h->present.size() == 1 && splines_pick(d, rows, mean_row(h))) {
+        const int rc = setup_splines(h);
+        if (rc != UMLMD_OK || !use_splines(h, rows)) return rc;
+        if (rows * spline_pitch(h) > h->moments_cap) API_CUDA(h, dev_ensure(&h->moments, &h->moments_cap, rows * spline_pitch(h)));
+        return UMLMD_OK;
+    }
     if (h->pair_tables || !moments_pick(d, rows)) return UMLMD_OK;
     const int64_t per_tile = moment_order_ints(d, B);
     int64_t c = 0;
@@ -583,7 +630,7 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->on_device) cudaStreamSynchronize(h->st);
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
-    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->moments, h->moment_order, h->moment_scratch, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
+    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->moments, h->moment_order, h->moment_scratch, h->spline, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
                     h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->uni, h->d_species};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
@@ -710,6 +757,8 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
     if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
+    constexpr int64_t kMostSplineRows = 264;            // rows of coefficients of the largest fit
+    if (splines_pick(d, Bt, 1.0e9)) t += buf(Bt * kMostSplineRows, 4) + buf(kMostSplineRows * d.C0, 4);
     if (moments_pick(d, Bt)) t += buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);

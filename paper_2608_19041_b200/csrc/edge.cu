@@ -258,8 +258,32 @@ __device__ __forceinline__ void eval_modes(const EdgeArgs& a, const int4* qes, i
 }
 
 // What a kernel does about shared radial modes (without per-pair tables): there are none; every edge reads its pair's mixing
-// rows; or the scalar channels get them, and beta, from the row's moments (moments.cu)
-enum : int { kNoModes = 0, kModesPerEdge = 1, kMoments = 2 };
+// rows; or the scalar channels get them, and beta, from the row's moments (moments.cu).  kSplines: one species, whose scalar
+// channels are B-splines and enter through the row's spline weights (moments.cu)
+enum : int { kNoModes = 0, kModesPerEdge = 1, kMoments = 2, kSplines = 3 };
+
+// interval of a distance and place in it
+__device__ __forceinline__ int spline_interval(const EdgeArgs& a, float rho, float* t) {
+    const int k = min((int)(rho * a.spline_inv_h), a.spline_n - 1);
+    *t = fmaf(rho, a.spline_inv_h, -(float)k);
+    return k;
+}
+// basis functions of degree six (times 6!) and seven (times 7!) that are not zero on the interval, by their recursion
+__device__ __forceinline__ void spline_basis(float t, float* u6, float* u7) {
+    float u[7];
+    u[0] = 1.0f;
+#pragma unroll
+    for (int d = 1; d <= 6; ++d) {
+#pragma unroll
+        for (int j = d; j >= 0; --j)
+            u[j] = j == d ? t * u[j - 1] : (j == 0 ? (1.0f - t) * u[0] : fmaf(t + (float)(d - j), u[j - 1], ((float)(j + 1) - t) * u[j]));
+    }
+#pragma unroll
+    for (int j = 0; j < 7; ++j) u6[j] = u[j];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        u7[j] = j == 7 ? t * u[6] : (j == 0 ? (1.0f - t) * u[0] : fmaf(t + (float)(7 - j), u[j - 1], ((float)(j + 1) - t) * u[j]));
+}
 
 // adds sum_mu U_c,mu q_mu of four channels; pm: the pair's rows at the channel
 template <int C0, bool PAIR = true>
@@ -369,7 +393,7 @@ template <int C0, int L, int G = 1, bool ROWS = false> struct Widths {
 // registers and one wave beat 85 and two (4000 atoms at C0 = 64: 41 -> 35 us; 597 atoms 25 against 21, 32,400
 // atoms 254 against 234).
 template <int C0, int L, int MODES, bool UNI, bool FEW> struct BwdShape {
-    static constexpr bool two = C0 >= 128 && (MODES == kModesPerEdge || (UNI && L == 2));
+    static constexpr bool two = C0 >= 128 && (MODES == kModesPerEdge || (MODES == kNoModes && UNI && L == 2));
     static constexpr int G = C0 >= 128 ? (two ? 2 : 4) : (C0 >= 32 ? 2 : 1);
     static constexpr int warps = C0 >= 128 ? (two ? 24 : 16) : (MODES == kMoments ? 16 : (FEW ? 32 : 24));
     static constexpr bool tight = two || FEW;
@@ -378,9 +402,9 @@ template <int C0, int L, int MODES, bool UNI, bool FEW> struct BwdShape {
 template <int C0, int L, int MODES, bool UNI> struct BwdSmem {          // dynamic shared memory of the backward kernel
     using W = Widths<C0, L, BwdShape<C0, L, MODES, UNI, false>::G>;
     static constexpr int queue_floats = 32 * 4 + 5 * 32;    // queue of in-range edges: int4 and five scalars per slot
-    static constexpr int mode_floats = MODES ? 2 * 32 * kMaxR : 0;   // parked radial modes and their derivatives or products
+    static constexpr int mode_floats = MODES == kModesPerEdge || MODES == kMoments ? 2 * 32 * kMaxR : 0;   // parked radial modes and their derivatives or products
     static constexpr bool products = wide_channels(C0);             // reads the product table (product_piece)
-    static constexpr int n_red = products ? 1 : 2;                  // partial dot products per edge and lane pair
+    static constexpr int n_red = MODES == kSplines ? 0 : (products ? 1 : 2);                  // partial dot products per edge and lane pair
     static constexpr int per_warp = (32 * W::PB + n_red * 32 * (W::LH + 1) + W::NHI + 3) / 4 * 4 + mode_floats + queue_floats;   // floats
     static constexpr size_t bytes = kWarpsPerBlock * 9 * sizeof(double) + sizeof(float) * kWarpsPerBlock * per_warp;
 };
@@ -420,7 +444,7 @@ k_edge_forward(const EdgeArgs a) {
     constexpr int G = FwdShape<C0, MODES, UNI>::G;          // channel groups of a lane
     constexpr bool PAIR = C0 < 128 || UNI;                  // see axpy2
     using W = Widths<C0, L, G, !UNI>;
-    constexpr bool HASR = MODES != kNoModes;
+    constexpr bool HASR = MODES == kModesPerEdge || MODES == kMoments, SPL = MODES == kSplines;
     static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");
     // scratch per warp: the parked amplitudes of the batch, first the radial modes and then (once the
     // amplitudes are done) the harmonic weights chi^2 B_lm
@@ -480,9 +504,10 @@ k_edge_forward(const EdgeArgs a) {
     }
     const bool swapped = job >= W::JFULL + W::JLOW && job < W::NJ;      // (weights and amplitudes change places in the jobs of one channel)
     const int pitch_v = swapped ? W::PW : W::PP, pitch_s = swapped ? W::PP : W::PW;
-    float* const mom = moments_s + (MODES == kMoments ? wid * a.n_moments : 0);
-    if (MODES == kMoments) {
-        for (int v = lane; v < a.n_moments; v += 32) mom[v] = 0.f;
+    // (splines: four partial rows, one for each group of eight lanes)
+    float* const mom = moments_s + (MODES == kMoments ? 1 : (SPL ? 4 : 0)) * wid * a.n_moments;
+    if (MODES == kMoments || SPL) {
+        for (int v = lane; v < (SPL ? 4 : 1) * a.n_moments; v += 32) mom[v] = 0.f;
         __syncwarp();
     }
     double s0 = 0.0, s1 = 0.0;   // normaliser sums in double: the calibration subtracts their mean
@@ -523,10 +548,41 @@ k_edge_forward(const EdgeArgs a) {
                 }
             }
         }
+        if constexpr (SPL) {
+            // lane = edge: eight spline weights times the envelope, parked in rows of twelve with their first place; then
+            // eight lanes per edge add them to their group's row
+            constexpr int TP = 12;
+            static_assert(32 * TP <= W::SCRATCH, "spline weights of a batch");
+            if (lane < nb) {
+                const int4 es = qes[lane];
+                float t, u6[7], u7[8];
+                const int k = spline_interval(a, __int_as_float(es.y), &t);
+                spline_basis(t, u6, u7);
+                const float w = __int_as_float(es.w) * (1.0f / 5040.0f);
+                float4* const o = reinterpret_cast<float4*>(psi_s + lane * TP);
+                o[0] = make_float4(w * u7[0], w * u7[1], w * u7[2], w * u7[3]);
+                o[1] = make_float4(w * u7[4], w * u7[5], w * u7[6], w * u7[7]);
+                psi_s[lane * TP + 8] = __int_as_float(k);
+            }
+            __syncwarp();
+            float* const part = mom + (lane >> 3) * a.n_moments + (lane & 7);
+            for (int e = lane >> 3; e < nb; e += 4) part[__float_as_int(psi_s[e * TP + 8])] += psi_s[e * TP + (lane & 7)];
+            __syncwarp();
+            // amplitudes of the leading channels, four channels of an edge per lane
+            constexpr int LE = 32 / W::NL1;
+            for (int b0 = 0; b0 < nb; b0 += LE) {
+                const int b = b0 + lane / W::NL1, cc = 4 * (lane % W::NL1);
+                if (b < nb) {
+                    float psi[4];
+                    value_eval4(a.vtable_uni, C0, qes[b].x, cc, __int_as_float(qes[b].z), k2, k3, psi);
+                    *reinterpret_cast<float4*>(psi_s + b * W::PP + cc) = make_float4(psi[0], psi[1], psi[2], psi[3]);
+                }
+            }
+        }
         // lanes = channels, a group of lanes per edge
         constexpr int UNR = C0 >= 32 ? 1 : 2;     // (unrolled as the compiler would: C0 = 64, 32,400 atoms 185 us, so 160)
 #pragma unroll UNR
-        for (int it = 0; it * W::EPI < nb; ++it) {
+        for (int it = 0; !SPL && it * W::EPI < nb; ++it) {
             const int b = it * W::EPI + sub;
             if (b >= nb) continue;
             const int4 es = qes[b];
@@ -596,7 +652,7 @@ k_edge_forward(const EdgeArgs a) {
         const int p = qn + __popc(vmask & lt_mask);       // queue slot of this lane's edge, if it has one
         if (g.valid) { const double c2 = (double)g.chi * (double)g.chi; s0 += c2; s1 += c2 * c2; }
         if (g.valid && p < 32) {
-            qes[p] = make_int4(g.row, g.pair, __float_as_int(g.t), __float_as_int(g.chi));
+            qes[p] = make_int4(g.row, SPL ? __float_as_int(g.rho) : g.pair, __float_as_int(g.t), __float_as_int(g.chi));
             qd[p] = g.dx; qd[32 + p] = g.dy; qd[64 + p] = g.dz;
         }
         qn += __popc(vmask);
@@ -604,7 +660,7 @@ k_edge_forward(const EdgeArgs a) {
         if (qn >= 32) {                                   // a full batch; the overflow waits in registers
             run_batch(32);
             if (g.valid && p >= 32) {
-                qes[p - 32] = make_int4(g.row, g.pair, __float_as_int(g.t), __float_as_int(g.chi));
+                qes[p - 32] = make_int4(g.row, SPL ? __float_as_int(g.rho) : g.pair, __float_as_int(g.t), __float_as_int(g.chi));
                 qd[p - 32] = g.dx; qd[p] = g.dy; qd[32 + p] = g.dz;
             }
             qn -= 32;
@@ -625,7 +681,7 @@ k_edge_forward(const EdgeArgs a) {
     }
     float* const row_glob = a.state + (size_t)(i - a.a0) * a.d.SP;
     float* const row_out = SPLIT ? psi_s : row_glob;        // (the batches are done with the scratch)
-    if (sub == 0) {
+    if (!SPL && sub == 0) {
 #pragma unroll
         for (int gq = 0; gq < G; ++gq)
             *reinterpret_cast<float4*>(row_out + c + gq * W::GOFF) = make_float4(acc0[4 * gq], acc0[4 * gq + 1], acc0[4 * gq + 2], acc0[4 * gq + 3]);
@@ -653,6 +709,11 @@ k_edge_forward(const EdgeArgs a) {
     if (MODES == kMoments) {
         float* const out = a.moments + (size_t)(i - a.a0) * a.n_moments;
         for (int v = lane; v < a.n_moments; v += 32) out[v] = mom[v];
+    }
+    if (SPL) {
+        float* const out = a.moments + (size_t)(i - a.a0) * a.n_moments;
+        const float *p1 = mom + a.n_moments, *p2 = p1 + a.n_moments, *p3 = p2 + a.n_moments;
+        for (int v = lane; v < a.n_moments; v += 32) out[v] = (mom[v] + p1[v]) + (p2[v] + p3[v]);
     }
     if (SPLIT) {
         if (lane == 0) { s_part[wid][0] = s0; s_part[wid][1] = s1; }
@@ -689,7 +750,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, BwdShape<C0, L, MODES, UN
 k_edge_backward(const EdgeArgs a) {
     using SM = BwdSmem<C0, L, MODES, UNI>;
     constexpr int G = BwdShape<C0, L, MODES, UNI, FEW>::G;
-    constexpr bool PR = SM::products, HASR = MODES != kNoModes;
+    constexpr bool PR = SM::products, HASR = MODES == kModesPerEdge || MODES == kMoments, SPL = MODES == kSplines;
     using W = Widths<C0, L, G>;
     extern __shared__ __align__(16) unsigned char dsm[];
     double (*vsum)[9] = reinterpret_cast<double (*)[9]>(dsm);
@@ -703,7 +764,7 @@ k_edge_backward(const EdgeArgs a) {
     int4* const qes = reinterpret_cast<int4*>(wbase + SM::per_warp - SM::queue_floats);
     float* const qm = reinterpret_cast<float*>(qes) - SM::mode_floats;   // [2][32][kMaxR]
     float* const qd = reinterpret_cast<float*>(qes + 32);        // [5][32]
-    float* const mom = reinterpret_cast<float*>(dsm + SM::bytes) + (MODES == kMoments ? wid * a.n_moments : 0);   // [n_moments]
+    float* const mom = reinterpret_cast<float*>(dsm + SM::bytes) + (MODES == kMoments || SPL ? wid * a.n_moments : 0);   // [n_moments]
     const int i = a.a0 + (SPLIT ? blockIdx.x : blockIdx.x * kWarpsPerBlock + wid);
     const bool active = i < a.a1;
     const int sub = lane / W::LPE, cl = lane % W::LPE, c = 4 * cl;
@@ -726,12 +787,12 @@ k_edge_backward(const EdgeArgs a) {
         const float* grow = a.state + (size_t)(i - a.a0) * a.d.SP;
         float h0[4 * G];
 #pragma unroll
-        for (int gq = 0; gq < G; ++gq) {
+        for (int gq = 0; gq < (SPL ? 0 : G); ++gq) {
             const float4 v = *reinterpret_cast<const float4*>(grow + c + gq * W::GOFF);
             h0[4 * gq] = v.x; h0[4 * gq + 1] = v.y; h0[4 * gq + 2] = v.z; h0[4 * gq + 3] = v.w;
         }
         for (int v = lane; v < W::NHI; v += 32) hi_s[v] = grow[a.d.offA[1] + v];
-        if (MODES == kMoments)
+        if (MODES == kMoments || SPL)
             for (int v = lane; v < a.n_moments; v += 32) mom[v] = a.moments[(size_t)(i - a.a0) * a.n_moments + v];
         const float ds0 = grow[a.d.S], ds1 = grow[a.d.S + 1];
         __syncwarp();
@@ -754,7 +815,12 @@ k_edge_backward(const EdgeArgs a) {
                         const int4 es = qes[b];
                         const float t = __int_as_float(es.z);
                         float psi[4];
-                        if constexpr (MODES == kMoments) {         // their products as well, from the same pair rows
+                        if constexpr (SPL) {                       // and their products
+                            float d[4];
+                            value_eval4(a.vtable_uni, C0, es.x, cc, t, k2, k3, psi);
+                            value_eval4(a.dtable_uni, C0, es.x, cc, t, d1, d2, d);
+                            *reinterpret_cast<float4*>(psi_s + b * W::PB + W::C1 + cc) = make_float4(d[0], d[1], d[2], d[3]);
+                        } else if constexpr (MODES == kMoments) {  // the same, from the same pair rows
                             float d[4];
                             const float* pm = a.pairmod + (size_t)es.y * (2 + a.d.R) * C0 + cc;
                             const float dchi = qd[96 + b];
@@ -779,7 +845,7 @@ k_edge_backward(const EdgeArgs a) {
                     }
                 }
                 // all channels: sum_c G_c (chi psi_c)'
-                for (int it = 0; it * W::EPI < nb; ++it) {
+                for (int it = 0; !SPL && it * W::EPI < nb; ++it) {
                     const int b = it * W::EPI + sub;
                     const bool act = b < nb;
                     float2 p2 = make_float2(0.f, 0.f);
@@ -843,7 +909,7 @@ k_edge_backward(const EdgeArgs a) {
                 const float gux = gdx * inv_rho, guy = gdy * inv_rho, guz = gdz * inv_rho;
                 float sa = 0.f, sb = 0.f;
 #pragma unroll
-                for (int j = 0; j < W::LH; ++j) {
+                for (int j = 0; !SPL && j < W::LH; ++j) {
                     sa += red[lane * (W::LH + 1) + j];
                     if (!PR) sb += red[(32 + lane) * (W::LH + 1) + j];
                 }
@@ -851,6 +917,18 @@ k_edge_backward(const EdgeArgs a) {
                 // pr1 = sum_lm B_lm sum_c dps_c G_lmc.  By component, all channels in registers; where the registers are
                 // few (BwdShape), by four channels, which keeps the components' sums instead: 0.94 against 1.02 ms for
                 // the 128,000 atoms of five species, but 1.12 against 1.10 at 128 registers.
+                if (SPL) {           // (chi S)' of the spline of the row's coefficients
+                    float t, u6[7], u7[8], v = 0.f, dv = 0.f;
+                    const float* const h = mom + spline_interval(a, __int_as_float(qes[lane].y), &t);
+                    spline_basis(t, u6, u7);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float hj = h[j];
+                        v = fmaf(hj, u7[j], v);
+                        dv = fmaf(hj, j == 0 ? -u6[0] : (j == 7 ? u6[6] : u6[j - 1] - u6[j]), dv);
+                    }
+                    sa = dchi * (1.0f / 5040.0f) * v + chi * (a.spline_inv_h * (1.0f / 720.0f)) * dv;
+                }
                 if (MODES == kMoments) {
                     const float* hr = mom + (qes[lane].y - ti * a.d.T) * (1 + a.d.R);
                     sa += dchi * hr[0];
@@ -1026,7 +1104,7 @@ k_edge_backward(const EdgeArgs a) {
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
             if (g.valid && p < 32) {
-                qes[p] = make_int4(g.row, g.pair, __float_as_int(g.t), __float_as_int(g.chi));
+                qes[p] = make_int4(g.row, SPL ? __float_as_int(g.rho) : g.pair, __float_as_int(g.t), __float_as_int(g.chi));
                 qd[p] = g.dx; qd[32 + p] = g.dy; qd[64 + p] = g.dz; qd[96 + p] = g.dchi;
                 qd[128 + p] = __int_as_float(e);
             } else if (!g.valid && e < len) {
@@ -1039,7 +1117,7 @@ k_edge_backward(const EdgeArgs a) {
                 run_batch(32);
                 if (g.valid && p >= 32) {
                     const int r = p - 32;
-                    qes[r] = make_int4(g.row, g.pair, __float_as_int(g.t), __float_as_int(g.chi));
+                    qes[r] = make_int4(g.row, SPL ? __float_as_int(g.rho) : g.pair, __float_as_int(g.t), __float_as_int(g.chi));
                     qd[r] = g.dx; qd[32 + r] = g.dy; qd[64 + r] = g.dz; qd[96 + r] = g.dchi;
                     qd[128 + r] = __int_as_float(e);
                 }
@@ -1083,6 +1161,16 @@ template <int C0, int L, bool SPLIT>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
     auto kern = a.uni ? k_edge_forward<C0, L, kNoModes, true, SPLIT>
                       : (a.d.R > 0 ? k_edge_forward<C0, L, kModesPerEdge, false, SPLIT> : k_edge_forward<C0, L, kNoModes, false, SPLIT>);
+    if constexpr (C0 >= 64 && !SPLIT) {
+        if (a.spline_n) {
+            kern = k_edge_forward<C0, L, kSplines, true, false>;
+            const size_t bytes = sizeof(float) * kWarpsPerBlock * 4 * a.n_moments;
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            if (e != cudaSuccess) return e;
+            kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
     if constexpr (wide_channels(C0) && !SPLIT) {
         if (a.moments) {
             kern = k_edge_forward<C0, L, kMoments, false, false>;
@@ -1099,10 +1187,10 @@ cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
 template <int C0, int L, int MODES, bool UNI>
 cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
     const bool few = a.a1 - a.a0 > 148 * 24 && a.a1 - a.a0 <= 148 * 32;
-    constexpr bool FEW = C0 <= 64 && MODES != kMoments;           // (the others have no such variant)
+    constexpr bool FEW = C0 <= 64 && MODES < kMoments;           // (the others have no such variant)
     size_t bytes = BwdSmem<C0, L, MODES, UNI>::bytes;
     auto kern = few ? k_edge_backward<C0, L, MODES, UNI, FEW, false> : k_edge_backward<C0, L, MODES, UNI, false, false>;
-    if constexpr (MODES == kMoments) bytes += sizeof(float) * kWarpsPerBlock * a.n_moments;
+    if constexpr (MODES >= kMoments) bytes += sizeof(float) * kWarpsPerBlock * a.n_moments;
     else if (split) kern = k_edge_backward<C0, L, MODES, UNI, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
@@ -1112,6 +1200,9 @@ cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t
 template <bool FWD, int C0, int L>
 cudaError_t launch(const EdgeArgs& a, int blocks, bool split, cudaStream_t st) {
     if (FWD) return split ? launch_fwd_r<C0, L, true>(a, blocks, st) : launch_fwd_r<C0, L, false>(a, blocks, st);
+    if constexpr (C0 >= 64) {
+        if (a.spline_n) return launch_bwd_r<C0, L, kSplines, true>(a, blocks, false, st);
+    }
     if (a.uni) return launch_bwd_r<C0, L, kNoModes, true>(a, blocks, split, st);
     if constexpr (wide_channels(C0)) {
         if (a.moments) return launch_bwd_r<C0, L, kMoments, false>(a, blocks, false, st);

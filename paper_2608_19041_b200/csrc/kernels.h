@@ -77,6 +77,10 @@ struct EdgeArgs {
     // or gradients of them (backward), see moments.cu; null: every edge reads its pair's mode mixing
     float* moments;
     int n_moments;
+    // one species, from enough rows on: n_moments spline weights per row (moments.cu); spline_n intervals of 1 / spline_inv_h,
+    // 0: not by splines
+    int spline_n;
+    float spline_inv_h;
 };
 constexpr int kEdgeRowsPerBlock = 4, kEdgeSplitRows = 1184;
 // present: device array of the n_present species indices, ascending
@@ -134,10 +138,12 @@ struct MomentArgs {
     Dims d;
     const float* pairmod;
     const int* type_s;
-    const int* order;       // rows of the tile by species (launch_moment_groups)
+    const int* order;       // rows of the tile by species (launch_moment_groups); null with splines
     int a0, n;              // tile start (sorted index) and row count
     float* state;           // [n][SP]
-    float* moments;         // [n][moment_pitch]
+    float* moments;         // [n][pitch]
+    int pitch;
+    const float* spline;    // [pitch][C0] spline coefficients of the pair's amplitude, null: the pair rows of the modes
 };
 // From 2048 rows on (the two edge kernels and the products, C0 = 128 with 64 species and four modes, by moments against every
 // edge reading its pair's rows: 2100 rows 150 against 211 us, 4000 235 against 406, 40,009 1510 against 2638); below, whole
@@ -149,8 +155,17 @@ bool moments_pick(const Dims& d, int64_t rows);
 int64_t moment_order_ints(const Dims& d, int64_t rows);
 // type_s: of the tile; scratch: 2 T ints
 cudaError_t launch_moment_groups(const Dims& d, const int* type_s, int n, int* scratch, int* order, cudaStream_t st);
-cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st);    // state += (beta | U)^T moments
-cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st);   // moments = (beta | U) state
+cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st);    // state += (beta | U)^T moments; = spline^T moments
+cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st);   // moments = (beta | U) state; spline state
+// Whether the scalar channels of a tile of so many rows, all of one species and with so many listed neighbours on average, go by
+// splines (true for n implies true for more).  The products with the coefficients cost the same for every row, the edges save
+// with their number and the width.  Edge kernels and products, tables against splines, us: C0 = 64 with 274 listed neighbours
+// 30,000 rows 609 and 484, 9000 197 and 178, with 122 neighbours 10,000 rows 118 and 132; C0 = 128 with 274 30,000 rows 966 and
+// 675, 9000 304 and 223.
+constexpr int kSplineRows = 8192;
+inline bool splines_pick(const Dims& d, int64_t rows, double row_length) {
+    return d.C0 >= 64 && rows >= kSplineRows && row_length * d.C0 >= 64 * 180;
+}
 
 // ---- invariants.cu -------------------------------------------------------------------
 struct InvArgs {

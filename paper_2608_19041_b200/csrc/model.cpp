@@ -179,6 +179,93 @@ bool derive_dims(int C0, int L, int R, Dims* d) {
     return true;
 }
 
+void spline_weights(double t, double w[8], double dw[8]) {
+    double u[8] = {1, 0, 0, 0, 0, 0, 0, 0};
+    for (int d = 1; d <= 7; ++d) {
+        if (d == 7)
+            for (int j = 0; j <= 7; ++j) dw[j] = (j > 0 ? u[j - 1] : 0.0) - (j < 7 ? u[j] : 0.0);
+        for (int j = d; j >= 0; --j) u[j] = ((j > 0 ? (t + d - j) * u[j - 1] : 0.0) + (j < d ? (j + 1 - t) * u[j] : 0.0)) / d;
+    }
+    for (int j = 0; j <= 7; ++j) w[j] = u[j];
+}
+
+int fit_radial_splines(const HostModel& m, std::vector<double>* coef) {
+    const Dims& d = m.d;
+    const int NC = d.C0 + d.R, n = d.n_rows + 1;
+    if (m.knots.empty()) return 0;
+    for (const int K : {160, 192, 256}) {
+        const int stride = n / (8 * K);                   // about eight knots per interval; the ones half way between are checked
+        if (stride < 1) return 0;
+        const int M = K + 7;
+        const double inv_h = K / m.rc;
+        std::vector<double> A((size_t)M * 8, 0.0);         // lower band of the normal equations, A[i][i - j]
+        coef->assign((size_t)M * NC, 0.0);
+        double* const B = coef->data();
+        auto basis = [&](int s, double* w, double* dw) {
+            const double x = s * m.dx * inv_h;
+            const int k = std::min((int)x, K - 1);
+            spline_weights(x - k, w, dw);
+            return k;
+        };
+        double w[8], dw[8];
+        for (int s = 0; s < n; s += stride) {
+            const int k = basis(s, w, dw);
+            const double* y = &m.knots[(size_t)s * 2 * NC];
+            for (int a = 0; a < 8; ++a) {
+                for (int b = 0; b <= a; ++b) A[(size_t)(k + a) * 8 + (a - b)] += w[a] * w[b];
+                double* r = B + (size_t)(k + a) * NC;
+                for (int c = 0; c < NC; ++c) r[c] += w[a] * y[c];
+            }
+        }
+        bool ok = true;                                    // Cholesky, then forward and backward substitution
+        for (int i = 0; i < M && ok; ++i)
+            for (int j = std::max(0, i - 7); j <= i; ++j) {
+                double v = A[(size_t)i * 8 + (i - j)];
+                for (int p = std::max(0, i - 7); p < j; ++p) v -= A[(size_t)i * 8 + (i - p)] * A[(size_t)j * 8 + (j - p)];
+                if (i == j) { ok = v > 0; A[(size_t)i * 8] = std::sqrt(v); }
+                else A[(size_t)i * 8 + (i - j)] = v / A[(size_t)j * 8];
+            }
+        if (!ok) continue;
+        auto eliminate = [&](int i, int p, double l) {
+            double* r = B + (size_t)i * NC;
+            const double* q = B + (size_t)p * NC;
+            for (int c = 0; c < NC; ++c) r[c] -= l * q[c];
+        };
+        auto divide = [&](int i) {
+            double* r = B + (size_t)i * NC;
+            const double inv = 1 / A[(size_t)i * 8];
+            for (int c = 0; c < NC; ++c) r[c] *= inv;
+        };
+        for (int i = 0; i < M; ++i) {
+            for (int p = std::max(0, i - 7); p < i; ++p) eliminate(i, p, A[(size_t)i * 8 + (i - p)]);
+            divide(i);
+        }
+        for (int i = M - 1; i >= 0; --i) {
+            for (int p = i + 1; p < std::min(M, i + 8); ++p) eliminate(i, p, A[(size_t)p * 8 + (p - i)]);
+            divide(i);
+        }
+        std::vector<double> v(NC), dv(NC);
+        double ev = 0, ed = 0, mv = 0, md = 0;
+        for (int s = stride / 2; s < n; s += stride) {
+            const int k = basis(s, w, dw);
+            const double *y = &m.knots[(size_t)s * 2 * NC], *y1 = y + NC;
+            std::fill(v.begin(), v.end(), 0.0);
+            std::fill(dv.begin(), dv.end(), 0.0);
+            for (int a = 0; a < 8; ++a) {
+                const double *q = B + (size_t)(k + a) * NC, wa = w[a], da = dw[a] * inv_h;
+                for (int c = 0; c < NC; ++c) { v[c] += wa * q[c]; dv[c] += da * q[c]; }
+            }
+            for (int c = 0; c < NC; ++c) {
+                ev = std::max(ev, std::fabs(v[c] - y[c])); mv = std::max(mv, std::fabs(y[c]));
+                ed = std::max(ed, std::fabs(dv[c] - y1[c])); md = std::max(md, std::fabs(y1[c]));
+            }
+        }
+        // (the tables: 2^-24 and 2^-23)
+        if (std::isfinite(ev) && std::isfinite(ed) && ev <= 0x1p-24 * mv && ed <= 0x1p-23 * md) return K;
+    }
+    return 0;
+}
+
 int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostModel* m,
                      std::string* err) {
     const unsigned char* blob = static_cast<const unsigned char*>(blob_v);
@@ -397,6 +484,8 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         m->dtable.clear();
         if (wide) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
     }
+
+    if (C0 >= 64) m->knots = std::move(Y);
 
     // ---- ordered type-pair cache -----------------------------------------------------
     {

@@ -8,6 +8,14 @@
 // The edge kernel leaves the T (1 + R) moments m of each row; here they meet the rows of the centre's species, once per row and
 // not per edge, as a matrix product whose rows are grouped by species.  The backward pass forms H = (beta | U) G_0 the same way,
 // and its edge kernel adds sum_c G_0,c (chi (beta_c + U q))' = chi' H_t,0 + sum_mu (chi q_mu)' H_t,mu for each edge.
+//
+// Scalar channels by splines.
+//
+// Where all atoms are of one species, psi_c(rho) of the one pair is written as a B-spline of degree seven on a few hundred intervals,
+// psi_c = sum_a B_a(t) S_{k + a, c}, and the sum over a row becomes sum_j chi_j psi_c = sum_k S_k,c p_k with
+// p_{k + a} = sum_j chi_j B_a(t_j): an edge adds eight numbers whatever C0 is, where it read 8 bytes per channel and multiplied them out.
+// The rows of p meet S in the same matrix product, and the backward pass reads H = S G_0 of its row: sum_c G_0,c (chi psi_c)' is
+// the derivative of chi times the spline of coefficients H.
 #include "kernels.h"
 
 namespace umd {
@@ -15,9 +23,7 @@ namespace umd {
 namespace {
 
 constexpr int kRows = 64;            // rows of a block, all of one species
-constexpr int KC = 32;               // depth of a step
-constexpr int AP = kRows + 4;        // pitch of the transposed operands (16-byte reads of four rows)
-constexpr int kThreads = 256;
+constexpr int KC = 16;               // depth of a step
 
 // ---- rows of a tile grouped by the species of their atom --------------------------------------------------------------
 // order: rows of the first species, then of the second ..., each padded with -1 to whole blocks; which place a row gets inside its
@@ -45,118 +51,136 @@ __global__ void k_group_fill(int n, int T, const int* __restrict__ type, const i
 }
 
 // ---- C[64 x NT] = A[64 x K] B[K x NT] in single precision -----------------------------------------------------------------
-// FORWARD: A = moments of the rows, B = beta and U of the centre's species, added to the scalar channels' sums.
-// Backward: A = gradient of those sums, B the transpose, into the moments' place.
-// A thread holds four rows and NT / 16 columns; a step's operands are fetched while the one before is multiplied, pairs of
-// multiply-adds in one instruction.  40,009 rows of 320 moments and 128 channels (3.3 GFLOP) take 142 us forward, 134 backward, a
-// third of the FMA rate: 689 blocks are 2.3 rounds of the machine, and the L1 data pipe, which a thread's twelve words per 32
-// multiply-adds occupy, is 65 to 80 % busy.  The edge kernels, which read these rows for every edge, took 543 us and 820 us more.
+// FORWARD: A = moments of the rows, B = beta and U of the centre's species (or the spline coefficients), added to (or put into) the
+// scalar channels' sums.  Backward: A = gradient of those sums, B the transpose, into the moments' place.
+// NT threads of eight rows and eight columns each: sixteen words from shared memory for 64 multiply-adds, pairs of them in one
+// instruction.  The L1 data pipe takes a cycle for every word that the lanes of a warp read, the FMA pipe one for every
+// multiply-add, so that both are busy alike.
+// A step's products are added up by themselves first: in one chain of 168 the rounding of a row of splines is 2.7e-7 of the sums'
+// rms, in two levels 1.1e-7 to 1.5e-7, as the sums over the edges have it (1.1e-7 to 1.6e-7).  Operands come by asynchronous
+// copies, two steps ahead; those whose depth is contiguous in memory lie in rows of KC + 4.
 template <bool FORWARD, int NT>
-__global__ void __launch_bounds__(kThreads) k_moments(int a0, int K, int N, Dims d, const float* __restrict__ pairmod, const int* __restrict__ type_s,
-                                                      const int* __restrict__ order, float* __restrict__ state, float* __restrict__ moments, int km) {
-    constexpr int TC = NT / 16;                                   // columns of a thread: TC / 4 runs of four (or one of two)
-    constexpr int BP = FORWARD ? NT : NT + 4;
-    __shared__ __align__(16) float As[KC][AP];
-    __shared__ __align__(16) float Bs[KC][BP];
+__global__ void __launch_bounds__(NT, 256 / NT) k_moments(int a0, int K, int N, Dims d, const float* __restrict__ pairmod, const int* __restrict__ type_s,
+                                                          const int* __restrict__ order, float* __restrict__ state, float* __restrict__ moments, int km,
+                                                          const float* __restrict__ spline, int n) {
+    constexpr int STAGES = 3, AP = KC + 4, BP = FORWARD ? NT : KC + 4, BROWS = FORWARD ? KC : NT;
+    __shared__ __align__(16) float As[STAGES][kRows * AP];
+    __shared__ __align__(16) float Bs[STAGES][BROWS * BP];
     __shared__ int row_s[kRows];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    if (tid < kRows) row_s[tid] = order[(size_t)blockIdx.x * kRows + tid];
+    const int tid = threadIdx.x, tx = tid % (NT / 8), ty = tid / (NT / 8);
+    for (int r = tid; r < kRows; r += NT) {
+        const int at = blockIdx.x * kRows + r;
+        row_s[r] = spline ? (at < n ? at : -1) : order[at];
+    }
     __syncthreads();
     if (row_s[0] < 0) return;                                    // past the last group
-    const int ti = type_s[a0 + row_s[0]], R1 = 1 + d.R, C0 = d.C0;
+    const int R1 = 1 + d.R, C0 = d.C0, ti = spline ? 0 : type_s[a0 + row_s[0]], kb = spline ? km : d.T * R1;
     const int n0 = FORWARD ? 0 : blockIdx.y * NT;                 // first column
     // row k of (beta | U) of the centre's species: moment k = t (1 + R) + mu
-    auto mixing = [&](int k) { const int t = k / R1; return pairmod + ((size_t)(ti * d.T + t) * (2 + d.R) + 1 + (k - t * R1)) * C0; };
+    auto mixing = [&](int k) {
+        if (spline) return spline + (size_t)k * C0;
+        const int t = k / R1;
+        return pairmod + ((size_t)(ti * d.T + t) * (2 + d.R) + 1 + (k - t * R1)) * C0;
+    };
     const int lda = FORWARD ? km : d.SP;
     const float* const A = FORWARD ? moments : state;
-    float4 ra[2];
-    constexpr int NB = KC * NT / 4 / kThreads;                    // 16-byte pieces of B per thread
-    float4 rb[NB];
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto fetch = [&](int k0) {
+    auto copy16 = [](float* dst, const float* src, bool on) {     // 16 bytes, zeros where there is nothing
+        const unsigned at = (unsigned)__cvta_generic_to_shared(dst);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at), "l"(src), "r"(on ? 16 : 0) : "memory");
+    };
+    auto fetch = [&](int step) {
+        const int k0 = step * KC, st = step % STAGES;
+        if (k0 < K) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int row = row_s[(tid >> 3) + 32 * h], k = k0 + 4 * (tid & 7);
-            ra[h] = row >= 0 && k < K ? *reinterpret_cast<const float4*>(A + (size_t)row * lda + k) : zero;
-        }
+            for (int p = 0; p < kRows * KC / 4 / NT; ++p) {
+                const int at = tid + p * NT, r = at / (KC / 4), k = 4 * (at % (KC / 4)), row = row_s[r];
+                const bool on = row >= 0 && k0 + k < K;
+                copy16(&As[st][r * AP + k], on ? A + (size_t)row * lda + k0 + k : A, on);
+            }
 #pragma unroll
-        for (int p = 0; p < NB; ++p) {
-            const int at = tid + p * kThreads;
-            if (FORWARD) {
-                const int k = k0 + at / (NT / 4), c = 4 * (at % (NT / 4));
-                rb[p] = k < K && k < d.T * R1 ? *reinterpret_cast<const float4*>(mixing(k) + c) : zero;
-            } else {
-                const int m = n0 + (at >> 3), k = k0 + 4 * (at & 7);
-                rb[p] = m < d.T * R1 ? *reinterpret_cast<const float4*>(mixing(m) + k) : zero;
+            for (int p = 0; p < KC / 4; ++p) {
+                const int at = tid + p * NT;
+                const int k = FORWARD ? k0 + at / (NT / 4) : n0 + at / (KC / 4), c = FORWARD ? 4 * (at % (NT / 4)) : k0 + 4 * (at % (KC / 4));
+                const bool on = k < kb && (FORWARD || c < C0);
+                copy16(&Bs[st][FORWARD ? (at / (NT / 4)) * BP + c : (at / (KC / 4)) * BP + 4 * (at % (KC / 4))], on ? mixing(k) + c : pairmod, on);
             }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto park = [&]() {
+    float2 acc[8][4], part[8][4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int r = (tid >> 3) + 32 * h, k = 4 * (tid & 7);
-            As[k][r] = ra[h].x; As[k + 1][r] = ra[h].y; As[k + 2][r] = ra[h].z; As[k + 3][r] = ra[h].w;
-        }
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int p = 0; p < NB; ++p) {
-            const int at = tid + p * kThreads;
-            if (FORWARD) {
-                *reinterpret_cast<float4*>(&Bs[at / (NT / 4)][4 * (at % (NT / 4))]) = rb[p];
-            } else {
-                const int m = at >> 3, k = 4 * (at & 7);
-                Bs[k][m] = rb[p].x; Bs[k + 1][m] = rb[p].y; Bs[k + 2][m] = rb[p].z; Bs[k + 3][m] = rb[p].w;
-            }
-        }
-    };
-    float2 acc[4][TC / 2];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < TC / 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
-    // columns of a thread: runs of four at 4 tx + 64 run, or two at 2 tx
-    auto column = [&](int c) { return TC == 2 ? 2 * tx : 4 * tx + 64 * (c >> 1) + 2 * (c & 1); };
+        for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.f, 0.f);
+    // rows of a thread: four at 4 ty, four at 32 + 4 ty; columns: forward four at 4 tx and four at NT / 2 + 4 tx, backward every NT / 8-th
+    auto row_of = [&](int r) { return 4 * ty + (r & 3) + 32 * (r >> 2); };
+    auto column = [&](int c) { return tx + NT / 8 * c; };
+    const int steps = (K + KC - 1) / KC;
     fetch(0);
-    for (int k0 = 0; k0 < K; k0 += KC) {
-        park();
-        __syncthreads();
-        if (k0 + KC < K) fetch(k0 + KC);
-#pragma unroll 8
-        for (int k = 0; k < KC; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&As[k][4 * ty]);
-            float2 b[TC / 2];
-            if (TC == 2) b[0] = *reinterpret_cast<const float2*>(&Bs[k][2 * tx]);
-            else {
+    fetch(1);
+    for (int s = 0; s < steps; ++s) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();                                         // (this step is there, and nobody reads the stage that is filled next)
+        fetch(s + 2);
+        const float *as = As[s % STAGES], *bs = Bs[s % STAGES];
 #pragma unroll
-                for (int c = 0; c < TC / 2; c += 2) {
-                    const float4 v = *reinterpret_cast<const float4*>(&Bs[k][column(c)]);
-                    b[c] = make_float2(v.x, v.y);
-                    b[c + 1 < TC / 2 ? c + 1 : c] = make_float2(v.z, v.w);
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[r][c] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < KC; k += 4) {
+            float4 a[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) a[r] = *reinterpret_cast<const float4*>(as + row_of(r) * AP + k);
+            float4 bt[8];                                        // backward: four depths of eight columns
+            if (!FORWARD) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) bt[c] = *reinterpret_cast<const float4*>(bs + column(c) * BP + k);
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                auto at = [&](const float4& v) { return kk == 0 ? v.x : (kk == 1 ? v.y : (kk == 2 ? v.z : v.w)); };
+                float2 b[4];
+                if (FORWARD) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 v = *reinterpret_cast<const float4*>(bs + (k + kk) * BP + 4 * tx + NT / 2 * h);
+                        b[2 * h] = make_float2(v.x, v.y); b[2 * h + 1] = make_float2(v.z, v.w);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) b[c] = make_float2(at(bt[2 * c]), at(bt[2 * c + 1]));
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const float2 ar = make_float2(at(a[r]), at(a[r]));
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) part[r][c] = ffma2(ar, b[c], part[r][c]);
                 }
             }
-#pragma unroll
-            for (int c = 0; c < TC / 2; ++c) {
-                acc[0][c] = ffma2(make_float2(a.x, a.x), b[c], acc[0][c]);
-                acc[1][c] = ffma2(make_float2(a.y, a.y), b[c], acc[1][c]);
-                acc[2][c] = ffma2(make_float2(a.z, a.z), b[c], acc[2][c]);
-                acc[3][c] = ffma2(make_float2(a.w, a.w), b[c], acc[3][c]);
-            }
         }
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) { acc[r][c].x += part[r][c].x; acc[r][c].y += part[r][c].y; }
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int row = row_s[4 * ty + r];
+    for (int r = 0; r < 8; ++r) {
+        const int row = row_s[row_of(r)];
         if (row < 0) continue;
+        if (FORWARD) {
 #pragma unroll
-        for (int c = 0; c < TC / 2; ++c) {
-            const int n = n0 + column(c);
-            if (n >= N) continue;                                // (N is even)
-            if (FORWARD) {
-                float2* const o = reinterpret_cast<float2*>(state + (size_t)row * d.SP + n);
-                const float2 v = *o;
-                *o = make_float2(v.x + acc[r][c].x, v.y + acc[r][c].y);
-            } else {
-                *reinterpret_cast<float2*>(moments + (size_t)row * km + n) = acc[r][c];
+            for (int h = 0; h < 2; ++h) {
+                float4* const o = reinterpret_cast<float4*>(state + (size_t)row * d.SP + 4 * tx + NT / 2 * h);
+                const float4 v = spline ? make_float4(0.f, 0.f, 0.f, 0.f) : *o;
+                const float2 x = acc[r][2 * h], y = acc[r][2 * h + 1];
+                *o = make_float4(v.x + x.x, v.y + x.y, v.z + y.x, v.w + y.y);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int m = n0 + column(c);
+                if (m < N) moments[(size_t)row * km + m] = c & 1 ? acc[r][c >> 1].y : acc[r][c >> 1].x;
             }
         }
     }
@@ -182,14 +206,16 @@ cudaError_t launch_moment_groups(const Dims& d, const int* type_s, int n, int* s
 template <bool FORWARD>
 static cudaError_t launch(const MomentArgs& a, cudaStream_t st) {
     const Dims& d = a.d;
-    const int km = moment_pitch(d), K = FORWARD ? km : d.C0, N = FORWARD ? d.C0 : km;
-    const unsigned groups = (unsigned)(moment_order_ints(d, a.n) / kRows);
+    const int km = a.pitch, K = FORWARD ? km : d.C0, N = FORWARD ? d.C0 : km;
+    const unsigned groups = a.spline ? (unsigned)((a.n + kRows - 1) / kRows) : (unsigned)(moment_order_ints(d, a.n) / kRows);
     auto go = [&](auto kern, int NT) {
-        kern<<<dim3(groups, (unsigned)((N + NT - 1) / NT)), kThreads, 0, st>>>(a.a0, K, N, d, a.pairmod, a.type_s, a.order, a.state, a.moments, km);
+        kern<<<dim3(groups, (unsigned)((N + NT - 1) / NT)), NT, 0, st>>>(a.a0, K, N, d, a.pairmod, a.type_s, a.order, a.state, a.moments, km, a.spline, a.n);
         return cudaGetLastError();
     };
-    if (!FORWARD || d.C0 == 128) return go(k_moments<FORWARD, 128>, 128);
-    return d.C0 == 64 ? go(k_moments<FORWARD, 64>, 64) : go(k_moments<FORWARD, 32>, 32);
+    // (backward: the width that pads fewer columns)
+    const int width = FORWARD ? d.C0 : ((N + 63) / 64 * 64 < (N + 127) / 128 * 128 ? 64 : 128);
+    if (width == 128) return go(k_moments<FORWARD, 128>, 128);
+    return width == 64 ? go(k_moments<FORWARD, 64>, 64) : go(k_moments<true, 32>, 32);
 }
 cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st) { return launch<true>(a, st); }
 cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st) { return launch<false>(a, st); }

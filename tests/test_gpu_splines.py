@@ -1,0 +1,74 @@
+"""Scalar channels by splines (one species, many rows) against the same kernels reading the pair's tables (few rows)."""
+
+import numpy as np
+import pytest
+import torch
+
+from tests.test_host_tables import _steep_blob
+from workloads import SMALL_PROFILES, make_blob, make_system
+
+pytestmark = pytest.mark.gpu
+
+SPLINE_ROWS = 8192      # the fewest rows that take the way over splines
+
+
+def _frames():
+    # 29 atoms with long rows, some closer than any material has them, and three with rows of at most two edges
+    dense = make_system(dict(kind="random_box", atoms=29, edges=(4.6, 5.0, 5.4), min_dist=0.9, seed=81, n_types=1, masses=[1.0]))
+    sparse = make_system(dict(kind="random_box", atoms=3, edges=(30.0, 30.0, 30.0), min_dist=1.6, seed=82, n_types=1, masses=[1.0]))
+    sparse["pos"][:2] = [[3.0, 3.0, 3.0], [4.7, 3.2, 3.1]]
+    return (29, 3), [np.diag(np.diag(np.asarray(f["cell"], dtype=np.float64))) for f in (dense, sparse)], np.concatenate([dense["pos"], sparse["pos"]])
+
+
+def _evaluate(model, copies, species=0):
+    sizes, cells, frame = _frames()
+    off = np.concatenate([[0], np.cumsum(np.tile(sizes, copies))])
+    pos = torch.as_tensor(np.tile(frame, (copies, 1)), dtype=torch.float64).cuda().contiguous()
+    types = torch.full((32 * copies,), species, dtype=torch.int32, device="cuda")
+    out = model.compute_batch(off, pos, types, np.stack(cells * copies), (1, 1, 1), atom_energy=True)
+    return (out["forces"].cpu().numpy().reshape(copies, 32, 3), out["atom_energy"].cpu().numpy().reshape(copies, 32),
+            np.asarray(out["virials"]).reshape(copies, 2, -1))
+
+
+def _compare(a, b):
+    (F, E, V), (Fb, Eb, Vb) = a, b
+    f_scale, e_scale = np.abs(Fb).max(), np.abs(Eb).max()
+    # either side keeps 2e-5 of the largest force and 1e-5 of the largest energy from the oracle
+    assert np.abs(F - Fb[:1]).max() <= 2 * (2e-5 * f_scale + 2e-7)
+    assert np.abs(E - Eb[:1]).max() <= 2e-5 * e_scale
+    assert np.abs(V - Vb[:1]).max() <= 2e-5 * 32 * max(1.0, f_scale)
+
+
+@pytest.mark.parametrize("basis", ["bessel", "gaussian"])
+@pytest.mark.parametrize("name", ["p64_3_8", "p128_2_0", "p128_3_4", "p128_4_4"])
+def test_splines_match_tables(name, basis):
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES[name]
+    blob = make_blob(p, seed=83, bias_scale=0.2, e_ref_scale=0.5, basis=basis)
+    m = binding.Model(blob)
+    tiled = binding.Model(blob, node_tile=SPLINE_ROWS + 1)       # a tile by splines, one of 95 rows without
+    most = SPLINE_ROWS // 32
+    ref = _evaluate(m, most - 1)                                  # tables
+    by_splines = False
+    for model, copies in ((m, most), (m, most + 3), (tiled, most + 3)):
+        out = _evaluate(model, copies)
+        _compare(out, ref)
+        by_splines = by_splines or not np.array_equal(out[0][:1], ref[0][:1])
+        if model is m:
+            assert np.array_equal(out[0], np.repeat(out[0][:1], copies, axis=0))      # copies agree bit for bit
+    assert by_splines
+    _compare(_evaluate(m, most, species=p["T"] - 1), _evaluate(m, most - 1, species=p["T"] - 1))     # another pair, same fit
+    m.close()
+    tiled.close()
+
+
+@pytest.mark.parametrize("case", ["steep", "coarse"])
+def test_maps_without_a_fit_keep_their_tables(case):
+    from paper_2608_19041_b200 import binding
+    p = SMALL_PROFILES["p128_3_4"]
+    # a high frequency that a few hundred intervals cannot follow; a table with fewer knots than intervals
+    m = binding.Model(_steep_blob(p, 3, 1.0, 250)) if case == "steep" else binding.Model(make_blob(p, seed=83), table_dx=0.05)
+    most = SPLINE_ROWS // 32
+    a, b = _evaluate(m, most), _evaluate(m, most - 1)
+    assert np.array_equal(a[0][:-1], b[0]) and np.array_equal(a[1][:-1], b[1])
+    m.close()
