@@ -472,7 +472,7 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     int rc = ensure_device_model(h);
     if (rc != UMLMD_OK) return rc;
     h->have_list = false;            // (until it and the workspace for it are complete)
-    { Scope sc(h, kNeighbor, 5 + (fetch && N > 0)); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, fetch, h->st, &h->err); }
+    { Scope sc(h, kNeighbor, neighbor_launches(N, fetch != nullptr)); rc = neighbor_build(&h->nb, N, h->n_owned, d_pos, d_type, cell, pbc, skin, h->hm.rc, h->d_err, fetch, h->st, &h->err); }
     if (rc != UMLMD_OK) return rc;
     h->have_edge_grad = false;       // edges were renumbered
     h->have_groups = false;          // rows as well

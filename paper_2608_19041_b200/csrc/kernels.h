@@ -21,6 +21,7 @@ struct BuildFetch { int T; int* d_flags; int* h_flags; int* h_err; };
 int neighbor_build(NeighborDev* nb, int64_t N, int64_t n_owned, const double* d_pos, const int32_t* d_type,
                    const double cell[9], const int pbc[3], double skin, double rc, int* d_err,
                    const BuildFetch* fetch, cudaStream_t st, std::string* err);   // cell: the three cell vectors as rows
+int neighbor_launches(int64_t N, bool fetch);     // kernels of this library that a build launches
 void neighbor_free(NeighborDev* nb);
 // Export the list in caller numbering (device buffers of the caller).
 int neighbor_export(NeighborDev* nb, int32_t* d_row_ptr, int32_t* d_src, int8_t* d_shift,

@@ -106,12 +106,8 @@ __global__ void k_bounds(int N, const double* __restrict__ pos, Grid g, unsigned
     }
 }
 
-// fold positions into the cell, bin them
-__global__ void k_fold_bin(int N, const double* __restrict__ pos, Grid g, double* __restrict__ wpos,
-                           int* __restrict__ img_o, int* __restrict__ key, int* __restrict__ idx,
-                           int* __restrict__ err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+// fold the position of atom i into the cell; its bin
+__device__ __forceinline__ int fold_atom(int i, const double* __restrict__ pos, const Grid& g, double* wpos, int* img_o, int* __restrict__ err) {
     int c[3];
     bool bad = false;
     if (g.tri) {
@@ -156,8 +152,32 @@ __global__ void k_fold_bin(int N, const double* __restrict__ pos, Grid g, double
         atomicOr(err, kErrNonFinite);
         c[0] = c[1] = c[2] = 0;
     }
-    key[i] = (c[2] * g.nc[1] + c[1]) * g.nc[0] + c[0] + (i >= g.n_owned ? g.ncell : 0);
+    return (c[2] * g.nc[1] + c[1]) * g.nc[0] + c[0] + (i >= g.n_owned ? g.ncell : 0);
+}
+__global__ void k_fold_bin(int N, const double* __restrict__ pos, Grid g, double* __restrict__ wpos,
+                           int* __restrict__ img_o, int* __restrict__ key, int* __restrict__ idx,
+                           int* __restrict__ err) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    key[i] = fold_atom(i, pos, g, wpos, img_o, err);
     idx[i] = i;
+}
+
+// atom o as the i-th of the internal order
+__device__ __forceinline__ void sorted_atom(int i, int o, const double* wpos, const int* img_o, const int* __restrict__ type,
+                                            int* __restrict__ perm, double* __restrict__ xs0, double* __restrict__ xs, float4* __restrict__ rec,
+                                            int* __restrict__ img, int* __restrict__ type_s) {
+    perm[i] = o;
+    type_s[i] = type[o];
+    float hi[3];
+    for (int k = 0; k < 3; ++k) {
+        const double w = wpos[3 * (size_t)o + k];
+        xs0[3 * (size_t)i + k] = w;
+        xs[3 * (size_t)i + k] = w;
+        img[3 * (size_t)i + k] = img_o[3 * (size_t)o + k];
+        hi[k] = (float)w;
+    }
+    rec[i] = make_float4(hi[0], hi[1], hi[2], 0.f);   // what the scans read
 }
 
 // gather the per-atom arrays into sorted order; where the sorted key rises from one atom to the next,
@@ -182,18 +202,94 @@ __global__ void k_gather_sorted(int N, int nkeys, const int* __restrict__ skey, 
         for (int c = lane; c < n_l; c += 32) cell_start[lo_l + c] = i_l;
     }
     if (i >= N) return;
-    const int o = sidx[i];
-    perm[i] = o;
-    type_s[i] = type[o];
-    float hi[3];
-    for (int k = 0; k < 3; ++k) {
-        const double w = wpos[3 * (size_t)o + k];
-        xs0[3 * (size_t)i + k] = w;
-        xs[3 * (size_t)i + k] = w;
-        img[3 * (size_t)i + k] = img_o[3 * (size_t)o + k];
-        hi[k] = (float)w;
+    sorted_atom(i, sidx[i], wpos, img_o, type, perm, xs0, xs, rec, img, type_s);
+}
+
+// Up to kBinTogether atoms: bins, their order and the sorted arrays by one block in one launch (fold, sort and gather as three
+// took 3.5 + 6.1 + 4.9 us at 597 atoms, and the gaps between them).
+constexpr int kBinTogether = 4096, kBinThreads = 1024;
+template <int ITEMS>
+__global__ void __launch_bounds__(kBinThreads) k_bin_together(int N, int nkeys, int end_bit, const double* __restrict__ pos, Grid g,
+                                                              const int* __restrict__ type, double* wpos, int* img_o,
+                                                              int* __restrict__ skey, int* __restrict__ perm, double* __restrict__ xs0,
+                                                              double* __restrict__ xs, float4* __restrict__ rec, int* __restrict__ img,
+                                                              int* __restrict__ type_s, int* __restrict__ cell_start, int* __restrict__ err) {
+    using Sort = cub::BlockRadixSort<int, kBinThreads, ITEMS, int>;
+    __shared__ union { typename Sort::TempStorage sort; int keys[kBinThreads * ITEMS]; } sh;
+    int key[ITEMS], idx[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = threadIdx.x * ITEMS + k;
+        idx[k] = i;
+        key[k] = i < N ? fold_atom(i, pos, g, wpos, img_o, err) : nkeys;       // (what is no atom comes last: nkeys < 2^end_bit)
     }
-    rec[i] = make_float4(hi[0], hi[1], hi[2], 0.f);   // what the scans read
+    Sort(sh.sort).Sort(key, idx, 0, end_bit);
+    __syncthreads();                                  // (the folded positions of the block are there, the sort is done with its area)
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = threadIdx.x * ITEMS + k;
+        sh.keys[i] = key[k];
+        if (i < N) {
+            skey[i] = key[k];
+            sorted_atom(i, idx[k], wpos, img_o, type, perm, xs0, xs, rec, img, type_s);
+        }
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c <= nkeys; c += kBinThreads) {                   // first atom of every bin, and N
+        int lo = 0, hi = N;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sh.keys[mid] < c) lo = mid + 1;
+            else hi = mid;
+        }
+        cell_start[c] = lo;
+    }
+}
+
+// Up to kOffsetsTogether rows: row offsets from row lengths and all that the host waits for, by one block, which writes the results
+// to the host's pinned memory itself (otherwise the scan's two launches, the flags' kernel, three clears and four copies).
+// h_flags null: the totals alone.
+constexpr int kOffsetsTogether = 8192;
+__global__ void __launch_bounds__(1024) k_row_offsets(int N, int n_owned, const int* __restrict__ deg, eidx_t* __restrict__ row_ptr,
+                                                      const int* __restrict__ type, int T, eidx_t* __restrict__ h_totals,
+                                                      int* __restrict__ h_flags, int* __restrict__ h_err, int* __restrict__ err) {
+    __shared__ eidx_t warp_sum[32];
+    __shared__ int present[1024];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (N + 1023) / 1024, first = tid * per, last = min(first + per, N);
+    present[tid] = 0;
+    __syncthreads();
+    eidx_t sum = 0;
+    bool bad = false;
+    for (int i = first; i < last; ++i) {
+        sum += deg[i];
+        if (h_flags) {
+            const int t = type[i];
+            if (t < 0 || t >= T) bad = true;
+            else present[t] = 1;
+        }
+    }
+    eidx_t upto = sum;                                // inclusive over the warp
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const eidx_t v = __shfl_up_sync(0xffffffffu, upto, off);
+        if (lane >= off) upto += v;
+    }
+    if (lane == 31) warp_sum[warp] = upto;
+    if (bad) atomicOr(err, kErrSpecies);
+    __syncthreads();
+    eidx_t at = upto - sum;
+    for (int w = 0; w < warp; ++w) at += warp_sum[w];
+    for (int i = first; i < last; ++i) {
+        row_ptr[i] = at;
+        if (i == n_owned) h_totals[1] = at;
+        at += deg[i];
+    }
+    if (tid == 1023) { row_ptr[N] = at; h_totals[0] = at; }     // (the last thread's end is everyone's)
+    if (h_flags) {
+        for (int t = tid; t < T; t += 1024) h_flags[t] = present[t];
+        if (tid == 0) *h_err = atomicExch(err, 0);
+    }
 }
 
 // Squared list radius, its single-precision value, and a band around that outside of which a squared
@@ -690,13 +786,23 @@ void neighbor_free(NeighborDev* nb) {
 // know by then, and the edge arrays grow to hold the list.
 static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, int* d_err, const BuildFetch* fetch, cudaStream_t st,
                        std::string* err) {
-    NB_CHECK(cudaMemcpyAsync(nb->h_totals, nb->row_ptr + N, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
-    if (n_owned < N) NB_CHECK(cudaMemcpyAsync(nb->h_totals + 1, nb->row_ptr + n_owned, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
-    if (fetch) {
-        NB_CHECK(launch_species_present(N, d_type, fetch->T, fetch->d_flags, d_err, st));
-        NB_CHECK(cudaMemcpyAsync(fetch->h_flags, fetch->d_flags, sizeof(int) * (size_t)fetch->T, cudaMemcpyDeviceToHost, st));
-        NB_CHECK(cudaMemcpyAsync(fetch->h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-        NB_CHECK(cudaMemsetAsync(d_err, 0, sizeof(int), st));
+    if (N <= kOffsetsTogether) {
+        k_row_offsets<<<1, 1024, 0, st>>>(N, n_owned, nb->deg, nb->row_ptr, d_type, fetch ? fetch->T : 0, nb->h_totals,
+                                          fetch ? fetch->h_flags : nullptr, fetch ? fetch->h_err : nullptr, d_err);
+        NB_CHECK(cudaGetLastError());
+    } else {
+        NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
+        size_t tmp_bytes = nb->cub_bytes;
+        auto deg_wide = thrust::make_transform_iterator(static_cast<const int*>(nb->deg), WidenDeg());
+        NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, N + 1, st));
+        NB_CHECK(cudaMemcpyAsync(nb->h_totals, nb->row_ptr + N, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
+        if (n_owned < N) NB_CHECK(cudaMemcpyAsync(nb->h_totals + 1, nb->row_ptr + n_owned, sizeof(eidx_t), cudaMemcpyDeviceToHost, st));
+        if (fetch) {
+            NB_CHECK(launch_species_present(N, d_type, fetch->T, fetch->d_flags, d_err, st));
+            NB_CHECK(cudaMemcpyAsync(fetch->h_flags, fetch->d_flags, sizeof(int) * (size_t)fetch->T, cudaMemcpyDeviceToHost, st));
+            NB_CHECK(cudaMemcpyAsync(fetch->h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+            NB_CHECK(cudaMemsetAsync(d_err, 0, sizeof(int), st));
+        }
     }
     NB_CHECK(cudaStreamSynchronize(st));
     const int64_t total = nb->h_totals[0];
@@ -711,6 +817,8 @@ static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, i
     }
     return UMLMD_OK;
 }
+
+int neighbor_launches(int64_t N, bool fetch) { return N <= kBinTogether ? 5 : (N <= kOffsetsTogether ? 6 : 5 + fetch); }
 
 int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double* d_pos, const int32_t* d_type,
                    const double cell[9], const int pbc[3], double skin, double rc, int* d_err,
@@ -844,7 +952,6 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     int* img_o = nb->img + 3 * (size_t)(N + 1);
 
     const int TB = 256;
-    k_fold_bin<<<(N + TB - 1) / TB, TB, 0, st>>>(N, d_pos, g, nb->wpos, img_o, nb->key, nb->idx, d_err);
     int end_bit = 1;
     while ((1LL << end_bit) < nkeys) ++end_bit;
     size_t need_tmp = 0, need_scan = 0;
@@ -862,11 +969,20 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
         NB_CHECK(dev_malloc(&nb->cub_tmp, need_tmp + 256));
         nb->cub_bytes = need_tmp + 256;
     }
-    size_t tmp_bytes = nb->cub_bytes;
-    NB_CHECK(cub::DeviceRadixSort::SortPairs(nb->cub_tmp, tmp_bytes, nb->key, nb->key2, nb->idx, nb->idx2, N,
-                                             0, end_bit, st));
-    k_gather_sorted<<<N / TB + 1, TB, 0, st>>>(N, (int)nkeys, nb->key2, nb->idx2, nb->wpos, img_o, d_type, nb->perm, nb->xs0,
-                                              nb->xs, nb->rec, nb->img, nb->type_s, nb->cell_start);
+    if (N <= kBinTogether) {
+        int bits = 1;
+        while ((1LL << bits) <= nkeys) ++bits;           // (one key more: no atom)
+        auto bin = N <= kBinThreads ? k_bin_together<1> : k_bin_together<kBinTogether / kBinThreads>;
+        bin<<<1, kBinThreads, 0, st>>>(N, (int)nkeys, bits, d_pos, g, d_type, nb->wpos, img_o, nb->key2, nb->perm, nb->xs0, nb->xs, nb->rec,
+                                       nb->img, nb->type_s, nb->cell_start, d_err);
+    } else {
+        k_fold_bin<<<(N + TB - 1) / TB, TB, 0, st>>>(N, d_pos, g, nb->wpos, img_o, nb->key, nb->idx, d_err);
+        size_t tmp_bytes = nb->cub_bytes;
+        NB_CHECK(cub::DeviceRadixSort::SortPairs(nb->cub_tmp, tmp_bytes, nb->key, nb->key2, nb->idx, nb->idx2, N,
+                                                 0, end_bit, st));
+        k_gather_sorted<<<N / TB + 1, TB, 0, st>>>(N, (int)nkeys, nb->key2, nb->idx2, nb->wpos, img_o, d_type, nb->perm, nb->xs0,
+                                                  nb->xs, nb->rec, nb->img, nb->type_s, nb->cell_start);
+    }
     // Eight centres per warp and a block of four warps per cell; below 16384 atoms, where the cells are
     // too few to fill the machine that way, two centres per warp and four blocks per cell (4000 atoms,
     // 125 cells: count and fill 19 + 24 us; with one block per cell they took 34 + 45).
@@ -886,9 +1002,6 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     auto scan = apart ? (few ? k_scan_cells<false, 2, true> : k_scan_cells<false, 8, true>)
                        : (few ? k_scan_cells<false, 2, false> : k_scan_cells<false, 8, false>);
     scan<<<scan_blocks, scan_threads, 0, st>>>(N, span, g, nr, nb->key2, nb->cell_start, nb->rec, nb->xs0, nb->deg, nullptr, nullptr, d_err);
-    NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
-    tmp_bytes = nb->cub_bytes;
-    NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, N + 1, st));
     int code = read_totals(nb, N, n_owned, d_type, d_err, fetch, st, err);
     if (code != UMLMD_OK) return code;
     if (nb->E > 0) {
@@ -1001,9 +1114,6 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
     k_batch_fold<<<n_frames, TB, 0, st>>>(nb->frames, d_pos, d_type, T, rc, 1.0 / nb->quantum, nb->xs, nb->rec, nb->fix, nb->type_s, nb->frame_of, nb->perm, d_err);
     const int wb = (int)((N + TB / 32 - 1) / (TB / 32));
     k_batch_scan<false><<<wb, TB, 0, st>>>((int)N, nb->frames, nb->frame_of, rc, nb->xs, nb->rec, nb->deg, nullptr, nullptr);
-    NB_CHECK(cudaMemsetAsync(nb->deg + N, 0, sizeof(int), st));
-    size_t tmp_bytes = nb->cub_bytes;
-    NB_CHECK(cub::DeviceScan::ExclusiveScan(nb->cub_tmp, tmp_bytes, deg_wide, nb->row_ptr, cub::Sum(), (eidx_t)0, (int)N + 1, st));
     nb->n_owned = N;
     int code = read_totals(nb, (int)N, (int)N, nb->type_s, d_err, fetch, st, err);
     if (code != UMLMD_OK) return code;
