@@ -41,7 +41,7 @@ struct umlmd {
     std::vector<double> spline_coef;                 // of the radial map and modes
     bool have_groups = false;                        // moment_order belongs to the current list
     float* g = nullptr; int64_t g_cap = 0;
-    double* e_atom = nullptr; double* f_sorted = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
+    double* e_atom = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
     double* virial_part = nullptr; int64_t vpart_cap = 0;
     double* frame_out = nullptr; int64_t frame_out_cap = 0;     // batched evaluation: [n_frames][10] energy, virial
     double* h_frame = nullptr; int64_t h_frame_cap = 0;         // pinned copy of it: part of `pinned`, or frame_pinned for many frames
@@ -194,11 +194,10 @@ int ensure_workspace(umlmd_t* h) {
         int64_t c;
         h->n_cap = 0;
         c = 0; API_CUDA(h, dev_ensure(&h->e_atom, &c, N));
-        c = 0; API_CUDA(h, dev_ensure(&h->f_sorted, &c, N * 3));
         c = 0; API_CUDA(h, dev_ensure(&h->type_o, &c, N));
         h->n_cap = N;
     }
-    const int64_t vneed = (edge_blocks_max(N, B) + 2) * 9;
+    const int64_t vneed = std::max(edge_blocks_max(N, B) + 2, h->nb.batch ? N : 0) * 9;       // (a batch keeps them by row)
     if (vneed > h->vpart_cap || !h->virial_part) API_CUDA(h, dev_ensure(&h->virial_part, &h->vpart_cap, vneed));
     return UMLMD_OK;
 }
@@ -294,20 +293,13 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         }
     }
     h->have_edge_grad = want_grad;
-    if (nb.batch) {                   // frames are reduced one by one
-        if (want_grad) {
-            Scope sc(h, kForce, 1);
-            API_CUDA(h, launch_force_assembly(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, h->d_err, h->st));
-        }
-        if (d_atom_energy) { Scope sc(h, kReduce, 1); API_CUDA(h, launch_scatter_atom_energy(nb, h->e_atom, d_atom_energy, h->st)); }
-        return UMLMD_OK;
-    }
+    if (nb.batch) return UMLMD_OK;    // (frames are reduced one by one: umlmd_compute_batch)
     double* const ho = to_host ? h->h_out : nullptr;
     int* const he = to_host ? h->h_err : nullptr;
     unsigned* const counter = (unsigned*)h->d_err + 1;
-    if (want_grad) {
+    if (d_force) {
         Scope sc(h, kForce, assemble_launches(N));
-        API_CUDA(h, launch_assemble(nb, h->g, d_force ? nullptr : h->f_sorted, d_force, tail ? *tail : StepTail{}, h->e_atom, d_atom_energy,
+        API_CUDA(h, launch_assemble(nb, h->g, d_force, tail ? *tail : StepTail{}, h->e_atom, d_atom_energy,
                                     h->virial_part, vpart_used, h->scratch, counter, h->d_out, h->d_err, ho, he, h->st));
     } else {
         Scope sc(h, kReduce, 1);
@@ -630,7 +622,7 @@ int umlmd_destroy(umlmd_t* h) {
     if (h->on_device) cudaStreamSynchronize(h->st);
     for (void* p : h->model_allocs) dev_free(p);
     neighbor_free(&h->nb);
-    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->moments, h->moment_order, h->moment_scratch, h->spline, h->g, h->e_atom, h->f_sorted, h->type_o, h->virial_part,
+    void* ptrs[] = {h->frame_out, h->state, h->desc, h->pre, h->hbuf, h->tc_hi, h->tc_lo, h->fused_scratch, h->moments, h->moment_order, h->moment_scratch, h->spline, h->g, h->e_atom, h->type_o, h->virial_part,
                     h->scratch, h->d_out, h->d_err, h->md_force, h->d_mass, h->d_inv_mass, h->d_nhc, h->uni, h->d_species};
     for (void* p : ptrs) dev_free(p);
     for (auto& sp : h->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }
@@ -763,8 +755,8 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
     t += grown(3 * n_edges, 4);
-    t += buf(N, 8) + buf(3 * N, 8) + buf(N, 4);
-    t += buf((edge_blocks_max(N, Bt) + 2) * 9, 8);
+    t += buf(N, 8) + buf(N, 4);
+    t += buf(std::max(edge_blocks_max(N, Bt) + 2, N) * 9, 8);
     t += buf(3 * N, 8) + 2 * buf(d.T, 8) + buf(2 * kNhcChain + 2, 8);
     *bytes = t;
     return UMLMD_OK;
@@ -858,8 +850,10 @@ int umlmd_compute_batch(umlmd_t* h, int32_t n_frames, const int64_t* frame_offse
         h->h_frame_cap = n_out;
     }
     if (N > 0) {
+        double* const row_virial = virials ? h->virial_part : nullptr;         // (the edge kernels' partial sums are not needed)
+        if (want_grad) { Scope sc(h, kForce, 1); API_CUDA(h, launch_frame_rows(h->nb, h->g, d_force, row_virial, h->d_err, h->st)); }
         Scope sc(h, kReduce, 1);
-        API_CUDA(h, launch_frame_reduce(h->nb, h->e_atom, h->g, virials != nullptr, h->frame_out, h->d_err, h->st));
+        API_CUDA(h, launch_frame_reduce(h->nb, h->e_atom, d_atom_energy, row_virial, h->frame_out, h->d_err, h->st));
     } else {
         API_CUDA(h, cudaMemsetAsync(h->frame_out, 0, sizeof(double) * (size_t)n_out, h->st));
     }

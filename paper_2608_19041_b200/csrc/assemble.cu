@@ -78,25 +78,6 @@ __device__ __forceinline__ void force_of_row(int row, const eidx_t* __restrict__
     f[0] = fx; f[1] = fy; f[2] = fz;
 }
 
-// out (caller numbering, through perm) and / or f (sorted numbering) may be null
-__global__ void k_force_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
-                             const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
-                             double* __restrict__ out, int* __restrict__ err) {
-    chain_begin();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= N) return;
-    double v[3];
-    force_of_row(warp, row_ptr, rev, g, v);
-    if (lane == 0) {
-        if (f) { f[3 * (size_t)warp] = v[0]; f[3 * (size_t)warp + 1] = v[1]; f[3 * (size_t)warp + 2] = v[2]; }
-        if (out) {
-            const size_t o = 3 * (size_t)perm[warp];
-            out[o] = v[0]; out[o + 1] = v[1]; out[o + 2] = v[2];
-            if (!isfinite(v[0]) || !isfinite(v[1]) || !isfinite(v[2])) atomicOr(err, kErrNonFinite);
-        }
-    }
-}
-
 // Per-atom share of the virial, one warp per atom over its own row: every directed edge gives half
 // of -g_e (x) r_e to its centre and half to its neighbour, so atom i collects
 // -1/2 sum_{e in row(i)} (g_e - g_rev(e)) (x) r_e (the reverse edge has the opposite vector).
@@ -141,27 +122,6 @@ __global__ void k_atom_virial(int N, const eidx_t* __restrict__ row_ptr, const i
         for (int k = 0; k < 9; ++k) if (lane == k) v = w[k];
         out[9 * (size_t)perm[warp] + lane] = -0.5 * v;
     }
-}
-
-__global__ void k_scatter3(int N, const int* __restrict__ perm, const double* __restrict__ in,
-                           double* __restrict__ out, int* __restrict__ err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int o = perm[i];
-    bool bad = false;
-    for (int k = 0; k < 3; ++k) {
-        const double v = in[3 * (size_t)i + k];
-        if (!isfinite(v)) bad = true;
-        out[3 * (size_t)o + k] = v;
-    }
-    if (bad) atomicOr(err, kErrNonFinite);
-}
-
-__global__ void k_scatter1(int N, const int* __restrict__ perm, const double* __restrict__ in,
-                           double* __restrict__ out) {
-    chain_begin();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) out[perm[i]] = in[i];
 }
 
 __global__ void k_unsort_rows(int N, const int* __restrict__ perm, const float* __restrict__ in, int stride,
@@ -213,37 +173,67 @@ __device__ __forceinline__ double block_sums(double* v, double* sh) {
     return s;
 }
 
-// Segmented reduction of a batched evaluation: block f sums the atomic energies of frame f and,
-// when asked, -g (x) r over the edges of the frame's rows (edge vectors recomputed from the
-// positions and the frame's cell): a warp per row, lanes over its edges, then one fixed-order block
-// sum.  Latency-bound: a frame is one block (64 frames of 54 to 108 atoms: 15 us; with a thread per row,
-// whose edges followed one another, 74 us).
-constexpr int kFrameBlock = 1024;
+// Rows of a batched evaluation, a warp each: the force on the row's atom (caller order is internal order) and, when asked
+// (row_virial), the nine sums of g (x) r over its edges, edge vectors recomputed in double from the positions and the
+// frame's cell.  With the virial in the reduction by frame, a block each, 64 frames of 54 to 108 atoms took 6.7 + 15 us.
+__global__ void k_frame_rows(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev, const int2* __restrict__ nbr,
+                             const float* __restrict__ g, const double* __restrict__ xs, const FrameCell* __restrict__ frames,
+                             const int* __restrict__ frame_of, double* __restrict__ out, double* __restrict__ row_virial, int* __restrict__ err) {
+    chain_begin();
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (row >= N) return;
+    if (out) {
+        double f[3];
+        force_of_row(row, row_ptr, rev, g, f);
+        if (lane < 3) {
+            const double mine = lane == 0 ? f[0] : (lane == 1 ? f[1] : f[2]);
+            out[3 * (size_t)row + lane] = mine;
+            if (!isfinite(mine)) atomicOr(err, kErrNonFinite);
+        }
+    }
+    if (!row_virial) return;
+    const double* const H = frames[frame_of[row]].H;
+    const double xi = xs[3 * (size_t)row], yi = xs[3 * (size_t)row + 1], zi = xs[3 * (size_t)row + 2];
+    double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    const eidx_t e1 = row_ptr[row + 1];
+    for (eidx_t k = row_ptr[row] + lane; k < e1; k += 32) {
+        const int2 js = nbr[k];
+        const int j = js.x, s = js.y;
+        const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff), nz = (int)(signed char)((s >> 16) & 0xff);
+        const double r[3] = {(xs[3 * (size_t)j] + ((nx * H[0] + ny * H[3]) + nz * H[6])) - xi,
+                             (xs[3 * (size_t)j + 1] + ((nx * H[1] + ny * H[4]) + nz * H[7])) - yi,
+                             (xs[3 * (size_t)j + 2] + ((nx * H[2] + ny * H[5]) + nz * H[8])) - zi};
+        const double gg[3] = {(double)g[3 * (size_t)k], (double)g[3 * (size_t)k + 1], (double)g[3 * (size_t)k + 2]};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) v[3 * a + b] += gg[a] * r[b];
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+        if (lane == k) row_virial[9 * (size_t)row + k] = v[k];
+    }
+}
+
+// Segmented reduction of a batched evaluation: block f sums the atomic energies of frame f, which go to e_out (may be null) on
+// the way, and, when asked, its rows' virials, in a fixed order.
+constexpr int kFrameBlock = 256;
 __global__ void __launch_bounds__(kFrameBlock) k_frame_reduce(const FrameCell* __restrict__ frames, const double* __restrict__ e_atom,
-                                                              const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr,
-                                                              const float* __restrict__ g, const double* __restrict__ xs, bool want_virial,
+                                                              double* __restrict__ e_out, const double* __restrict__ row_virial,
                                                               double* __restrict__ out, int* __restrict__ err) {
     __shared__ double sh[kFrameBlock / 32 * 10];
     chain_begin();
     const FrameCell& fc = frames[blockIdx.x];
-    const int lane = threadIdx.x & 31;
     double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i = fc.a0 + threadIdx.x; i < fc.a1; i += kFrameBlock) v[0] += e_atom[i];
-    for (int i = fc.a0 + (threadIdx.x >> 5); want_virial && i < fc.a1; i += kFrameBlock / 32) {
-        const double xi = xs[3 * (size_t)i], yi = xs[3 * (size_t)i + 1], zi = xs[3 * (size_t)i + 2];
-        const eidx_t e1 = row_ptr[i + 1];
-        for (eidx_t k = row_ptr[i] + lane; k < e1; k += 32) {
-            const int2 js = nbr[k];
-            const int j = js.x, s = js.y;
-            const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff), nz = (int)(signed char)((s >> 16) & 0xff);
-            const double r[3] = {(xs[3 * (size_t)j] + ((nx * fc.H[0] + ny * fc.H[3]) + nz * fc.H[6])) - xi,
-                                 (xs[3 * (size_t)j + 1] + ((nx * fc.H[1] + ny * fc.H[4]) + nz * fc.H[7])) - yi,
-                                 (xs[3 * (size_t)j + 2] + ((nx * fc.H[2] + ny * fc.H[5]) + nz * fc.H[8])) - zi};
-            const double gg[3] = {(double)g[3 * (size_t)k], (double)g[3 * (size_t)k + 1], (double)g[3 * (size_t)k + 2]};
+    for (int i = fc.a0 + threadIdx.x; i < fc.a1; i += kFrameBlock) {
+        const double e = e_atom[i];
+        v[0] += e;
+        if (e_out) e_out[i] = e;
+        if (row_virial) {
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) v[1 + 3 * a + b] += gg[a] * r[b];
+            for (int k = 0; k < 9; ++k) v[1 + k] += row_virial[9 * (size_t)i + k];
         }
     }
     const double s = block_sums<10>(v, sh);
@@ -324,7 +314,7 @@ __global__ void __launch_bounds__(kRedBlock) k_reduce(const ReduceArgs a) {
 constexpr int kReduceTogether = 32768;
 template <bool REDUCE>
 __global__ void __launch_bounds__(kRedBlock) k_assemble(int N, const eidx_t* __restrict__ row_ptr, const eidx_t* __restrict__ rev,
-                                                        const float* __restrict__ g, double* __restrict__ f, const int* __restrict__ perm,
+                                                        const float* __restrict__ g, const int* __restrict__ perm,
                                                         double* __restrict__ out, int* __restrict__ err, const ReduceArgs a, const StepTail t) {
     __shared__ double sh[kRedBlock / 32 * 10];
     __shared__ bool last;
@@ -339,11 +329,8 @@ __global__ void __launch_bounds__(kRedBlock) k_assemble(int N, const eidx_t* __r
             const int o = perm[row];
             const double mine = lane == 0 ? v[0] : (lane == 1 ? v[1] : v[2]);
             if (lane < 3) {
-                if (f) f[3 * (size_t)row + lane] = mine;
-                if (out) {
-                    out[3 * (size_t)o + lane] = mine;
-                    if (!isfinite(mine)) atomicOr(err, kErrNonFinite);
-                }
+                out[3 * (size_t)o + lane] = mine;
+                if (!isfinite(mine)) atomicOr(err, kErrNonFinite);
             }
             if (t.pos) {
                 // (of the positions that this step has evaluated: the next ones may be binned anew first)
@@ -507,14 +494,6 @@ inline void slices(int64_t N, int* blocks, int64_t* chunk) {
 
 int reduce_scratch_doubles(int64_t) { return kReduceBlocks * 10; }      // (more than kRedMaxBlocks)
 
-// forces in sorted numbering (f_sorted) and / or scattered to the caller's numbering (d_force)
-cudaError_t launch_force_assembly(const NeighborDev& nb, const float* g, double* f_sorted, double* d_force,
-                                  int* d_err, cudaStream_t st) {
-    const int N = (int)nb.N;
-    if (N == 0) return cudaSuccess;
-    return launch_chained(k_force_rows, (N + 7) / 8, 256, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err);
-}
-
 cudaError_t launch_atom_virial(const NeighborDev& nb, const float* g, double* d_out, cudaStream_t st) {
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
@@ -524,19 +503,17 @@ cudaError_t launch_atom_virial(const NeighborDev& nb, const float* g, double* d_
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_forces(const NeighborDev& nb, const double* f_sorted, double* d_force, int* d_err,
-                                  cudaStream_t st) {
+cudaError_t launch_frame_rows(const NeighborDev& nb, const float* g, double* d_force, double* row_virial, int* d_err, cudaStream_t st) {
     const int N = (int)nb.N;
-    if (N == 0) return cudaSuccess;
-    k_scatter3<<<(N + 255) / 256, 256, 0, st>>>(N, nb.perm, f_sorted, d_force, d_err);
-    return cudaGetLastError();
+    if (N == 0 || (!d_force && !row_virial)) return cudaSuccess;
+    return launch_chained(k_frame_rows, (N + 7) / 8, 256, 0, st, N, nb.row_ptr, nb.rev, nb.nbr, g, nb.xs, nb.frames, nb.frame_of, d_force,
+                          row_virial, d_err);
 }
 
-cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
-                                double* d_out, int* d_err, cudaStream_t st) {
+cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* row_virial, double* d_out,
+                                int* d_err, cudaStream_t st) {
     if (nb.n_frames <= 0) return cudaSuccess;
-    return launch_chained(k_frame_reduce, nb.n_frames, kFrameBlock, 0, st, nb.frames, e_atom, nb.row_ptr, nb.nbr, g, nb.xs, want_virial,
-                          d_out, d_err);
+    return launch_chained(k_frame_reduce, nb.n_frames, kFrameBlock, 0, st, nb.frames, e_atom, d_atom_energy, row_virial, d_out, d_err);
 }
 
 static ReduceArgs reduce_args(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part,
@@ -554,15 +531,15 @@ cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_a
 }
 
 int assemble_launches(int64_t N) { return N <= kReduceTogether ? 1 : 2; }
-cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* f_sorted, double* d_force, const StepTail& tail,
+cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* d_force, const StepTail& tail,
                             const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part, double* scratch,
                             unsigned* counter, double* out, int* d_err, double* h_out, int* h_err, cudaStream_t st) {
     const int N = (int)nb.N;
     const ReduceArgs a = reduce_args(nb, e_atom, d_atom_energy, virial_part, n_part, scratch, counter, out, d_err, h_out, h_err);
     const int rows = (N + kRedBlock / 32 - 1) / (kRedBlock / 32);
     if (N <= kReduceTogether)
-        return launch_chained(k_assemble<true>, a.n_blocks + rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err, a, tail);
-    const cudaError_t e = launch_chained(k_assemble<false>, rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, f_sorted, nb.perm, d_force, d_err, a, tail);
+        return launch_chained(k_assemble<true>, a.n_blocks + rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, nb.perm, d_force, d_err, a, tail);
+    const cudaError_t e = launch_chained(k_assemble<false>, rows, kRedBlock, 0, st, N, nb.row_ptr, nb.rev, g, nb.perm, d_force, d_err, a, tail);
     return e != cudaSuccess ? e : launch_chained(k_reduce, a.n_blocks, kRedBlock, 0, st, a);
 }
 
@@ -581,12 +558,6 @@ cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, 
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
     return launch_chained(k_gather_positions, (N + 255) / 256, 256, 0, st, N, nb.perm, d_pos, gather_args(nb, species_slot), d_err);
-}
-
-cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out, cudaStream_t st) {
-    const int N = (int)nb.N;
-    if (N == 0) return cudaSuccess;
-    return launch_chained(k_scatter1, (N + 255) / 256, 256, 0, st, N, nb.perm, e_sorted, d_out);
 }
 
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width, float* out,

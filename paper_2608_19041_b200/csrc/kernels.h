@@ -32,10 +32,12 @@ int neighbor_export(NeighborDev* nb, int32_t* d_row_ptr, int32_t* d_src, int8_t*
 int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, const double* cells, const int pbc[3],
                          const double* d_pos, const int32_t* d_type, int T, double rc, int* d_err, const BuildFetch* fetch,
                          cudaStream_t st, std::string* err);
-// per-frame energy and virial: out[10 f] = sum of e_atom over the frame, out[10 f + 1 ..] = -sum over
-// the frame's edges of g (x) r, each by one block in a fixed order
-cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, const float* g, bool want_virial,
-                                double* d_out, int* d_err, cudaStream_t st);
+// batched evaluation: forces (caller order is internal order; may be null) and per-row sums of g (x) r (may be null)
+cudaError_t launch_frame_rows(const NeighborDev& nb, const float* g, double* d_force, double* row_virial, int* d_err, cudaStream_t st);
+// per-frame energy and virial: out[10 f] = sum of e_atom over the frame, out[10 f + 1 ..] = -sum over the frame's rows of
+// row_virial (may be null), each by one block in a fixed order; the atomic energies go to d_atom_energy (may be null) as well
+cudaError_t launch_frame_reduce(const NeighborDev& nb, const double* e_atom, double* d_atom_energy, const double* row_virial, double* d_out,
+                                int* d_err, cudaStream_t st);
 // Rows first .. first + n - 1 of the caller's numbering with 64-bit offsets: d_row_ptr [n + 1] is
 // always filled; edges are copied while they fit `cap` (cap = 0 or null buffers: offsets only).
 int neighbor_export_rows(NeighborDev* nb, int64_t first, int64_t n, int64_t* d_row_ptr, int32_t* d_src,
@@ -239,15 +241,9 @@ struct StepTail {
 // d_flags[t] = 1 for every species t in [0, T) that occurs among the N atoms, 0 otherwise;
 // kErrSpecies is or-ed into *d_err when an index lies outside [0, T)
 cudaError_t launch_species_present(int64_t N, const int* type, int T, int* d_flags, int* d_err, cudaStream_t st);
-cudaError_t launch_force_assembly(const NeighborDev& nb, const float* g, double* d_force_sorted, double* d_force,
-                                  int* d_err, cudaStream_t st);
 // per-atom virial shares [N][9] in the caller's numbering from the edge gradients of the last
 // backward pass: W_i = -1/2 sum over the edges that touch atom i of g_e (x) r_e
 cudaError_t launch_atom_virial(const NeighborDev& nb, const float* g, double* d_out, cudaStream_t st);
-cudaError_t launch_scatter_forces(const NeighborDev& nb, const double* f_sorted, double* d_force,
-                                  int* d_err, cudaStream_t st);
-cudaError_t launch_scatter_atom_energy(const NeighborDev& nb, const double* e_sorted, double* d_out,
-                                       cudaStream_t st);
 // out[0] = sum e_atom, out[1..9] = -sum virial partials (fixed order, double), in one launch; the atomic
 // energies go to d_atom_energy (caller's numbering, may be null) on the way.  counter: a zero that comes
 // back as zero.  h_out, h_err (pinned, may be null): results and error word for the host; clears the word.
@@ -257,7 +253,7 @@ cudaError_t launch_reduce_energy_virial(const NeighborDev& nb, const double* e_a
 int reduce_scratch_doubles(int64_t N);
 // the same and the force assembly (in one launch, where few atoms make that the better one), with the rest of an MD step (tail)
 int assemble_launches(int64_t N);
-cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* d_force_sorted, double* d_force, const StepTail& tail,
+cudaError_t launch_assemble(const NeighborDev& nb, const float* g, double* d_force, const StepTail& tail,
                             const double* e_atom, double* d_atom_energy, const double* virial_part, int n_part, double* scratch,
                             unsigned* counter, double* out, int* d_err, double* h_out, int* h_err, cudaStream_t st);
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width,
