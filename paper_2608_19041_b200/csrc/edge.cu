@@ -565,9 +565,13 @@ k_edge_forward(const EdgeArgs a) {
                 psi_s[lane * TP + 8] = __int_as_float(k);
             }
             __syncwarp();
+            // (the places of successive edges overlap: a lane adds to what another lane of its group left there)
             float* const part = mom + (lane >> 3) * a.n_moments + (lane & 7);
-            for (int e = lane >> 3; e < nb; e += 4) part[__float_as_int(psi_s[e * TP + 8])] += psi_s[e * TP + (lane & 7)];
-            __syncwarp();
+            for (int e0 = 0; e0 < nb; e0 += 4) {
+                const int e = e0 + (lane >> 3);
+                if (e < nb) part[__float_as_int(psi_s[e * TP + 8])] += psi_s[e * TP + (lane & 7)];
+                __syncwarp();
+            }
             // amplitudes of the leading channels, four channels of an edge per lane
             constexpr int LE = 32 / W::NL1;
             for (int b0 = 0; b0 < nb; b0 += LE) {

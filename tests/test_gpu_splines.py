@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import dpa4c as orc
 from tests.test_host_tables import _steep_blob
 from workloads import SMALL_PROFILES, make_blob, make_system
 
@@ -72,3 +73,45 @@ def test_maps_without_a_fit_keep_their_tables(case):
     a, b = _evaluate(m, most), _evaluate(m, most - 1)
     assert np.array_equal(a[0][:-1], b[0]) and np.array_equal(a[1][:-1], b[1])
     m.close()
+
+
+def _lattice(atoms, spacing, jitter, seed):
+    n = int(np.ceil(atoms ** (1 / 3) - 1e-9))
+    rng = np.random.default_rng(seed)
+    pos = spacing * np.stack(np.meshgrid(*[np.arange(n)] * 3, indexing="ij"), -1).reshape(-1, 3)[rng.permutation(n ** 3)[:atoms]]
+    return pos + jitter * rng.standard_normal(pos.shape), np.diag([spacing * n] * 3)
+
+
+def _row_sums(blob, m, pos, cell, species, centers):
+    """Scalar channels' sums of the given rows: the library's, and those of the oracle."""
+    types = np.full(len(pos), species, dtype=np.int32)
+    p = torch.as_tensor(pos, dtype=torch.float64).cuda().contiguous()
+    m.build_neighbors(p, torch.as_tensor(types).cuda(), cell, (1, 1, 1), 0.0)
+    m.compute(p, forces=False, virial=False)
+    C0 = m.query()["C0"]
+    got = m.get_intermediates()[0][:, :C0].cpu().numpy()[centers].astype(np.float64)
+    o = orc.Oracle(blob)
+    w = orc.wrap_positions(pos, cell, (1, 1, 1))
+    dst, _, rij = orc.rows_to_edges(orc.neighbor_rows(w, cell, (1, 1, 1), o.p["rc"], centers=centers), centers, w, cell)
+    t = torch.full((len(dst),), species, dtype=torch.int64)
+    A = orc.aggregate(o.p, o.prm, o.pair, len(centers), torch.from_numpy(dst), t, t, torch.from_numpy(rij))[0]
+    return got, A[0].reshape(len(centers), C0).numpy()
+
+
+# neighbours at few distances: the weights of successive edges fall on the same or on the next places of the row; odd counts
+@pytest.mark.parametrize("jitter", [0.004, 0.1])
+@pytest.mark.parametrize("name,spacing", [("p64_3_8", 1.6), ("p128_2_0", 1.9)])
+def test_row_sums_follow_the_definition(name, spacing, jitter):
+    from paper_2608_19041_b200 import binding
+    blob = make_blob(SMALL_PROFILES[name], seed=84, bias_scale=0.2, e_ref_scale=0.5)
+    m = binding.Model(blob)
+    pos, cell = _lattice(SPLINE_ROWS + 7, spacing, jitter, 85)
+    got, ref = _row_sums(blob, m, pos, cell, 0, np.arange(5, len(pos), 8))
+    m.close()
+    # a row's sum of products has the rounding of its 168 single-precision terms in two levels: below 2^-22 of the sums' rms,
+    # six times that for the largest of 65,000 and more; a weight that is lost is 1e-3 and more
+    rms = np.sqrt((ref ** 2).mean())
+    err = got - ref
+    print(name, jitter, "rms %.2e max %.2e scale %.2e" % (np.sqrt((err ** 2).mean()) / rms, np.abs(err).max() / rms, (got * ref).sum() / (ref * ref).sum() - 1))
+    assert np.sqrt((err ** 2).mean()) <= 2.0 ** -22 * rms
+    assert np.abs(err).max() <= 6 * 2.0 ** -22 * rms
