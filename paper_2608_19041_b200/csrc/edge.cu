@@ -270,10 +270,12 @@ enum : int { kNoModes = 0, kModesPerEdge = 1, kMoments = 2, kSplines = 3 };
 // interval of a distance and place in it
 __device__ __forceinline__ int spline_interval(const EdgeArgs& a, float rho, float* t) {
     const int k = min((int)(rho * a.spline_inv_h), a.spline_n - 1);
-    *t = fmaf(rho, a.spline_inv_h, -(float)k);
+    *t = fmaf(rho, a.spline_inv_h_lo, fmaf(rho, a.spline_inv_h, -(float)k));
     return k;
 }
-// basis functions of degree six (times 6!) and seven (times 7!) that are not zero on the interval, by their recursion
+// basis functions of degree six (times 6!) and seven (times 7!) that are not zero on the interval, by their recursion.  The
+// coefficients (moments.cu) are divided by 7!, in double: a factor of 1 / 5040 in single precision is 1.4e-8 off, the same way for
+// every edge of every atom.
 __device__ __forceinline__ void spline_basis(float t, float* u6, float* u7) {
     float u[7];
     u[0] = 1.0f;
@@ -564,7 +566,7 @@ k_edge_forward(const EdgeArgs a) {
                 float t, u6[7], u7[8];
                 const int k = spline_interval(a, __int_as_float(es.y), &t);
                 spline_basis(t, u6, u7);
-                const float w = __int_as_float(es.w) * (1.0f / 5040.0f);
+                const float w = __int_as_float(es.w);            // (the coefficients hold 1 / 7!)
                 float4* const o = reinterpret_cast<float4*>(psi_s + lane * TP);
                 o[0] = make_float4(w * u7[0], w * u7[1], w * u7[2], w * u7[3]);
                 o[1] = make_float4(w * u7[4], w * u7[5], w * u7[6], w * u7[7]);
@@ -938,7 +940,7 @@ k_edge_backward(const EdgeArgs a) {
                         v = fmaf(hj, u7[j], v);
                         dv = fmaf(hj, j == 0 ? -u6[0] : (j == 7 ? u6[6] : u6[j - 1] - u6[j]), dv);
                     }
-                    sa = dchi * (1.0f / 5040.0f) * v + chi * (a.spline_inv_h * (1.0f / 720.0f)) * dv;
+                    sa = dchi * v + chi * (7.0f * a.spline_inv_h) * dv;
                 }
                 if (MODES == kMoments) {
                     const float* hr = mom + (qes[lane].y - ti * a.d.T) * (1 + a.d.R);

@@ -83,7 +83,7 @@ struct EdgeArgs {
     // one species, from enough rows on: n_moments spline weights per row (moments.cu); spline_n intervals of 1 / spline_inv_h,
     // 0: not by splines
     int spline_n;
-    float spline_inv_h;
+    float spline_inv_h, spline_inv_h_lo;      // (as two numbers)
 };
 constexpr int kEdgeRowsPerBlock = 4, kEdgeSplitRows = 1184;
 // present: device array of the n_present species indices, ascending

@@ -112,6 +112,8 @@ def test_row_sums_follow_the_definition(name, spacing, jitter):
     # six times that for the largest of 65,000 and more; a weight that is lost is 1e-3 and more
     rms = np.sqrt((ref ** 2).mean())
     err = got - ref
-    print(name, jitter, "rms %.2e max %.2e scale %.2e" % (np.sqrt((err ** 2).mean()) / rms, np.abs(err).max() / rms, (got * ref).sum() / (ref * ref).sum() - 1))
     assert np.sqrt((err ** 2).mean()) <= 2.0 ** -22 * rms
     assert np.abs(err).max() <= 6 * 2.0 ** -22 * rms
+    # what is common to all sums: gamma, beta and U of the pair are rounded by up to 2^-25, at random over the dozen channels and
+    # more that carry them
+    assert abs((got * ref).sum() / (ref * ref).sum() - 1) <= 8e-9
