@@ -382,6 +382,14 @@ int umlmd_eval_edge_tables(const umlmd_t* h, int32_t type_i, int32_t type_j, int
                            double* out_psi, double* out_dchipsi);
 
 /*
+ * The same for a system of one species whose scalar channels go by splines (from C0 = 64, 8192 rows and rows long enough on):
+ * psi_c of the pair (type, type) and its derivative with respect to rho at n distances in [0, rc] (host arrays, [n, C0];
+ * out_dpsi may be NULL), from the rounded coefficients that the kernels read.  The splines are fitted at umlmd_create, for
+ * models that they follow within the bounds of the tables; UMLMD_E_UNSUPPORTED_PROFILE where there are none.
+ */
+int umlmd_eval_edge_splines(umlmd_t* h, int32_t type, int64_t n, const double* rho, double* out_psi, double* out_dpsi);
+
+/*
  * Per-kernel-class accounting.  The handle always counts the kernels it launches; with
  * profiling enabled it also brackets each class with CUDA events on its stream (a few
  * microseconds of overhead per launch group, so leave it off when timing whole steps).

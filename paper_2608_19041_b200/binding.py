@@ -28,6 +28,7 @@ EXPORTS = [
     "umlmd_get_profile", "umlmd_profile_class_name", "umlmd_kinetic_energy_static", "umlmd_static_last_error",
     "umlmd_probe_fma_peak", "umlmd_get_neighbor_rows", "umlmd_workspace_bytes", "umlmd_get_nvt_state", "umlmd_set_nvt_state",
     "umlmd_compute_batch", "umlmd_set_owned_atoms", "umlmd_vv_update", "umlmd_eval_edge_tables",
+    "umlmd_eval_edge_splines",
 ]
 
 
@@ -78,6 +79,7 @@ def load_library(path=_LIB_PATH):
     lib.umlmd_get_intermediates.argtypes = [vp, vp, vp]
     lib.umlmd_eval_radial_table.argtypes = [vp, i64, ctypes.POINTER(dbl), ctypes.POINTER(dbl), ctypes.POINTER(dbl)]
     lib.umlmd_eval_edge_tables.argtypes = [vp, i32, i32, i32, i64, ctypes.POINTER(dbl), ctypes.POINTER(dbl), ctypes.POINTER(dbl)]
+    lib.umlmd_eval_edge_splines.argtypes = [vp, i32, i64, ctypes.POINTER(dbl), ctypes.POINTER(dbl), ctypes.POINTER(dbl)]
     lib.umlmd_eval_pair_cache.argtypes = [vp, i32, i32, ctypes.POINTER(dbl)]
     lib.umlmd_set_profiling.argtypes = [vp, ctypes.c_int]
     lib.umlmd_get_profile.argtypes = [vp, i32, ctypes.POINTER(dbl), ctypes.POINTER(i64), ctypes.POINTER(i32)]
@@ -416,6 +418,19 @@ class Model:
         if rc != OK:
             self._raise(rc)
         return g, dg
+
+    def eval_edge_splines(self, species, rho):
+        """(psi, d psi / d rho) [n, C0] of the pair (species, species) from the splines of a system of one species."""
+        rho = np.ascontiguousarray(rho, dtype=np.float64)
+        C0 = self.query()["C0"]
+        psi = np.empty((len(rho), C0), dtype=np.float64)
+        dpsi = np.empty((len(rho), C0), dtype=np.float64)
+        P = ctypes.POINTER(ctypes.c_double)
+        rc = self._lib.umlmd_eval_edge_splines(self._h, int(species), len(rho), rho.ctypes.data_as(P), psi.ctypes.data_as(P),
+                                               dpsi.ctypes.data_as(P))
+        if rc != OK:
+            self._raise(rc)
+        return psi, dpsi
 
     def eval_edge_tables(self, type_i, type_j, rho, per_pair):
         """(psi, d(chi psi)/d rho) [n, C0] of an ordered species pair as the edge kernels read them."""

@@ -34,11 +34,10 @@ struct umlmd {
     float* moments = nullptr; int64_t moments_cap = 0;
     int* moment_order = nullptr; int64_t order_cap = 0;
     int* moment_scratch = nullptr;
-    // scalar channels by splines (moments.cu): coefficients of the pair of spline_species, intervals
-    float* spline = nullptr; int64_t spline_cap = 0;
-    int spline_n = 0, spline_species = -1;
-    bool spline_failed = false;                      // the radial map takes more intervals than are worth it
-    std::vector<double> spline_coef;                 // of the radial map and modes
+    // scalar channels by splines (moments.cu): coefficients of the radial map and modes, and of the pair of spline_species
+    double* spline_coef = nullptr;
+    float* spline = nullptr;
+    int spline_species = -1;
     bool have_groups = false;                        // moment_order belongs to the current list
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
@@ -214,9 +213,9 @@ int decode_device_errors(umlmd_t* h, int word) {
 
 double mean_row(const umlmd_t* h) { return h->nb.N > 0 ? (double)h->nb.E / (double)h->nb.N : 0.0; }      // listed neighbours
 // rows of spline coefficients, padded to whole 16-byte pieces
-int spline_pitch(const umlmd_t* h) { return (h->spline_n + 7 + 3) / 4 * 4; }
+int spline_pitch(const umlmd_t* h) { return (h->hm.spline_n + 7 + 3) / 4 * 4; }
 bool use_splines(const umlmd_t* h, int64_t rows) {
-    return h->pair_tables && h->present.size() == 1 && h->spline_n > 0 && h->spline_species == h->present[0] && splines_pick(h->d, rows, mean_row(h));
+    return h->pair_tables && h->present.size() == 1 && h->spline_species == h->present[0] && splines_pick(h->d, rows, mean_row(h));
 }
 
 // what the records of the edge kernels hold in place of the species, null for the species itself
@@ -251,8 +250,8 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
         ea.a0 = a0; ea.a1 = a0 + n; ea.state = h->state; ea.g = h->g;
         const bool by_splines = use_splines(h, n), by_moments = by_splines || (h->have_groups && !h->pair_tables && moments_pick(d, n));
         ea.moments = by_moments ? h->moments : nullptr; ea.n_moments = by_splines ? spline_pitch(h) : moment_pitch(d);
-        ea.spline_n = by_splines ? h->spline_n : 0; ea.spline_inv_h = (float)(h->spline_n / h->hm.rc);
-        ea.spline_inv_h_lo = (float)(h->spline_n / h->hm.rc - (double)ea.spline_inv_h);
+        ea.spline_n = by_splines ? h->hm.spline_n : 0; ea.spline_inv_h = (float)(h->hm.spline_n / h->hm.rc);
+        ea.spline_inv_h_lo = (float)(h->hm.spline_n / h->hm.rc - (double)ea.spline_inv_h);
         const int* order = by_splines || !by_moments ? nullptr : h->moment_order + (a0 / B) * moment_order_ints(d, B);
         const MomentArgs mo = {d, h->md.pairmod, nb.type_s, order, a0, n, h->state, h->moments, ea.n_moments, by_splines ? h->spline : nullptr};
         ea.virial_part = h->virial_part + (size_t)vpart_used * 9;
@@ -484,35 +483,15 @@ int build_list(umlmd_t* h, int64_t N, const double* d_pos, const int32_t* d_type
     return UMLMD_OK;
 }
 
-// Spline coefficients of the one pair of a system of one species; the fit (2 to 5 ms) is made once per model, by the first system
-// that uses it.
+// Spline coefficients of the one pair of a system of one species.
 int setup_splines(umlmd_t* h) {
-    const Dims& d = h->d;
-    const int t = h->present[0], NC = d.C0 + d.R;
-    if (h->spline_failed || h->spline_species == t) return UMLMD_OK;
-    if (h->spline_n == 0) h->spline_n = fit_radial_splines(h->hm, &h->spline_coef);
-    h->spline_failed = h->spline_n == 0;
-    if (h->spline_failed) return UMLMD_OK;
-    std::vector<float> S((size_t)spline_pitch(h) * d.C0, 0.0f);
-    const float* pm = &h->hm.pairmod[(size_t)(t * d.T + t) * (2 + d.R) * d.C0];
-    std::vector<double> left(d.C0, 0.0);
-    for (int k = 0; k < h->spline_n + 7; ++k) {
-        const double* g = &h->spline_coef[(size_t)k * NC];
-        for (int c = 0; c < d.C0; ++c) {
-            double v = (double)pm[c] * g[c] + (double)pm[d.C0 + c];          // (the basis functions add up to one)
-            for (int q = 0; q < d.R; ++q) v += (double)pm[(size_t)(2 + q) * d.C0 + c] * g[d.C0 + q];
-            // the kernels' basis functions are 7! times them; what a coefficient loses by rounding the next one makes up for
-            // (a row's mean error over its channels 3e-9 of the sums, so 3e-10; by the tables it is 7e-10 to 1e-9)
-            const double w = v / 5040 - left[c];
-            const float r = (float)w;
-            S[(size_t)k * d.C0 + c] = r;
-            left[c] = (double)r - w;
-        }
-    }
-    h->spline_species = -1;
-    if ((int64_t)S.size() > h->spline_cap) API_CUDA(h, dev_ensure(&h->spline, &h->spline_cap, (int64_t)S.size()));
-    API_CUDA(h, cudaMemcpyAsync(h->spline, S.data(), sizeof(float) * S.size(), cudaMemcpyHostToDevice, h->st));
-    API_CUDA(h, cudaStreamSynchronize(h->st));       // (S is pageable host memory)
+    const int t = h->present[0];
+    if (h->spline_species == t) return UMLMD_OK;
+    if (!h->spline_coef) API_CUDA(h, upload(h, h->hm.spline, &h->spline_coef));
+    int64_t c = 0;
+    if (!h->spline) API_CUDA(h, dev_ensure(&h->spline, &c, (int64_t)spline_pitch(h) * h->d.C0));
+    Scope sc(h, kNeighbor, 1);
+    API_CUDA(h, launch_spline_pair(h->d, h->spline_coef, h->md.pairmod, t, h->hm.spline_n, spline_pitch(h), h->spline, h->st));
     h->spline_species = t;
     return UMLMD_OK;
 }
@@ -522,9 +501,9 @@ int setup_moments(umlmd_t* h) {
     const Dims& d = h->d;
     const int64_t NR = h->nb.n_owned, B = h->nb.N < h->node_tile ? h->nb.N : h->node_tile, rows = NR < B ? NR : B;
     h->have_groups = false;
-    if (h->pair_tables && h->present.size() == 1 && splines_pick(d, rows, mean_row(h))) {
+    if (h->pair_tables && h->present.size() == 1 && h->hm.spline_n > 0 && splines_pick(d, rows, mean_row(h))) {
         const int rc = setup_splines(h);
-        if (rc != UMLMD_OK || !use_splines(h, rows)) return rc;
+        if (rc != UMLMD_OK) return rc;
         if (rows * spline_pitch(h) > h->moments_cap) API_CUDA(h, dev_ensure(&h->moments, &h->moments_cap, rows * spline_pitch(h)));
         return UMLMD_OK;
     }
@@ -1131,6 +1110,33 @@ int umlmd_eval_radial_table(const umlmd_t* h, int64_t n, const double* rho, doub
             const double c0 = p[c], c1 = p[d.CP + c], c2 = h2, c3 = h3;
             out_g[i * NC + c] = ((c3 * t + c2) * t + c1) * t + c0;
             if (out_dg) out_dg[i * NC + c] = (3 * c3 * t + 2 * c2) * t + c1;
+        }
+    }
+    return UMLMD_OK;
+}
+
+int umlmd_eval_edge_splines(umlmd_t* h, int32_t type, int64_t n, const double* rho, double* out_psi, double* out_dpsi) {
+    if (!h || n < 0 || (n > 0 && (!rho || !out_psi)) || type < 0 || type >= h->d.T) return UMLMD_E_INVALID_ARG;
+    const Dims& d = h->d;
+    const HostModel& m = h->hm;
+    if (m.spline_n == 0) return fail(h, UMLMD_E_UNSUPPORTED_PROFILE, "this model has no splines");
+    const int rows = m.spline_n + 7;
+    std::vector<float> S((size_t)rows * d.C0);
+    const float* pm = &m.pairmod[(size_t)(type * d.T + type) * (2 + d.R) * d.C0];
+    for (int c = 0; c < d.C0; ++c) {
+        double left = 0;
+        for (int k = 0; k < rows; ++k) S[(size_t)k * d.C0 + c] = spline_coefficient(d, &m.spline[(size_t)k * (d.C0 + d.R)], pm + c, c, &left);
+    }
+    for (int64_t i = 0; i < n; ++i) {
+        const double x = std::min(std::max(rho[i], 0.0), m.rc) * (m.spline_n / m.rc);
+        const int k = std::min((int)x, m.spline_n - 1);
+        double w[8], dw[8];
+        spline_weights(x - k, w, dw);
+        for (int c = 0; c < d.C0; ++c) {
+            double v = 0, dv = 0;
+            for (int a = 0; a < 8; ++a) { const double q = 5040.0 * S[(size_t)(k + a) * d.C0 + c]; v += w[a] * q; dv += dw[a] * q; }
+            out_psi[i * d.C0 + c] = v;
+            if (out_dpsi) out_dpsi[i * d.C0 + c] = dv * (m.spline_n / m.rc);
         }
     }
     return UMLMD_OK;

@@ -185,6 +185,18 @@ __host__ __device__ inline void pair_cubic(const Dims& d, const float* row, cons
         if (q < 0) v[0] += (double)pm[d.C0];
     }
 }
+// One spline coefficient of the amplitude psi_c of a pair from those of the radial map and modes: `coef` their row, `pm` channel c of
+// the pair's row.  The basis functions add up to one; the kernels' are 7! times them.  *left: what the coefficient before has lost by
+// rounding, which this one makes up for (a row's mean error over its channels 3e-9 of the sums, so 3e-10; by the tables it is 7e-10
+// to 1e-9).
+__host__ __device__ inline float spline_coefficient(const Dims& d, const double* coef, const float* pm, int c, double* left) {
+    double v = (double)pm[0] * coef[c] + (double)pm[d.C0];
+    for (int q = 0; q < d.R; ++q) v += (double)pm[(size_t)(2 + q) * d.C0] * coef[d.C0 + q];
+    v = v / 5040 - *left;
+    const float r = (float)v;
+    *left = (double)r - v;
+    return r;
+}
 // Models of at least 32 channels use the product table and none with derivatives.  At C0 = 8 and 16 a quarter or more of the
 // channels are leading ones, which need both: there the table with derivatives is less to read.
 __host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }

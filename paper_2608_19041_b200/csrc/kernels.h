@@ -158,6 +158,8 @@ bool moments_pick(const Dims& d, int64_t rows);
 int64_t moment_order_ints(const Dims& d, int64_t rows);
 // type_s: of the tile; scratch: 2 T ints
 cudaError_t launch_moment_groups(const Dims& d, const int* type_s, int n, int* scratch, int* order, cudaStream_t st);
+// spline coefficients [pitch][C0] of psi of the pair (t, t) from those of the radial map, coef [n + 7][C0 + R]
+cudaError_t launch_spline_pair(const Dims& d, const double* coef, const float* pairmod, int t, int n, int pitch, float* spline, cudaStream_t st);
 cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st);    // state += (beta | U)^T moments; = spline^T moments
 cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st);   // moments = (beta | U) state; spline state
 // Whether the scalar channels of a tile of so many rows, all of one species and with so many listed neighbours on average, go by

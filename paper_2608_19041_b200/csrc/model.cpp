@@ -189,20 +189,18 @@ void spline_weights(double t, double w[8], double dw[8]) {
     for (int j = 0; j <= 7; ++j) w[j] = u[j];
 }
 
-int fit_radial_splines(const HostModel& m, std::vector<double>* coef) {
-    const Dims& d = m.d;
+int fit_radial_splines(const Dims& d, double rc, double dx, const std::vector<double>& knots, std::vector<double>* coef) {
     const int NC = d.C0 + d.R, n = d.n_rows + 1;
-    if (m.knots.empty()) return 0;
     for (const int K : {160, 192, 256}) {
         const int stride = n / (8 * K);                   // about eight knots per interval; the ones half way between are checked
         if (stride < 1) return 0;
         const int M = K + 7;
-        const double inv_h = K / m.rc;
+        const double inv_h = K / rc;
         std::vector<double> A((size_t)M * 8, 0.0);         // lower band of the normal equations, A[i][i - j]
         coef->assign((size_t)M * NC, 0.0);
         double* const B = coef->data();
         auto basis = [&](int s, double* w, double* dw) {
-            const double x = s * m.dx * inv_h;
+            const double x = s * dx * inv_h;
             const int k = std::min((int)x, K - 1);
             spline_weights(x - k, w, dw);
             return k;
@@ -210,7 +208,7 @@ int fit_radial_splines(const HostModel& m, std::vector<double>* coef) {
         double w[8], dw[8];
         for (int s = 0; s < n; s += stride) {
             const int k = basis(s, w, dw);
-            const double* y = &m.knots[(size_t)s * 2 * NC];
+            const double* y = &knots[(size_t)s * 2 * NC];
             for (int a = 0; a < 8; ++a) {
                 for (int b = 0; b <= a; ++b) A[(size_t)(k + a) * 8 + (a - b)] += w[a] * w[b];
                 double* r = B + (size_t)(k + a) * NC;
@@ -248,7 +246,7 @@ int fit_radial_splines(const HostModel& m, std::vector<double>* coef) {
         double ev = 0, ed = 0, mv = 0, md = 0;
         for (int s = stride / 2; s < n; s += stride) {
             const int k = basis(s, w, dw);
-            const double *y = &m.knots[(size_t)s * 2 * NC], *y1 = y + NC;
+            const double *y = &knots[(size_t)s * 2 * NC], *y1 = y + NC;
             std::fill(v.begin(), v.end(), 0.0);
             std::fill(dv.begin(), dv.end(), 0.0);
             for (int a = 0; a < 8; ++a) {
@@ -486,7 +484,8 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         if (wide) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
     }
 
-    if (C0 >= 64) m->knots = std::move(Y);
+    // (2 to 6 ms here; with the first system that uses them the fit was an eighth of a handle's first list build)
+    if (C0 >= 64) m->spline_n = fit_radial_splines(d, m->rc, m->dx, Y, &m->spline);
 
     // ---- ordered type-pair cache -----------------------------------------------------
     {

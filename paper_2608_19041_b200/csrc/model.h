@@ -18,7 +18,8 @@ struct HostModel {
     std::vector<float> table;      // [n_rows][3][CP]: c0, c1, packed (c2, c3) (see tab_pack)
     std::vector<float> vtable;     // [n_vrows][2][CP]: a0, packed (a1, a2) (see value_piece)
     std::vector<float> dtable;     // [n_vrows][2][CP]: derivative of envelope times g (see product_piece)
-    std::vector<double> knots;     // [n_rows + 1][2][C0 + R] value and slope of [g, q] at the knots of the table (C0 >= 64: for splines)
+    std::vector<double> spline;    // [spline_n + 7][C0 + R] [g, q] as B-splines (C0 >= 64, see fit_radial_splines)
+    int spline_n = 0;              // their intervals on [0, rc]; 0: there are none
     std::vector<float> pairmod;    // [T*T][2+R][C0]
     std::vector<float> X0, W1p, W2p, A1, A2, mu, inv_sigma;
     std::vector<std::vector<float>> theta, thetaT, bias;   // per hidden layer
@@ -36,10 +37,11 @@ struct HostModel {
 // Fills `d` widths for (C0, L, R); false when the triple is unsupported.
 bool derive_dims(int C0, int L, int R, Dims* d);
 
-// The radial map and modes as uniform B-splines of degree seven, fitted to the table's knots: intervals of rc / n, coefficient
-// rows 0 .. n + 6 of C0 + R columns in `coef`, value on interval k = sum_a B_a(t) coef[k + a].  n is the smallest of a few numbers
-// for which values and slopes meet the knots that the fit has left out to the bounds of the tables; 0 when none does.
-int fit_radial_splines(const HostModel& m, std::vector<double>* coef);
+// The radial map and modes as uniform B-splines of degree seven (de Boor, A Practical Guide to Splines, 1978), fitted by least
+// squares to knots of the table: `knots` [n_rows + 1][2][C0 + R] holds values and slopes.  Intervals of rc / n, coefficient rows
+// 0 .. n + 6 of C0 + R columns in `coef`, value on interval k = sum_a B_a(t) coef[k + a].  n is the smallest of a few numbers for
+// which values and slopes meet the knots that the fit has left out to the bounds of the tables; 0 when none does.
+int fit_radial_splines(const Dims& d, double rc, double dx, const std::vector<double>& knots, std::vector<double>* coef);
 // the eight basis functions at t in [0, 1], and their derivatives with respect to t
 void spline_weights(double t, double w[8], double dw[8]);
 

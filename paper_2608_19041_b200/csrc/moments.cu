@@ -186,6 +186,17 @@ __global__ void __launch_bounds__(NT, 256 / NT) k_moments(int a0, int K, int N, 
     }
 }
 
+// A thread per channel, the rows one after the other (spline_coefficient); once per species that a handle meets.
+__global__ void k_spline_pair(Dims d, const double* __restrict__ coef, const float* __restrict__ pairmod, int t, int n, int pitch,
+                              float* __restrict__ spline) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= d.C0) return;
+    const float* const pm = pairmod + (size_t)(t * d.T + t) * (2 + d.R) * d.C0 + c;
+    double left = 0;
+    for (int k = 0; k < pitch; ++k)
+        spline[(size_t)k * d.C0 + c] = k < n + 7 ? spline_coefficient(d, coef + (size_t)k * (d.C0 + d.R), pm, c, &left) : 0.0f;
+}
+
 }  // namespace
 
 int moment_pitch(const Dims& d) { return (d.T * (1 + d.R) + 3) / 4 * 4; }
@@ -216,6 +227,10 @@ static cudaError_t launch(const MomentArgs& a, cudaStream_t st) {
     const int width = FORWARD ? d.C0 : ((N + 63) / 64 * 64 < (N + 127) / 128 * 128 ? 64 : 128);
     if (width == 128) return go(k_moments<FORWARD, 128>, 128);
     return width == 64 ? go(k_moments<FORWARD, 64>, 64) : go(k_moments<true, 32>, 32);
+}
+cudaError_t launch_spline_pair(const Dims& d, const double* coef, const float* pairmod, int t, int n, int pitch, float* spline, cudaStream_t st) {
+    k_spline_pair<<<(d.C0 + 31) / 32, 32, 0, st>>>(d, coef, pairmod, t, n, pitch, spline);
+    return cudaGetLastError();
 }
 cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st) { return launch<true>(a, st); }
 cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st) { return launch<false>(a, st); }

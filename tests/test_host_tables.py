@@ -90,3 +90,15 @@ def test_a_steep_map_with_shared_modes_is_cut_for_the_products_too():
     m = binding.Model(_steep_blob(p, 3, 3e-6, 250))
     psi, product = _distance(m, p, 1, 0.002)
     assert psi <= PSI and product <= PRODUCT
+
+
+def test_splines_are_fitted_when_the_model_is_made():
+    p = SMALL_PROFILES["p128_2_0"]
+    m = binding.Model(make_blob(p, seed=5))              # (no list build waits for it)
+    assert m.eval_edge_splines(0, [1.0, 2.0])[0].shape == (2, p["C0"])
+
+
+def test_narrow_models_have_no_splines():
+    m = binding.Model(make_blob(SMALL_PROFILES["p32_2_4"], seed=5))
+    with pytest.raises(binding.UmlmdError, match="splines"):
+        m.eval_edge_splines(0, [1.0])
