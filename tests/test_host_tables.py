@@ -3,7 +3,9 @@ cubic pieces they are derived from, on the host."""
 
 import numpy as np
 import pytest
+import torch
 
+from oracle import dpa4c as orc
 from paper_2608_19041_b200 import binding
 from workloads import SMALL_PROFILES, make_blob
 from workloads.weights import HEADER_BYTES, blob_array_shapes
@@ -92,10 +94,27 @@ def test_a_steep_map_with_shared_modes_is_cut_for_the_products_too():
     assert psi <= PSI and product <= PRODUCT
 
 
-def test_splines_are_fitted_when_the_model_is_made():
-    p = SMALL_PROFILES["p128_2_0"]
-    m = binding.Model(make_blob(p, seed=5))              # (no list build waits for it)
-    assert m.eval_edge_splines(0, [1.0, 2.0])[0].shape == (2, p["C0"])
+@pytest.mark.parametrize("basis", ["bessel", "gaussian"])
+@pytest.mark.parametrize("name", ["p64_3_8", "p128_2_0", "p128_3_4"])
+def test_splines_follow_the_radial_map_between_the_knots(name, basis):
+    p = SMALL_PROFILES[name]
+    blob = make_blob(p, seed=5, basis=basis)
+    m, o = binding.Model(blob), orc.Oracle(blob)        # (fitted when the model is made: no list build waits for it)
+    rho = torch.from_numpy(np.random.default_rng(1).uniform(1e-3, p["rc"], 3000)).requires_grad_(True)
+    g, q = orc.radial_map(rho, o.prm, o.p.get("basis", "bessel"), o.p["rc"])
+    gs = [torch.autograd.grad(c.sum(), rho, retain_graph=True)[0].numpy() for c in torch.cat([g, q], dim=1).T]
+    y, dy = torch.cat([g, q], dim=1).detach().numpy(), np.stack(gs, axis=1)
+    C0 = p["C0"]
+    for t in range(p["T"]):
+        gamma, beta, U = (x[t, t].numpy() for x in o.pair)
+        psi, dpsi = gamma * y[:, :C0] + beta, gamma * dy[:, :C0]
+        if p["R"]:
+            psi, dpsi = psi + y[:, C0:] @ U.T, dpsi + dy[:, C0:] @ U.T
+        got = m.eval_edge_splines(t, rho.detach().numpy())
+        # the fit's bounds, 2^-24 and 2^-23 of the largest, one more for gamma, beta and U in single precision, and the coefficients'
+        # own 2^-25: of the value half a unit, of the slope 32 of their differences per Angstrom against a slope of about twice the value
+        assert np.abs(got[0] - psi).max() <= 3 * U24 * np.abs(psi).max()
+        assert np.abs(got[1] - dpsi).max() <= 3 * 2 * U24 * np.abs(dpsi).max() + 32 * U24 * np.abs(psi).max()
 
 
 def test_narrow_models_have_no_splines():
