@@ -38,6 +38,7 @@ struct umlmd {
     double* spline_coef = nullptr;
     float* spline = nullptr;
     int spline_species = -1;
+    bool splines = false;                            // the list that the caller has built goes that way, and so do the driver's rebuilds of it
     bool have_groups = false;                        // moment_order belongs to the current list
     float* g = nullptr; int64_t g_cap = 0;
     double* e_atom = nullptr; int* type_o = nullptr; int64_t n_cap = 0;
@@ -214,9 +215,7 @@ int decode_device_errors(umlmd_t* h, int word) {
 double mean_row(const umlmd_t* h) { return h->nb.N > 0 ? (double)h->nb.E / (double)h->nb.N : 0.0; }      // listed neighbours
 // rows of spline coefficients, padded to whole 16-byte pieces
 int spline_pitch(const umlmd_t* h) { return (h->hm.spline_n + 7 + 3) / 4 * 4; }
-bool use_splines(const umlmd_t* h, int64_t rows) {
-    return h->pair_tables && h->present.size() == 1 && h->spline_species == h->present[0] && splines_pick(h->d, rows, mean_row(h));
-}
+bool use_splines(const umlmd_t* h, int64_t rows) { return h->splines && splines_pick(h->d, rows); }
 
 // what the records of the edge kernels hold in place of the species, null for the species itself
 const int* record_slots(const umlmd_t* h) { return h->pair_tables ? h->d_species + h->d.T : nullptr; }
@@ -497,15 +496,16 @@ int setup_splines(umlmd_t* h) {
 }
 
 // Makes room for the moments of a tile's rows, and groups the rows of the current list by species, where its kernels take that way.
-int setup_moments(umlmd_t* h) {
+// rebuild: of the same atoms by an MD driver, which keeps what the caller's list has decided, so that the way, and with it the
+// energy in its last digits, does not change in the middle of a run.
+int setup_moments(umlmd_t* h, bool rebuild = false) {
     const Dims& d = h->d;
     const int64_t NR = h->nb.n_owned, B = h->nb.N < h->node_tile ? h->nb.N : h->node_tile, rows = NR < B ? NR : B;
     h->have_groups = false;
-    if (h->pair_tables && h->present.size() == 1 && h->hm.spline_n > 0 && splines_pick(d, rows, mean_row(h))) {
-        const int rc = setup_splines(h);
-        if (rc != UMLMD_OK) return rc;
+    if (!rebuild) h->splines = h->pair_tables && h->present.size() == 1 && h->hm.spline_n > 0 && splines_pick(d, rows) && splines_pay(d, mean_row(h));
+    if (h->splines) {
         if (rows * spline_pitch(h) > h->moments_cap) API_CUDA(h, dev_ensure(&h->moments, &h->moments_cap, rows * spline_pitch(h)));
-        return UMLMD_OK;
+        return setup_splines(h);
     }
     if (h->pair_tables || !moments_pick(d, rows)) return UMLMD_OK;
     const int64_t per_tile = moment_order_ints(d, B);
@@ -736,7 +736,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
     if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
     constexpr int64_t kMostSplineRows = 264;            // rows of coefficients of the largest fit
-    if (splines_pick(d, Bt, 1.0e9)) t += buf(Bt * kMostSplineRows, 4) + buf(kMostSplineRows * d.C0, 4);
+    if (splines_pick(d, Bt)) t += buf(Bt * kMostSplineRows, 4) + buf(kMostSplineRows * d.C0, 4);
     if (moments_pick(d, Bt)) t += buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
@@ -915,7 +915,7 @@ static int maybe_rebuild(umlmd_t* h, int rebuild_every) {
             API_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
             return decode_device_errors(h, word);
         }
-        if ((rc = setup_moments(h)) != UMLMD_OK) return rc;
+        if ((rc = setup_moments(h, true)) != UMLMD_OK) return rc;
     }
     return UMLMD_OK;
 }

@@ -162,15 +162,14 @@ cudaError_t launch_moment_groups(const Dims& d, const int* type_s, int n, int* s
 cudaError_t launch_spline_pair(const Dims& d, const double* coef, const float* pairmod, int t, int n, int pitch, float* spline, cudaStream_t st);
 cudaError_t launch_moments_forward(const MomentArgs& a, cudaStream_t st);    // state += (beta | U)^T moments; = spline^T moments
 cudaError_t launch_moments_backward(const MomentArgs& a, cudaStream_t st);   // moments = (beta | U) state; spline state
-// Whether the scalar channels of a tile of so many rows, all of one species and with so many listed neighbours on average, go by
-// splines (true for n implies true for more).  The products with the coefficients cost the same for every row, the edges save
-// with their number and the width.  Edge kernels and products, tables against splines, us: C0 = 64 with 274 listed neighbours
-// 30,000 rows 609 and 484, 9000 197 and 178, with 122 neighbours 10,000 rows 118 and 132; C0 = 128 with 274 30,000 rows 966 and
-// 675, 9000 304 and 223.
+// Whether the scalar channels of a tile of so many rows, all of one species, go by splines (true for n implies true for more), given
+// that the list's rows, with so many listed neighbours on average, are long enough for it to pay.  The products with the coefficients
+// cost the same for every row, the edges save with their number and the width.  Edge kernels and products, tables against splines,
+// us: C0 = 64 with 274 listed neighbours 30,000 rows 609 and 484, 9000 197 and 178, with 122 neighbours 10,000 rows 118 and 132;
+// C0 = 128 with 274 30,000 rows 966 and 675, 9000 304 and 223.
 constexpr int kSplineRows = 8192;
-inline bool splines_pick(const Dims& d, int64_t rows, double row_length) {
-    return d.C0 >= 64 && rows >= kSplineRows && row_length * d.C0 >= 64 * 180;
-}
+inline bool splines_pick(const Dims& d, int64_t rows) { return d.C0 >= 64 && rows >= kSplineRows; }
+inline bool splines_pay(const Dims& d, double row_length) { return row_length * d.C0 >= 64 * 180; }
 
 // ---- invariants.cu -------------------------------------------------------------------
 struct InvArgs {

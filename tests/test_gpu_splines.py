@@ -117,3 +117,28 @@ def test_row_sums_follow_the_definition(name, spacing, jitter):
     # what is common to all sums: gamma, beta and U of the pair are rounded by up to 2^-25, at random over the dozen channels and
     # more that carry them
     assert abs((got * ref).sum() / (ref * ref).sum() - 1) <= 8e-9
+
+
+# some 97 and 79 listed neighbours on average: either side of where splines are taken at this width
+@pytest.mark.parametrize("spacing,growth", [(2.29, 0.02), (2.33, -0.02)])
+def test_a_run_keeps_the_way_its_list_was_built_for(spacing, growth):
+    from paper_2608_19041_b200 import binding
+    m = binding.Model(make_blob(SMALL_PROFILES["p128_2_0"], seed=84))
+    pos, cell = _lattice(21 ** 3, spacing, 0.02, 86)
+    steps, dt = 10, 0.001
+    pos = pos - pos.mean(axis=0)
+    vel = pos * (growth / (steps * dt))                # the cluster grows or shrinks by 2 % in all
+    p, v = (torch.as_tensor(x, dtype=torch.float64).cuda().contiguous() for x in (pos, vel))
+    types = torch.zeros(len(pos), dtype=torch.int32, device="cuda")
+    m.build_neighbors(p, types, 4 * cell, (0, 0, 0), 0.9)
+    listed = [m.query()["n_edges"] / len(pos)]
+    m.get_profile()
+    m.compute(p)
+    per_call = m.get_profile()["edge_forward"][1]      # one launch more by splines
+    assert per_call == (2 if growth > 0 else 1)
+    m.set_md_state(p, v, np.full(SMALL_PROFILES["p128_2_0"]["T"], 1.0e9))
+    m.step(steps, dt, rebuild_every=2)
+    listed.append(m.query()["n_edges"] / len(pos))
+    assert min(listed) < 90 < max(listed)              # (the mean row has crossed the switch)
+    assert m.get_profile()["edge_forward"][1] == (steps + 1) * per_call
+    m.close()
