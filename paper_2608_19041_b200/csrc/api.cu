@@ -735,8 +735,7 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
     if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
-    constexpr int64_t kMostSplineRows = 264;            // rows of coefficients of the largest fit
-    if (splines_pick(d, Bt)) t += buf(Bt * kMostSplineRows, 4) + buf(kMostSplineRows * d.C0, 4);
+    if (splines_pick(d, Bt)) t += buf(Bt * kMaxSplinePitch, 4) + buf(kMaxSplinePitch * d.C0, 4);
     if (moments_pick(d, Bt)) t += buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);

@@ -1170,6 +1170,8 @@ k_edge_backward(const EdgeArgs a) {
 
 
 // per-pair amplitude tables already hold the modes, so the kernels without them are used
+// (The limit of dynamic shared memory belongs to the kernel, whichever thread and model launches it: always the largest that
+// any model takes, so that one thread's cannot come between another's limit and launch.)
 template <int C0, int L, bool SPLIT>
 cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
     auto kern = a.uni ? k_edge_forward<C0, L, kNoModes, true, SPLIT>
@@ -1178,7 +1180,7 @@ cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
         if (a.spline_n) {
             kern = k_edge_forward<C0, L, kSplines, true, false>;
             const size_t bytes = sizeof(float) * kWarpsPerBlock * 4 * a.n_moments;
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * kWarpsPerBlock * 4 * kMaxSplinePitch));
             if (e != cudaSuccess) return e;
             kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
             return cudaGetLastError();
@@ -1188,7 +1190,7 @@ cudaError_t launch_fwd_r(const EdgeArgs& a, int blocks, cudaStream_t st) {
         if (a.moments) {
             kern = k_edge_forward<C0, L, kMoments, false, false>;
             const size_t bytes = sizeof(float) * kWarpsPerBlock * a.n_moments;
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * kWarpsPerBlock * kMaxMoments));
             if (e != cudaSuccess) return e;
             kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
             return cudaGetLastError();
@@ -1203,9 +1205,12 @@ cudaError_t launch_bwd_r(const EdgeArgs& a, int blocks, bool split, cudaStream_t
     constexpr bool FEW = C0 <= 64 && MODES < kMoments;           // (the others have no such variant)
     size_t bytes = BwdSmem<C0, L, MODES, UNI>::bytes;
     auto kern = few ? k_edge_backward<C0, L, MODES, UNI, FEW, false> : k_edge_backward<C0, L, MODES, UNI, false, false>;
-    if constexpr (MODES >= kMoments) bytes += sizeof(float) * kWarpsPerBlock * a.n_moments;
-    else if (split) kern = k_edge_backward<C0, L, MODES, UNI, false, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    size_t most = bytes;
+    if constexpr (MODES >= kMoments) {
+        most += sizeof(float) * kWarpsPerBlock * (MODES == kSplines ? kMaxSplinePitch : kMaxMoments);
+        bytes += sizeof(float) * kWarpsPerBlock * a.n_moments;
+    } else if (split) kern = k_edge_backward<C0, L, MODES, UNI, false, true>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
     kern<<<blocks, kWarpsPerBlock * 32, bytes, st>>>(a);
     return cudaGetLastError();

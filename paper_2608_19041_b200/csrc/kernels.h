@@ -152,6 +152,7 @@ struct MomentArgs {
 // edge reading its pair's rows: 2100 rows 150 against 211 us, 4000 235 against 406, 40,009 1510 against 2638); below, whole
 // blocks of 64 rows of a species are mostly padding.  640 moments (2.5 KB a row) keep the blocks that fit on an SM.
 constexpr int kMaxMoments = 640, kMomentRows = 2048;
+constexpr int kMaxSplinePitch = 264;            // rows of spline coefficients of the largest fit, 256 intervals
 int moment_pitch(const Dims& d);
 // whether a tile of so many rows, without per-pair tables, takes the way over moments (true for n implies true for more)
 bool moments_pick(const Dims& d, int64_t rows);

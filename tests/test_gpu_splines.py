@@ -1,5 +1,9 @@
 """Scalar channels by splines (one species, many rows) against the same kernels reading the pair's tables (few rows)."""
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -142,3 +146,43 @@ def test_a_run_keeps_the_way_its_list_was_built_for(spacing, growth):
     assert min(listed) < 90 < max(listed)              # (the mean row has crossed the switch)
     assert m.get_profile()["edge_forward"][1] == (steps + 1) * per_call
     m.close()
+
+
+THREADS = """
+import threading
+import numpy as np, torch
+from paper_2608_19041_b200 import binding
+from workloads import SMALL_PROFILES, make_blob
+import tests.test_gpu_splines as base
+# (models whose kernels are the same and whose rows of spline weights are not)
+blobs = [make_blob(SMALL_PROFILES["p64_3_8"], seed=83, bias_scale=0.2, e_ref_scale=0.5, basis=b) for b in ("bessel", "gaussian")]
+pos, cell = base._lattice(8200, 1.6, 0.05, 87)
+jobs = []
+for t in range(4):
+    st = torch.cuda.Stream()
+    jobs.append((st, binding.Model(blobs[t % 2], stream=st, launch_graphs=-1), torch.tensor(pos, device="cuda"), torch.zeros(len(pos), dtype=torch.int32, device="cuda")))
+torch.cuda.synchronize()
+gate, out = threading.Barrier(len(jobs)), [None] * len(jobs)
+
+def work(i):
+    st, m, p, types = jobs[i]
+    with torch.cuda.stream(st):
+        m.build_neighbors(p, types, cell, (1, 1, 1), 0.0)
+        ref = m.compute(p)["forces"].clone()
+        gate.wait()
+        same = True
+        for _ in range(300):
+            same = same and torch.equal(m.compute(p)["forces"], ref)
+        out[i] = same
+
+threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+print(out)
+"""
+
+
+def test_models_with_other_rows_of_weights_in_several_threads():
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", THREADS], cwd=root, capture_output=True, text=True, timeout=180)
+    assert r.returncode == 0 and r.stdout.strip() == str([True] * 4), r.stdout + r.stderr
