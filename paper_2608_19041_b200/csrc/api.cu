@@ -231,19 +231,20 @@ int enqueue_compute(umlmd_t* h, const double* d_pos, bool want_grad, double* d_f
     const int NR = (int)nb.n_owned;      // rows that are evaluated: the owned atoms, first in the internal order
     // (a batched list was built from these very positions: nothing to gather)
     if (!nb.batch && !tail) { Scope sc(h, kGather, 1); API_CUDA(h, launch_gather_positions(nb, d_pos, record_slots(h), h->d_err, h->st)); }
+    if (nb.per_edge) { Scope sc(h, kGather, 1); API_CUDA(h, launch_edge_records(nb, h->hm.rc, h->st)); }
     const int B = N < h->node_tile ? N : h->node_tile;
     int vpart_used = 0;
     for (int a0 = 0; a0 < NR; a0 += B) {
         const int n = NR - a0 < B ? NR - a0 : B;
         EdgeArgs ea;
-        ea.d = d; ea.table = h->md.table; ea.pairmod = h->md.pairmod; ea.fix = nb.fix; ea.quantum = (float)nb.quantum;
+        ea.d = d; ea.table = h->md.table; ea.pairmod = h->md.pairmod; ea.fix = nb.per_edge ? nb.edge_fix : nb.fix; ea.quantum = (float)(nb.per_edge ? position_quantum(kEdgeRecordReach * h->hm.rc) : nb.quantum);
         ea.uni = h->pair_tables; ea.table_uni = h->table_uni;
         ea.vtable = h->md.vtable; ea.vtable_uni = h->vtable_uni;
         ea.dtable = h->md.dtable; ea.dtable_uni = h->dtable_uni;
         ea.uni_scale = h->uni_scale;
         ea.species_slot = nb.batch ? h->d_species + d.T : nullptr; ea.n_present = (int)h->present.size();
         ea.frames = nb.batch ? nb.frames : nullptr; ea.frame_of = nb.frame_of;
-        ea.row_ptr = nb.row_ptr; ea.nbr = nb.nbr;
+        ea.row_ptr = nb.row_ptr; ea.nbr = nb.per_edge ? nb.edge_nbr : nb.nbr;
         for (int k = 0; k < 9; ++k) ea.Hq[k] = to_quanta(nb.H[k], 1.0 / nb.quantum);
         ea.tri = nb.tri;
         ea.a0 = a0; ea.a1 = a0 + n; ea.state = h->state; ea.g = h->g;

@@ -124,6 +124,32 @@ __global__ void k_atom_virial(int N, const eidx_t* __restrict__ row_ptr, const i
     }
 }
 
+// Records of the edges of a row, a warp per row: edge vectors in double, rounded to quanta.  An edge beyond the cutoff, whose vector
+// may be longer than the quanta reach, is put just outside it.  frames: of a batched list, whose cells differ (null: the cell H).
+struct CellRows { double h[9]; };
+__global__ void k_edge_records(int n_rows, int N, const eidx_t* __restrict__ row_ptr, const int2* __restrict__ nbr, const double* __restrict__ xs,
+                               const int4* __restrict__ fix, CellRows cell, const FrameCell* __restrict__ frames, const int* __restrict__ frame_of,
+                               double inv_q, double far, int4* __restrict__ out, int2* __restrict__ out_nbr) {
+    chain_begin();
+    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (row >= n_rows) return;
+    double H[9];
+    for (int k = 0; k < 9; ++k) H[k] = frames ? frames[frame_of[row]].H[k] : cell.h[k];
+    if (lane == 0) out[row] = make_int4(0, 0, 0, fix[row].w);
+    const eidx_t e1 = row_ptr[row + 1];
+    for (eidx_t e = row_ptr[row] + lane; e < e1; e += 32) {
+        const int2 js = nbr[e];
+        const int s = js.y;
+        const int nx = (int)(signed char)(s & 0xff), ny = (int)(signed char)((s >> 8) & 0xff), nz = (int)(signed char)((s >> 16) & 0xff);
+        double r[3];
+        for (int k = 0; k < 3; ++k)
+            r[k] = (xs[3 * (size_t)js.x + k] + ((nx * H[k] + ny * H[3 + k]) + nz * H[6 + k])) - xs[3 * (size_t)row + k];
+        const bool near = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] < far * far;
+        out[N + e] = make_int4(to_quanta(near ? r[0] : far, inv_q), near ? to_quanta(r[1], inv_q) : 0, near ? to_quanta(r[2], inv_q) : 0, fix[js.x].w);
+        out_nbr[e] = make_int2((int)(N + e), 0);
+    }
+}
+
 __global__ void k_unsort_rows(int N, const int* __restrict__ perm, const float* __restrict__ in, int stride,
                               int width, float* __restrict__ out) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -558,6 +584,16 @@ cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, 
     const int N = (int)nb.N;
     if (N == 0) return cudaSuccess;
     return launch_chained(k_gather_positions, (N + 255) / 256, 256, 0, st, N, nb.perm, d_pos, gather_args(nb, species_slot), d_err);
+}
+
+cudaError_t launch_edge_records(const NeighborDev& nb, double rc, cudaStream_t st) {
+    const int N = (int)nb.n_owned;
+    if (N == 0) return cudaSuccess;
+    CellRows cell;
+    for (int k = 0; k < 9; ++k) cell.h[k] = nb.H[k];
+    return launch_chained(k_edge_records, (N + 7) / 8, 256, 0, st, N, (int)nb.N, nb.row_ptr, nb.nbr, nb.xs, nb.fix, cell,
+                          nb.batch ? nb.frames : nullptr, nb.frame_of, 1.0 / position_quantum(kEdgeRecordReach * rc), kEdgeRecordReach * rc,
+                          nb.edge_fix, nb.edge_nbr);
 }
 
 cudaError_t launch_unsort_state(const NeighborDev& nb, const float* in, int stride, int width, float* out,

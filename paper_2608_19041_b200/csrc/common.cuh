@@ -206,10 +206,18 @@ __host__ __device__ constexpr bool wide_channels(int C0) { return C0 >= 32; }
 // beyond the list radius rc + skin a component up to that wraps to itself; the longest edge of a list that is not stale is rc + 2 skin,
 // and what lies beyond R comes out as at least 2 R - (rc + 2 skin) > rc, outside the cutoff as it is.  Half a quantum is 1.9e-9 at
 // a list radius of 6 or 7 Angstrom, where the rounding of a component between 1 and 8 to single precision is 6e-8 to 2.4e-7.
+// The quantum grows with the list radius, and an image offset's rounding with the number of the image.  From a list radius of 16
+// Angstrom on, and in cells so small that offsets could be 3e-8 off, every edge gets a record of its own instead, formed in double
+// and in quanta for the cutoff (edge_records_needed, k_edge_records).
 inline double position_quantum(double r_list) {
     int e;
     std::frexp(r_list, &e);
     return std::ldexp(1.0, e - 31);
+}
+constexpr double kEdgeRecordReach = 1.001;      // times the cutoff: where the records of edges beyond it are
+inline bool edge_records_needed(double r_list, int images) {
+    const double q = position_quantum(r_list);
+    return q > 0x1p-27 || 0.5 * q * images > 0x1p-25;
 }
 __host__ __device__ inline int to_quanta(double x, double inv_q) {
 #ifdef __CUDA_ARCH__
@@ -262,6 +270,11 @@ struct NeighborDev {
     // modulo 2^32: differences of two coordinates wrap to the true one, whatever the size of the box (position_quantum)
     int4* fix = nullptr;
     double quantum = 1;
+    // where `fix` is too coarse (edge_records_needed): a record for every row, at the origin, and for every edge, at its edge vector,
+    // and a list that names them
+    bool per_edge = false;
+    int4* edge_fix = nullptr; int64_t edge_fix_cap = 0;
+    int2* edge_nbr = nullptr; int64_t edge_nbr_cap = 0;
     eidx_t* row_ptr = nullptr;   // [N+1]
     int2* nbr = nullptr;         // [E] x: sorted index of the neighbour, y: its image n, packed int8 x3
     eidx_t* rev = nullptr;       // [E] index of the reverse edge, -1 if absent

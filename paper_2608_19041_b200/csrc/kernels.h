@@ -233,6 +233,8 @@ struct GatherArgs {
 GatherArgs gather_args(const NeighborDev& nb, const int* species_slot);
 // xs[i] = pos[perm[i]] - img[i]*L and the records of the edge kernels; flags stale / non-finite atoms in *d_err
 cudaError_t launch_gather_positions(const NeighborDev& nb, const double* d_pos, const int* species_slot, int* d_err, cudaStream_t st);
+// the records of every edge, from the current positions (nb.xs) and the records' species (nb.fix): nb.edge_fix and nb.edge_nbr
+cudaError_t launch_edge_records(const NeighborDev& nb, double rc, cudaStream_t st);
 // What an MD step does with the forces of an atom once they are there (pos null: nothing): kicks and, if drift, the drift and
 // the records of the next evaluation
 struct StepTail {

@@ -775,7 +775,7 @@ struct WidenDeg {
 }  // namespace
 
 void neighbor_free(NeighborDev* nb) {
-    void* ptrs[] = {nb->frames, nb->rec, nb->fix, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->nbr, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
+    void* ptrs[] = {nb->frames, nb->rec, nb->fix, nb->edge_fix, nb->edge_nbr, nb->wpos, nb->img, nb->perm, nb->type_s, nb->xs0, nb->xs, nb->row_ptr, nb->nbr, nb->rev, nb->key, nb->key2, nb->idx, nb->idx2, nb->cell_start, nb->deg,
                     nb->cub_tmp, nb->bounds};
     for (void* p : ptrs)
         dev_free(p);
@@ -814,6 +814,11 @@ static int read_totals(NeighborDev* nb, int N, int n_owned, const int* d_type, i
         c = 0; NB_CHECK(dev_ensure(&nb->nbr, &c, total, 1.1));
         c = 0; NB_CHECK(dev_ensure(&nb->rev, &c, total, 1.1));
         nb->E_cap = c;
+    }
+    if (nb->per_edge && N + total > 0x7fffffffLL) nb->per_edge = false;         // (more than the list can name: the coarse ones)
+    if (nb->per_edge) {
+        if (N + total > nb->edge_fix_cap) NB_CHECK(dev_ensure(&nb->edge_fix, &nb->edge_fix_cap, N + total, 1.1));
+        if (total > nb->edge_nbr_cap) NB_CHECK(dev_ensure(&nb->edge_nbr, &nb->edge_nbr_cap, total, 1.1));
     }
     return UMLMD_OK;
 }
@@ -921,7 +926,10 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     g.ncell = (int)ncell; g.n_owned = n_owned; g.halves = n_owned < N ? 2 : 1;
     const int64_t nkeys = (int64_t)g.halves * ncell;
 
+    int images = 0;                             // the farthest along a cell vector
+    for (int k = 0; k < 3; ++k) if (pbc[k]) images = std::max(images, (int)std::floor(r_list / height[k]) + 1);
     nb->N = N; nb->skin = skin; nb->r_list = r_list; nb->quantum = position_quantum(r_list); nb->n_owned = n_owned; nb->E_owned = 0;
+    nb->per_edge = edge_records_needed(r_list, images);
     for (int k = 0; k < 3; ++k) { nb->L[k] = L[k]; nb->pbc[k] = pbc[k] ? 1 : 0; }
     for (int k = 0; k < 9; ++k) nb->H[k] = cell[k];
     nb->tri = g.tri;
@@ -1040,6 +1048,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
                          cudaStream_t st, std::string* err) {
     const int64_t N = offsets[n_frames];
     std::vector<FrameCell> fr((size_t)n_frames);
+    int images = 0;                             // the farthest along a cell vector
     for (int f = 0; f < n_frames; ++f) {
         FrameCell& c = fr[f];
         const double* H = cells + 9 * (size_t)f;
@@ -1063,6 +1072,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
             c.pbc[k] = pbc[k] ? 1 : 0;
             c.reach[k] = rc / height + 1e-6;
             c.m[k] = pbc[k] ? (int)std::ceil(rc / height) : 0;
+            images = std::max(images, c.m[k]);
             if (c.m[k] > 127) { *err = "frame cell much smaller than the cutoff (more than 127 images)"; return UMLMD_E_UNSUPPORTED_CELL; }
         }
         // coordinates of a folded atom are bounded by the cell along periodic directions only (else see k_batch_fold)
@@ -1072,6 +1082,7 @@ int neighbor_build_batch(NeighborDev* nb, int n_frames, const int64_t* offsets, 
         c.a0 = (int)offsets[f]; c.a1 = (int)offsets[f + 1];
     }
     nb->N = N; nb->skin = 0; nb->r_list = rc; nb->quantum = position_quantum(rc); nb->tri = 1; nb->batch = true; nb->n_frames = n_frames;
+    nb->per_edge = edge_records_needed(rc, images);
     for (int k = 0; k < 3; ++k) { nb->pbc[k] = pbc[k] ? 1 : 0; nb->L[k] = 0; }
     for (int k = 0; k < 9; ++k) nb->H[k] = 0;
     nb->E = 0;

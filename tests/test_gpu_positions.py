@@ -100,3 +100,38 @@ def test_a_stale_list_is_reported_by_the_step_that_evaluates_it():
         else:
             m.step(steps, 0.001, rebuild_every=rebuild)
         m.close()
+
+
+# list radii past those whose quanta are fine enough, and a cell of many images: edge vectors as they are at a usual list radius
+@pytest.mark.parametrize("case", ["open", "periodic", "images", "batch"])
+@pytest.mark.parametrize("skin", [0.0, 9.9, 10.1, 100.0, 2500.0])
+def test_edge_vectors_do_not_lose_precision_with_the_list_radius(case, skin):
+    p = SMALL_PROFILES["p16_2_0"]
+    s = make_system(dict(kind="random_box", atoms=24, edges=(7.0, 8.0, 9.0), min_dist=1.6, seed=92, n_types=p["T"], masses=[1.0] * p["T"]))
+    pos, types, cell, pbc = s["pos"], s["types"], np.diag(np.diag(np.asarray(s["cell"], dtype=np.float64))), (0, 0, 0)
+    if case == "periodic":
+        cell, pbc = cell * 3.0, (1, 1, 1)
+        if skin > 100.0:
+            pytest.skip("a list of 1e8 edges")
+    elif case == "images":               # 18 images along a direction at a list radius of 6
+        if skin:
+            pytest.skip("the images are what this case is about")
+        pos, types, cell, pbc = np.array([[0.1, 1.0, 1.0], [0.2, 5.0, 4.0]]), types[:2], np.diag([0.345, 9.0, 8.0]), (1, 1, 1)
+    elif case == "batch":
+        if skin:
+            pytest.skip("a batch has no skin")
+        pos, types, cell, pbc = np.array([[0.1, 1.0, 1.0], [0.2, 5.0, 4.0]]), types[:2], np.diag([0.345, 9.0, 8.0]), (1, 1, 1)
+    blob, m = _model()
+    if case == "batch":
+        off = np.array([0, len(pos), 2 * len(pos)])
+        out = m.compute_batch(off, _cuda(np.concatenate([pos, pos])), _cuda(np.concatenate([types, types]), torch.int32), np.stack([cell, cell]), pbc,
+                              atom_energy=True)
+    else:
+        m.build_neighbors(_cuda(pos), _cuda(types, torch.int32), cell, pbc, skin)
+        out = m.compute(_cuda(pos), atom_energy=True)
+    ref = orc.Oracle(blob).compute(pos, types, cell, pbc)
+    E, F = np.asarray(ref["E_i"]), np.asarray(ref["F"])
+    # as at a usual list radius; with quanta that grow with it atomic energies were 1.7e-6 off at the largest one
+    assert np.abs(out["atom_energy"].cpu().numpy()[:len(pos)] - E).max() <= 8e-7 * np.abs(E).max()
+    assert np.abs(out["forces"].cpu().numpy()[:len(pos)] - F).max() <= 8e-7 * np.abs(F).max()
+    m.close()
