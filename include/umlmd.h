@@ -138,8 +138,12 @@ const char* umlmd_last_error(const umlmd_t* h);
  * tile of evaluation workspace, per-edge gradients and per-atom results.  Known before anything
  * is allocated (library plumbing, no counterpart in the paper; the paper's memory-scaling note is
  * the model: a fixed tile workspace plus terms linear in atoms and in edges).  An upper estimate
- * within a few per cent; per-pair amplitude tables, when the species present are few enough for
- * them, add at most umlmd_options.pair_table_mb on top (320 MiB where that is 0).
+ * within a few per cent for the system of the handle's list; for another one, whose species are not
+ * known, it counts the larger of what rows of one species (from C0 = 64 and 8192 rows on) and rows of
+ * many with shared modes (from C0 = 32 and 2048 rows on) may need, up to 2560 bytes a row.  Per-pair
+ * amplitude tables, when the species present are few enough for them, add at most
+ * umlmd_options.pair_table_mb on top (320 MiB where that is 0), and a list radius of 16 Angstrom or
+ * more 24 bytes an edge.
  */
 int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t* bytes);
 

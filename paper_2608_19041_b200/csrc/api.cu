@@ -736,8 +736,13 @@ int umlmd_workspace_bytes(const umlmd_t* h, int64_t N, int64_t n_edges, int64_t*
     const int64_t wmax = d.DP > d.F ? d.DP : d.F;
     t += buf(Bt * d.SP, 4) + buf(Bt * d.DP, 4);
     if (const int64_t need = fused_floats(h, N, Bt)) t += buf(need, 4);
-    if (splines_pick(d, Bt)) t += buf(Bt * kMaxSplinePitch, 4) + buf(kMaxSplinePitch * d.C0, 4);
-    if (moments_pick(d, Bt)) t += buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4);
+    // rows of spline weights or of moments, never both; which, the species decide: those of this handle's list where that is the
+    // system asked for, else the larger
+    const bool known = h->have_list && h->nb.N == N && h->nb.E == n_edges;
+    const bool splines = known ? h->splines : m.spline_n > 0 && N > 0 && splines_pick(d, Bt) && splines_pay(d, (double)n_edges / (double)N);
+    const bool moments = known ? h->have_groups : moments_pick(d, Bt);
+    t += std::max(splines ? buf(Bt * spline_pitch(h), 4) + buf((int64_t)spline_pitch(h) * d.C0, 4) + buf((int64_t)m.spline.size(), 8) : 0,
+                  moments ? buf(Bt * moment_pitch(d), 4) + buf((N + Bt - 1) / Bt * moment_order_ints(d, Bt), 4) + buf(2 * d.T, 4) : 0);
     if (!mlp_needs_chain(h, Bt)) t += 2 * buf(Bt * d.DP, 2);
     else t += buf(Bt * d.F * d.n_hidden, 4) + buf(Bt * d.F * 2, 4) + 2 * buf(2 * Bt * wmax, 2);
     t += grown(3 * n_edges, 4);

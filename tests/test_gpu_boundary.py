@@ -82,6 +82,36 @@ def test_workspace_estimate_covers_what_a_run_allocates():
     m.close()
 
 
+# rows of spline weights (one species), of moments (shared modes, no per-pair tables), and neither
+@pytest.mark.parametrize("name,species,mb", [("p64_3_8", 1, 0), ("p128_2_0", 1, 0), ("p128_3_4", 3, -1), ("p64_3_8", 2, 0)])
+def test_workspace_estimate_of_many_rows(name, species, mb):
+    m = _binding().Model(make_blob(SMALL_PROFILES[name], seed=46), pair_table_mb=mb)
+    before = m.query()["device_bytes"]
+    n, spacing = 21, 1.8
+    rng = np.random.default_rng(47)
+    pos = spacing * np.stack(np.meshgrid(*[np.arange(n)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.05 * rng.standard_normal((n ** 3, 3))
+    pos, types = _dev(pos, torch.float64), _dev(rng.integers(0, species, n ** 3), torch.int32)
+    edges = 0
+    for skin in (0.5, 0.5):                      # before anything is allocated (from a like system's count) and with the list there
+        first = m.workspace_bytes(n ** 3, edges) if edges else None
+        m.build_neighbors(pos, types, np.diag([spacing * n] * 3), (1, 1, 1), skin)
+        edges = m.query()["n_edges"]
+    m.compute(pos)
+    m.set_md_state(pos, torch.zeros_like(pos), np.ones(SMALL_PROFILES[name]["T"]))
+    held, est = m.query()["device_bytes"] - before, m.workspace_bytes(n ** 3, edges)
+    tables = 0
+    if mb == 0:                                  # (the per-pair tables come on top of the estimate: 4/3 of rows x 3 x C0 words a pair, kept)
+        p = SMALL_PROFILES[name]
+        tables = species ** 2 * m.query()["table_rows"] * 4 * p["C0"] * 4
+    print(f"{name} {species}: held {held / 2**20:.1f} MiB, tables {tables / 2**20:.1f}, estimate {est / 2**20:.1f} MiB")
+    assert held - tables <= est + 4096 and est <= 1.1 * (held - tables) + (4 << 20)
+    assert first == est
+    # a handle without a list does not know the species
+    fresh = _binding().Model(make_blob(SMALL_PROFILES[name], seed=46), pair_table_mb=mb).workspace_bytes(n ** 3, edges)
+    assert est <= fresh <= est + n ** 3 * 2560 + (2 << 20)
+    m.close()
+
+
 @pytest.mark.parametrize("variant", ["one_tile", "persistent", "cta_pairs"])
 def test_expired_pipeline_wait_is_reported_and_the_handle_recovers(variant):
     # The diagnostic option leaves one operand stage of the first MLP layer unloaded; nothing sets
