@@ -373,8 +373,8 @@ int umlmd_eval_radial_table(const umlmd_t* h, int64_t n, const double* rho, doub
  * What the edge kernels read for centre species type_i and neighbour species type_j at n distances
  * (host arrays): out_psi [n, C0] the amplitudes psi_c of the forward pass (quadratic pieces), and
  * out_dchipsi [n, C0] (may be NULL) the derivative of envelope times amplitude that the backward
- * pass works with -- from C0 = 32 on, without shared modes or from per-pair tables, quadratic pieces
- * of that product, otherwise formed from the cubic pieces.  per_pair = 0: shared table and pair
+ * pass works with -- from C0 = 32 on quadratic pieces of that product, below formed from the cubic
+ * pieces (scalar channels of one species by splines: umlmd_eval_edge_splines).  per_pair = 0: shared table and pair
  * cache; 1: the tables that umlmd_build_neighbors makes for a system of just these two species.
  * Pieces are at most 0.0025 Angstrom long, and cut finer until those of g, q and of the envelope's
  * products follow the cubic pieces within 2^-24 (psi) and 2^-23 (product) of their largest magnitude,
@@ -402,6 +402,11 @@ int umlmd_eval_edge_splines(umlmd_t* h, int32_t type, int64_t n, const double* r
  * receives the number of classes) and resets them.  Class names: gather_positions,
  * edge_forward, invariants_forward, mlp_forward, mlp_backward, invariants_backward,
  * edge_backward, force_assembly, energy_virial_reduce, integrate, neighbor_build.
+ * A launch counts under one class, though it may do more: the matrix products of rows by moments
+ * or splines are edge_forward and edge_backward; up to 32768 atoms the launch that assembles the
+ * forces also reduces energy and virial; in umlmd_step it also applies kicks and drift and gathers
+ * the positions of the next step, so that integrate is left with the opening kick and the kinetic
+ * energy of a call, and gather_positions with the evaluations behind a list build.
  */
 int umlmd_set_profiling(umlmd_t* h, int enabled);
 int umlmd_get_profile(umlmd_t* h, int32_t max_classes, double* ms, int64_t* launches, int32_t* n_classes);
