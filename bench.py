@@ -152,6 +152,27 @@ def work_model(p, n_atoms, e_rc, e_list, one_species=False):
     }
 
 
+def work_done(work, prof, steps, n_atoms, nve):
+    """(work, times): the work of one pass of each class and how many passes `steps` steps made, by what the launches of
+    the class in `prof` do.  In a constant-energy run (nve) the launch that assembles the forces also applies kicks and
+    drift and leaves the records of the next evaluation: what is left of "integrate" are the opening kick and drift and
+    the two launches of the kinetic energy of each call, and of "gather_positions" the evaluations behind a list build."""
+    work = dict(work)
+    times = {c: steps for c in work}
+    launches = {c: v[1] for c, v in prof.items()}
+    times["neighbor_build"] = max(1, launches.get("neighbor_build", 0) // 5)
+    times["gather_positions"] = launches.get("gather_positions", 0)
+    if not launches.get("mlp_backward"):       # one kernel for both passes, under the forward pass's name
+        work["mlp_forward"] = dict(work["mlp_forward"], flops=work["mlp_forward"]["flops"] + work["mlp_backward"]["flops"],
+                                   bytes=work["mlp_forward"]["bytes"] + work["mlp_backward"]["bytes"])
+    if nve:
+        # per atom: positions and velocities in and out, species; then image, build position, position and record
+        work["force_assembly"] = dict(work["force_assembly"], bytes=work["force_assembly"]["bytes"] + n_atoms * (4 * 24 + 4 + 12 + 24 + 24 + 16))
+        work["integrate"] = dict(work["integrate"], bytes=n_atoms * ((5 * 24 + 4) + (24 + 4)))
+        times["integrate"] = launches.get("integrate", 0) / 3
+    return work, times
+
+
 def roofline_entry(name, ms, launches, evals, work, peaks):
     """achieved = algorithmic work of `evals` evaluations / time; against the binding peak."""
     w = work[name]
@@ -343,16 +364,13 @@ class Workload:
         prof = m.get_profile()
         m.set_profiling(False)
         work = work_model(self.p, self.N, self.e_rc, self.e_list, one_species=len(np.unique(self.s["types"])) == 1)
-        if not prof["mlp_backward"][1]:        # one kernel for both passes, under the forward pass's name
-            work["mlp_forward"] = dict(work["mlp_forward"], flops=work["mlp_forward"]["flops"] + work["mlp_backward"]["flops"],
-                                       bytes=work["mlp_forward"]["bytes"] + work["mlp_backward"]["bytes"])
+        work, times = work_done(work, prof, steps, self.N, not self.static and not self.nvt)
         total_ms = sum(v[0] for v in prof.values()) or 1.0
         kernels = []
         for cname, (kms, kl) in prof.items():
             if kl == 0 or cname not in work:
                 continue
-            evals = steps if cname != "neighbor_build" else max(1, kl // 5)
-            ent = roofline_entry(cname, kms, kl, evals, work, peaks)
+            ent = roofline_entry(cname, kms, kl, times[cname], work, peaks)
             if ent:
                 ent["share"] = round(kms / total_ms, 4)
                 kernels.append(ent)

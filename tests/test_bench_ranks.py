@@ -62,3 +62,25 @@ def test_reference_arm_runs_on_rank_zero_only(monkeypatch, capsys):
     args = argparse.Namespace(workload="cfg1_al108", steps=1, warmup=1, cpu_seconds=1.0, gpus=2, impl="reference", modes=-1)
     bench.run_reference(args)                           # returns at once, prints nothing
     assert capsys.readouterr().out == ""
+
+
+def test_work_of_a_class_is_what_its_launches_do():
+    import bench
+    from workloads import workload_profile
+    n, steps = 1000, 20
+    work = bench.work_model(workload_profile("cfg5_amorphous1m"), n, 50 * n, 100 * n)
+    # twenty steps of one constant-energy call with two list builds, and the launches of each class
+    prof = {c: (1.0, steps) for c in work}
+    prof.update(gather_positions=(1.0, 3), integrate=(1.0, 3), neighbor_build=(1.0, 10), mlp_backward=(0.0, 0))
+    done, times = bench.work_done(work, prof, steps, n, nve=True)
+    assert times["gather_positions"] == 3 and times["integrate"] == 1 and times["neighbor_build"] == 2
+    assert times["force_assembly"] == times["edge_forward"] == steps
+    # what those two classes no longer do is what the force launch does more
+    per_step = work["gather_positions"]["bytes"] + work["integrate"]["bytes"]
+    moved = done["force_assembly"]["bytes"] - work["force_assembly"]["bytes"]
+    assert 0.4 * per_step <= moved <= per_step
+    assert done["mlp_forward"]["flops"] == work["mlp_forward"]["flops"] + work["mlp_backward"]["flops"]
+    # a thermostatted run launches both every step
+    prof.update(gather_positions=(1.0, steps), integrate=(1.0, 2 * steps))
+    done, times = bench.work_done(work, prof, steps, n, nve=False)
+    assert times["gather_positions"] == times["integrate"] == steps and done["force_assembly"] == work["force_assembly"]
