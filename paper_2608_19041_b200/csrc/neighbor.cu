@@ -206,36 +206,28 @@ __global__ void k_gather_sorted(int N, int nkeys, const int* __restrict__ skey, 
 }
 
 // Up to kBinTogether atoms: bins, their order and the sorted arrays by one block in one launch (fold, sort and gather as three
-// took 3.5 + 6.1 + 4.9 us at 597 atoms, and the gaps between them).
-constexpr int kBinTogether = 4096, kBinThreads = 1024;
-template <int ITEMS>
-__global__ void __launch_bounds__(kBinThreads) k_bin_together(int N, int nkeys, int end_bit, const double* __restrict__ pos, Grid g,
-                                                              const int* __restrict__ type, double* wpos, int* img_o,
-                                                              int* __restrict__ skey, int* __restrict__ perm, double* __restrict__ xs0,
-                                                              double* __restrict__ xs, float4* __restrict__ rec, int* __restrict__ img,
-                                                              int* __restrict__ type_s, int* __restrict__ cell_start, int* __restrict__ err) {
-    using Sort = cub::BlockRadixSort<int, kBinThreads, ITEMS, int>;
-    __shared__ union { typename Sort::TempStorage sort; int keys[kBinThreads * ITEMS]; } sh;
-    int key[ITEMS], idx[ITEMS];
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const int i = threadIdx.x * ITEMS + k;
-        idx[k] = i;
-        key[k] = i < N ? fold_atom(i, pos, g, wpos, img_o, err) : nkeys;       // (what is no atom comes last: nkeys < 2^end_bit)
-    }
+// took 3.5 + 6.1 + 4.9 us at 597 atoms, and the gaps between them).  Builds in us, together and apart: 108 atoms 94 and 100, 512 72 and
+// 77, 1024 81 and 82; from two atoms per thread on the block's sort and its passes take longer than several blocks': 1500 atoms 100
+// and 91, 4096 128 and 88, and 119 and 63 where most bins are empty.
+constexpr int kBinTogether = 1024;
+__global__ void __launch_bounds__(kBinTogether) k_bin_together(int N, int nkeys, int end_bit, const double* __restrict__ pos, Grid g,
+                                                               const int* __restrict__ type, double* wpos, int* img_o,
+                                                               int* __restrict__ skey, int* __restrict__ perm, double* __restrict__ xs0,
+                                                               double* __restrict__ xs, float4* __restrict__ rec, int* __restrict__ img,
+                                                               int* __restrict__ type_s, int* __restrict__ cell_start, int* __restrict__ err) {
+    using Sort = cub::BlockRadixSort<int, kBinTogether, 1, int>;
+    __shared__ union { typename Sort::TempStorage sort; int keys[kBinTogether]; } sh;
+    const int i = threadIdx.x;
+    int key[1] = {i < N ? fold_atom(i, pos, g, wpos, img_o, err) : nkeys}, idx[1] = {i};     // (what is no atom comes last: nkeys < 2^end_bit)
     Sort(sh.sort).Sort(key, idx, 0, end_bit);
     __syncthreads();                                  // (the folded positions of the block are there, the sort is done with its area)
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const int i = threadIdx.x * ITEMS + k;
-        sh.keys[i] = key[k];
-        if (i < N) {
-            skey[i] = key[k];
-            sorted_atom(i, idx[k], wpos, img_o, type, perm, xs0, xs, rec, img, type_s);
-        }
+    sh.keys[i] = key[0];
+    if (i < N) {
+        skey[i] = key[0];
+        sorted_atom(i, idx[0], wpos, img_o, type, perm, xs0, xs, rec, img, type_s);
     }
     __syncthreads();
-    for (int c = threadIdx.x; c <= nkeys; c += kBinThreads) {                   // first atom of every bin, and N
+    for (int c = i; c <= nkeys; c += kBinTogether) {                            // first atom of every bin, and N
         int lo = 0, hi = N;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
@@ -248,7 +240,8 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_together(int N, int nkeys, 
 
 // Up to kOffsetsTogether rows: row offsets from row lengths and all that the host waits for, by one block, which writes the results
 // to the host's pinned memory itself (otherwise the scan's two launches, the flags' kernel, three clears and four copies).
-// h_flags null: the totals alone.
+// h_flags null: the totals alone.  Builds of 8192 and 8193 atoms, us: 142 and 165, 144 and 168 in an open box, 99 and 128 where most
+// bins are empty.
 constexpr int kOffsetsTogether = 8192;
 __global__ void __launch_bounds__(1024) k_row_offsets(int N, int n_owned, const int* __restrict__ deg, eidx_t* __restrict__ row_ptr,
                                                       const int* __restrict__ type, int T, eidx_t* __restrict__ h_totals,
@@ -980,8 +973,7 @@ int neighbor_build(NeighborDev* nb, int64_t N64, int64_t n_owned64, const double
     if (N <= kBinTogether) {
         int bits = 1;
         while ((1LL << bits) <= nkeys) ++bits;           // (one key more: no atom)
-        auto bin = N <= kBinThreads ? k_bin_together<1> : k_bin_together<kBinTogether / kBinThreads>;
-        bin<<<1, kBinThreads, 0, st>>>(N, (int)nkeys, bits, d_pos, g, d_type, nb->wpos, img_o, nb->key2, nb->perm, nb->xs0, nb->xs, nb->rec,
+        k_bin_together<<<1, kBinTogether, 0, st>>>(N, (int)nkeys, bits, d_pos, g, d_type, nb->wpos, img_o, nb->key2, nb->perm, nb->xs0, nb->xs, nb->rec,
                                        nb->img, nb->type_s, nb->cell_start, d_err);
     } else {
         k_fold_bin<<<(N + TB - 1) / TB, TB, 0, st>>>(N, d_pos, g, nb->wpos, img_o, nb->key, nb->idx, d_err);

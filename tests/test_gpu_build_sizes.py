@@ -15,7 +15,7 @@ def _model():
     return binding.Model(make_blob(SMALL_PROFILES["p16_2_0"], 3))      # three species
 
 
-# one atom; the sort's one and four atoms per thread; bins in one block and in several; offsets in one block and in several
+# one atom; bins in one block and in several; offsets in one block and in several
 @pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 4095, 4096, 4097, 8192, 8193])
 @pytest.mark.parametrize("case", ["periodic", "clustered", "ghosts"])
 def test_rows_where_the_launches_change(n, case):
