@@ -392,8 +392,9 @@ template <int C0, int L, int G = 1, bool ROWS = false> struct Widths {
 // The channel-parallel phase of the backward pass waits on load latency, and what hides it best
 // depends on the width and on what is read (all measured on the edge backward kernel).  C0 = 128 with shared
 // table and pair cache, or degree three: four channel groups per lane, that many times the loads in flight,
-// at 16 resident warps per SM (128 registers): 64,007 atoms of one species 1.10 ms against 1.19 with two
-// groups at 24 warps (85 registers, spilled words), the 64-species mixture 12.6 against 14.6.  With shared modes,
+// at 16 resident warps per SM (128 registers): 64,007 atoms of one species by tables (as its rows go below 8192, or
+// where they are short) 1.10 ms against 1.19 with two groups at 24 warps (85 registers, spilled words), a million atoms of
+// the 64-species mixture, when its kernel took 12.6 ms, 14.6.  By splines the same.  With shared modes,
 // and with per-pair tables at degree two (fewer registers spilled): the latter, 1.62 -> 1.49 ms for 40,009 atoms
 // with four modes, 1.00 -> 0.94 for 128,000 atoms of five species.  C0 = 32 and 64: two groups at 24 warps;
 // C0 <= 16: one group, 24 warps.  FEW: rows for more than 24 but not more than 32 warps per SM (3553 to 4736): 64
@@ -426,10 +427,11 @@ template <int C0, int L, int MODES, bool UNI> struct BwdSmem {          // dynam
 //      degree-0 sums accumulated in registers; the leading C1 amplitudes of each edge are
 //      parked in shared memory.
 //   3. lane = edge again: harmonics of the lane's own edge, parked as weights chi^2 B_lm; then
-//      lane = job: a lane owns four consecutive channels of one harmonic component (or up to four
-//      components of a one-channel degree) for the whole row, and for every edge of its group of
-//      edges adds vector x scalar from the parked row: two shared-memory reads per edge and group of
+//      lane = job: a lane owns four consecutive channels of two harmonic components (of one below C0 = 32,
+//      or up to four components of a one-channel degree) for the whole row, and for every edge of its group
+//      of edges adds vector x scalar from the parked row: two shared-memory reads per edge and group of
 //      lanes, where summing per-edge products by transposition took six.
+// One species by splines: phase 2 adds eight spline weights per edge to the row's, and forms the leading amplitudes alone.
 // What hides the load latency of the channel-parallel phase best depends on the width and on what is read.  Up to C0 = 64, 32
 // warps per SM (64 registers, a few spilled words; 24 were 6 to 10 % slower).  C0 = 128: with per-pair tables an edge per half
 // warp, two channel groups per lane, at 24 warps (40,009 atoms of five species 196 us; two at 16 warps 242, four at 20 warps
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, FwdShape<C0, MODES, UNI>:
 k_edge_forward(const EdgeArgs a) {
     constexpr int G = FwdShape<C0, MODES, UNI>::G;          // channel groups of a lane
     constexpr bool PAIR = C0 < 128 || UNI;                  // see axpy2
-    constexpr bool DIV = C0 >= 128 && UNI && MODES == kNoModes;      // (40,009 atoms of five species 197 us, 211 the other way; C0 = 8 in both 230)
+    constexpr bool DIV = C0 >= 128 && UNI && MODES == kNoModes;      // (40,009 atoms of five species 199 us, 211 the other way)
     using W = Widths<C0, L, G, !UNI>;
     constexpr bool HASR = MODES == kModesPerEdge || MODES == kMoments, SPL = MODES == kSplines;
     static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");

@@ -123,6 +123,70 @@ def test_row_sums_follow_the_definition(name, spacing, jitter):
     assert abs((got * ref).sum() / (ref * ref).sum() - 1) <= 8e-9
 
 
+# whole systems, by splines and (tiles of fewer rows) by tables
+@pytest.mark.parametrize("case", ["periodic", "sheared", "slab", "ghosts"])
+@pytest.mark.parametrize("name,spacing", [("p64_3_8", 1.6), ("p128_2_0", 1.9)])
+def test_systems_by_splines_match_tables(name, spacing, case):
+    from paper_2608_19041_b200 import binding
+    blob = make_blob(SMALL_PROFILES[name], seed=88, bias_scale=0.2, e_ref_scale=0.5)
+    pos, cell = _lattice(21 ** 3, spacing, 0.1, 89)
+    pbc = {"periodic": (1, 1, 1), "sheared": (1, 1, 1), "slab": (1, 1, 0), "ghosts": (0, 0, 0)}[case]
+    if case == "sheared":
+        shear = np.array([[1.0, 0.0, 0.0], [0.12, 1.0, 0.0], [0.07, -0.05, 1.0]])
+        pos, cell = pos @ shear, cell @ shear
+    types = torch.ones(len(pos), dtype=torch.int32, device="cuda")
+    p = torch.as_tensor(pos, dtype=torch.float64).cuda().contiguous()
+    results = []
+    for kw, launches in (dict(), 2), (dict(node_tile=SPLINE_ROWS - 1), 2):            # edge and product; two tiles
+        m = binding.Model(blob, **kw)
+        if case == "ghosts":
+            m.set_owned_atoms(SPLINE_ROWS + 40)
+        m.build_neighbors(p, types, cell, pbc, 0.5)
+        m.get_profile()
+        out = m.compute(p, atom_energy=True)
+        assert m.get_profile()["edge_forward"][1] == launches
+        alone = m.compute(p, forces=False, virial=False, atom_energy=True)
+        assert torch.equal(alone["atom_energy"], out["atom_energy"]) and alone["energy"] == out["energy"]
+        results.append((out["forces"].cpu().numpy(), out["atom_energy"].cpu().numpy(), out["virial"]))
+        m.close()
+    (F, E, V), (Fb, Eb, Vb) = results
+    assert not np.array_equal(F, Fb)                   # (they did go different ways)
+    # either side keeps 2e-5 of the largest force and 1e-5 of the largest energy from the oracle
+    f_scale, e_scale = np.abs(Fb).max(), np.abs(Eb).max()
+    assert np.abs(F - Fb).max() <= 2 * (2e-5 * f_scale + 2e-7)
+    assert np.abs(E - Eb).max() <= 2e-5 * e_scale
+    assert np.abs(V - Vb).max() <= 2e-5 * len(pos) * max(1.0, f_scale)
+    if case == "sheared":
+        Fk, near = orc.Oracle(blob).force_on(pos, np.ones(len(pos), dtype=np.int32), cell, pbc, 4567)
+        assert np.abs(F[4567] - Fk).max() <= 2e-5 * f_scale + 2e-7
+        assert max(abs(E[a] - e) for a, e in near.items()) <= 1e-5 * e_scale
+
+
+def test_a_run_by_splines_follows_the_run_by_tables():
+    from paper_2608_19041_b200 import binding
+    blob = make_blob(SMALL_PROFILES["p128_2_0"], seed=88, bias_scale=0.2)
+    pos, cell = _lattice(21 ** 3, 1.9, 0.05, 90)
+    vel = np.random.default_rng(91).standard_normal(pos.shape)
+    masses = np.full(SMALL_PROFILES["p128_2_0"]["T"], 20.0)
+    runs = []
+    for kw in dict(), dict(node_tile=SPLINE_ROWS - 1):
+        m = binding.Model(blob, **kw)
+        p, v = (torch.as_tensor(x, dtype=torch.float64).cuda().contiguous() for x in (pos, vel))
+        m.build_neighbors(p, torch.zeros(len(pos), dtype=torch.int32, device="cuda"), cell, (1, 1, 1), 0.6)
+        m.set_md_state(p, v, masses)
+        e = m.step(13, 0.0005, rebuild_every=5)
+        f = m.compute(p)["forces"]
+        runs.append((p, v, f, sum(e)))
+        m.close()
+    (p, v, f, e), (pb, vb, fb, eb) = runs
+    # forces agree to 4e-5 of the largest; the positions' difference after n steps is at most n^2 / 2 times what one step makes of that
+    f_scale = fb.abs().max().item()
+    step = 4e-5 * f_scale / 20.0 * 9648.53321 * 0.0005 ** 2
+    assert (p - pb).abs().max().item() <= 13 ** 2 / 2 * step
+    assert (f - fb).abs().max().item() <= 8e-5 * f_scale
+    assert abs(e - eb) <= 2e-5 * len(pos)
+
+
 # some 97 and 79 listed neighbours on average: either side of where splines are taken at this width
 @pytest.mark.parametrize("spacing,growth", [(2.29, 0.02), (2.33, -0.02)])
 def test_a_run_keeps_the_way_its_list_was_built_for(spacing, growth):
