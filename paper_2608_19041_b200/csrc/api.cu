@@ -1134,7 +1134,7 @@ int umlmd_eval_edge_splines(umlmd_t* h, int32_t type, int64_t n, const double* r
     }
     for (int64_t i = 0; i < n; ++i) {
         const double x = std::min(std::max(rho[i], 0.0), m.rc) * (m.spline_n / m.rc);
-        const int k = std::min((int)x, m.spline_n - 1);
+        const int k = std::max(0, std::min((int)x, m.spline_n - 1));          // (a distance that is no number gives no number)
         double w[8], dw[8];
         spline_weights(x - k, w, dw);
         for (int c = 0; c < d.C0; ++c) {

@@ -121,3 +121,11 @@ def test_narrow_models_have_no_splines():
     m = binding.Model(make_blob(SMALL_PROFILES["p32_2_4"], seed=5))
     with pytest.raises(binding.UmlmdError, match="splines"):
         m.eval_edge_splines(0, [1.0])
+
+
+def test_splines_at_the_ends_and_at_no_number():
+    p = SMALL_PROFILES["p128_2_0"]
+    m = binding.Model(make_blob(p, seed=5))
+    psi, dpsi = m.eval_edge_splines(1, [-1.0, 0.0, p["rc"], 2 * p["rc"], np.nan, -np.nan])
+    assert np.array_equal(psi[0], psi[1]) and np.array_equal(psi[2], psi[3]) and np.isfinite(psi[:4]).all() and np.isfinite(dpsi[:4]).all()
+    assert np.isnan(psi[4:]).all() and np.isnan(dpsi[4:]).all()
