@@ -50,7 +50,6 @@ struct Dims {
     float tab_v1, tab_v2;    // steps of its packed linear and quadratic coefficients
     float tab_d1, tab_d2;    // the same for the product table
     float rc, dx, inv_dx;
-    float inv_rc, inv_rc_lo, rc_lo;      // 1 / rc as two numbers; what rc is more than its rounded value, over rc
 };
 
 struct GauntSparse {         // non-zeros of one unit-norm coupling tensor

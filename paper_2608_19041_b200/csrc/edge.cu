@@ -52,9 +52,7 @@ struct Geom {
 // addition in double per component, this phase was half of what the narrow kernels sent through the L1 data pipe (32 scattered
 // 16-byte loads are 32 of its wavefronts) and a quarter of their instructions.
 // VALUE: row and offset in the value table, else in the table with derivatives
-// DIVIDE: 1 / rc by a division ahead of the loop instead of from the arguments: the same number in registers, which some of the
-// kernels are scheduled better with (figures where they say so)
-template <bool VALUE, bool DIVIDE = false>
+template <bool VALUE>
 __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool in_range, const int4& c, int ti,
                                               const int* __restrict__ Hf) {
     Geom g;
@@ -87,11 +85,8 @@ __device__ __forceinline__ Geom edge_geometry(const EdgeArgs& a, eidx_t e, bool 
     g.valid = true;
     g.inv_rho = 1.0f / g.rho;
     g.ux = g.dx * g.inv_rho; g.uy = g.dy * g.inv_rho; g.uz = g.dz * g.inv_rho;
-    // Envelope: t = (rc - rho) / rc with rc and 1 / rc as two numbers, x as what is left to one: the rounding of t hardly moves
-    // chi, whose partial derivatives by t and x cancel where it is flat.  From x = rho * (1 / rc), whose factor is 3e-8 off at
-    // rc = 6, and t = 1 - x, chi came out 1.1e-7 too small on average, which was half and more of the error of the atomic energies.
-    const float inv_rc = DIVIDE ? 1.0f / a.d.rc : a.d.inv_rc, inv_lo = DIVIDE ? (fmaf(-inv_rc, a.d.rc, 1.0f) - a.d.rc_lo) * inv_rc : a.d.inv_rc_lo;
-    const float left = a.d.rc - g.rho, t = fmaf(left, inv_rc, fmaf(left, inv_lo, a.d.rc_lo)), x = 1.0f - t;
+    const float inv_rc = 1.0f / a.d.rc;
+    const float x = g.rho * inv_rc, t = 1.0f - x;
     const float t2 = t * t, x2 = x * x;
     const float poly = 1.0f + x * (4.0f + x * (10.0f + x * (20.0f + 35.0f * x)));
     g.chi = t2 * t2 * poly;
@@ -452,7 +447,6 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, FwdShape<C0, MODES, UNI>:
 k_edge_forward(const EdgeArgs a) {
     constexpr int G = FwdShape<C0, MODES, UNI>::G;          // channel groups of a lane
     constexpr bool PAIR = C0 < 128 || UNI;                  // see axpy2
-    constexpr bool DIV = C0 >= 128 && UNI && MODES == kNoModes;      // (40,009 atoms of five species 199 us, 211 the other way)
     using W = Widths<C0, L, G, !UNI>;
     constexpr bool HASR = MODES == kModesPerEdge || MODES == kMoments, SPL = MODES == kSplines;
     static_assert(C0 + W::NHI <= W::SCRATCH, "a split row's partial sums take the place of the batch");
@@ -661,7 +655,7 @@ k_edge_forward(const EdgeArgs a) {
 
     int qn = 0;
     for (int base = 0; base < len; base += 32) {
-        const Geom g = edge_geometry<true, DIV>(a, e0 + base + lane, base + lane < len, ci, ti, Hf);
+        const Geom g = edge_geometry<true>(a, e0 + base + lane, base + lane < len, ci, ti, Hf);
         const unsigned vmask = __ballot_sync(kFull, g.valid);
         const int p = qn + __popc(vmask & lt_mask);       // queue slot of this lane's edge, if it has one
         if (g.valid) { const double c2 = (double)g.chi * (double)g.chi; s0 += c2; s1 += c2 * c2; }
@@ -765,7 +759,6 @@ k_edge_backward(const EdgeArgs a) {
     using SM = BwdSmem<C0, L, MODES, UNI>;
     constexpr int G = BwdShape<C0, L, MODES, UNI, FEW>::G;
     constexpr bool PR = SM::products, HASR = MODES == kModesPerEdge || MODES == kMoments, SPL = MODES == kSplines;
-    constexpr bool DIV = C0 == 64 && L >= 3 && UNI;         // (32,400 atoms of water 211 us, 214 the other way; degree two 275 and 271)
     using W = Widths<C0, L, G>;
     extern __shared__ __align__(16) unsigned char dsm[];
     double (*vsum)[9] = reinterpret_cast<double (*)[9]>(dsm);
@@ -1115,7 +1108,7 @@ k_edge_backward(const EdgeArgs a) {
         int qn = 0;
         for (int base = 0; base < len; base += 32) {
             const int e = base + lane;
-            const Geom g = edge_geometry<PR, DIV>(a, e0 + e, e < len, ci, ti, Hf);
+            const Geom g = edge_geometry<PR>(a, e0 + e, e < len, ci, ti, Hf);
             const unsigned vmask = __ballot_sync(kFull, g.valid);
             const int p = qn + __popc(vmask & lt_mask);   // queue slot of this lane's edge, if it has one
             if (g.valid && p < 32) {

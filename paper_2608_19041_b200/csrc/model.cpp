@@ -335,7 +335,6 @@ int build_host_model(const void* blob_v, size_t bytes, double dx_override, HostM
     const int n_rows = (int)std::ceil(m->rc / m->dx - 1e-9);
     d.n_rows = n_rows;
     d.rc = (float)m->rc; d.dx = (float)m->dx; d.inv_dx = (float)(1.0 / m->dx);
-    d.inv_rc = 1.0f / d.rc; d.inv_rc_lo = (float)(1.0 / m->rc - (double)d.inv_rc); d.rc_lo = (float)((m->rc - (double)d.rc) / m->rc);
     const int CP = d.CP, NC = C0 + R;
     std::vector<double> Y((size_t)(n_rows + 1) * 2 * NC);  // [knot][deriv][channel]
     {

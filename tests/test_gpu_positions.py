@@ -105,7 +105,7 @@ def test_a_stale_list_is_reported_by_the_step_that_evaluates_it():
 # list radii past those whose quanta are fine enough, and a cell of many images: edge vectors as they are at a usual list radius
 @pytest.mark.parametrize("case,skin", [("open", 0.0), ("open", 9.9), ("open", 10.1), ("open", 100.0), ("open", 2500.0), ("periodic", 0.0),
                                        ("periodic", 9.9), ("periodic", 10.1), ("periodic", 100.0), ("images", 0.0), ("batch", 0.0)])
-def test_edge_vectors_do_not_lose_precision_with_the_list_radius(case, skin):
+def test_edge_vectors_do_not_lose_precision_with_the_list_radius(case, skin, kernel_envelope):
     p = SMALL_PROFILES["p16_2_0"]
     s = make_system(dict(kind="random_box", atoms=24, edges=(7.0, 8.0, 9.0), min_dist=1.6, seed=92, n_types=p["T"], masses=[1.0] * p["T"]))
     pos, types, cell, pbc = s["pos"], s["types"], np.diag(np.diag(np.asarray(s["cell"], dtype=np.float64))), (0, 0, 0)

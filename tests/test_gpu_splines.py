@@ -105,7 +105,7 @@ def _row_sums(blob, m, pos, cell, species, centers):
 # neighbours at few distances: the weights of successive edges fall on the same or on the next places of the row; odd counts
 @pytest.mark.parametrize("jitter", [0.004, 0.1])
 @pytest.mark.parametrize("name,spacing", [("p64_3_8", 1.6), ("p128_2_0", 1.9)])
-def test_row_sums_follow_the_definition(name, spacing, jitter):
+def test_row_sums_follow_the_definition(name, spacing, jitter, kernel_envelope):
     from paper_2608_19041_b200 import binding
     blob = make_blob(SMALL_PROFILES[name], seed=84, bias_scale=0.2, e_ref_scale=0.5)
     m = binding.Model(blob)
@@ -118,9 +118,6 @@ def test_row_sums_follow_the_definition(name, spacing, jitter):
     err = got - ref
     assert np.sqrt((err ** 2).mean()) <= 2.0 ** -22 * rms
     assert np.abs(err).max() <= 6 * 2.0 ** -22 * rms
-    # what is common to all sums: gamma, beta and U of the pair are rounded by up to 2^-25, at random over the dozen channels and
-    # more that carry them
-    assert abs((got * ref).sum() / (ref * ref).sum() - 1) <= 8e-9
 
 
 # whole systems, by splines and (tiles of fewer rows) by tables

@@ -129,3 +129,18 @@ def test_splines_at_the_ends_and_at_no_number():
     psi, dpsi = m.eval_edge_splines(1, [-1.0, 0.0, p["rc"], 2 * p["rc"], np.nan, -np.nan])
     assert np.array_equal(psi[0], psi[1]) and np.array_equal(psi[2], psi[3]) and np.isfinite(psi[:4]).all() and np.isfinite(dpsi[:4]).all()
     assert np.isnan(psi[4:]).all() and np.isnan(dpsi[4:]).all()
+
+
+@pytest.mark.parametrize("name", ["p64_3_8", "p128_2_0"])
+def test_splines_have_no_common_factor(name):
+    p = SMALL_PROFILES[name]
+    blob = make_blob(p, seed=84)
+    m, o = binding.Model(blob), orc.Oracle(blob)
+    rho = np.random.default_rng(2).uniform(1.0, p["rc"], 3000)
+    with torch.no_grad():
+        g, q = (x.numpy() for x in orc.radial_map(torch.from_numpy(rho), o.prm, o.p.get("basis", "bessel"), o.p["rc"]))
+    gamma, beta, U = (x[0, 0].numpy() for x in o.pair)
+    psi = gamma * g + beta + (q @ U.T if p["R"] else 0.0)
+    got = m.eval_edge_splines(0, rho)[0]
+    # gamma, beta and U of the pair are rounded by up to 2^-25, at random over the dozen channels and more that carry them
+    assert abs((got * psi).sum() / (psi * psi).sum() - 1) <= 8e-9
